@@ -23,8 +23,6 @@ constexpr uint32_t kFull       = 0xFFFFFFFFu;
 constexpr int      kMaxWindows = 5;                   // the grid never exceeds 32 * kMaxWindows CTAs
 constexpr int      kHdrSeq     = 0;                   // header words (64-bit): launch sequence number,
 constexpr int      kHdrAbort   = 1;                   //   abort word (== the launch's tag once a wait ran out)
-constexpr int      kCountShift = 40;                  // wave total word: (tiles added << 40) | sum of counts
-
 
 __device__ __forceinline__ uint64_t now_ns()
 {
@@ -120,206 +118,548 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     }
 }
 
-// shared-memory accesses by 32-bit shared address, kept in program order among themselves
-// register type that holds one element: 64 bits for 8-byte elements, 32 bits otherwise
+// ---------------------------------------------------------------------------------------------
+// A segment of a tile as one warp compacts it: kRows rows of 32 * kE elements, lane l owning the kE consecutive
+// elements l * kE .. of every row.  A lane keeps its elements in registers and four flag bits per row (bit j of nibble
+// r: element j of row r survives) in ONE 32-bit word; the ranks come from counts packed four rows to a register (bytes:
+// at most 128 survivors of a row), so that a warp scan of two registers ranks all eight rows at once.
+//
+// Four elements per lane and row keep the survivors of a row within 256 (2-byte) or 512 bytes, so that the predicated
+// stores of a row meet in few banks (eight 2-byte elements per lane were measured to lose there what they save).
 template <typename U>
-using Reg = std::conditional_t<sizeof(U) == 8, uint64_t, uint32_t>;
+struct Rows {
+    static constexpr int kE    = sizeof(U) == 8 ? 2 : 4;                 // consecutive elements of a lane in a row
+    static constexpr int kRows = 8;
+    static constexpr int kSeg  = kRows * 32 * kE;                        // 1024 elements (512 of 8 bytes)
+    static constexpr int kRegs = kE * static_cast<int>(sizeof(U)) / 4;   // registers of a lane per row: 2 or 4
+    uint32_t x[kRows][kRegs];
+};
 
 template <typename U>
-__device__ __forceinline__ Reg<U> lds_elem(uint32_t addr)
+__device__ __forceinline__ void load_rows(Rows<U> &s, const uint32_t seg_addr, const uint32_t lane)
 {
-    Reg<U> v;
-    if constexpr (sizeof(U) == 8) asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(addr));
-    else if constexpr (sizeof(U) == 4) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-    else asm volatile("ld.shared.s16 %0, [%1];" : "=r"(v) : "r"(addr));   // sign-extended
-    return v;
+    using R = Rows<U>;
+#pragma unroll
+    for (int r = 0; r < R::kRows; ++r) {
+        const uint32_t at = seg_addr + static_cast<uint32_t>(r) * (128u * R::kRegs) + lane * (4u * R::kRegs);
+        if constexpr (R::kRegs == 4)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(s.x[r][0]), "=r"(s.x[r][1]), "=r"(s.x[r][2]), "=r"(s.x[r][3]) : "r"(at));
+        else
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(s.x[r][0]), "=r"(s.x[r][1]) : "r"(at));
+    }
 }
 
-// ---------------------------------------------------------------------------------------------
-// One warp compacts its segment of kSteps * 32 elements in place.  Returns the number of packed
-// values; lane k leaves with the ballot of step k, which is bitmap word k of the segment, in `word`
-// (kept in registers through a tree of selects: a store to shared memory per step costs more).
-// `y` (fused form with dense output) points at the segment's first element of the dense ReLU
-// output, `yvalid` is how many of them exist.  seg_addr is a shared-window address.
-//
-// The loads of a batch of 8 steps are issued before the stores of the batch before it: a store of
-// step k lands below element 32(k+1) and a later batch reads at or above it, so they never meet.
-//
-// Which pipe an instruction runs on decides the speed of this loop: with 2-byte elements the kernel is bound by
-// the SM's integer/logic pipe (73 % busy, the top stall reason "math pipe throttle"), which the compare, the
-// mask of the ballot, the address arithmetic and the selects of a step all queue at.  So what can be a
-// multiply-add is one (those run on the FMA pipe): the ballot bits below the lane are b * 2^(32 - lane) instead
-// of b & lanemask_lt, addresses are rank * size + base with the size in a register the compiler cannot see
-// through, and lane k takes ballot k as a sum of ballots times 0/1 factors instead of through a tree of selects.
-// On the 392 MiB bf16 tensor: 0.1485 -> 0.139 ms plain, 0.165 -> 0.138 ms fused (with the compare below).
-template <typename U, int RELU_DT, bool WRITE_Y, bool kGuardY, int kSteps>
-__device__ __forceinline__ uint32_t compact_segment(const uint32_t seg_addr, uint32_t &word, const uint32_t lane,
-                                                    U *y, const uint32_t yvalid, const float tau, const Extent yx)
+// acc += bit where the element is not the zero pattern / is kept by the ReLU (greater than zero, or a NaN); the latter
+// also gives the ReLU's dense value.
+__device__ __forceinline__ void flag_nonzero(uint32_t &acc, const uint32_t x, const uint32_t bit)
 {
-    constexpr int      kBatch = 8;
-    static_assert(kSteps % kBatch == 0 && kSteps <= 32, "whole batches; one bitmap word per lane");
-    constexpr uint32_t kES    = sizeof(U);
-    const uint32_t     in0    = seg_addr + lane * kES;
-    uint32_t           out    = seg_addr;               // address of the next free packed slot
-    Reg<U>             v[kBatch], vn[kBatch];
-    const uint32_t     below  = lane ? (1u << (32u - lane)) : 0u;   // b * below: the ballot bits of the lanes below, at the top
-    uint32_t           size, pick[kBatch];              // element size; pick[j] = 1 on the lanes that keep ballot j of a batch
-    asm volatile("mov.u32 %0, %1;" : "=r"(size) : "n"(kES));
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p add.u32 %0, %0, %2;\n\t}" : "+r"(acc) : "r"(x), "r"(bit));
+}
+__device__ __forceinline__ uint32_t flag_relu(uint32_t &acc, const uint32_t x, const uint32_t bit)
+{
+    uint32_t y;
+    asm("{\n\t.reg .pred p;\n\tsetp.gtu.f32 p, %2, 0f00000000;\n\t@p add.u32 %0, %0, %3;\n\tselp.b32 %1, %2, 0, p;\n\t}"
+        : "+r"(acc), "=r"(y) : "f"(__uint_as_float(x)), "r"(bit));
+    return y;
+}
+
+// Two packed 2-byte elements compared in their own type: 0xFFFF in the half of an element that is kept by the ReLU
+// (greater than zero or a NaN) resp. saturated by the ReLU6 (at least 6), else 0.
+template <int DT>
+__device__ __forceinline__ uint32_t relu_keeps_pair(const uint32_t x)
+{
+    uint32_t m;
+    if constexpr (DT == BT_F16) asm("set.gtu.u32.f16x2 %0, %1, %2;" : "=r"(m) : "r"(x), "r"(0u));
+    else asm("set.gtu.u32.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(x), "r"(0u));
+    return m;
+}
+template <int DT>
+__device__ __forceinline__ uint32_t relu6_saturates_pair(const uint32_t x)
+{
+    uint32_t m;
+    if constexpr (DT == BT_F16) asm("set.ge.u32.f16x2 %0, %1, %2;" : "=r"(m) : "r"(x), "r"(0x46004600u));
+    else asm("set.ge.u32.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(x), "r"(0x40C040C0u));
+    return m;
+}
+
+// The flag word of the lane's elements; the fused forms replace the elements by their forward value on the way (the
+// forms decided by one compare leave elements that are not kept as they are: their flag is clear) and, with WRITE_Y,
+// store it (kGuardY: only the first yvalid elements of the segment exist).
+template <typename U, int FUSED, bool WRITE_Y, bool kGuardY>
+__device__ __forceinline__ uint32_t flag_rows(Rows<U> &s, const uint32_t lane, U *y, const uint32_t yvalid, const float tau,
+                                              const Extent yx)
+{
+    using R = Rows<U>;
+    constexpr bool kDirect = FUSED >= kFusedReluDirect;
+    uint32_t acc[4] = {0, 0, 0, 0};                       // byte b of the flag word: rows 2b and 2b + 1
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) asm volatile("mov.u32 %0, %1;" : "=r"(pick[j]) : "r"((lane & 7u) == static_cast<uint32_t>(j) ? 1u : 0u));
-    word = 0;
+    for (int r = 0; r < R::kRows; ++r) {
+        uint32_t yv[R::kRegs];
+        if constexpr (sizeof(U) == 2) {
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) v[j] = lds_elem<U>(in0 + j * 32 * kES);
+            for (int h = 0; h < R::kRegs; ++h) {
+                uint32_t &x = s.x[r][h];
+                const int i = 4 * (r & 1) + 2 * h;        // bit of the pair's first element within the byte
+                if constexpr (FUSED < 0) {
+                    // 1 per non-zero half, then both flags into place by one multiply-add of bytes
+                    acc[r >> 1] = __dp4a(__vminu2(x, 0x00010001u), (1u << i) | ((2u << i) << 16), acc[r >> 1]);
+                } else if constexpr (kDirect) {
+                    const uint32_t m = relu_keeps_pair<FUSED & 3>(x);
+                    if constexpr (FUSED >= kFusedRelu6Direct) {
+                        const uint32_t q = relu6_saturates_pair<FUSED & 3>(x);
+                        x                = (x & ~q) | (Elem<FUSED & 3>::kSix * 0x00010001u & q);
+                    }
+                    // bytes 0 and 2 of the mask are 0 or -1
+                    const uint32_t c = (static_cast<uint32_t>(-(1 << i)) & 0xFFu) | ((static_cast<uint32_t>(-(2 << i)) & 0xFFu) << 16);
+                    acc[r >> 1]      = static_cast<uint32_t>(__dp4a(static_cast<int>(m), static_cast<int>(c), static_cast<int>(acc[r >> 1])));
+                    yv[h]            = x & m;
+                } else {
+                    const uint32_t lo = fused_forward<FUSED>(x & 0xFFFFu, tau), hi = fused_forward<FUSED>(x >> 16, tau);
+                    flag_nonzero(acc[r >> 1], lo, 1u << i);
+                    flag_nonzero(acc[r >> 1], hi, 2u << i);
+                    x     = lo | (hi << 16);
+                    yv[h] = x;
+                }
+            }
+        } else {
 #pragma unroll
-    for (int kb = 0; kb < kSteps; kb += kBatch) {
-        if (kb + kBatch < kSteps) {
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) vn[j] = lds_elem<U>(in0 + (kb + kBatch + j) * 32 * kES);
+            for (int j = 0; j < R::kE; ++j) {
+                const uint32_t bit = 1u << (4 * (r & 1) + j);
+                if constexpr (sizeof(U) == 4) {
+                    uint32_t &x = s.x[r][j];
+                    if constexpr (kDirect) {
+                        yv[j] = flag_relu(acc[r >> 1], x, bit);
+                    } else {
+                        if constexpr (FUSED >= 0) x = fused_forward<FUSED>(x, tau);
+                        flag_nonzero(acc[r >> 1], x, bit);
+                        yv[j] = x;
+                    }
+                } else {
+                    uint64_t x = s.x[r][2 * j] | (static_cast<uint64_t>(s.x[r][2 * j + 1]) << 32);
+                    if constexpr (FUSED >= 0) {
+                        x                 = fused_forward<FUSED>(x, tau);
+                        s.x[r][2 * j]     = static_cast<uint32_t>(x);
+                        s.x[r][2 * j + 1] = static_cast<uint32_t>(x >> 32);
+                    }
+                    flag_nonzero(acc[r >> 1], static_cast<uint32_t>(x) | static_cast<uint32_t>(x >> 32), bit);
+                    yv[2 * j] = static_cast<uint32_t>(x), yv[2 * j + 1] = static_cast<uint32_t>(x >> 32);
+                }
+            }
         }
-        uint32_t w = 0;
-#pragma unroll
-        for (int j = 0; j < kBatch; ++j) {
-            Reg<U> x = v[j];
-            bool   nz;
-            if constexpr (RELU_DT >= kFusedReluHalf) {
-                nz = relu_keeps_half<RELU_DT & 3>(x);        // a kept element is never the zero pattern
-                if constexpr (RELU_DT >= kFusedRelu6Half) x = relu6_saturates_half<RELU_DT & 3>(x) ? Elem<RELU_DT & 3>::kSix : x;
-                if constexpr (WRITE_Y) {
-                    const uint32_t e = (kb + j) * 32 + lane;
-                    if ((!kGuardY || e < yvalid) && yx.holds(y + e, sizeof(U))) y[e] = nz ? static_cast<U>(x) : U(0);
+        if constexpr (WRITE_Y) {
+            const uint32_t e = static_cast<uint32_t>(r * 32 * R::kE) + lane * R::kE;       // the lane's first element of the row
+            if (!kGuardY || e + R::kE <= yvalid) {
+                if (yx.holds(y + e, R::kE * sizeof(U))) {
+                    if constexpr (R::kRegs == 4) *reinterpret_cast<uint4 *>(y + e) = make_uint4(yv[0], yv[1], yv[2], yv[3]);
+                    else *reinterpret_cast<uint2 *>(y + e) = make_uint2(yv[0], yv[1]);
                 }
             } else {
-                if constexpr (RELU_DT >= 0) {
-                    x = fused_forward<RELU_DT>(x, tau);
-                    if constexpr (WRITE_Y) {
-                        const uint32_t e = (kb + j) * 32 + lane;
-                        if ((!kGuardY || e < yvalid) && yx.holds(y + e, sizeof(U))) y[e] = static_cast<U>(x);
-                    }
-                }
-                nz = x != Reg<U>(0);
-            }
-            const uint32_t b = __ballot_sync(kFull, nz);
-            uint32_t       lower, at;
-            asm("mul.lo.u32 %0, %1, %2;" : "=r"(lower) : "r"(b), "r"(below));
-            asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(at) : "r"(__popc(lower)), "r"(size), "r"(out));
-            if (nz) {
-                if constexpr (kES == 8) asm volatile("st.shared.u64 [%0], %1;" ::"r"(at), "l"(x));
-                else if constexpr (kES == 4) asm volatile("st.shared.u32 [%0], %1;" ::"r"(at), "r"(x));
-                else asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"(static_cast<uint16_t>(x)));
-            }
-            asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(out) : "r"(__popc(b)), "r"(size));
-            asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(w) : "r"(b), "r"(pick[j]));
-        }
-        word = (lane >> 3) == static_cast<uint32_t>(kb / 8) ? w : word;     // lane kb + j keeps ballot j of this batch
 #pragma unroll
-        for (int j = 0; j < kBatch; ++j) v[j] = vn[j];
+                for (int j = 0; j < R::kE; ++j) {
+                    U v;
+                    if constexpr (sizeof(U) == 2) v = static_cast<U>(yv[j >> 1] >> (16 * (j & 1)));
+                    else if constexpr (sizeof(U) == 4) v = yv[j];
+                    else v = yv[2 * j] | (static_cast<uint64_t>(yv[2 * j + 1]) << 32);
+                    if (e + j < yvalid && yx.holds(y + e + j, sizeof(U))) y[e + j] = v;
+                }
+            }
+        }
     }
-    return (out - seg_addr) / kES;
+    return acc[0] | (acc[1] << 8) | (acc[2] << 16) | (acc[3] << 24);
 }
 
-// Down-cast on stash: a binary32 pattern narrowed to binary16 (CAST 1) or bfloat16 (CAST 2), round to nearest
-// even by the hardware conversion, every NaN to the one quiet NaN 0x7FFF.  CAST 0 passes the element through.
-template <int CAST, typename U>
-__device__ __forceinline__ auto narrowed(const U v)
+// Ranks: byte k of excl[i] is the number of survivors in the lanes below within row 2k + i, of total[i] the survivors
+// of that row.
+struct RowRanks {
+    uint32_t excl[2], total[2];
+    __device__ __forceinline__ uint32_t count() const { return __dp4a(total[0], 0x01010101u, __dp4a(total[1], 0x01010101u, 0u)); }
+};
+
+template <int kBy>
+__device__ __forceinline__ void scan_step(uint32_t &v)
 {
-    if constexpr (CAST == 0) {
-        return v;
-    } else {
-        static_assert(sizeof(U) == 4, "the narrowing forms take binary32 tensors");
-        const float f = __uint_as_float(v);
-        uint16_t    h;
-        if constexpr (CAST == 1) asm("cvt.rn.f16.f32 %0, %1;" : "=h"(h) : "f"(f));
-        else asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(h) : "f"(f));
-        return (v & 0x7FFFFFFFu) > 0x7F800000u ? static_cast<uint16_t>(0x7FFFu) : h;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tshfl.sync.up.b32 t|p, %0, %1, 0, 0xFFFFFFFF;\n\t@p add.u32 %0, %0, t;\n\t}" : "+r"(v) : "n"(kBy));
+}
+
+__device__ __forceinline__ void rank_rows(RowRanks &k, const uint32_t flags)
+{
+    // survivors per row: population counts of the nibbles, all eight at once
+    uint32_t c = flags - ((flags >> 1) & 0x55555555u);
+    c          = (c & 0x33333333u) + ((c >> 2) & 0x33333333u);
+    const uint32_t own0 = c & 0x0F0F0F0Fu, own1 = (c >> 4) & 0x0F0F0F0Fu;
+    uint32_t       v0 = own0, v1 = own1;
+    scan_step<1>(v0), scan_step<1>(v1);
+    scan_step<2>(v0), scan_step<2>(v1);
+    scan_step<4>(v0), scan_step<4>(v1);
+    scan_step<8>(v0), scan_step<8>(v1);
+    scan_step<16>(v0), scan_step<16>(v1);
+    k.total[0] = __shfl_sync(kFull, v0, 31), k.total[1] = __shfl_sync(kFull, v1, 31);
+    k.excl[0] = v0 - own0, k.excl[1] = v1 - own1;
+}
+
+// The segment's bitmap words.  A lane's nibbles are exchanged with three neighbours (four for 8-byte elements, whose
+// rows give a lane two bits) until it holds one whole word; `index` receives the word's place within the segment.
+// True if this lane has a word (all lanes; every other one for 8-byte elements).
+template <int kE>
+__device__ __forceinline__ bool segment_word(const uint32_t flags, const uint32_t lane, uint32_t &word, uint32_t &index)
+{
+    uint32_t a = flags, v = lane;                          // v: lane number among those that hold distinct bits
+    if constexpr (kE == 2) {
+        const uint32_t b = __shfl_xor_sync(kFull, a, 1);   // two lanes' pairs of bits make a nibble, on both lanes
+        a                = (lane & 1u) ? (b | (a << 2)) : (a | (b << 2));
+        v                = lane >> 1;
     }
+    constexpr int kX = kE == 2 ? 2 : 1;
+    // rows 0..3 to the even, rows 4..7 to the odd holder: the nibbles of the two, interleaved into four bytes
+    uint32_t b = __shfl_xor_sync(kFull, a, kX);
+    a          = __byte_perm(a, b, (v & 1u) ? 0x3726u : 0x5140u);
+    const uint32_t m = (a ^ (a >> 4)) & 0x00F000F0u;
+    a                = a ^ m ^ (m << 4);
+    b = __shfl_xor_sync(kFull, a, 2 * kX);                 // two rows each: 16 bits per row
+    a = __byte_perm(a, b, (v & 2u) ? 0x3726u : 0x5140u);
+    b = __shfl_xor_sync(kFull, a, 4 * kX);                 // one row each: 32 bits
+    a = __byte_perm(a, b, (v & 4u) ? 0x3276u : 0x5410u);
+    word               = a;
+    const uint32_t row = 4u * (v & 1u) + (v & 2u) + ((v >> 2) & 1u);
+    index              = row * static_cast<uint32_t>(kE) + (v >> 3);
+    return kE == 4 || (lane & 1u) == 0;
+}
+
+// The survivors to shared memory, packed from address `out` on.  kES: bytes of a stored value, kE: a lane's elements
+// per row; x[r] holds row r.
+template <int kES, int kE>
+__device__ __forceinline__ void place_rows(const uint32_t (&x)[8][kES * kE / 4], const uint32_t flags, const RowRanks &k, uint32_t out)
+{
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const uint32_t f  = static_cast<uint32_t>(kES) << (8 * (r >> 1));   // picks the row's byte and scales it
+        uint32_t       at = __dp4a(k.excl[r & 1], f, out);
+        out               = __dp4a(k.total[r & 1], f, out);
+#pragma unroll
+        for (int j = 0; j < kE; ++j) {
+            const uint32_t bit = 1u << (4 * r + j);
+            if constexpr (kES == 2)
+                asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %1, %2;\n\tsetp.ne.u32 p, t, 0;\n\t@p st.shared.u16 [%0], %3;\n\t@p add.u32 %0, %0, 2;\n\t}"
+                             : "+r"(at) : "r"(flags), "r"(bit), "h"(static_cast<uint16_t>(x[r][j >> 1] >> (16 * (j & 1)))) : "memory");
+            else if constexpr (kES == 4)
+                asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %1, %2;\n\tsetp.ne.u32 p, t, 0;\n\t@p st.shared.u32 [%0], %3;\n\t@p add.u32 %0, %0, 4;\n\t}"
+                             : "+r"(at) : "r"(flags), "r"(bit), "r"(x[r][j]) : "memory");
+            else
+                asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %1, %2;\n\tsetp.ne.u32 p, t, 0;\n\t@p st.shared.v2.u32 [%0], {%3, %4};\n\t@p add.u32 %0, %0, 8;\n\t}"
+                             : "+r"(at) : "r"(flags), "r"(bit), "r"(x[r][2 * j]), "r"(x[r][2 * j + 1]) : "memory");
+        }
+    }
+}
+
+// Down-cast on stash: two binary32 patterns narrowed to a packed pair of binary16 (CAST 1) or bfloat16 (CAST 2), round
+// to nearest even by the hardware conversion, every NaN to the one quiet NaN 0x7FFF (a NaN always narrows to a NaN and
+// nothing else does, so the packed result is what is asked).
+template <int CAST>
+__device__ __forceinline__ uint32_t narrowed_pair(const uint32_t lo, const uint32_t hi)
+{
+    uint32_t h, m;
+    if constexpr (CAST == 1) {
+        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
+        asm("set.nan.u32.f16x2 %0, %1, %1;" : "=r"(m) : "r"(h));
+    } else {
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
+        asm("set.nan.u32.bf16x2 %0, %1, %1;" : "=r"(m) : "r"(h));
+    }
+    return (h & ~m) | (0x7FFF7FFFu & m);
 }
 template <int CAST, typename U>
 using Stored = std::conditional_t<CAST == 0, U, uint16_t>;
 
-// One warp copies the `cnt` packed slots of its segment to out[0..cnt): contiguous, coalesced.
-template <typename U, int CAST, bool kGuard>
-__device__ __forceinline__ void copy_out_segment(const U *__restrict__ seg, const uint32_t lane, const uint32_t cnt,
-                                                 Stored<CAST, U> *__restrict__ out, const uint64_t room, const Extent vx)
+__device__ __forceinline__ uint4 lds_vec(const uint32_t addr)
 {
-    // (Pairing narrowed values into 4-byte stores was measured and is no faster: at half zeros the narrowing
-    // forms run at the speed of the compaction, not of the copy-out.)
-    uint32_t j = lane;
-    for (; j + 96 < cnt; j += 128) {
-        const auto v0 = narrowed<CAST>(seg[j]), v1 = narrowed<CAST>(seg[j + 32]), v2 = narrowed<CAST>(seg[j + 64]),
-                   v3 = narrowed<CAST>(seg[j + 96]);
-        if ((!kGuard || j < room) && vx.holds(out + j, sizeof(*out))) out[j] = v0;
-        if ((!kGuard || j + 32 < room) && vx.holds(out + j + 32, sizeof(*out))) out[j + 32] = v1;
-        if ((!kGuard || j + 64 < room) && vx.holds(out + j + 64, sizeof(*out))) out[j + 64] = v2;
-        if ((!kGuard || j + 96 < room) && vx.holds(out + j + 96, sizeof(*out))) out[j + 96] = v3;
-    }
-    for (; j < cnt; j += 32) {
-        const auto v = narrowed<CAST>(seg[j]);
-        if ((!kGuard || j < room) && vx.holds(out + j, sizeof(*out))) out[j] = v;
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+template <typename V>
+__device__ __forceinline__ V lds_value(const uint32_t addr)
+{
+    V v;
+    if constexpr (sizeof(V) == 8) asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(addr));
+    else if constexpr (sizeof(V) == 4) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    else asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+    return v;
+}
+
+// 16 bytes of a packed run kBytes (0 .. 14) behind a 16-byte boundary of shared memory.
+template <int kWords, bool kHalf>
+__device__ __forceinline__ uint4 lds_vec_shifted(const uint32_t addr)
+{
+    const uint4 a = lds_vec(addr);
+    if constexpr (kWords == 0 && !kHalf) {
+        return a;
+    } else {
+        const uint4    b    = lds_vec(addr + 16);
+        const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        if constexpr (kHalf)
+            return make_uint4(__byte_perm(w[kWords], w[kWords + 1], 0x5432), __byte_perm(w[kWords + 1], w[kWords + 2], 0x5432),
+                              __byte_perm(w[kWords + 2], w[kWords + 3], 0x5432), __byte_perm(w[kWords + 3], w[kWords + 4], 0x5432));
+        else return make_uint4(w[kWords], w[kWords + 1], w[kWords + 2], w[kWords + 3]);
     }
 }
 
-// The copy-out of a packed run of 2-byte values through the copy engine.  A lane-by-lane copy costs a shared load
-// and a 2-byte global store per survivor on the port the compactors' votes, counts and stores also queue at; a
-// bulk copy reads shared memory by itself.  It wants source and destination on 16-byte boundaries, and the
-// destination is wherever the run's rank puts it: so the up to 7 values in front of the destination's first
-// boundary and the up to 7 behind its last one leave as single elements, and the rest is first moved down inside
-// the segment by that many elements (two 16-byte loads, four funnel shifts, one 16-byte store per 8 values;
-// loads of a round before its stores, rounds in rising order, so nothing is overwritten before it is read).
-// The caller waits for the copy engine's reads (bulk_store_wait_read) before it releases the slot.
-constexpr bool kBulkCopyOut16 = true;
-
-__device__ __forceinline__ void bulk_store_wait_read()
+template <typename V, int kWords, bool kHalf>
+__device__ __forceinline__ void copy_vectors(const uint32_t from, const uint32_t lane, const uint32_t vecs, V *to, const Extent vx)
 {
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    constexpr uint32_t kPer = 16 / sizeof(V);
+#pragma unroll 2
+    for (uint32_t v = lane; v < vecs; v += 32) {
+        const uint4 d = lds_vec_shifted<kWords, kHalf>(from + 16u * v);
+        if (vx.holds(to + kPer * v, 16)) *reinterpret_cast<uint4 *>(to + kPer * v) = d;
+    }
 }
 
-__device__ __forceinline__ void copy_out_run16(uint16_t *seg, const uint32_t lane, const uint32_t cnt, uint16_t *out,
-                                               const Extent vx)
+// One warp copies the `cnt` packed values at the 16-byte aligned shared address `from` to out[0 .. cnt).  The
+// destination is wherever the run's rank puts it: the values in front of its first 16-byte boundary and behind its last
+// one leave as single elements, the rest as 16-byte vectors put together from two shared vectors (the shift is the same
+// for the whole warp).  Never reads past the last whole 16 bytes that the run touches.
+template <typename V>
+__device__ __forceinline__ void copy_out_run(const uint32_t from, const uint32_t lane, const uint32_t cnt, V *out, const Extent vx)
 {
-    const uint32_t sa = smem_addr(seg);
-    uint32_t       h  = (static_cast<uint32_t>(16u - (reinterpret_cast<uintptr_t>(out) & 15u)) & 15u) >> 1;
-    h                 = h < cnt ? h : cnt;                       // values in front of the first boundary
-    const uint32_t vecs = (cnt - h) >> 3;                        // whole 16-byte units behind them
-    const uint32_t tail = h + 8u * vecs;                         // first of the values behind the last unit
-    // the ragged ends: lanes 0..6 the head, lanes 8..14 the tail; read now, the move below overwrites the head
-    const bool     is_head = lane < h, is_tail = lane >= 8u && tail + (lane - 8u) < cnt;
-    const uint32_t ei      = is_head ? lane : tail + (lane - 8u);
-    uint16_t       edge    = 0;
-    if (is_head || is_tail) edge = seg[ei];
-    if (vecs) {
-        if (h) {
-            __syncwarp();
-            const uint32_t sh = (h & 1u) * 16u;
-            for (uint32_t v0 = 0; v0 < vecs; v0 += 32) {
-                const uint32_t v  = v0 + lane;
-                const uint32_t at = sa + 16u * v;
-                uint32_t       w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0, w6 = 0, w7 = 0;
-                if (v < vecs) {
-                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3) : "r"(at));
-                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w4), "=r"(w5), "=r"(w6), "=r"(w7) : "r"(at + 16u));
-                }
-                __syncwarp();
-                if (v < vecs) {
-                    uint32_t o0, o1, o2, o3;
-                    switch (h >> 1) {                              // the same for the whole warp
-                    case 0: o0 = __funnelshift_r(w0, w1, sh), o1 = __funnelshift_r(w1, w2, sh), o2 = __funnelshift_r(w2, w3, sh), o3 = __funnelshift_r(w3, w4, sh); break;
-                    case 1: o0 = __funnelshift_r(w1, w2, sh), o1 = __funnelshift_r(w2, w3, sh), o2 = __funnelshift_r(w3, w4, sh), o3 = __funnelshift_r(w4, w5, sh); break;
-                    case 2: o0 = __funnelshift_r(w2, w3, sh), o1 = __funnelshift_r(w3, w4, sh), o2 = __funnelshift_r(w4, w5, sh), o3 = __funnelshift_r(w5, w6, sh); break;
-                    default: o0 = __funnelshift_r(w3, w4, sh), o1 = __funnelshift_r(w4, w5, sh), o2 = __funnelshift_r(w5, w6, sh), o3 = __funnelshift_r(w6, w7, sh); break;
-                    }
-                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(o0), "r"(o1), "r"(o2), "r"(o3) : "memory");
-                }
-            }
-            fence_proxy_async();                                  // the moved values, before the copy engine reads them
+    constexpr uint32_t kPer = 16 / sizeof(V);
+    uint32_t           h    = (static_cast<uint32_t>(16u - (reinterpret_cast<uintptr_t>(out) & 15u)) & 15u) / static_cast<uint32_t>(sizeof(V));
+    h                       = h < cnt ? h : cnt;                 // values in front of the first boundary
+    const uint32_t vecs = (cnt - h) / kPer;                      // whole 16-byte units behind them
+    const uint32_t tail = h + kPer * vecs;                       // first of the values behind the last unit
+    const bool     is_head = lane < h, is_tail = lane >= 16u && tail + (lane - 16u) < cnt;
+    if (is_head || is_tail) {
+        const uint32_t e = is_head ? lane : tail + (lane - 16u);
+        const V        v = lds_value<V>(from + e * static_cast<uint32_t>(sizeof(V)));
+        if (vx.holds(out + e, sizeof(V))) out[e] = v;
+    }
+    V *const to = out + h;
+    if constexpr (sizeof(V) == 8) {
+        if (h == 0) copy_vectors<V, 0, false>(from, lane, vecs, to, vx);
+        else copy_vectors<V, 2, false>(from, lane, vecs, to, vx);
+    } else if constexpr (sizeof(V) == 4) {
+        switch (h) {
+        case 0: copy_vectors<V, 0, false>(from, lane, vecs, to, vx); break;
+        case 1: copy_vectors<V, 1, false>(from, lane, vecs, to, vx); break;
+        case 2: copy_vectors<V, 2, false>(from, lane, vecs, to, vx); break;
+        default: copy_vectors<V, 3, false>(from, lane, vecs, to, vx); break;
         }
+    } else {
+        switch (h) {
+        case 0: copy_vectors<V, 0, false>(from, lane, vecs, to, vx); break;
+        case 1: copy_vectors<V, 0, true>(from, lane, vecs, to, vx); break;
+        case 2: copy_vectors<V, 1, false>(from, lane, vecs, to, vx); break;
+        case 3: copy_vectors<V, 1, true>(from, lane, vecs, to, vx); break;
+        case 4: copy_vectors<V, 2, false>(from, lane, vecs, to, vx); break;
+        case 5: copy_vectors<V, 2, true>(from, lane, vecs, to, vx); break;
+        case 6: copy_vectors<V, 3, false>(from, lane, vecs, to, vx); break;
+        default: copy_vectors<V, 3, true>(from, lane, vecs, to, vx); break;
+        }
+    }
+}
+
+// The same where the values buffer ends inside the run: only the first `room` values leave.
+template <typename V>
+__device__ __forceinline__ void copy_out_clipped(const uint32_t from, const uint32_t lane, const uint32_t cnt, V *out, const uint64_t room,
+                                                 const Extent vx)
+{
+    for (uint32_t j = lane; j < cnt && j < room; j += 32) {
+        const V v = lds_value<V>(from + j * static_cast<uint32_t>(sizeof(V)));
+        if (vx.holds(out + j, sizeof(V))) out[j] = v;
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Shared memory of a CTA besides the ring of tiles and the worker warps' rings of packed values.  A tile goes round
+// through five mbarriers: its ring slot through `full` and `empty`, its place in the queue of the last kQueue tiles
+// through `counted`, `ready` and `done`.
+constexpr int kQueue = 8;   // tiles of a CTA between their count and the end of their copy-out
+template <int kSegs, int kStages>
+struct CtaState {
+    uint64_t full[kStages];           // the bulk copy of the tile has landed               (copy engine -> workers)
+    uint64_t empty[kStages];          // every segment of the tile is in registers          (workers -> load warp)
+    uint64_t counted[kQueue];         // every segment's count is posted                    (workers -> scan warps)
+    uint64_t ready[kQueue];           // base and offsets are in shared                     (scan warps -> workers)
+    uint64_t done[kQueue];            // every segment has been copied out                  (workers -> workers)
+    uint64_t base[kQueue];            // exclusive base of the tile
+    uint64_t dst[kQueue];             // batched arena form: byte offset of the tile's tensor in the arena
+    uint32_t job[kQueue];             // batched form: the tile's tensor
+    uint32_t agg[kQueue];             // packed count of the tile
+    uint32_t cnt[kQueue][kSegs];      // packed count of each segment
+    uint32_t off[kQueue][kSegs];      // exclusive offset of each segment in the tile
+    uint32_t at[kQueue][kSegs];       // where in its worker's ring a segment's values start
+    volatile uint64_t tag;            // this launch's tag once a scan warp has it, else 0
+    uint64_t          arena_c0;       // arena forms: the cursor as the launch found it
+    volatile uint32_t abort;
+    // by one thread; a fence and a CTA-wide barrier follow
+    __device__ __forceinline__ void init(const uint64_t *arena_cursor)
+    {
+        arena_c0 = arena_cursor ? *reinterpret_cast<const volatile uint64_t *>(arena_cursor) : 0;
+        abort    = 0;
+        tag      = 0;
+        for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], kSegs);
+        for (int q = 0; q < kQueue; ++q) mbar_init(&counted[q], kSegs), mbar_init(&ready[q], 1), mbar_init(&done[q], kSegs);
+        fence_proxy_async();
+    }
+};
+
+// One CTA per SM; the input ring and the workers' rings take nearly all of its shared memory.  Three slots of 32 KB keep
+// the loads going (measured with loads alone: 6.2 to 6.4 TB/s with 3 to 7 slots), since a slot is free again as soon as
+// its tile is in registers.
+template <size_t kElemBytes>
+struct Shape {
+    static constexpr int kSegs = 8, kWorkers = 24, kStages = 3, kRing = 5376;
+};
+template <>
+struct Shape<2> {
+    static constexpr int kSegs = 16, kWorkers = 21, kStages = 3, kRing = 6144;
+};
+
+// The tile a worker looks at, and where a tile's values go.
+struct TileIn {
+    uint64_t    n, first;       // elements of the tensor, first element of the tile
+    const void *src;
+    void       *y;
+    uint32_t   *bitmap;
+};
+struct TileOut {
+    void    *values;
+    uint64_t capacity;          // in values
+};
+
+// One worker warp of a CTA (worker w of kWorkers): takes the segments w, w + kWorkers, w + 2 kWorkers, ... of the CTA's
+// stream of tiles -- into registers, flags, ranks, count posted, packed into its own ring in shared memory -- and copies
+// each out once its base is known, a few tiles later.  False if a wait ran out.
+//
+// Every worker does everything, so that what one waits for (a shuffle, a shared load, a base) is filled by the others;
+// a warp's chain of dependent steps per segment is about 1500 cycles, as long as a tile takes at full bandwidth, and
+// eight warps in step with each tile (which the first version of this kernel had) left the SM waiting half the time.
+//
+// No worker waits for a base before it has posted the counts that the base needs: the scan makes tile t ready once the
+// tiles up to t + 2 are counted, and a worker that waits for tile t has posted its segments of the tiles up to t + 2.
+// (After placing a segment of tile `it` it copies out what is left of tiles up to it - 3; a lack of room in its ring can
+// only make it wait for segments at least 2 tiles back, because the ring holds the segments nearer than that: kNear.)
+template <typename U, int FUSED, bool WRITE_Y, int CAST, int kSegs, int kWorkers, int kStages, int kRing, typename Stream>
+__device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, const uint32_t ring, const uint32_t w, const uint32_t lane,
+                                     Stream &stream, const float tau, const uint64_t wait_ns)
+{
+    using V                  = Stored<CAST, U>;
+    constexpr int      kE    = Rows<U>::kE;
+    constexpr int      kSeg  = Rows<U>::kSeg;
+    constexpr int      kTile = kSegs * kSeg;
+    constexpr uint32_t kES   = sizeof(V);
+    constexpr int      kNear = (2 * kSegs - 1) / kWorkers;          // a worker's earlier segments that can be less than two tiles back
+    constexpr int      kMax  = kSeg * static_cast<int>(kES);        // a segment without zeros
+    static_assert(kNear <= 1 && kRing % 16 == 0 && kRing >= (kNear == 0 ? kMax : 3 * kMax - 16),
+                  "the near segments and one more always fit, wherever they lie");
+    static_assert(3 * kSegs <= kQueue * kSegs - kWorkers - kSegs, "the queue holds every tile not copied out");
+
+    uint32_t it = w / kSegs, seg = w % kSegs;                       // the segment in hand
+    uint32_t o_it = it, o_seg = seg, pending = 0, head = 0;         // the oldest not yet copied out; their number; the ring's next free byte
+    auto     next = [](uint32_t &i, uint32_t &s) {
+        i += kWorkers / kSegs, s += kWorkers % kSegs;
+        if (kWorkers % kSegs != 0 && s >= static_cast<uint32_t>(kSegs)) s -= kSegs, ++i;
+    };
+    auto copy_oldest = [&]() -> bool {
+        const uint32_t q = o_it % kQueue;
+        if (!mbar_wait(&sh.ready[q], (o_it / kQueue) & 1u, &sh.abort, wait_ns)) return false;
+        const TileOut  o   = stream.out(q);
+        const uint32_t cnt = sh.cnt[q][o_seg], from = ring + sh.at[q][o_seg];
+        const uint64_t dst = sh.base[q] + sh.off[q][o_seg];
+        V *const       to  = static_cast<V *>(o.values) + dst;
+        const Extent   vx  = extent_of(o.values, o.capacity * sizeof(V));
+        if (dst + cnt <= o.capacity) copy_out_run<V>(from, lane, cnt, to, vx);
+        else copy_out_clipped<V>(from, lane, cnt, to, dst < o.capacity ? o.capacity - dst : 0, vx);
         __syncwarp();
-        if (lane == 0 && vx.holds(out + h, 16u * vecs)) {
-            fence_proxy_async();                                  // the compactors' stores (ordered before this by the mbarriers)
-            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(out + h), "r"(sa), "r"(16u * vecs) : "memory");
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        if (lane == 0) mbar_arrive(&sh.done[q]);
+        next(o_it, o_seg);
+        --pending;
+        return true;
+    };
+
+    TileIn t;
+    for (; stream.seek(it, t); next(it, seg)) {
+        const uint32_t s    = it % kStages, q = it % kQueue;
+        U *const       tile = tiles + static_cast<size_t>(s) * kTile;
+        if (!mbar_wait(&sh.full[s], (it / kStages) & 1u, &sh.abort, wait_ns)) return false;
+        if (t.n - t.first < static_cast<uint64_t>(kTile)) {
+            // Ragged last tile: each warp completes its own segment -- what the 16-byte granular bulk copy left out,
+            // zeros behind the end of the tensor -- and meets no other warp over it.  (A barrier among the workers here
+            // would never open if one of them had left the kernel because its wait ran out.)
+            const U *const src     = static_cast<const U *>(t.src);
+            const uint32_t have    = static_cast<uint32_t>(t.n - t.first);
+            const uint32_t by_bulk = ((have * static_cast<uint32_t>(sizeof(U))) & ~15u) / sizeof(U);
+            const uint32_t seg0    = seg * kSeg;
+            for (uint32_t e = (by_bulk > seg0 ? by_bulk : seg0) + lane; e < seg0 + kSeg; e += 32)
+                tile[e] = (e < have) ? src[t.first + e] : U(0);
+            __syncwarp();
         }
+        // the segment into registers; the slot is free for the next tile once every segment is
+        Rows<U> rows;
+        load_rows<U>(rows, smem_addr(tile + seg * kSeg), lane);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.empty[s]);
+
+        const uint64_t e0 = t.first + seg * kSeg;                   // first element of the segment
+        uint32_t       flags;
+        if constexpr (WRITE_Y) {
+            U *const       y      = static_cast<U *>(t.y) + e0;
+            const Extent   yx     = extent_of(t.y, t.n * sizeof(U));
+            const uint32_t yvalid = e0 + kSeg <= t.n ? static_cast<uint32_t>(kSeg) : (e0 < t.n ? static_cast<uint32_t>(t.n - e0) : 0u);
+            if (yvalid == static_cast<uint32_t>(kSeg)) flags = flag_rows<U, FUSED, true, false>(rows, lane, y, yvalid, tau, yx);
+            else flags = flag_rows<U, FUSED, true, true>(rows, lane, y, yvalid, tau, yx);
+        } else {
+            flags = flag_rows<U, FUSED, false, false>(rows, lane, nullptr, 0, tau, extent_of(nullptr, 0));
+        }
+        RowRanks ranks;
+        rank_rows(ranks, flags);
+        const uint32_t run = ranks.count();
+        // the count first: the exchange of counts waits for nothing else
+        if (it >= static_cast<uint32_t>(kQueue) && !mbar_wait(&sh.done[q], ((it / kQueue) - 1) & 1u, &sh.abort, wait_ns)) return false;
+        if (lane == 0) {
+            sh.cnt[q][seg] = run;
+            mbar_arrive(&sh.counted[q]);
+        }
+        uint32_t word, index;
+        if (segment_word<kE>(flags, lane, word, index)) {
+            const uint64_t wd = e0 / 32 + index;
+            if (wd < ((t.n + 31) >> 5) && extent_of(t.bitmap, 4 * ((t.n + 31) >> 5)).holds(t.bitmap + wd, 4)) t.bitmap[wd] = word;
+        }
+        // room in the ring: the pending segments lie one behind the other from the oldest one to `head`, each in one
+        // piece, so the end of the ring may stay unused
+        const uint32_t need = run ? (run * kES + 15u) & ~15u : 16u;
+        uint32_t       at   = 0;
+        while (pending) {
+            const uint32_t tail = sh.at[o_it % kQueue][o_seg];
+            if (head > tail) {
+                at = head;
+                if (head + need <= static_cast<uint32_t>(kRing)) break;
+                at = 0;
+                if (need <= tail) break;
+            } else {
+                at = head;
+                if (head + need <= tail) break;
+            }
+            at = 0;
+            if (!copy_oldest()) return false;
+        }
+        head = at + need;
+        ++pending;
+        if constexpr (CAST != 0) {
+            uint32_t h[8][2];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) h[r][0] = narrowed_pair<CAST>(rows.x[r][0], rows.x[r][1]), h[r][1] = narrowed_pair<CAST>(rows.x[r][2], rows.x[r][3]);
+            place_rows<2, 4>(h, flags, ranks, ring + at);
+        } else {
+            place_rows<sizeof(U), kE>(rows.x, flags, ranks, ring + at);
+        }
+        if (lane == 0) sh.at[q][seg] = at;
+        __syncwarp();
+        while (pending && o_it + 3 <= it)
+            if (!copy_oldest()) return false;
     }
-    if ((is_head || is_tail) && vx.holds(out + ei, 2)) out[ei] = edge;
+    while (pending)
+        if (!copy_oldest()) return false;
+    return true;
 }
 
 // Launch shape of one kernel instantiation on one device: the opt-in shared

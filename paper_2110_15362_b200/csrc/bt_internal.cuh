@@ -14,9 +14,6 @@ namespace bt {
 // The workspace arrives with unspecified contents.  It holds
 //   a 256-byte header, 64-bit words: [0] seq, the launch sequence number of this workspace; [1] abort, equal to
 //     the launch's tag once a bounded wait of that launch ran out;
-//   one 64-bit total per wave of tiles of every tensor of the launch (an even number of words): sums made by
-//     reductions, zeroed by the launch itself before the grid's one meeting, used only by tensors of more than
-//     one wave;
 //   one 16-byte descriptor per tile, never cleared: word 0 = (tag >> 32) << 32 | count, word 1 = (tag & 0xFFFFFFFF)
 //     << 32 | count.  A reader takes a descriptor only if both halves carry its own launch's tag and agree on
 //     the count (the two halves may be written and read separately).
@@ -25,7 +22,7 @@ namespace bt {
 // the last tile adds 1 once all counts are in; a CTA that gives up adds 2^32), so replays of one captured launch
 // -- same call_tag -- get different tags too.  Memory this library never wrote matches by chance only: 2^-64
 // per word for the tag, and the repeated count on top.
-// Sized for the smallest tile: 24 bytes per 4096 elements.
+// Sized for the smallest tile, with 8 bytes per 4096 elements to spare: 24 bytes per 4096 elements.
 constexpr size_t   kWsHeaderBytes = 256;
 constexpr uint32_t kMinTileElems  = BT_CHUNK_ELEMS;
 constexpr uint32_t kMaxBatch      = 32;                        // tensors of one batched launch
@@ -44,8 +41,7 @@ struct CompressArgs {
     uint64_t   *nnz_out;
     int32_t    *dev_status;
     uint64_t   *ws_header;
-    uint64_t   *ws_desc;    // wave totals, then tile descriptors
-    uint32_t    ws_waves;   // number of wave-total words (even; set by launch_compress)
+    uint64_t   *ws_desc;    // tile descriptors
     uint64_t    call_tag;   // unique to the call (set by launch_compress)
     uint64_t    wait_ns;    // bound of every in-kernel wait (set by launch_compress)
     int         cast;       // 0, or the 16-bit type (BT_F16 / BT_BF16) the stashed values of a binary32 tensor are narrowed to
@@ -74,16 +70,13 @@ struct CompressJob {
     // set by launch_compress_batch:
     uint32_t    tiles;      // number of tiles of the tensor
     uint32_t    rot;        // the CTA that takes the tensor's tile 0 (tile t goes to CTA (rot + t) mod grid)
-    uint32_t    total0;     // index of the tensor's first wave-total word
     uint32_t    desc0;      // index of the tensor's first tile descriptor
 };
 
 // What the tensors of a batched launch share (all set by launch_compress_batch but tau).
 struct CompressCommon {
     uint64_t   *ws_header;
-    uint64_t   *ws_total;   // wave totals
     uint64_t   *ws_desc;    // tile descriptors
-    uint32_t    ws_totals;  // number of wave-total words (even)
     uint64_t    ws_words;   // 8-byte words of the workspace behind its header (what the size query promises)
     uint32_t    jobs;       // number of tensors
     uint64_t    call_tag;   // unique to the call
@@ -371,40 +364,12 @@ __device__ __forceinline__ uint32_t greater_or_nan(double v, double b)
 }
 
 // The fused forward forms are numbered by one template argument: -1 none (plain compressor), DT (0..3) keep
-// what exceeds the threshold (tau = 0: ReLU), 4 + DT ReLU6, and for the 2-byte types 8 + DT the ReLU and 12 + DT
-// the ReLU6 decided by compares in the element's own type.
-constexpr int kFusedRelu6     = 4;
-constexpr int kFusedReluHalf  = 8;
-constexpr int kFusedRelu6Half = 12;
-
-// ReLU and ReLU6 of a 2-byte element (x: its pattern, possibly sign-extended) without widening it, by binary16 /
-// bfloat16 compare instructions: kept iff x > 0 or x is a NaN -- exactly the elements for which x <= 0 is false
-// under IEEE comparison --, saturated iff x >= 6 (false for a NaN).  One instruction per decision instead of a
-// conversion, a float compare, a select and the zero test, and not on the integer pipe that the rest of the
-// compaction step loads (integer compares of the bit pattern, two per decision, measured slower than the float
-// form without the dense output; these are faster than both, with and without it).
-template <int DT>
-__device__ __forceinline__ bool relu_keeps_half(const uint32_t x)
-{
-    static_assert(DT == BT_F16 || DT == BT_BF16, "2-byte element types");
-    uint32_t r;
-    if constexpr (DT == BT_F16)
-        asm("{\n\t.reg .pred p;\n\t.reg .b16 h, z;\n\tcvt.u16.u32 h, %1;\n\tmov.b16 z, 0;\n\tsetp.gtu.f16 p, h, z;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"(x));
-    else
-        asm("{\n\t.reg .pred p;\n\t.reg .b16 h, z;\n\tcvt.u16.u32 h, %1;\n\tmov.b16 z, 0;\n\tsetp.gtu.bf16 p, h, z;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"(x));
-    return r != 0;
-}
-template <int DT>
-__device__ __forceinline__ bool relu6_saturates_half(const uint32_t x)
-{
-    static_assert(DT == BT_F16 || DT == BT_BF16, "2-byte element types");
-    uint32_t r;
-    if constexpr (DT == BT_F16)
-        asm("{\n\t.reg .pred p;\n\t.reg .b16 h, z;\n\tcvt.u16.u32 h, %1;\n\tmov.b16 z, 0x4600;\n\tsetp.ge.f16 p, h, z;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"(x));
-    else
-        asm("{\n\t.reg .pred p;\n\t.reg .b16 h, z;\n\tcvt.u16.u32 h, %1;\n\tmov.b16 z, 0x40C0;\n\tsetp.ge.bf16 p, h, z;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"(x));
-    return r != 0;
-}
+// what exceeds the threshold, 4 + DT ReLU6, and 8 + DT the ReLU (tau = 0; 2- and 4-byte types) and 12 + DT the ReLU6
+// (2-byte types) decided by compares in the element's own type: kept iff x > 0 or x is a NaN -- exactly the elements for
+// which x <= 0 is false under IEEE comparison, none of them the zero pattern --, saturated iff x >= 6 (false for a NaN).
+constexpr int kFusedRelu6       = 4;
+constexpr int kFusedReluDirect  = 8;
+constexpr int kFusedRelu6Direct = 12;
 
 // y = (x <= tau) ? +0 : x, and for ReLU6 additionally 6 where x >= 6; IEEE comparisons, so a NaN is kept.
 template <int FUSED, typename R>
