@@ -511,7 +511,7 @@ struct Shape {
 };
 template <>
 struct Shape<2> {
-    static constexpr int kSegs = 16, kWorkers = 21, kStages = 3, kRing = 6144;
+    static constexpr int kSegs = 16, kWorkers = 16, kStages = 3, kRing = 8064;
 };
 
 // The tile a worker looks at, and where a tile's values go.
@@ -552,6 +552,9 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
     static_assert(kNear <= 1 && kRing % 16 == 0 && kRing >= (kNear == 0 ? kMax : 3 * kMax - 16),
                   "the near segments and one more always fit, wherever they lie");
     static_assert(3 * kSegs <= kQueue * kSegs - kWorkers - kSegs, "the queue holds every tile not copied out");
+    // A wait on a barrier's parity tells two phases apart, not three: a worker that comes to a ring slot must have seen
+    // the slot's tile before.  (The copies of different slots may land in any order.)
+    static_assert((kStages * kSegs) % kWorkers == 0, "a worker visits a ring slot once per round, in its turn");
 
     uint32_t it = w / kSegs, seg = w % kSegs;                       // the segment in hand
     uint32_t o_it = it, o_seg = seg, pending = 0, head = 0;         // the oldest not yet copied out; their number; the ring's next free byte
