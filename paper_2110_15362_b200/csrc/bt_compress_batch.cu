@@ -485,7 +485,7 @@ cudaError_t launch_shaped(const CompressCommon &c, const CompressJob *jobs, uint
 template <typename U, int FUSED, bool WRITE_Y>
 cudaError_t launch_typed(const CompressCommon &c, const CompressJob *jobs, uint32_t count, void *workspace, cudaStream_t stream)
 {
-    using S = Shape<sizeof(U)>;   // as the single-tensor kernel
+    using S = Shape;   // as the single-tensor kernel
     return launch_shaped<U, FUSED, WRITE_Y, kMaxBatch, S::kSegs, S::kWorkers, S::kStages, S::kRing>(c, jobs, count, workspace, stream);
 }
 
