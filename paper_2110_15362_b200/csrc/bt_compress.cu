@@ -99,7 +99,9 @@ __global__ void __launch_bounds__((kWorkers + 3) * 32) compress_kernel(const Com
 
     // The arena's cursor is read before the barrier below: the kernel's one update of it follows the last tile's base,
     // which needs a publication from every CTA, and a CTA publishes only after this barrier.
-    if (tid == 0) sh.init(a.arena_cursor);
+    if (tid == 0) sh.init();
+    in_stream_order();
+    if (tid == 0) sh.arena_c0 = a.arena_cursor ? *reinterpret_cast<const volatile uint64_t *>(a.arena_cursor) : 0;
     __syncthreads();
 
     // bulk copy of tile `it` of this CTA into its ring slot (issued by lane 0 of the load warp)
@@ -353,10 +355,7 @@ cudaError_t launch_shaped(const CompressArgs &a, cudaStream_t stream)
     CompressArgs args = a;
     args.call_tag     = next_call_tag();
     args.wait_ns      = compress_wait_ns();
-    uint32_t     nt   = num_tiles;
-    void *params[] = {&args, &nt};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kernel), dim3(grid), dim3(kThreads), params, kSmem,
-                                       stream);
+    return launch_cooperative(kernel, grid, kThreads, kSmem, stream, args, num_tiles);
 }
 
 template <typename U, int FUSED, bool WRITE_Y, int CAST = 0>

@@ -157,7 +157,9 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
     // The arena's cursor is read before the barrier below: the launch's first update of it follows a tensor's last base,
     // which needs a publication from every CTA in front of it, and the sequence number moves only behind all of them.
     const bool in_arena = p.c.arena != nullptr;
-    if (tid == 0) sh.init(in_arena ? p.c.arena_cursor : nullptr);
+    if (tid == 0) sh.init();
+    in_stream_order();
+    if (tid == 0) sh.arena_c0 = in_arena ? *reinterpret_cast<const volatile uint64_t *>(p.c.arena_cursor) : 0;
     __syncthreads();
 
     const Extent wsx = extent_of(p.c.ws_desc, 8 * p.c.ws_words);
@@ -478,8 +480,7 @@ cudaError_t launch_shaped(const CompressCommon &c, const CompressJob *jobs, uint
     p.c.call_tag  = next_call_tag();
     p.c.wait_ns   = compress_wait_ns();
     // cooperative launch: the runtime guarantees that all `grid` CTAs are resident together
-    void *params[] = {&p};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kernel), dim3(grid), dim3(kThreads), params, kSmem, stream);
+    return launch_cooperative(kernel, grid, kThreads, kSmem, stream, p);
 }
 
 template <typename U, int FUSED, bool WRITE_Y>

@@ -496,12 +496,11 @@ struct CtaState {
     volatile uint64_t tag;            // this launch's tag once a scan warp has it, else 0
     uint64_t          arena_c0;       // arena forms: the cursor as the launch found it
     volatile uint32_t abort;
-    // by one thread; a fence and a CTA-wide barrier follow
-    __device__ __forceinline__ void init(const uint64_t *arena_cursor)
+    // by one thread; a CTA-wide barrier follows
+    __device__ __forceinline__ void init()
     {
-        arena_c0 = arena_cursor ? *reinterpret_cast<const volatile uint64_t *>(arena_cursor) : 0;
-        abort    = 0;
-        tag      = 0;
+        abort = 0;
+        tag   = 0;
         for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], kSegs);
         for (int q = 0; q < kQueue; ++q) mbar_init(&counted[q], kSegs), mbar_init(&ready[q], 1), mbar_init(&done[q], kSegs);
         fence_proxy_async();

@@ -217,6 +217,7 @@ decompress_kernel(const uint32_t *__restrict__ bitmap, const U *values,
                   const uint64_t *__restrict__ values_offset, const uint64_t *__restrict__ prefix, const uint64_t n,
                   U *__restrict__ out)
 {
+    in_stream_order();
     decompress_body<U, kE, kGrp, kWarps>(bitmap, values, values_offset, prefix, n, out, blockIdx.x);
 }
 
@@ -225,6 +226,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1536 / (kWarps * 32))
 decompress16_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *values, const uint64_t *__restrict__ values_offset,
                     const uint64_t *__restrict__ prefix, const uint64_t n, uint16_t *__restrict__ out)
 {
+    in_stream_order();
     decompress16_body<kWarps>(bitmap, values, values_offset, prefix, n, out, blockIdx.x);
 }
 
@@ -233,6 +235,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1536 / (kWarps * 32))
 decompress16_widen_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *values, const uint64_t *__restrict__ values_offset,
                           const uint64_t *__restrict__ prefix, const uint64_t n, uint32_t *__restrict__ out)
 {
+    in_stream_order();
     decompress16_body<kWarps, WIDEN>(bitmap, values, values_offset, prefix, n, out, blockIdx.x);
 }
 
@@ -251,6 +254,7 @@ template <typename U, int kE, int kGrp, int kWarps, int kJobs>
 __global__ void __launch_bounds__(kWarps * 32)
 decompress_batch_kernel(const __grid_constant__ RestoreParams<kJobs> p)
 {
+    in_stream_order();
     const RestoreJob &j = p.job[job_of_block(p)];
     decompress_body<U, kE, kGrp, kWarps>(j.bitmap, static_cast<const U *>(j.values), j.values_offset, j.prefix, j.n, static_cast<U *>(j.out),
                                             blockIdx.x - j.first_block);
@@ -260,6 +264,7 @@ template <int kWarps, int kJobs>
 __global__ void __launch_bounds__(kWarps * 32, 1536 / (kWarps * 32))
 decompress16_batch_kernel(const __grid_constant__ RestoreParams<kJobs> p)
 {
+    in_stream_order();
     const RestoreJob &j = p.job[job_of_block(p)];
     decompress16_body<kWarps>(j.bitmap, static_cast<const uint16_t *>(j.values), j.values_offset, j.prefix, j.n, static_cast<uint16_t *>(j.out),
                               blockIdx.x - j.first_block);
@@ -273,7 +278,7 @@ cudaError_t launch_typed(const uint32_t *bitmap, const void *values, const uint6
     const uint64_t quarters = (n + 1023) >> 10;
     const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    decompress_kernel<U, kE, kGrp, kWarps><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(
+    launch(decompress_kernel<U, kE, kGrp, kWarps>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
         bitmap, static_cast<const U *>(values), values_offset, prefix, n, static_cast<U *>(out));
     return cudaGetLastError();
 }
@@ -290,8 +295,8 @@ cudaError_t launch_decompress_widen(const uint32_t *bitmap, const void *values16
     const auto *v = static_cast<const uint16_t *>(values16);
     auto       *o = static_cast<uint32_t *>(out_f32);
     // the 2-byte decompressor (packed run staged in shared memory) with the widening in its store path
-    if (from_dtype == BT_F16) decompress16_widen_kernel<kWarps, 1><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(bitmap, v, values_offset, prefix, n, o);
-    else decompress16_widen_kernel<kWarps, 2><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(bitmap, v, values_offset, prefix, n, o);
+    if (from_dtype == BT_F16) launch(decompress16_widen_kernel<kWarps, 1>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, bitmap, v, values_offset, prefix, n, o);
+    else launch(decompress16_widen_kernel<kWarps, 2>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, bitmap, v, values_offset, prefix, n, o);
     return cudaGetLastError();
 }
 
@@ -304,7 +309,7 @@ cudaError_t launch_decompress(const uint32_t *bitmap, const void *values, const 
     const uint64_t quarters = (n + 1023) >> 10;
     const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    decompress16_kernel<kWarps><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(
+    launch(decompress16_kernel<kWarps>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
         bitmap, static_cast<const uint16_t *>(values), values_offset, prefix, n, static_cast<uint16_t *>(out));
     return cudaGetLastError();
 }
@@ -323,9 +328,9 @@ cudaError_t launch_decompress_batch(const DecompressJob *jobs, uint32_t count, i
     }
     p.jobs = count;
     const unsigned grid = static_cast<unsigned>(blocks);
-    if (elem_size == 8) decompress_batch_kernel<uint64_t, 2, 16, kWarps, kMaxBatch><<<grid, kWarps * 32, 0, stream>>>(p);
-    else if (elem_size == 4) decompress_batch_kernel<uint32_t, 4, 8, kWarps, kMaxBatch><<<grid, kWarps * 32, 0, stream>>>(p);
-    else decompress16_batch_kernel<kWarps, kMaxBatch><<<grid, kWarps * 32, 0, stream>>>(p);
+    if (elem_size == 8) launch(decompress_batch_kernel<uint64_t, 2, 16, kWarps, kMaxBatch>, grid, kWarps * 32, 0, stream, p);
+    else if (elem_size == 4) launch(decompress_batch_kernel<uint32_t, 4, 8, kWarps, kMaxBatch>, grid, kWarps * 32, 0, stream, p);
+    else launch(decompress16_batch_kernel<kWarps, kMaxBatch>, grid, kWarps * 32, 0, stream, p);
     return cudaGetLastError();
 }
 

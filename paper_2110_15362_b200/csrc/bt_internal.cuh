@@ -145,6 +145,40 @@ cudaError_t launch_maxpool2x2_bwd(const uint32_t *codes, const uint32_t *mask, c
 cudaError_t launch_relu_bwd(const uint32_t *bitmap, const void *gout, uint64_t n, int elem_size,
                             void *gin, cudaStream_t s);
 
+// ---------------------------------------------------------------- launches
+// Every kernel of the library is launched with programmatic stream serialisation: the launch need not wait until the
+// kernel before it in the stream is complete, and the kernel begins with in_stream_order(), which returns once that one
+// is complete and its writes are visible.  So the launch itself (parameters, CTA set-up, 1 to 2 us between two kernels of
+// a stream) overlaps the tail of the kernel before.  No kernel gives the next one leave to start early
+// (cudaTriggerProgrammaticLaunchCompletion): the launch begins when the last CTAs exit.  With leave given at the start
+// the next kernel's CTAs take SM slots from the streaming kernels' own: four calls on fp32 2^28 elements 1093 -> 1164 us,
+// against 1090 this way; three calls on fp16 [64,512,28,28] 66.0 -> 61.5 us this way.
+template <typename... P, typename... A>
+inline cudaError_t launch_as(bool cooperative, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)
+{
+    cudaLaunchAttribute attr[2];
+    attr[0].id                                         = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id                                         = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative                            = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid), c.blockDim = dim3(threads), c.dynamicSmemBytes = smem, c.stream = stream;
+    c.attrs = attr, c.numAttrs = cooperative ? 2 : 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)
+{
+    return launch_as(false, kernel, grid, threads, smem, stream, static_cast<A &&>(args)...);
+}
+// all CTAs resident together, or an error
+template <typename... P, typename... A>
+inline cudaError_t launch_cooperative(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)
+{
+    return launch_as(true, kernel, grid, threads, smem, stream, static_cast<A &&>(args)...);
+}
+__device__ __forceinline__ void in_stream_order() { cudaGridDependencySynchronize(); }
+
 // ---------------------------------------------------------------- PTX wrappers
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
 {

@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 mask_gather_kernel(const U *x, const uint32_t *__restrict__ bitmap, const uint64_t *__restrict__ prefix,
                    const uint64_t n, U *y, U *__restrict__ values, const uint64_t capacity)   // y may alias x
 {
+    in_stream_order();
     constexpr int kVec          = 16 / sizeof(U);          // elements per 16-byte vector
     constexpr int kLanesPerWord = 32 / kE;
     constexpr int kWordsPerStep = kE;
@@ -234,10 +235,10 @@ cudaError_t launch_typed(const void *x, const uint32_t *bitmap, const uint64_t *
     const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     if (y)
-        mask_gather_kernel<U, kE, kWarps, true><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(
+        launch(mask_gather_kernel<U, kE, kWarps, true>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
             static_cast<const U *>(x), bitmap, prefix, n, static_cast<U *>(y), static_cast<U *>(values), capacity);
     else
-        mask_gather_kernel<U, kE, kWarps, false><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(
+        launch(mask_gather_kernel<U, kE, kWarps, false>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
             static_cast<const U *>(x), bitmap, prefix, n, nullptr, static_cast<U *>(values), capacity);
     return cudaGetLastError();
 }

@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(kThreads)
 maxpool2x2_fwd_kernel(const U *__restrict__ x, const uint64_t outputs, const I wo, const I width, U *__restrict__ y,
                       uint32_t *__restrict__ codes)
 {
+    in_stream_order();
     using P             = Pair<U>;
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t o64  = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x;
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(kThreads)
 maxpool2x2_bwd_kernel(const uint32_t *__restrict__ codes, const uint32_t *__restrict__ mask, const U *__restrict__ gout,
                       const uint64_t outputs, const I wo, const I width, U *__restrict__ gin)
 {
+    in_stream_order();
     // mask (may be NULL): bitmap over the outputs; the gradient of an output whose bit is clear counts as +0
     using P            = Pair<U>;
     const uint64_t o64 = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x;
@@ -132,6 +134,7 @@ __global__ void __launch_bounds__(kThreads)
 maxpool2x2_fwd_vec_kernel(const U *__restrict__ x, const uint64_t groups, const I groups_per_row, const I width,
                           U *__restrict__ y, uint32_t *__restrict__ codes)
 {
+    in_stream_order();
     constexpr int      kOut          = 8 / sizeof(U);          // outputs per thread
     constexpr uint32_t kLanesPerWord = 16 / kOut;
     const uint32_t     lane          = threadIdx.x & 31u;
@@ -182,6 +185,7 @@ __global__ void __launch_bounds__(kThreads)
 maxpool2x2_bwd_vec_kernel(const uint32_t *__restrict__ codes, const uint32_t *__restrict__ mask, const U *__restrict__ gout,
                           const uint64_t groups, const I groups_per_row, const I width, U *__restrict__ gin)
 {
+    in_stream_order();
     constexpr int  kOut = 8 / sizeof(U);
     const uint64_t g64  = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x;
     if (g64 >= groups) return;
@@ -224,11 +228,11 @@ cudaError_t fwd_typed(const void *x, uint64_t outputs, uint64_t wo, uint64_t wid
             const uint64_t groups = outputs / kOut, per_row = wo / kOut, vgrid = (groups + kThreads - 1) / kThreads;
             if (vgrid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
             if (elements <= 0xFFFFFFFFull)
-                maxpool2x2_fwd_vec_kernel<U, DT, uint32_t><<<static_cast<unsigned>(vgrid), kThreads, 0, s>>>(
+                launch(maxpool2x2_fwd_vec_kernel<U, DT, uint32_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
                     static_cast<const U *>(x), groups, static_cast<uint32_t>(per_row), static_cast<uint32_t>(width),
                     static_cast<U *>(y), codes);
             else
-                maxpool2x2_fwd_vec_kernel<U, DT, uint64_t><<<static_cast<unsigned>(vgrid), kThreads, 0, s>>>(
+                launch(maxpool2x2_fwd_vec_kernel<U, DT, uint64_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
                     static_cast<const U *>(x), groups, per_row, width, static_cast<U *>(y), codes);
             return cudaGetLastError();
         }
@@ -236,10 +240,10 @@ cudaError_t fwd_typed(const void *x, uint64_t outputs, uint64_t wo, uint64_t wid
     const uint64_t grid = (outputs + kThreads - 1) / kThreads;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     if (elements <= 0xFFFFFFFFull)
-        maxpool2x2_fwd_kernel<U, DT, uint32_t><<<static_cast<unsigned>(grid), kThreads, 0, s>>>(
+        launch(maxpool2x2_fwd_kernel<U, DT, uint32_t>, static_cast<unsigned>(grid), kThreads, 0, s, 
             static_cast<const U *>(x), outputs, static_cast<uint32_t>(wo), static_cast<uint32_t>(width), static_cast<U *>(y), codes);
     else
-        maxpool2x2_fwd_kernel<U, DT, uint64_t><<<static_cast<unsigned>(grid), kThreads, 0, s>>>(
+        launch(maxpool2x2_fwd_kernel<U, DT, uint64_t>, static_cast<unsigned>(grid), kThreads, 0, s, 
             static_cast<const U *>(x), outputs, wo, width, static_cast<U *>(y), codes);
     return cudaGetLastError();
 }
@@ -254,11 +258,11 @@ cudaError_t bwd_typed(const uint32_t *codes, const uint32_t *mask, const void *g
             const uint64_t groups = outputs / kOut, per_row = wo / kOut, vgrid = (groups + kThreads - 1) / kThreads;
             if (vgrid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
             if (elements <= 0xFFFFFFFFull)
-                maxpool2x2_bwd_vec_kernel<U, uint32_t><<<static_cast<unsigned>(vgrid), kThreads, 0, s>>>(
+                launch(maxpool2x2_bwd_vec_kernel<U, uint32_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
                     codes, mask, static_cast<const U *>(gout), groups, static_cast<uint32_t>(per_row),
                     static_cast<uint32_t>(width), static_cast<U *>(gin));
             else
-                maxpool2x2_bwd_vec_kernel<U, uint64_t><<<static_cast<unsigned>(vgrid), kThreads, 0, s>>>(
+                launch(maxpool2x2_bwd_vec_kernel<U, uint64_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
                     codes, mask, static_cast<const U *>(gout), groups, per_row, width, static_cast<U *>(gin));
             return cudaGetLastError();
         }
@@ -266,11 +270,11 @@ cudaError_t bwd_typed(const uint32_t *codes, const uint32_t *mask, const void *g
     const uint64_t grid = (outputs + kThreads - 1) / kThreads;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     if (elements <= 0xFFFFFFFFull)
-        maxpool2x2_bwd_kernel<U, uint32_t><<<static_cast<unsigned>(grid), kThreads, 0, s>>>(
+        launch(maxpool2x2_bwd_kernel<U, uint32_t>, static_cast<unsigned>(grid), kThreads, 0, s, 
             codes, mask, static_cast<const U *>(gout), outputs, static_cast<uint32_t>(wo), static_cast<uint32_t>(width),
             static_cast<U *>(gin));
     else
-        maxpool2x2_bwd_kernel<U, uint64_t><<<static_cast<unsigned>(grid), kThreads, 0, s>>>(
+        launch(maxpool2x2_bwd_kernel<U, uint64_t>, static_cast<unsigned>(grid), kThreads, 0, s, 
             codes, mask, static_cast<const U *>(gout), outputs, wo, width, static_cast<U *>(gin));
     return cudaGetLastError();
 }

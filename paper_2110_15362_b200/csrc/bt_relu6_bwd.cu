@@ -26,6 +26,7 @@ relu6_bwd_kernel(const uint32_t *__restrict__ bitmap, const U *__restrict__ valu
                  const uint64_t *__restrict__ values_offset, const uint64_t *__restrict__ prefix, const U *gout,
                  const uint64_t n, U *gin)   // gin may alias gout
 {
+    in_stream_order();
     // arena form: the packed values start *values_offset bytes into `values`
     if (values_offset) values = reinterpret_cast<const U *>(reinterpret_cast<const unsigned char *>(values) + *values_offset);
     constexpr int kVec          = 16 / sizeof(U);
@@ -169,6 +170,7 @@ relu6_bwd16_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *__restri
                    const uint64_t *__restrict__ values_offset, const uint64_t *__restrict__ prefix, const uint16_t *gout,
                    const uint64_t n, uint16_t *gin)   // gin may alias gout
 {
+    in_stream_order();
     const uint32_t lane        = threadIdx.x & 31u;
     const uint64_t warp_global = static_cast<uint64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
     if (warp_global >= ((n + 1023) >> 10)) return;
@@ -217,7 +219,7 @@ cudaError_t launch_16(const uint32_t *bitmap, const void *values, const uint64_t
     const uint64_t quarters = (n + 1023) >> 10;
     const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    relu6_bwd16_kernel<DT, kWarps><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(
+    launch(relu6_bwd16_kernel<DT, kWarps>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
         bitmap, static_cast<const uint16_t *>(values), values_offset, prefix, static_cast<const uint16_t *>(gout), n,
         static_cast<uint16_t *>(gin));
     return cudaGetLastError();
@@ -231,7 +233,7 @@ cudaError_t launch_typed(const uint32_t *bitmap, const void *values, const uint6
     const uint64_t quarters = (n + 1023) >> 10;
     const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    relu6_bwd_kernel<U, DT, kE, kBlk, kWarps><<<static_cast<unsigned>(grid), kWarps * 32, 0, stream>>>(
+    launch(relu6_bwd_kernel<U, DT, kE, kBlk, kWarps>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
         bitmap, static_cast<const U *>(values), values_offset, prefix, static_cast<const U *>(gout), n, static_cast<U *>(gin));
     return cudaGetLastError();
 }

@@ -88,6 +88,7 @@ template <typename U>
 __global__ void __launch_bounds__(kThreads)
 relu_bwd_kernel(const uint32_t *__restrict__ bitmap, const U *gout, const uint64_t n, U *gin)
 {
+    in_stream_order();
     relu_bwd_body<U>(bitmap, gout, n, gin, blockIdx.x);
 }
 
@@ -110,6 +111,7 @@ template <typename U, int kJobs>
 __global__ void __launch_bounds__(kThreads)
 relu_bwd_batch_kernel(const __grid_constant__ MaskParams<kJobs> p)
 {
+    in_stream_order();
     uint32_t k = 0;
     for (uint32_t j = 1; j < p.jobs; ++j) k = p.job[j].first_block <= blockIdx.x ? j : k;
     const MaskJob &j = p.job[k];
@@ -124,7 +126,7 @@ cudaError_t launch_typed(const uint32_t *bitmap, const void *gout, uint64_t n, v
     uint64_t       grid = (vecs + kThreads * kUnroll - 1) / (kThreads * kUnroll);
     if (grid == 0) grid = 1;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    relu_bwd_kernel<U><<<static_cast<unsigned>(grid), kThreads, 0, stream>>>(bitmap, static_cast<const U *>(gout), n,
+    launch(relu_bwd_kernel<U>, static_cast<unsigned>(grid), kThreads, 0, stream, bitmap, static_cast<const U *>(gout), n,
                                                                              static_cast<U *>(gin));
     return cudaGetLastError();
 }
@@ -154,9 +156,9 @@ cudaError_t launch_relu_bwd_batch(const DecompressJob *jobs, uint32_t count, int
     }
     p.jobs = count;
     const unsigned grid = static_cast<unsigned>(blocks);
-    if (elem_size == 8) relu_bwd_batch_kernel<uint64_t, kMaxBatch><<<grid, kThreads, 0, stream>>>(p);
-    else if (elem_size == 4) relu_bwd_batch_kernel<uint32_t, kMaxBatch><<<grid, kThreads, 0, stream>>>(p);
-    else relu_bwd_batch_kernel<uint16_t, kMaxBatch><<<grid, kThreads, 0, stream>>>(p);
+    if (elem_size == 8) launch(relu_bwd_batch_kernel<uint64_t, kMaxBatch>, grid, kThreads, 0, stream, p);
+    else if (elem_size == 4) launch(relu_bwd_batch_kernel<uint32_t, kMaxBatch>, grid, kThreads, 0, stream, p);
+    else launch(relu_bwd_batch_kernel<uint16_t, kMaxBatch>, grid, kThreads, 0, stream, p);
     return cudaGetLastError();
 }
 
