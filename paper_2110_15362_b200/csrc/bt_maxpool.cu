@@ -120,18 +120,57 @@ __device__ __forceinline__ void unpack16(const uint4 v, U (&e)[16 / sizeof(U)])
         e[4] = static_cast<U>(v.z), e[5] = static_cast<U>(v.z >> 16), e[6] = static_cast<U>(v.w), e[7] = static_cast<U>(v.w >> 16);
     }
 }
-template <typename U>
-__device__ __forceinline__ uint4 pack16(const U (&e)[16 / sizeof(U)])
+// Two windows of 2-byte elements at once: A, B, C, D hold the two windows' elements (0,0), (0,1), (1,0), (1,1), one
+// window per half.  The comparison rule on packed pairs in the element's own type (an exact widening changes no
+// comparison); `code` receives the winner's position per half.
+template <int DT>
+__device__ __forceinline__ uint32_t later_wins(const uint32_t v, const uint32_t best)
 {
-    if constexpr (sizeof(U) == 4) return make_uint4(e[0], e[1], e[2], e[3]);
-    else
-        return make_uint4(e[0] | (uint32_t(e[1]) << 16), e[2] | (uint32_t(e[3]) << 16), e[4] | (uint32_t(e[5]) << 16),
-                          e[6] | (uint32_t(e[7]) << 16));
+    uint32_t gt, nan;
+    if constexpr (DT == BT_F16) {
+        asm("set.gt.u32.f16x2 %0, %1, %2;" : "=r"(gt) : "r"(v), "r"(best));
+        asm("set.nan.u32.f16x2 %0, %1, %1;" : "=r"(nan) : "r"(v));
+    } else {
+        asm("set.gt.u32.bf16x2 %0, %1, %2;" : "=r"(gt) : "r"(v), "r"(best));
+        asm("set.nan.u32.bf16x2 %0, %1, %1;" : "=r"(nan) : "r"(v));
+    }
+    return gt | nan;                                        // 0xFFFF in the half of a window where v replaces the maximum
+}
+template <int DT>
+__device__ __forceinline__ uint32_t pool_pair(const uint32_t a, const uint32_t b, const uint32_t c, const uint32_t d, uint32_t &code)
+{
+    uint32_t m = later_wins<DT>(b, a), best = (b & m) | (a & ~m);
+    code       = 0x00010001u & m;
+    m          = later_wins<DT>(c, best), best = (c & m) | (best & ~m);
+    code       = (0x00020002u & m) | (code & ~m);
+    m          = later_wins<DT>(d, best), best = (d & m) | (best & ~m);
+    code       = (0x00030003u & m) | (code & ~m);
+    return best;
 }
 
-template <typename U, int DT, typename I>
+// g / d for g < 2^31 by one multiplication (d >= 1): floor(g (2^32 + m) / 2^(32 + s)) with s = ceil(log2 d) and
+// m = floor(2^32 (2^s - d) / d) + 1 is exact (Granlund and Montgomery, Division by invariant integers).
+struct DivBy {
+    uint32_t m, s;
+    static DivBy of(const uint32_t d)
+    {
+        uint32_t s = 0;
+        while ((1ull << s) < d) ++s;
+        return DivBy{static_cast<uint32_t>((((1ull << s) - d) << 32) / d + 1), s};
+    }
+    __device__ __forceinline__ uint32_t operator()(const uint32_t g) const { return (__umulhi(g, m) + g) >> s; }
+};
+// rows of more than 2^31 groups in all: the plain division
+struct DivWide {
+    uint64_t d;
+    __device__ __forceinline__ uint64_t operator()(const uint64_t g) const { return g / d; }
+};
+
+// A thread's group starts at element 2 * kOut * g + row * width of the input: the rows of outputs in front of it cover
+// two input rows each, and a row of groups covers one.
+template <typename U, int DT, typename I, typename Div>
 __global__ void __launch_bounds__(kThreads)
-maxpool2x2_fwd_vec_kernel(const U *__restrict__ x, const uint64_t groups, const I groups_per_row, const I width,
+maxpool2x2_fwd_vec_kernel(const U *__restrict__ x, const uint64_t groups, const Div row_of, const I width,
                           U *__restrict__ y, uint32_t *__restrict__ codes)
 {
     in_stream_order();
@@ -142,33 +181,40 @@ maxpool2x2_fwd_vec_kernel(const U *__restrict__ x, const uint64_t groups, const 
     const bool         live          = g64 < groups;
     uint32_t           bits          = 0;
     if (live) {
-        const I        g   = static_cast<I>(g64);
-        const I        row = g / groups_per_row;
-        const I        cg  = g - row * groups_per_row;
-        const uint64_t at  = 2ull * row * width + 2ull * kOut * cg;
-        U              top[2 * kOut], bot[2 * kOut], win[kOut];
-        unpack16<U>(*reinterpret_cast<const uint4 *>(x + at), top);
-        unpack16<U>(*reinterpret_cast<const uint4 *>(x + at + width), bot);
+        const I        row = row_of(static_cast<I>(g64));
+        const uint64_t at  = 2ull * kOut * g64 + static_cast<uint64_t>(row) * width;
+        const uint4    top = *reinterpret_cast<const uint4 *>(x + at), bot = *reinterpret_cast<const uint4 *>(x + at + width);
+        uint2          pack;
+        if constexpr (sizeof(U) == 2) {
+            uint32_t c0, c1;
+            pack.x = pool_pair<DT>(__byte_perm(top.x, top.y, 0x5410), __byte_perm(top.x, top.y, 0x7632), __byte_perm(bot.x, bot.y, 0x5410),
+                                   __byte_perm(bot.x, bot.y, 0x7632), c0);
+            pack.y = pool_pair<DT>(__byte_perm(top.z, top.w, 0x5410), __byte_perm(top.z, top.w, 0x7632), __byte_perm(bot.z, bot.w, 0x5410),
+                                   __byte_perm(bot.z, bot.w, 0x7632), c1);
+            bits = __dp4a(c0, 0x00040001u, __dp4a(c1, 0x00400010u, 0u));
+        } else {
+            U t[2 * kOut], b[2 * kOut], win[kOut];
+            unpack16<U>(top, t);
+            unpack16<U>(bot, b);
 #pragma unroll
-        for (int j = 0; j < kOut; ++j) {
-            const U  e[4]  = {top[2 * j], top[2 * j + 1], bot[2 * j], bot[2 * j + 1]};
-            U        best  = e[0];
-            auto     bestv = Elem<DT>::widen(e[0]);
-            uint32_t code  = 0;
+            for (int j = 0; j < kOut; ++j) {
+                const U  e[4]  = {t[2 * j], t[2 * j + 1], b[2 * j], b[2 * j + 1]};
+                U        best  = e[0];
+                auto     bestv = Elem<DT>::widen(e[0]);
+                uint32_t code  = 0;
 #pragma unroll
-            for (uint32_t k = 1; k < 4; ++k) {
-                const auto v    = Elem<DT>::widen(e[k]);
-                const bool take = greater_or_nan(v, bestv) != 0;
-                best            = take ? e[k] : best;
-                bestv           = take ? v : bestv;
-                code            = take ? k : code;
+                for (uint32_t k = 1; k < 4; ++k) {
+                    const auto v    = Elem<DT>::widen(e[k]);
+                    const bool take = greater_or_nan(v, bestv) != 0;
+                    best            = take ? e[k] : best;
+                    bestv           = take ? v : bestv;
+                    code            = take ? k : code;
+                }
+                win[j] = best;
+                bits |= code << (2 * j);
             }
-            win[j] = best;
-            bits |= code << (2 * j);
+            pack = make_uint2(win[0], win[1]);
         }
-        uint2 pack;
-        if constexpr (sizeof(U) == 4) pack = make_uint2(win[0], win[1]);
-        else pack = make_uint2(win[0] | (uint32_t(win[1]) << 16), win[2] | (uint32_t(win[3]) << 16));
         if (extent_of(y, groups * kOut * sizeof(U)).holds(y + g64 * kOut, 8)) *reinterpret_cast<uint2 *>(y + g64 * kOut) = pack;
     }
     if (codes) {
@@ -180,42 +226,60 @@ maxpool2x2_fwd_vec_kernel(const U *__restrict__ x, const uint64_t groups, const 
     }
 }
 
-template <typename U, typename I>
+// 0xFFFF or 0xFFFF0000 where the 2-bit code in bits 4 and 5 of s (all others clear) names that element of a pair of
+// codes 0 and 1, else 0: shifts past the register give 0.
+__device__ __forceinline__ uint32_t pair_mask(const uint32_t s)
+{
+    uint32_t m;
+    asm("shl.b32 %0, %1, %2;" : "=r"(m) : "r"(0x0000FFFFu), "r"(s));
+    return m;
+}
+
+template <typename U, typename I, typename Div>
 __global__ void __launch_bounds__(kThreads)
 maxpool2x2_bwd_vec_kernel(const uint32_t *__restrict__ codes, const uint32_t *__restrict__ mask, const U *__restrict__ gout,
-                          const uint64_t groups, const I groups_per_row, const I width, U *__restrict__ gin)
+                          const uint64_t groups, const Div row_of, const I width, U *__restrict__ gin)
 {
     in_stream_order();
     constexpr int  kOut = 8 / sizeof(U);
     const uint64_t g64  = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x;
     if (g64 >= groups) return;
-    const I        g    = static_cast<I>(g64);
-    const I        row  = g / groups_per_row;
-    const I        cg   = g - row * groups_per_row;
-    const uint64_t at   = 2ull * row * width + 2ull * kOut * cg;
+    const I        row  = row_of(static_cast<I>(g64));
+    const uint64_t at   = 2ull * kOut * g64 + static_cast<uint64_t>(row) * width;
     const uint64_t o0   = g64 * kOut;
     const uint32_t bits = codes[o0 >> 4] >> (2u * (static_cast<uint32_t>(o0) & 15u));
     // the kOut mask bits of this thread's outputs sit in one word (kOut divides 32)
     const uint32_t live = mask != nullptr ? mask[o0 >> 5] >> (static_cast<uint32_t>(o0) & 31u) : 0xFFFFFFFFu;
     const uint2    gv   = *reinterpret_cast<const uint2 *>(gout + o0);
-    U              gr[kOut], top[2 * kOut], bot[2 * kOut];
-    if constexpr (sizeof(U) == 4) {
-        gr[0] = gv.x, gr[1] = gv.y;
-    } else {
-        gr[0] = static_cast<U>(gv.x), gr[1] = static_cast<U>(gv.x >> 16), gr[2] = static_cast<U>(gv.y), gr[3] = static_cast<U>(gv.y >> 16);
-    }
+    uint4          top, bot;
+    if constexpr (sizeof(U) == 2) {
+        // an output's gradient in both halves of a word, +0 where its bit is clear; the code's mask picks one half of
+        // the top or of the bottom pair (code ^ 2 puts the bottom codes where the top ones are)
+        const uint32_t g[4] = {__byte_perm(gv.x, 0, 0x1010), __byte_perm(gv.x, 0, 0x3232), __byte_perm(gv.y, 0, 0x1010), __byte_perm(gv.y, 0, 0x3232)};
+        uint32_t       tp[4], bp[4];
 #pragma unroll
-    for (int j = 0; j < kOut; ++j) {
-        const uint32_t k = (bits >> (2 * j)) & 3u;
-        gr[j]            = (live >> j) & 1u ? gr[j] : U(0);
-        top[2 * j]       = k == 0 ? gr[j] : U(0);
-        top[2 * j + 1]   = k == 1 ? gr[j] : U(0);
-        bot[2 * j]       = k == 2 ? gr[j] : U(0);
-        bot[2 * j + 1]   = k == 3 ? gr[j] : U(0);
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t s = j < 2 ? (bits << (4 - 2 * j)) & 0x30u : (bits >> (2 * j - 4)) & 0x30u;
+            const uint32_t v = (live >> j) & 1u ? g[j] : 0u;
+            tp[j] = v & pair_mask(s), bp[j] = v & pair_mask(s ^ 0x20u);
+        }
+        top = make_uint4(tp[0], tp[1], tp[2], tp[3]), bot = make_uint4(bp[0], bp[1], bp[2], bp[3]);
+    } else {
+        U gr[2] = {gv.x, gv.y}, t[4], b[4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const uint32_t k = (bits >> (2 * j)) & 3u;
+            gr[j]            = (live >> j) & 1u ? gr[j] : U(0);
+            t[2 * j]         = k == 0 ? gr[j] : U(0);
+            t[2 * j + 1]     = k == 1 ? gr[j] : U(0);
+            b[2 * j]         = k == 2 ? gr[j] : U(0);
+            b[2 * j + 1]     = k == 3 ? gr[j] : U(0);
+        }
+        top = make_uint4(t[0], t[1], t[2], t[3]), bot = make_uint4(b[0], b[1], b[2], b[3]);
     }
     const Extent gx = extent_of(gin, 4 * groups * kOut * sizeof(U));
-    if (gx.holds(gin + at, 16)) *reinterpret_cast<uint4 *>(gin + at) = pack16<U>(top);
-    if (gx.holds(gin + at + width, 16)) *reinterpret_cast<uint4 *>(gin + at + width) = pack16<U>(bot);
+    if (gx.holds(gin + at, 16)) *reinterpret_cast<uint4 *>(gin + at) = top;
+    if (gx.holds(gin + at + width, 16)) *reinterpret_cast<uint4 *>(gin + at + width) = bot;
 }
 
 template <typename U, int DT>
@@ -228,12 +292,12 @@ cudaError_t fwd_typed(const void *x, uint64_t outputs, uint64_t wo, uint64_t wid
             const uint64_t groups = outputs / kOut, per_row = wo / kOut, vgrid = (groups + kThreads - 1) / kThreads;
             if (vgrid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
             if (elements <= 0xFFFFFFFFull)
-                launch(maxpool2x2_fwd_vec_kernel<U, DT, uint32_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
-                    static_cast<const U *>(x), groups, static_cast<uint32_t>(per_row), static_cast<uint32_t>(width),
+                launch(maxpool2x2_fwd_vec_kernel<U, DT, uint32_t, DivBy>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
+                    static_cast<const U *>(x), groups, DivBy::of(static_cast<uint32_t>(per_row)), static_cast<uint32_t>(width),
                     static_cast<U *>(y), codes);
             else
-                launch(maxpool2x2_fwd_vec_kernel<U, DT, uint64_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
-                    static_cast<const U *>(x), groups, per_row, width, static_cast<U *>(y), codes);
+                launch(maxpool2x2_fwd_vec_kernel<U, DT, uint64_t, DivWide>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
+                    static_cast<const U *>(x), groups, DivWide{per_row}, width, static_cast<U *>(y), codes);
             return cudaGetLastError();
         }
     }
@@ -258,12 +322,12 @@ cudaError_t bwd_typed(const uint32_t *codes, const uint32_t *mask, const void *g
             const uint64_t groups = outputs / kOut, per_row = wo / kOut, vgrid = (groups + kThreads - 1) / kThreads;
             if (vgrid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
             if (elements <= 0xFFFFFFFFull)
-                launch(maxpool2x2_bwd_vec_kernel<U, uint32_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
-                    codes, mask, static_cast<const U *>(gout), groups, static_cast<uint32_t>(per_row),
+                launch(maxpool2x2_bwd_vec_kernel<U, uint32_t, DivBy>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
+                    codes, mask, static_cast<const U *>(gout), groups, DivBy::of(static_cast<uint32_t>(per_row)),
                     static_cast<uint32_t>(width), static_cast<U *>(gin));
             else
-                launch(maxpool2x2_bwd_vec_kernel<U, uint64_t>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
-                    codes, mask, static_cast<const U *>(gout), groups, per_row, width, static_cast<U *>(gin));
+                launch(maxpool2x2_bwd_vec_kernel<U, uint64_t, DivWide>, static_cast<unsigned>(vgrid), kThreads, 0, s, 
+                    codes, mask, static_cast<const U *>(gout), groups, DivWide{per_row}, width, static_cast<U *>(gin));
             return cudaGetLastError();
         }
     }
