@@ -164,7 +164,7 @@ decompress_body(const uint32_t *__restrict__ bitmap, const U *values,
 }
 
 // ---------------------------------------------------------------------------------------------
-// The decompressor for 2-byte elements: the quarter's packed run staged in shared memory, expanded from there
+// The decompressor for 2-byte elements: half a chunk's packed run staged in shared memory, expanded from there
 // (bt_quarter16.cuh).  WIDEN: 0 restores 2-byte elements; 1 (binary16) / 2 (bfloat16) widens every restored value
 // to binary32 on its way out.
 template <int kWarps, int WIDEN = 0>
@@ -173,17 +173,16 @@ decompress16_body(const uint32_t *__restrict__ bitmap, const uint16_t *values, c
                   const uint64_t *__restrict__ prefix, const uint64_t n,
                   std::conditional_t<WIDEN != 0, uint32_t, uint16_t> *__restrict__ out, const uint64_t block)
 {
-    q16::Quarter qt;
-    if (!q16::stage_quarter<kWarps>(bitmap, values, values_offset, prefix, n, block, qt)) return;
+    q16::Part pt;
+    if (!q16::stage_part<kWarps>(bitmap, values, values_offset, prefix, n, block, pt)) return;
     const uint32_t lane = threadIdx.x & 31u;
     const Extent   ox   = extent_of(out, n * sizeof(*out));
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        uint32_t       bits;
-        const uint2    v  = q16::expand_step(qt, k, lane, bits);
-        const uint64_t at = qt.e0 + static_cast<uint64_t>(k) * 128 + lane * 4;
+    for (int k = 0; k < q16::kPartSteps; ++k) {
+        const uint2    v  = q16::expand_step(pt, k, lane);
+        const uint64_t at = pt.e0 + static_cast<uint64_t>(k) * 128 + lane * 4;
         if constexpr (WIDEN == 0) {
-            if (qt.whole || at + 4 <= n) {
+            if (pt.whole || at + 4 <= n) {
                 if (ox.holds(out + at, 8)) *reinterpret_cast<uint2 *>(out + at) = v;
             } else {
                 const uint32_t h[2] = {v.x, v.y};
@@ -200,7 +199,7 @@ decompress16_body(const uint32_t *__restrict__ bitmap, const uint16_t *values, c
                 f[0] = widened<WIDEN>(static_cast<uint16_t>(v.x)), f[1] = widened<WIDEN>(static_cast<uint16_t>(v.x >> 16));
                 f[2] = widened<WIDEN>(static_cast<uint16_t>(v.y)), f[3] = widened<WIDEN>(static_cast<uint16_t>(v.y >> 16));
             }
-            if (qt.whole || at + 4 <= n) {
+            if (pt.whole || at + 4 <= n) {
                 if (ox.holds(out + at, 16)) *reinterpret_cast<uint4 *>(out + at) = make_uint4(f[0], f[1], f[2], f[3]);
             } else {
 #pragma unroll
@@ -288,9 +287,8 @@ cudaError_t launch_typed(const uint32_t *bitmap, const void *values, const uint6
 cudaError_t launch_decompress_widen(const uint32_t *bitmap, const void *values16, const uint64_t *values_offset,
                                     const uint64_t *prefix, uint64_t n, int from_dtype, void *out_f32, cudaStream_t stream)
 {
-    constexpr int  kWarps   = 4;
-    const uint64_t quarters = (n + 1023) >> 10;
-    const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
+    constexpr int  kWarps = 4;
+    const uint64_t grid   = q16::blocks_of(n, kWarps);
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     const auto *v = static_cast<const uint16_t *>(values16);
     auto       *o = static_cast<uint32_t *>(out_f32);
@@ -305,9 +303,8 @@ cudaError_t launch_decompress(const uint32_t *bitmap, const void *values, const 
 {
     if (elem_size == 8) return launch_typed<uint64_t, 2, 16>(bitmap, values, values_offset, prefix, n, out, stream);
     if (elem_size == 4) return launch_typed<uint32_t, 4, 8>(bitmap, values, values_offset, prefix, n, out, stream);
-    constexpr int  kWarps   = 4;
-    const uint64_t quarters = (n + 1023) >> 10;
-    const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
+    constexpr int  kWarps = 4;
+    const uint64_t grid   = q16::blocks_of(n, kWarps);
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     launch(decompress16_kernel<kWarps>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
         bitmap, static_cast<const uint16_t *>(values), values_offset, prefix, n, static_cast<uint16_t *>(out));
@@ -323,7 +320,7 @@ cudaError_t launch_decompress_batch(const DecompressJob *jobs, uint32_t count, i
     for (uint32_t k = 0; k < count; ++k) {
         const uint64_t quarters = (jobs[k].n + 1023) >> 10;
         p.job[k] = RestoreJob{jobs[k].bitmap, jobs[k].values, jobs[k].values_offset, jobs[k].prefix, jobs[k].out, jobs[k].n, static_cast<uint32_t>(blocks)};
-        blocks += (quarters + kWarps - 1) / kWarps;
+        blocks += elem_size == 2 ? q16::blocks_of(jobs[k].n, kWarps) : (quarters + kWarps - 1) / kWarps;
         if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     }
     p.jobs = count;

@@ -161,46 +161,45 @@ __device__ __forceinline__ uint32_t below_six_mask(const uint32_t pair)
     return m;
 }
 
-// 2-byte elements: the quarter's packed run staged in shared memory and gathered from there (bt_quarter16.cuh)
-// instead of one global gather per value.  The quarter's gradient -- eight 8-byte loads per lane that do not
-// depend on the stash -- is requested first, so that it arrives while the run is staged.
+// 2-byte elements: half a chunk's packed run staged in shared memory and gathered from there (bt_quarter16.cuh)
+// instead of one global gather per value.  The gradient does not depend on the stash: that of the first steps (an
+// 8-byte load per lane and step) is requested before the run is staged, that of a later step when the step kAhead before
+// it has used its registers.
 template <int DT, int kWarps>
-__global__ void __launch_bounds__(kWarps * 32, 1536 / (kWarps * 32))   // 40 registers, 12 CTAs per SM: 0.199 -> 0.178 ms against 8 CTAs
+__global__ void __launch_bounds__(kWarps * 32, 1536 / (kWarps * 32))   // 40 registers, 12 CTAs per SM
 relu6_bwd16_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *__restrict__ values,
                    const uint64_t *__restrict__ values_offset, const uint64_t *__restrict__ prefix, const uint16_t *gout,
                    const uint64_t n, uint16_t *gin)   // gin may alias gout
 {
     in_stream_order();
-    const uint32_t lane        = threadIdx.x & 31u;
-    const uint64_t warp_global = static_cast<uint64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
-    if (warp_global >= ((n + 1023) >> 10)) return;
-    const uint64_t e0 = warp_global << 10;
-    uint2          g[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t e0   = (static_cast<uint64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5)) * q16::kPartElems;
+    if (e0 >= n) return;
+    auto gradient = [&](const int k) {
         const uint64_t at = e0 + static_cast<uint64_t>(k) * 128 + lane * 4;
-        if (at + 4 <= n) {
-            g[k] = *reinterpret_cast<const uint2 *>(gout + at);
-        } else {
-            uint32_t h[4];
+        if (at + 4 <= n) return *reinterpret_cast<const uint2 *>(gout + at);
+        uint32_t h[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) h[j] = at + j < n ? gout[at + j] : 0u;
-            g[k] = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
-        }
-    }
-    q16::Quarter qt;
-    if (!q16::stage_quarter<kWarps>(bitmap, values, values_offset, prefix, n, blockIdx.x, qt)) return;
+        for (int j = 0; j < 4; ++j) h[j] = at + j < n ? gout[at + j] : 0u;
+        return make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+    };
+    constexpr int kAhead = 4;
+    uint2         g[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) g[k] = gradient(k);
+    q16::Part pt;
+    if (!q16::stage_part<kWarps>(bitmap, values, values_offset, prefix, n, blockIdx.x, pt)) return;
     const Extent ox = extent_of(gin, n * sizeof(uint16_t));
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < q16::kPartSteps; ++k) {
         // The gradient passes where the bit is set and the stashed value is below 6 (false for a stored 6 and for a
         // NaN).  Elements under a clear bit come out of the expansion as a NaN, so one compare of the packed pair in
         // its own type decides both conditions for two elements: a 16-bit mask of ones per element that passes.
-        uint32_t    bits;
-        const uint2 v = q16::expand_step<0x7FFFu>(qt, k, lane, bits);
-        const uint2 r = make_uint2(g[k].x & below_six_mask<DT>(v.x), g[k].y & below_six_mask<DT>(v.y));
+        const uint2 v = q16::expand_step<0x7FFFu>(pt, k, lane);
+        const uint2 r = make_uint2(g[k % kAhead].x & below_six_mask<DT>(v.x), g[k % kAhead].y & below_six_mask<DT>(v.y));
+        if (k + kAhead < q16::kPartSteps) g[k % kAhead] = gradient(k + kAhead);
         const uint64_t at = e0 + static_cast<uint64_t>(k) * 128 + lane * 4;
-        if (qt.whole || at + 4 <= n) {
+        if (pt.whole || at + 4 <= n) {
             if (ox.holds(gin + at, 8)) *reinterpret_cast<uint2 *>(gin + at) = r;
         } else {
             const uint32_t o[2] = {r.x, r.y};
@@ -215,9 +214,8 @@ template <int DT>
 cudaError_t launch_16(const uint32_t *bitmap, const void *values, const uint64_t *values_offset, const uint64_t *prefix,
                       const void *gout, uint64_t n, void *gin, cudaStream_t stream)
 {
-    constexpr int  kWarps   = 4;
-    const uint64_t quarters = (n + 1023) >> 10;
-    const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
+    constexpr int  kWarps = 4;
+    const uint64_t grid   = q16::blocks_of(n, kWarps);
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     launch(relu6_bwd16_kernel<DT, kWarps>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
         bitmap, static_cast<const uint16_t *>(values), values_offset, prefix, static_cast<const uint16_t *>(gout), n,
