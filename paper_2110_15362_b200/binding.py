@@ -1,6 +1,7 @@
-"""Thin ctypes binding of libbittrain.so: same names as the C ABI, argument
-marshalling only.  Every step of the codec runs in the library's CUDA kernels;
-there is no fallback: if the shared object is missing this module raises.
+"""Thin binding of libbittrain.so: same names as the C ABI, argument
+marshalling only (through the _pycall extension, csrc/bt_pycall.c; ctypes for the
+queries and the host-buffer forms).  Every step of the codec runs in the library's
+CUDA kernels; there is no fallback: if a shared object is missing this module raises.
 
 Tensors are torch CUDA tensors (device memory and streams are torch's); the
 functions pass their data pointers, the element count and the current stream.
@@ -36,6 +37,9 @@ EXPORTS = ("bt_compressed_bytes", "bt_workspace_bytes", "bt_compress", "bt_decom
            "bt_relu_bwd_from_bitmap_batch", "bt_compress_arena_batch", "bt_relu_fwd_compress_arena_batch",
            "bt_decompress_arena_batch")
 
+# what is called through _pycall: everything that takes a stream and no host buffers
+CALLS = tuple(n for n in EXPORTS if not n.endswith("_bytes") and not n.endswith("_host") and n != "bt_set_max_ctas")
+
 MAX_BATCH_PER_LAUNCH = 32
 
 
@@ -68,12 +72,29 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+class _Calls:
+    """The ABI's asynchronous calls of one build of the library (see _pycall): status codes out."""
+
+    def __init__(self, L: ctypes.CDLL, native_call):
+        for name in CALLS:
+            setattr(self, name, native_call(ctypes.cast(getattr(L, name), ctypes.c_void_p).value))
+
+
+def _calls() -> _Calls:
+    return (_lib or lib()).calls
+
+
 def load_library(path: str) -> ctypes.CDLL:
     """Open a build of the library and declare the C ABI's signatures on it."""
     if not os.path.exists(path):
         raise ImportError(f"{path} is missing: build it with "
                           "`python -m paper_2110_15362_b200.build` (needs nvcc); there is no CPU fallback")
+    try:
+        from . import _pycall
+    except ImportError as e:
+        raise ImportError(f"{_build.CALLER_PATH} is missing: build it with `python -m paper_2110_15362_b200.build`") from e
     L = ctypes.CDLL(path)
+    L.calls = _Calls(L, _pycall.native_call)
     u64, vp, i32, sz = ctypes.c_uint64, ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
     L.bt_compressed_bytes.restype = sz
     L.bt_compressed_bytes.argtypes = [u64, u64, i32]
@@ -158,9 +179,16 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> Optional[int]:
+_cuda_ready = False
+
+
+def _stream(stream) -> int:
+    global _cuda_ready
     if stream is None:
-        stream = torch.cuda.current_stream()
+        if not _cuda_ready:
+            torch.cuda.current_stream()                   # initialises CUDA where nothing has yet
+            _cuda_ready = True
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -185,9 +213,9 @@ def bt_compress(dense: torch.Tensor, bitmap: torch.Tensor, values: torch.Tensor,
                 check: bool = True) -> int:
     n = dense.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = lib().bt_compress(_ptr(dense), n, DTYPE_CODE[dense.dtype], _ptr(bitmap), _ptr(values), cap,
-                           _ptr(chunk_prefix), _ptr(nnz_out), _ptr(workspace),
-                           workspace.numel() * workspace.element_size(), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_compress(dense, n, DTYPE_CODE[dense.dtype], bitmap, values, cap,
+                              chunk_prefix, nnz_out, workspace,
+                              workspace.numel() * workspace.element_size(), dev_status, _stream(stream))
     return _check("bt_compress", st, check)
 
 
@@ -209,15 +237,15 @@ def batch_items(dense, stashes, y_out=None) -> "ctypes.Array":
 
 def bt_compress_batch(items, dtype: torch.dtype, workspace: torch.Tensor, *, stream=None, check: bool = True) -> int:
     """bt_compress of every tensor of `items` (from batch_items) in one pass."""
-    st = lib().bt_compress_batch(items, len(items), DTYPE_CODE[dtype], _ptr(workspace), _nbytes(workspace), _stream(stream))
+    st = _calls().bt_compress_batch(items, len(items), DTYPE_CODE[dtype], workspace, _nbytes(workspace), _stream(stream))
     return _check("bt_compress_batch", st, check)
 
 
 def bt_relu_fwd_compress_batch(items, dtype: torch.dtype, workspace: torch.Tensor, *, stream=None,
                                check: bool = True) -> int:
     """bt_relu_fwd_compress of every tensor of `items` (from batch_items) in one pass."""
-    st = lib().bt_relu_fwd_compress_batch(items, len(items), DTYPE_CODE[dtype], _ptr(workspace), _nbytes(workspace),
-                                          _stream(stream))
+    st = _calls().bt_relu_fwd_compress_batch(items, len(items), DTYPE_CODE[dtype], workspace, _nbytes(workspace),
+                                             _stream(stream))
     return _check("bt_relu_fwd_compress_batch", st, check)
 
 
@@ -226,28 +254,28 @@ def bt_compress_arena_batch(items, dtype: torch.dtype, arena: torch.Tensor, aren
                             check: bool = True) -> int:
     """The tensors of `items` pushed into the arena back to back by one pass (fused: ReLU forward first);
     values_offsets_out is a device int64 tensor with one word per item."""
-    fn = lib().bt_relu_fwd_compress_arena_batch if fused else lib().bt_compress_arena_batch
-    st = fn(items, len(items), DTYPE_CODE[dtype], _ptr(arena), _nbytes(arena), _ptr(arena_cursor), _ptr(values_offsets_out),
-            _ptr(workspace), _nbytes(workspace), _stream(stream))
+    fn = _calls().bt_relu_fwd_compress_arena_batch if fused else _calls().bt_compress_arena_batch
+    st = fn(items, len(items), DTYPE_CODE[dtype], arena, _nbytes(arena), arena_cursor, values_offsets_out, workspace,
+            _nbytes(workspace), _stream(stream))
     return _check("bt_compress_arena_batch", st, check)
 
 
 def bt_decompress_arena_batch(items, dtype: torch.dtype, arena: torch.Tensor, values_offsets: torch.Tensor, *, stream=None,
                               check: bool = True) -> int:
     """Every item's y_out restored from (bitmap, arena + values_offsets[k], chunk_prefix) in one pass."""
-    st = lib().bt_decompress_arena_batch(items, len(items), DTYPE_CODE[dtype], _ptr(arena), _ptr(values_offsets), _stream(stream))
+    st = _calls().bt_decompress_arena_batch(items, len(items), DTYPE_CODE[dtype], arena, values_offsets, _stream(stream))
     return _check("bt_decompress_arena_batch", st, check)
 
 
 def bt_decompress_batch(items, dtype: torch.dtype, *, stream=None, check: bool = True) -> int:
     """bt_decompress of every stash of `items` into its y_out, in one pass."""
-    st = lib().bt_decompress_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
+    st = _calls().bt_decompress_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
     return _check("bt_decompress_batch", st, check)
 
 
 def bt_relu_bwd_from_bitmap_batch(items, dtype: torch.dtype, *, stream=None, check: bool = True) -> int:
     """bt_relu_bwd_from_bitmap of every item (dense: upstream gradient, y_out: input gradient), in one pass."""
-    st = lib().bt_relu_bwd_from_bitmap_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
+    st = _calls().bt_relu_bwd_from_bitmap_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
     return _check("bt_relu_bwd_from_bitmap_batch", st, check)
 
 
@@ -258,8 +286,8 @@ def bt_compress_noalloc(dense: torch.Tensor, bitmap: torch.Tensor, values: torch
     call allocates nothing (for callers that may not); n is limited to NOALLOC_MAX_ELEMS."""
     n = dense.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = lib().bt_compress_noalloc(_ptr(dense), n, DTYPE_CODE[dense.dtype], _ptr(bitmap), _ptr(values), cap,
-                                   _ptr(chunk_prefix), _ptr(nnz_out), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_compress_noalloc(dense, n, DTYPE_CODE[dense.dtype], bitmap, values, cap,
+                                      chunk_prefix, nnz_out, dev_status, _stream(stream))
     return _check("bt_compress_noalloc", st, check)
 
 
@@ -270,10 +298,10 @@ def bt_relu_fwd_compress(pre_act: torch.Tensor, y_out: Optional[torch.Tensor], b
                          check: bool = True) -> int:
     n = pre_act.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = lib().bt_relu_fwd_compress(_ptr(pre_act), n, DTYPE_CODE[pre_act.dtype], _ptr(y_out), _ptr(bitmap),
-                                    _ptr(values), cap, _ptr(chunk_prefix), _ptr(nnz_out), _ptr(workspace),
-                                    workspace.numel() * workspace.element_size(), _ptr(dev_status),
-                                    _stream(stream))
+    st = _calls().bt_relu_fwd_compress(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
+                                       values, cap, chunk_prefix, nnz_out, workspace,
+                                       workspace.numel() * workspace.element_size(), dev_status,
+                                       _stream(stream))
     return _check("bt_relu_fwd_compress", st, check)
 
 
@@ -286,10 +314,10 @@ def bt_prune_fwd_compress(x: torch.Tensor, tau: float, y_out: Optional[torch.Ten
     """Activation pruning fused with the stash: elements <= tau (a binary32 threshold) become +0."""
     n = x.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = lib().bt_prune_fwd_compress(_ptr(x), n, DTYPE_CODE[x.dtype], ctypes.c_float(tau), _ptr(y_out), _ptr(bitmap),
-                                     _ptr(values), cap, _ptr(chunk_prefix), _ptr(nnz_out), _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _ptr(dev_status),
-                                     _stream(stream))
+    st = _calls().bt_prune_fwd_compress(x, n, DTYPE_CODE[x.dtype], float(tau), y_out, bitmap,
+                                        values, cap, chunk_prefix, nnz_out, workspace,
+                                        workspace.numel() * workspace.element_size(), dev_status,
+                                        _stream(stream))
     return _check("bt_prune_fwd_compress", st, check)
 
 def bt_set_max_ctas(max_ctas: int) -> int:
@@ -309,9 +337,9 @@ def bt_compress_narrow(dense: torch.Tensor, bitmap: torch.Tensor, values: torch.
     n = dense.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
     assert dense.dtype == torch.float32
-    st = lib().bt_compress_narrow(_ptr(dense), n, DTYPE_CODE[values.dtype], _ptr(bitmap), _ptr(values), cap,
-                                  _ptr(chunk_prefix), _ptr(nnz_out), _ptr(workspace), _nbytes(workspace),
-                                  _ptr(dev_status), _stream(stream))
+    st = _calls().bt_compress_narrow(dense, n, DTYPE_CODE[values.dtype], bitmap, values, cap,
+                                     chunk_prefix, nnz_out, workspace, _nbytes(workspace),
+                                     dev_status, _stream(stream))
     return _check("bt_compress_narrow", st, check)
 
 
@@ -324,9 +352,9 @@ def bt_prune_fwd_compress_narrow(x: torch.Tensor, tau: float, y_out: Optional[to
     n = x.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
     assert x.dtype == torch.float32
-    st = lib().bt_prune_fwd_compress_narrow(_ptr(x), n, DTYPE_CODE[values.dtype], ctypes.c_float(tau), _ptr(y_out),
-                                            _ptr(bitmap), _ptr(values), cap, _ptr(chunk_prefix), _ptr(nnz_out),
-                                            _ptr(workspace), _nbytes(workspace), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_prune_fwd_compress_narrow(x, n, DTYPE_CODE[values.dtype], float(tau), y_out,
+                                               bitmap, values, cap, chunk_prefix, nnz_out,
+                                               workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_prune_fwd_compress_narrow", st, check)
 
 
@@ -335,8 +363,8 @@ def bt_decompress_widen(bitmap: torch.Tensor, values: torch.Tensor, chunk_prefix
     """Restores a narrowed stash (16-bit `values`) into a float32 tensor."""
     n = dense_out.numel() if n is None else n
     assert dense_out.dtype == torch.float32
-    st = lib().bt_decompress_widen(_ptr(bitmap), _ptr(values), _ptr(chunk_prefix), n, DTYPE_CODE[values.dtype],
-                                   _ptr(dense_out), _stream(stream))
+    st = _calls().bt_decompress_widen(bitmap, values, chunk_prefix, n, DTYPE_CODE[values.dtype],
+                                      dense_out, _stream(stream))
     return _check("bt_decompress_widen", st, check)
 
 
@@ -347,7 +375,7 @@ def bt_maxpool2x2_fwd(x: torch.Tensor, y: torch.Tensor, codes: Optional[torch.Te
     height = x.shape[-2] if height is None else height
     width = x.shape[-1] if width is None else width
     planes = x.numel() // max(1, height * width) if planes is None else planes
-    st = lib().bt_maxpool2x2_fwd(_ptr(x), planes, height, width, DTYPE_CODE[x.dtype], _ptr(y), _ptr(codes), _stream(stream))
+    st = _calls().bt_maxpool2x2_fwd(x, planes, height, width, DTYPE_CODE[x.dtype], y, codes, _stream(stream))
     return _check("bt_maxpool2x2_fwd", st, check)
 
 
@@ -357,8 +385,8 @@ def bt_maxpool2x2_bwd(codes: torch.Tensor, grad_out: torch.Tensor, grad_in: torc
     height = grad_in.shape[-2] if height is None else height
     width = grad_in.shape[-1] if width is None else width
     planes = grad_in.numel() // max(1, height * width) if planes is None else planes
-    st = lib().bt_maxpool2x2_bwd(_ptr(codes), _ptr(grad_out), planes, height, width, DTYPE_CODE[grad_out.dtype],
-                                 _ptr(grad_in), _stream(stream))
+    st = _calls().bt_maxpool2x2_bwd(codes, grad_out, planes, height, width, DTYPE_CODE[grad_out.dtype],
+                                    grad_in, _stream(stream))
     return _check("bt_maxpool2x2_bwd", st, check)
 
 
@@ -370,8 +398,8 @@ def bt_maxpool2x2_bwd_masked(codes: torch.Tensor, pooled_bitmap: torch.Tensor, g
     height = grad_in.shape[-2] if height is None else height
     width = grad_in.shape[-1] if width is None else width
     planes = grad_in.numel() // max(1, height * width) if planes is None else planes
-    st = lib().bt_maxpool2x2_bwd_masked(_ptr(codes), _ptr(pooled_bitmap), _ptr(grad_out), planes, height, width,
-                                        DTYPE_CODE[grad_out.dtype], _ptr(grad_in), _stream(stream))
+    st = _calls().bt_maxpool2x2_bwd_masked(codes, pooled_bitmap, grad_out, planes, height, width,
+                                           DTYPE_CODE[grad_out.dtype], grad_in, _stream(stream))
     return _check("bt_maxpool2x2_bwd_masked", st, check)
 
 
@@ -381,8 +409,8 @@ def bt_mask_compress(x: torch.Tensor, mask_bitmap: torch.Tensor, mask_chunk_pref
     """Double-mask form: the values of x at the set bits of an existing stash's bitmap (and the masked dense y)."""
     n = x.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = lib().bt_mask_compress(_ptr(x), n, DTYPE_CODE[x.dtype], _ptr(mask_bitmap), _ptr(mask_chunk_prefix),
-                                _ptr(y_out), _ptr(values), cap, _stream(stream))
+    st = _calls().bt_mask_compress(x, n, DTYPE_CODE[x.dtype], mask_bitmap, mask_chunk_prefix,
+                                   y_out, values, cap, _stream(stream))
     return _check("bt_mask_compress", st, check)
 
 
@@ -392,9 +420,9 @@ def bt_compress_arena(dense: torch.Tensor, bitmap: torch.Tensor, arena: torch.Te
                       stream=None, check: bool = True) -> int:
     """bt_compress whose values go behind the cursor of a caller-owned arena (a uint8 device tensor)."""
     n = dense.numel() if n is None else n
-    st = lib().bt_compress_arena(_ptr(dense), n, DTYPE_CODE[dense.dtype], _ptr(bitmap), _ptr(arena), _nbytes(arena),
-                                 _ptr(arena_cursor), _ptr(values_offset_out), _ptr(chunk_prefix), _ptr(nnz_out),
-                                 _ptr(workspace), _nbytes(workspace), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_compress_arena(dense, n, DTYPE_CODE[dense.dtype], bitmap, arena, _nbytes(arena),
+                                    arena_cursor, values_offset_out, chunk_prefix, nnz_out,
+                                    workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_compress_arena", st, check)
 
 
@@ -405,10 +433,10 @@ def bt_prune_fwd_compress_arena(x: torch.Tensor, tau: float, y_out: Optional[tor
                                 check: bool = True) -> int:
     """Fused forward (tau = 0: ReLU) whose values go behind the cursor of a caller-owned arena."""
     n = x.numel() if n is None else n
-    st = lib().bt_prune_fwd_compress_arena(_ptr(x), n, DTYPE_CODE[x.dtype], ctypes.c_float(tau), _ptr(y_out),
-                                           _ptr(bitmap), _ptr(arena), _nbytes(arena), _ptr(arena_cursor),
-                                           _ptr(values_offset_out), _ptr(chunk_prefix), _ptr(nnz_out),
-                                           _ptr(workspace), _nbytes(workspace), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_prune_fwd_compress_arena(x, n, DTYPE_CODE[x.dtype], float(tau), y_out,
+                                              bitmap, arena, _nbytes(arena), arena_cursor,
+                                              values_offset_out, chunk_prefix, nnz_out,
+                                              workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_prune_fwd_compress_arena", st, check)
 
 
@@ -416,8 +444,8 @@ def bt_decompress_arena(bitmap: torch.Tensor, arena: torch.Tensor, values_offset
                         chunk_prefix: torch.Tensor, dense_out: torch.Tensor, *, n: Optional[int] = None, stream=None,
                         check: bool = True) -> int:
     n = dense_out.numel() if n is None else n
-    st = lib().bt_decompress_arena(_ptr(bitmap), _ptr(arena), _ptr(values_offset), _ptr(chunk_prefix), n,
-                                   DTYPE_CODE[dense_out.dtype], _ptr(dense_out), _stream(stream))
+    st = _calls().bt_decompress_arena(bitmap, arena, values_offset, chunk_prefix, n,
+                                      DTYPE_CODE[dense_out.dtype], dense_out, _stream(stream))
     return _check("bt_decompress_arena", st, check)
 
 
@@ -428,9 +456,9 @@ def bt_compress_narrow_arena(dense: torch.Tensor, to_dtype: torch.dtype, bitmap:
     """bt_compress_narrow whose 16-bit values (of `to_dtype`) go behind the cursor of a caller-owned arena."""
     n = dense.numel() if n is None else n
     assert dense.dtype == torch.float32
-    st = lib().bt_compress_narrow_arena(_ptr(dense), n, DTYPE_CODE[to_dtype], _ptr(bitmap), _ptr(arena), _nbytes(arena),
-                                        _ptr(arena_cursor), _ptr(values_offset_out), _ptr(chunk_prefix), _ptr(nnz_out),
-                                        _ptr(workspace), _nbytes(workspace), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_compress_narrow_arena(dense, n, DTYPE_CODE[to_dtype], bitmap, arena, _nbytes(arena),
+                                           arena_cursor, values_offset_out, chunk_prefix, nnz_out,
+                                           workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_compress_narrow_arena", st, check)
 
 
@@ -442,10 +470,10 @@ def bt_prune_fwd_compress_narrow_arena(x: torch.Tensor, to_dtype: torch.dtype, t
     """bt_prune_fwd_compress_narrow whose 16-bit values (of `to_dtype`) go behind the cursor of a caller-owned arena."""
     n = x.numel() if n is None else n
     assert x.dtype == torch.float32
-    st = lib().bt_prune_fwd_compress_narrow_arena(_ptr(x), n, DTYPE_CODE[to_dtype], ctypes.c_float(tau), _ptr(y_out),
-                                                  _ptr(bitmap), _ptr(arena), _nbytes(arena), _ptr(arena_cursor),
-                                                  _ptr(values_offset_out), _ptr(chunk_prefix), _ptr(nnz_out),
-                                                  _ptr(workspace), _nbytes(workspace), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_prune_fwd_compress_narrow_arena(x, n, DTYPE_CODE[to_dtype], float(tau), y_out,
+                                                     bitmap, arena, _nbytes(arena), arena_cursor,
+                                                     values_offset_out, chunk_prefix, nnz_out,
+                                                     workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_prune_fwd_compress_narrow_arena", st, check)
 
 
@@ -455,8 +483,8 @@ def bt_decompress_widen_arena(bitmap: torch.Tensor, arena: torch.Tensor, values_
     """Restores a narrowed stash whose 16-bit values (of `from_dtype`) sit in an arena into a float32 tensor."""
     n = dense_out.numel() if n is None else n
     assert dense_out.dtype == torch.float32
-    st = lib().bt_decompress_widen_arena(_ptr(bitmap), _ptr(arena), _ptr(values_offset), _ptr(chunk_prefix), n,
-                                         DTYPE_CODE[from_dtype], _ptr(dense_out), _stream(stream))
+    st = _calls().bt_decompress_widen_arena(bitmap, arena, values_offset, chunk_prefix, n,
+                                            DTYPE_CODE[from_dtype], dense_out, _stream(stream))
     return _check("bt_decompress_widen_arena", st, check)
 
 
@@ -467,10 +495,10 @@ def bt_relu6_fwd_compress_arena(pre_act: torch.Tensor, y_out: Optional[torch.Ten
                                 check: bool = True) -> int:
     """Fused ReLU6 forward whose values go behind the cursor of a caller-owned arena."""
     n = pre_act.numel() if n is None else n
-    st = lib().bt_relu6_fwd_compress_arena(_ptr(pre_act), n, DTYPE_CODE[pre_act.dtype], _ptr(y_out), _ptr(bitmap),
-                                           _ptr(arena), _nbytes(arena), _ptr(arena_cursor), _ptr(values_offset_out),
-                                           _ptr(chunk_prefix), _ptr(nnz_out), _ptr(workspace), _nbytes(workspace),
-                                           _ptr(dev_status), _stream(stream))
+    st = _calls().bt_relu6_fwd_compress_arena(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
+                                              arena, _nbytes(arena), arena_cursor, values_offset_out,
+                                              chunk_prefix, nnz_out, workspace, _nbytes(workspace),
+                                              dev_status, _stream(stream))
     return _check("bt_relu6_fwd_compress_arena", st, check)
 
 
@@ -479,8 +507,8 @@ def bt_relu6_bwd_from_stash_arena(bitmap: torch.Tensor, arena: torch.Tensor, val
                                   *, n: Optional[int] = None, stream=None, check: bool = True) -> int:
     """ReLU6 backward from a stash whose values sit in an arena."""
     n = grad_out.numel() if n is None else n
-    st = lib().bt_relu6_bwd_from_stash_arena(_ptr(bitmap), _ptr(arena), _ptr(values_offset), _ptr(chunk_prefix),
-                                             _ptr(grad_out), n, DTYPE_CODE[grad_out.dtype], _ptr(grad_in), _stream(stream))
+    st = _calls().bt_relu6_bwd_from_stash_arena(bitmap, arena, values_offset, chunk_prefix,
+                                                grad_out, n, DTYPE_CODE[grad_out.dtype], grad_in, _stream(stream))
     return _check("bt_relu6_bwd_from_stash_arena", st, check)
 
 
@@ -491,9 +519,9 @@ def bt_relu6_fwd_compress(pre_act: torch.Tensor, y_out: Optional[torch.Tensor], 
                           check: bool = True) -> int:
     n = pre_act.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = lib().bt_relu6_fwd_compress(_ptr(pre_act), n, DTYPE_CODE[pre_act.dtype], _ptr(y_out), _ptr(bitmap),
-                                     _ptr(values), cap, _ptr(chunk_prefix), _ptr(nnz_out), _ptr(workspace),
-                                     _nbytes(workspace), _ptr(dev_status), _stream(stream))
+    st = _calls().bt_relu6_fwd_compress(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
+                                        values, cap, chunk_prefix, nnz_out, workspace,
+                                        _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_relu6_fwd_compress", st, check)
 
 
@@ -501,24 +529,24 @@ def bt_relu6_bwd_from_stash(bitmap: torch.Tensor, values: torch.Tensor, chunk_pr
                             grad_out: torch.Tensor, grad_in: torch.Tensor, *, n: Optional[int] = None, stream=None,
                             check: bool = True) -> int:
     n = grad_out.numel() if n is None else n
-    st = lib().bt_relu6_bwd_from_stash(_ptr(bitmap), _ptr(values), _ptr(chunk_prefix), _ptr(grad_out), n,
-                                       DTYPE_CODE[grad_out.dtype], _ptr(grad_in), _stream(stream))
+    st = _calls().bt_relu6_bwd_from_stash(bitmap, values, chunk_prefix, grad_out, n,
+                                          DTYPE_CODE[grad_out.dtype], grad_in, _stream(stream))
     return _check("bt_relu6_bwd_from_stash", st, check)
 
 
 def bt_decompress(bitmap: torch.Tensor, values: torch.Tensor, chunk_prefix: torch.Tensor, dense_out: torch.Tensor,
                   *, n: Optional[int] = None, stream=None, check: bool = True) -> int:
     n = dense_out.numel() if n is None else n
-    st = lib().bt_decompress(_ptr(bitmap), _ptr(values), _ptr(chunk_prefix), n, DTYPE_CODE[dense_out.dtype],
-                             _ptr(dense_out), _stream(stream))
+    st = _calls().bt_decompress(bitmap, values, chunk_prefix, n, DTYPE_CODE[dense_out.dtype],
+                                dense_out, _stream(stream))
     return _check("bt_decompress", st, check)
 
 
 def bt_relu_bwd_from_bitmap(bitmap: torch.Tensor, grad_out: torch.Tensor, grad_in: torch.Tensor,
                             *, n: Optional[int] = None, stream=None, check: bool = True) -> int:
     n = grad_out.numel() if n is None else n
-    st = lib().bt_relu_bwd_from_bitmap(_ptr(bitmap), _ptr(grad_out), n, DTYPE_CODE[grad_out.dtype], _ptr(grad_in),
-                                       _stream(stream))
+    st = _calls().bt_relu_bwd_from_bitmap(bitmap, grad_out, n, DTYPE_CODE[grad_out.dtype], grad_in,
+                                          _stream(stream))
     return _check("bt_relu_bwd_from_bitmap", st, check)
 
 

@@ -1,15 +1,19 @@
-"""Builds the CUDA library (libbittrain.so) in-tree with nvcc for sm_100a."""
+"""Builds the CUDA library (libbittrain.so) in-tree with nvcc for sm_100a, and the extension module
+(_pycall) the binding calls it through."""
 from __future__ import annotations
 
 import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(os.path.dirname(PKG_DIR), "include")
 LIB_PATH = os.path.join(PKG_DIR, "libbittrain.so")
+CALLER_SRC = os.path.join(CSRC, "bt_pycall.c")
+CALLER_PATH = os.path.join(PKG_DIR, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
@@ -30,10 +34,22 @@ def is_stale(path: str = LIB_PATH) -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def build_caller(force: bool = False) -> str:
+    """Compile the extension module the binding calls the library through; returns its path."""
+    if not force and os.path.exists(CALLER_PATH) and os.path.getmtime(CALLER_PATH) >= os.path.getmtime(CALLER_SRC):
+        return CALLER_PATH
+    tmp = CALLER_PATH + ".tmp%d" % os.getpid()
+    subprocess.check_call(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp, CALLER_SRC])
+    os.replace(tmp, CALLER_PATH)
+    return CALLER_PATH
+
+
 def build_library(force: bool = False, verbose: bool = False, out: str = LIB_PATH, extra_flags=()) -> str:
     """Compile every .cu under csrc/ into one shared object; returns its path.  `out` and
     `extra_flags` (preprocessor defines and the like) are for the checking builds the tests use;
     the product library is the default."""
+    if out == LIB_PATH:
+        build_caller(force)
     if not force and not is_stale(out):
         return out
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
