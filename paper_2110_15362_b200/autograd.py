@@ -40,6 +40,7 @@ those calls); a ReLU6 stash is never narrowed.
 """
 from __future__ import annotations
 
+import threading
 import weakref
 from typing import Dict, Optional, Tuple
 
@@ -52,46 +53,95 @@ __all__ = ["PackedActivation", "stash_saved_activations", "relu_stash", "ReLUSta
            "ReLUMaxPool2x2Stash"]
 
 
+class _Record:
+    """What a stash keeps beside its values, in one allocation: the bitmap, the chunk prefix array and, in arena mode,
+    the words for the count and the byte offset of the values.  Views of it are made when somebody asks."""
+
+    __slots__ = ("buf", "n", "_bitmap", "_prefix")
+
+    def __init__(self, n: int, device, words: int = 0):
+        self.n = n
+        self.buf = torch.empty(_words_at(n) + 8 * words, dtype=torch.uint8, device=device)
+        self._bitmap = self._prefix = None
+
+    @property
+    def bitmap(self) -> torch.Tensor:
+        if self._bitmap is None:
+            self._bitmap = self.buf[:4 * ((self.n + 31) // 32)].view(torch.int32)
+        return self._bitmap
+
+    @property
+    def chunk_prefix(self) -> torch.Tensor:
+        if self._prefix is None:
+            self._prefix = self.buf[_prefix_at(self.n):_words_at(self.n)].view(torch.int64)
+        return self._prefix
+
+    def word(self, k: int) -> torch.Tensor:
+        at = _words_at(self.n) + 8 * k
+        return self.buf[at:at + 8].view(torch.int64)
+
+
+def _prefix_at(n: int) -> int:
+    """Byte offset of the prefix array in a record of n elements (the bitmap's bytes, up to 16)."""
+    return ((n + 31) // 32 * 4 + 15) & ~15
+
+
+def _words_at(n: int) -> int:
+    return _prefix_at(n) + (n + B.CHUNK - 1) // B.CHUNK * 8
+
+
 class PackedActivation:
     """What replaces a saved tensor: the stash and the metadata needed to rebuild it.  `values` is either the
     exact-size vector of values, or (arena mode) None with `arena`, `offset` (device word), `owner` and `stored`
     (the dtype of the values in the arena) set."""
 
-    __slots__ = ("bitmap", "values", "chunk_prefix", "shape", "dtype", "device", "nnz", "arena", "offset", "owner",
-                 "stored", "__weakref__")
+    __slots__ = ("record", "values", "shape", "dtype", "device", "_nnz", "arena", "owner", "stored", "__weakref__")
 
-    def __init__(self, bitmap, values, chunk_prefix, shape, dtype, device, nnz, arena=None, offset=None, owner=None,
-                 stored=None):
-        self.bitmap, self.values, self.chunk_prefix = bitmap, values, chunk_prefix
-        self.shape, self.dtype, self.device, self.nnz = shape, dtype, device, nnz
-        self.arena, self.offset, self.owner = arena, offset, owner
+    def __init__(self, record: _Record, values, shape, dtype, device, nnz, arena=None, owner=None, stored=None):
+        self.record, self.values = record, values
+        self.shape, self.dtype, self.device, self._nnz = shape, dtype, device, nnz
+        self.arena, self.owner = arena, owner
         self.stored = stored if stored is not None else (dtype if values is None else values.dtype)
 
     @property
+    def bitmap(self) -> torch.Tensor:
+        return self.record.bitmap
+
+    @property
+    def chunk_prefix(self) -> torch.Tensor:
+        return self.record.chunk_prefix
+
+    @property
+    def nnz(self):
+        """The number of values: an int, or (arena mode) the device word that holds it."""
+        return self._nnz if self.arena is None else self.record.word(0)
+
+    @property
+    def offset(self) -> Optional[torch.Tensor]:
+        return None if self.arena is None else self.record.word(1)
+
+    @property
     def numel(self) -> int:
-        n = 1
-        for s in self.shape:
-            n *= s
-        return n
+        return self.record.n
 
     def nbytes(self) -> int:
         """Bytes of the stash (arena mode: reads nnz from the device)."""
-        nnz = int(self.nnz.item()) if isinstance(self.nnz, torch.Tensor) else self.nnz
+        nnz = self._nnz if self.arena is None else int(self.nnz.item())
         return B.bt_compressed_bytes(self.numel, nnz, self.stored)
 
     def unpack(self) -> torch.Tensor:
         out = torch.empty(self.shape, dtype=self.dtype, device=self.device)
+        n, at, calls, stream = self.record.n, self.record.buf.data_ptr(), B._calls(), B._stream(None)
+        prefix, code = at + _prefix_at(n), B.DTYPE_CODE[self.stored]
         if self.arena is not None:
             self.owner.check_statuses()
-            if self.stored != self.dtype:              # a narrowed stash of a float32 tensor
-                B.bt_decompress_widen_arena(self.bitmap, self.arena, self.offset, self.chunk_prefix, self.stored,
-                                            out.view(-1))
-            else:
-                B.bt_decompress_arena(self.bitmap, self.arena, self.offset, self.chunk_prefix, out.view(-1))
-        elif self.values.dtype != self.dtype:          # a narrowed stash of a float32 tensor
-            B.bt_decompress_widen(self.bitmap, self.values, self.chunk_prefix, out.view(-1))
+            # a stash of another type than the tensor's is a narrowed stash of a float32 tensor
+            call = calls.bt_decompress_arena if self.stored is self.dtype else calls.bt_decompress_widen_arena
+            st = call(at, self.arena, at + _words_at(n) + 8, prefix, n, code, out, stream)
         else:
-            B.bt_decompress(self.bitmap, self.values, self.chunk_prefix, out.view(-1))
+            call = calls.bt_decompress if self.stored is self.dtype else calls.bt_decompress_widen
+            st = call(at, self.values, prefix, n, code, out, stream)
+        B._check("bt_decompress (autograd stash)", st, True)
         return out
 
 
@@ -110,15 +160,15 @@ class _Scratch:
 
     def __init__(self, two_pass: bool = True):
         self.ws: Dict[torch.device, torch.Tensor] = {}
+        self.ws_for: Dict[torch.device, int] = {}        # the largest element count a device's workspace serves
         self.values: Dict[Tuple[torch.device, torch.dtype], torch.Tensor] = {}
         self.two_pass = two_pass         # exact-size values without a full-capacity buffer (see _compress)
 
     def workspace(self, n: int, device) -> torch.Tensor:
-        need = B.bt_workspace_bytes(n)
-        ws = self.ws.get(device)
-        if ws is None or ws.numel() < need:
-            ws = self.ws[device] = torch.empty(need, dtype=torch.uint8, device=device)
-        return ws
+        if self.ws_for.get(device, -1) < n:
+            self.ws[device] = torch.empty(B.bt_workspace_bytes(n), dtype=torch.uint8, device=device)
+            self.ws_for[device] = n
+        return self.ws[device]
 
     def full_values(self, n: int, dtype, device) -> torch.Tensor:
         key = (device, dtype)
@@ -128,82 +178,133 @@ class _Scratch:
         return v
 
 
-def _compress(flat: torch.Tensor, scratch: _Scratch, relu_into: Optional[torch.Tensor] = None,
+class _StatusWords:
+    """Device status words of the calls of a pass, handed out from blocks; fresh blocks after every check."""
+
+    BLOCK = 64
+
+    def __init__(self):
+        self.blocks: list = []           # (block, words handed out)
+
+    def __bool__(self) -> bool:
+        return bool(self.blocks)
+
+    def next(self, device) -> int:
+        """The address of a new word on `device`."""
+        if not self.blocks or self.blocks[-1][1] == self.BLOCK or self.blocks[-1][0].device != device:
+            self.blocks.append([torch.empty(self.BLOCK, dtype=torch.int32, device=device), 0])
+        last = self.blocks[-1]
+        last[1] += 1
+        return last[0].data_ptr() + 4 * (last[1] - 1)
+
+    def drain(self) -> list:
+        """The words handed out since the last time (one host read per block)."""
+        words = [w for block, used in self.blocks for w in block[:used].tolist()]
+        self.blocks = []
+        return words
+
+
+class _HostWords(threading.local):
+    """Two words of page-locked memory per thread: the kernels store a count and a status straight into them, so that
+    reading the two back costs one wait for the stream instead of two copies."""
+
+    def __init__(self):
+        self.words = torch.zeros(2, dtype=torch.int64, pin_memory=True)
+        self.view = self.words.numpy()
+
+
+_host_words: Optional[_HostWords] = None
+
+
+def _read_back() -> _HostWords:
+    global _host_words
+    if _host_words is None:
+        _host_words = _HostWords()
+    return _host_words
+
+
+def _compress(x: torch.Tensor, scratch: _Scratch, relu_into: Optional[torch.Tensor] = None,
               narrow: Optional[torch.dtype] = None, relu6: bool = False):
-    """Runs the (fused) compressor on a flat tensor; returns bitmap, exact-size values, prefix, nnz.  `narrow`:
+    """Runs the (fused) compressor on a contiguous tensor; returns the record, the exact-size values and nnz.  `narrow`:
     16-bit dtype of the stashed values of a float32 tensor.  `relu6`: the fused form is ReLU6 (needs relu_into)."""
-    n, dev = flat.numel(), flat.device
-    if narrow is not None and flat.dtype != torch.float32:
+    n, dev = x.numel(), x.device
+    record = _Record(n, dev)
+    if n == 0:
+        return record, torch.empty(0, dtype=x.dtype, device=dev), 0
+    if narrow is not None and x.dtype != torch.float32:
         narrow = None
-    bitmap = torch.empty((n + 31) // 32, dtype=torch.int32, device=dev)
-    prefix = torch.empty((n + B.CHUNK - 1) // B.CHUNK, dtype=torch.int64, device=dev)
-    nnz_out = torch.empty(1, dtype=torch.int64, device=dev)
-    status = torch.empty(1, dtype=torch.int32, device=dev)
-    ws = scratch.workspace(n, dev)
-    if scratch.two_pass and narrow is None:
-        # Two passes instead of a values buffer of full capacity: the compressor with no room for values gives
-        # bitmap, prefix and nnz (BT_ERR_CAPACITY is its expected answer), the host reads nnz, and the masked
-        # gather fills a buffer of exactly that size from the activation.  Costs the gather (cheaper than a
-        # compaction); saves a buffer as large as the largest activation for the whole step.
-        if relu6:
-            B.bt_relu6_fwd_compress(flat, relu_into, bitmap, None, prefix, nnz_out, ws, status, n=n, values_capacity=0)
-        elif relu_into is None:
-            B.bt_compress(flat, bitmap, None, prefix, nnz_out, ws, status, n=n, values_capacity=0)
-        else:
-            B.bt_relu_fwd_compress(flat, relu_into, bitmap, None, prefix, nnz_out, ws, status, n=n, values_capacity=0)
-        nnz = int(nnz_out.item())
-        st = int(status.item())
-        if st not in (B.BT_OK, B.BT_ERR_CAPACITY):
-            raise B.BitTrainError("bt_compress (autograd stash)", st)
-        values = torch.empty(nnz, dtype=flat.dtype, device=dev)
-        if nnz:
-            B.bt_mask_compress(flat if relu_into is None else relu_into, bitmap, prefix, None, values, n=n)
-        return bitmap, values, prefix, nnz
-    full = scratch.full_values(n, narrow or flat.dtype, dev)
+    ws, host, calls = scratch.workspace(n, dev), _read_back(), B._calls()
+    at = record.buf.data_ptr()
+    nnz_word = host.words.data_ptr()
+    # Two passes instead of a values buffer of full capacity: the compressor with no room for values gives
+    # bitmap, prefix and nnz (BT_ERR_CAPACITY is its expected answer), the host reads nnz, and the masked
+    # gather fills a buffer of exactly that size from the activation.  Costs the gather (cheaper than a
+    # compaction); saves a buffer as large as the largest activation for the whole step.
+    two_pass = scratch.two_pass and narrow is None
+    full = None if two_pass else scratch.full_values(n, narrow or x.dtype, dev)
+    tail = (at, full, 0 if two_pass else n, at + _prefix_at(n), nnz_word, ws, ws.numel(), nnz_word + 8, B._stream(None))
+    code = B.DTYPE_CODE[narrow or x.dtype]
     if relu6:
-        B.bt_relu6_fwd_compress(flat, relu_into, bitmap, full, prefix, nnz_out, ws, status, n=n, values_capacity=n)
-    elif narrow is not None and relu_into is None:
-        B.bt_compress_narrow(flat, bitmap, full, prefix, nnz_out, ws, status, n=n, values_capacity=n)
-    elif narrow is not None:
-        B.bt_prune_fwd_compress_narrow(flat, 0.0, relu_into, bitmap, full, prefix, nnz_out, ws, status, n=n,
-                                       values_capacity=n)
+        st = calls.bt_relu6_fwd_compress(x, n, code, relu_into, *tail)
     elif relu_into is None:
-        B.bt_compress(flat, bitmap, full, prefix, nnz_out, ws, status, n=n, values_capacity=n)
+        st = (calls.bt_compress if narrow is None else calls.bt_compress_narrow)(x, n, code, *tail)
+    elif narrow is None:
+        st = calls.bt_relu_fwd_compress(x, n, code, relu_into, *tail)
     else:
-        B.bt_relu_fwd_compress(flat, relu_into, bitmap, full, prefix, nnz_out, ws, status, n=n, values_capacity=n)
-    nnz = int(nnz_out.item())                       # the one host read: sizes the values exactly
-    st = int(status.item())
-    if st != B.BT_OK:
+        st = calls.bt_prune_fwd_compress_narrow(x, n, code, 0.0, relu_into, *tail)
+    B._check("bt_compress (autograd stash)", st, True)
+    torch.cuda.current_stream().synchronize()       # the one host read: sizes the values exactly
+    nnz, st = int(host.view[0]), int(host.view[1]) & 0xFFFFFFFF
+    if st != B.BT_OK and not (two_pass and st == B.BT_ERR_CAPACITY):
         raise B.BitTrainError("bt_compress (autograd stash)", st)
-    return bitmap, full[:nnz].clone(), prefix, nnz
+    if not two_pass:
+        return record, full[:nnz].clone(), nnz
+    values = torch.empty(nnz, dtype=x.dtype, device=dev)
+    if nnz:
+        st = calls.bt_mask_compress(x if relu_into is None else relu_into, n, code, at, at + _prefix_at(n), None, values, nnz,
+                                    B._stream(None))
+        B._check("bt_mask_compress (autograd stash)", st, True)
+    return record, values, nnz
 
 
-def _compress_arena(flat: torch.Tensor, owner, relu_into: Optional[torch.Tensor] = None, relu6: bool = False):
-    """Arena form of `_compress`: nothing is read back; returns bitmap, prefix, nnz word, offset word and the
+def _compress_arena(x: torch.Tensor, owner, relu_into: Optional[torch.Tensor] = None, relu6: bool = False):
+    """Arena form of `_compress`: nothing is read back; returns the record (nnz and offset word included) and the
     dtype of the values pushed (the owner's narrow type for a float32 tensor, except under ReLU6)."""
-    n, dev = flat.numel(), flat.device
-    narrow = owner.narrow if (flat.dtype == torch.float32 and not relu6) else None
-    bitmap = torch.empty((n + 31) // 32, dtype=torch.int32, device=dev)
-    prefix = torch.empty((n + B.CHUNK - 1) // B.CHUNK, dtype=torch.int64, device=dev)
-    words = torch.empty(2, dtype=torch.int64, device=dev)               # nnz, byte offset of the values
-    status = torch.empty(1, dtype=torch.int32, device=dev)
-    ws = owner.scratch.workspace(n, dev)
+    n, dev = x.numel(), x.device
+    narrow = owner.narrow if (x.dtype == torch.float32 and not relu6) else None
+    record = _Record(n, dev, words=2)
+    ws, calls, arena = owner.scratch.workspace(n, dev), B._calls(), owner.arena
+    at = record.buf.data_ptr()
+    words = at + _words_at(n)
+    tail = (at, arena, arena.numel(), owner.cursor, words + 8, at + _prefix_at(n), words, ws, ws.numel(),
+            owner.statuses.next(dev), B._stream(None))
+    code = B.DTYPE_CODE[narrow or x.dtype]
     if relu6:
-        B.bt_relu6_fwd_compress_arena(flat, relu_into, bitmap, owner.arena, owner.cursor, words[1:], prefix, words[:1],
-                                      ws, status, n=n)
-    elif narrow is not None and relu_into is None:
-        B.bt_compress_narrow_arena(flat, narrow, bitmap, owner.arena, owner.cursor, words[1:], prefix, words[:1], ws,
-                                   status, n=n)
-    elif narrow is not None:
-        B.bt_prune_fwd_compress_narrow_arena(flat, narrow, 0.0, relu_into, bitmap, owner.arena, owner.cursor, words[1:],
-                                             prefix, words[:1], ws, status, n=n)
+        st = calls.bt_relu6_fwd_compress_arena(x, n, code, relu_into, *tail)
     elif relu_into is None:
-        B.bt_compress_arena(flat, bitmap, owner.arena, owner.cursor, words[1:], prefix, words[:1], ws, status, n=n)
+        st = (calls.bt_compress_arena if narrow is None else calls.bt_compress_narrow_arena)(x, n, code, *tail)
     else:
-        B.bt_prune_fwd_compress_arena(flat, 0.0, relu_into, bitmap, owner.arena, owner.cursor, words[1:], prefix,
-                                      words[:1], ws, status, n=n)
-    owner.statuses.append(status)
-    return bitmap, prefix, words[:1], words[1:], narrow or flat.dtype
+        st = (calls.bt_prune_fwd_compress_arena if narrow is None else calls.bt_prune_fwd_compress_narrow_arena)(
+            x, n, code, 0.0, relu_into, *tail)
+    B._check("bt_*_arena (autograd stash)", st, True)
+    return record, narrow or x.dtype
+
+
+def _packed(y: torch.Tensor, record: _Record, values, nnz) -> PackedActivation:
+    return PackedActivation(record, values, tuple(y.shape), y.dtype, y.device, nnz)
+
+
+def _packed_arena(y: torch.Tensor, record: _Record, owner, stored) -> PackedActivation:
+    return PackedActivation(record, None, tuple(y.shape), y.dtype, y.device, None, owner.arena, owner, stored)
+
+
+def _relu_bwd(bitmap: torch.Tensor, grad: torch.Tensor) -> torch.Tensor:
+    """The gradient under a bitmap (a record's buffer begins with it)."""
+    g = _flat_input(grad)
+    gin = torch.empty_like(g)
+    B._check("bt_relu_bwd_from_bitmap",
+             B._calls().bt_relu_bwd_from_bitmap(bitmap, g, g.numel(), B.DTYPE_CODE[g.dtype], gin, B._stream(None)), True)
+    return gin
 
 
 class stash_saved_activations(torch.autograd.graph.saved_tensors_hooks):
@@ -220,8 +321,8 @@ class stash_saved_activations(torch.autograd.graph.saved_tensors_hooks):
             raise ValueError("narrow must be torch.float16 or torch.bfloat16")
         self.min_numel, self.min_saving, self.narrow = min_numel, min_saving, narrow
         self.arena = self.cursor = None
-        self.statuses: list = []
-        self.loose_statuses: list = []   # status words of bitmap-only calls (BT_ERR_CAPACITY expected)
+        self.statuses = _StatusWords()
+        self.loose_statuses = _StatusWords()   # those of bitmap-only calls (BT_ERR_CAPACITY expected)
         if arena_bytes is not None:
             self.arena = torch.empty((arena_bytes + 15) // 16 * 16, dtype=torch.uint8, device=device)
             self.cursor = torch.zeros(1, dtype=torch.int64, device=device)
@@ -255,17 +356,13 @@ class stash_saved_activations(torch.autograd.graph.saved_tensors_hooks):
                 and not isinstance(t, torch.nn.Parameter) and not (t.requires_grad and t.is_leaf))
 
     def check_statuses(self) -> None:
-        """One host read for all status words collected so far; raises if an arena stash did not fit or a call
-        failed."""
+        """Reads all status words collected so far; raises if an arena stash did not fit or a call failed."""
         if self.loose_statuses:
-            words = torch.cat(self.loose_statuses)
-            self.loose_statuses.clear()
-            bad = words[(words != B.BT_OK) & (words != B.BT_ERR_CAPACITY)]
-            if bad.numel():
-                raise RuntimeError("a bitmap-only stash call failed: %s" % B.BitTrainError("bt_relu_fwd_compress", int(bad[0].item())))
+            bad = [w for w in self.loose_statuses.drain() if w not in (B.BT_OK, B.BT_ERR_CAPACITY)]
+            if bad:
+                raise RuntimeError("a bitmap-only stash call failed: %s" % B.BitTrainError("bt_relu_fwd_compress", bad[0]))
         if self.statuses:
-            worst = int(torch.cat(self.statuses).max().item())
-            self.statuses.clear()
+            worst = max(self.statuses.drain())
             if worst != B.BT_OK:
                 raise RuntimeError("stash arena too small or a stash call failed: %s" %
                                    B.BitTrainError("bt_*_arena", worst))
@@ -278,16 +375,15 @@ class stash_saved_activations(torch.autograd.graph.saved_tensors_hooks):
             return shared
         n, es = t.numel(), t.element_size()
         if self.arena is not None:
-            bitmap, prefix, nnz_word, off_word, stored = _compress_arena(t.detach().view(-1), self)
-            packed = PackedActivation(bitmap, None, prefix, tuple(t.shape), t.dtype, t.device, nnz_word,
-                                      arena=self.arena, offset=off_word, owner=self, stored=stored)
+            record, stored = _compress_arena(t, self)
+            packed = _packed_arena(t, record, self, stored)
             self.share(t, packed)
             self.dense_bytes += n * es
             return packed
-        bitmap, values, prefix, nnz = _compress(t.detach().view(-1), self.scratch, narrow=self.narrow)
+        record, values, nnz = _compress(t, self.scratch, narrow=self.narrow)
         if B.bt_compressed_bytes(n, nnz, values.dtype) > (1.0 - self.min_saving) * n * es:
             return t                                  # too few zeros: the stash would not be smaller
-        packed = PackedActivation(bitmap, values, prefix, tuple(t.shape), t.dtype, t.device, nnz)
+        packed = _packed(t, record, values, nnz)
         self.share(t, packed)
         self.packed_bytes += packed.nbytes()
         self.dense_bytes += n * es
@@ -327,33 +423,31 @@ class ReLUStash(torch.autograd.Function):
             # nobody will ask for the activation again (e.g. it only feeds a pooling layer that keeps winner codes):
             # the bitmap is all this ReLU's backward pass needs, so the values are not stored at all
             n, dev = xc.numel(), xc.device
-            bitmap = torch.empty((n + 31) // 32, dtype=torch.int32, device=dev)
-            prefix = torch.empty((n + B.CHUNK - 1) // B.CHUNK, dtype=torch.int64, device=dev)
-            nnz_out = torch.empty(1, dtype=torch.int64, device=dev)
-            status = torch.empty(1, dtype=torch.int32, device=dev)
+            record = _Record(n, dev, words=2)
+            statuses = hooks.loose_statuses if hooks is not None else _StatusWords()
             scratch = hooks.scratch if hooks is not None else _Scratch()
-            B.bt_relu_fwd_compress(xc.view(-1), y.view(-1), bitmap, None, prefix, nnz_out, scratch.workspace(n, dev), status,
-                                   n=n, values_capacity=0)
-            if hooks is not None:
-                hooks.loose_statuses.append(status)     # BT_ERR_CAPACITY is the expected answer here
-            elif int(status.item()) not in (B.BT_OK, B.BT_ERR_CAPACITY):
-                raise B.BitTrainError("bt_relu_fwd_compress (bitmap only)", int(status.item()))
-            ctx.save_for_backward(bitmap)
+            at, ws = record.buf.data_ptr(), scratch.workspace(n, dev)
+            st = B._calls().bt_relu_fwd_compress(xc, n, B.DTYPE_CODE[xc.dtype], y, at, None, 0, at + _prefix_at(n),
+                                                 at + _words_at(n), ws, ws.numel(), statuses.next(dev), B._stream(None))
+            B._check("bt_relu_fwd_compress (bitmap only)", st, True)
+            if hooks is None:                           # BT_ERR_CAPACITY is the expected answer here
+                st = statuses.drain()[0]
+                if st not in (B.BT_OK, B.BT_ERR_CAPACITY):
+                    raise B.BitTrainError("bt_relu_fwd_compress (bitmap only)", st)
+            ctx.save_for_backward(record.buf)
             return y
         if hooks is not None and hooks.arena is not None:
-            bitmap, prefix, nnz_word, off_word, stored = _compress_arena(xc.view(-1), hooks, relu_into=y.view(-1))
-            ctx.save_for_backward(bitmap)
-            hooks.share(y, PackedActivation(bitmap, None, prefix, tuple(y.shape), y.dtype, y.device, nnz_word,
-                                            arena=hooks.arena, offset=off_word, owner=hooks, stored=stored))
+            record, stored = _compress_arena(xc, hooks, relu_into=y)
+            ctx.save_for_backward(record.buf)
+            hooks.share(y, _packed_arena(y, record, hooks, stored))
             hooks.dense_bytes += y.numel() * y.element_size()
             return y
         scratch = hooks.scratch if hooks is not None else _Scratch()
-        bitmap, values, prefix, nnz = _compress(xc.view(-1), scratch, relu_into=y.view(-1),
-                                                narrow=hooks.narrow if hooks is not None else None)
-        ctx.save_for_backward(bitmap)     # released with the graph, like any saved tensor
+        record, values, nnz = _compress(xc, scratch, relu_into=y, narrow=hooks.narrow if hooks is not None else None)
+        ctx.save_for_backward(record.buf)     # released with the graph, like any saved tensor
         if hooks is not None:
             # the next layer will save y as its input: hand it this stash instead of compressing y again
-            packed = PackedActivation(bitmap, values, prefix, tuple(y.shape), y.dtype, y.device, nnz)
+            packed = _packed(y, record, values, nnz)
             hooks.share(y, packed)
             hooks.packed_bytes += packed.nbytes()
             hooks.dense_bytes += y.numel() * y.element_size()
@@ -361,11 +455,8 @@ class ReLUStash(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, grad: torch.Tensor):
-        g = _flat_input(grad)
-        gin = torch.empty_like(g)
-        (bitmap,) = ctx.saved_tensors
-        B.bt_relu_bwd_from_bitmap(bitmap, g.view(-1), gin.view(-1))
-        return gin, None, None, None
+        (buf,) = ctx.saved_tensors
+        return _relu_bwd(buf, grad), None, None, None
 
 
 def relu_stash(x: torch.Tensor, hooks: Optional[stash_saved_activations] = None, inplace: bool = False,
@@ -393,19 +484,17 @@ class ReLU6Stash(torch.autograd.Function):
             y = torch.empty_like(xc)
         ctx.owner = None
         if hooks is not None and hooks.arena is not None:
-            bitmap, prefix, nnz_word, off_word, stored = _compress_arena(xc.view(-1), hooks, relu_into=y.view(-1),
-                                                                         relu6=True)
+            record, stored = _compress_arena(xc, hooks, relu_into=y, relu6=True)
             ctx.owner = hooks
-            ctx.save_for_backward(bitmap, off_word, prefix)
-            hooks.share(y, PackedActivation(bitmap, None, prefix, tuple(y.shape), y.dtype, y.device, nnz_word,
-                                            arena=hooks.arena, offset=off_word, owner=hooks, stored=stored))
+            ctx.save_for_backward(record.buf)
+            hooks.share(y, _packed_arena(y, record, hooks, stored))
             hooks.dense_bytes += y.numel() * y.element_size()
             return y
         scratch = hooks.scratch if hooks is not None else _Scratch()
-        bitmap, values, prefix, nnz = _compress(xc.view(-1), scratch, relu_into=y.view(-1), relu6=True)
-        ctx.save_for_backward(bitmap, values, prefix)
+        record, values, nnz = _compress(xc, scratch, relu_into=y, relu6=True)
+        ctx.save_for_backward(record.buf, values)
         if hooks is not None:
-            packed = PackedActivation(bitmap, values, prefix, tuple(y.shape), y.dtype, y.device, nnz)
+            packed = _packed(y, record, values, nnz)
             hooks.share(y, packed)
             hooks.packed_bytes += packed.nbytes()
             hooks.dense_bytes += y.numel() * y.element_size()
@@ -415,12 +504,18 @@ class ReLU6Stash(torch.autograd.Function):
     def backward(ctx, grad: torch.Tensor):
         g = _flat_input(grad)
         gin = torch.empty_like(g)
-        bitmap, values, prefix = ctx.saved_tensors
-        if ctx.owner is not None:                      # arena mode: `values` is the offset word
+        n, calls, code = g.numel(), B._calls(), B.DTYPE_CODE[g.dtype]
+        if ctx.owner is not None:                      # arena mode: the record holds the offset word
+            (buf,) = ctx.saved_tensors
             ctx.owner.check_statuses()
-            B.bt_relu6_bwd_from_stash_arena(bitmap, ctx.owner.arena, values, prefix, g.view(-1), gin.view(-1))
+            at = buf.data_ptr()
+            st = calls.bt_relu6_bwd_from_stash_arena(at, ctx.owner.arena, at + _words_at(n) + 8, at + _prefix_at(n), g, n, code,
+                                                     gin, B._stream(None))
         else:
-            B.bt_relu6_bwd_from_stash(bitmap, values, prefix, g.view(-1), gin.view(-1))
+            buf, values = ctx.saved_tensors
+            at = buf.data_ptr()
+            st = calls.bt_relu6_bwd_from_stash(at, values, at + _prefix_at(n), g, n, code, gin, B._stream(None))
+        B._check("bt_relu6_bwd_from_stash", st, True)
         return gin, None, None
 
 
@@ -443,8 +538,7 @@ class DoubleMask(torch.autograd.Function):
         if src is None or src.arena is not None or src.values.dtype != like.dtype:
             # no reusable stash of `like` (none yet, or one whose size only the device knows): make one
             scratch = hooks.scratch if hooks is not None else _Scratch()
-            bitmap, values, prefix, nnz = _compress(_flat_input(like.detach()).view(-1), scratch)
-            src = PackedActivation(bitmap, values, prefix, tuple(like.shape), like.dtype, like.device, nnz)
+            src = _packed(like, *_compress(_flat_input(like.detach()), scratch))
         if inplace and _usable(out):
             xc = y = out
             ctx.mark_dirty(out)
@@ -453,10 +547,9 @@ class DoubleMask(torch.autograd.Function):
             y = torch.empty_like(xc)
         values = torch.empty(max(src.nnz, 1), dtype=out.dtype, device=out.device)
         B.bt_mask_compress(xc.view(-1), src.bitmap, src.chunk_prefix, y.view(-1), values, values_capacity=src.nnz)
-        ctx.save_for_backward(src.bitmap)
+        ctx.save_for_backward(src.record.buf)
         if hooks is not None:
-            packed = PackedActivation(src.bitmap, values[:src.nnz], src.chunk_prefix, tuple(y.shape), y.dtype, y.device,
-                                      src.nnz)
+            packed = _packed(y, src.record, values[:src.nnz], src.nnz)
             hooks.share(y, packed)
             hooks.packed_bytes += src.nnz * y.element_size()          # bitmap and prefix are the source's
             hooks.dense_bytes += y.numel() * y.element_size()
@@ -464,11 +557,8 @@ class DoubleMask(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, grad: torch.Tensor):
-        g = _flat_input(grad)
-        gin = torch.empty_like(g)
-        (bitmap,) = ctx.saved_tensors
-        B.bt_relu_bwd_from_bitmap(bitmap, g.view(-1), gin.view(-1))
-        return gin, None, None, None
+        (buf,) = ctx.saved_tensors
+        return _relu_bwd(buf, grad), None, None, None
 
 
 def double_mask(out: torch.Tensor, like: torch.Tensor, hooks: Optional[stash_saved_activations] = None,
@@ -523,22 +613,19 @@ class ReLUMaxPool2x2Stash(torch.autograd.Function):
         y = torch.empty(xc.shape[:-2] + (xc.shape[-2] // 2, xc.shape[-1] // 2), dtype=x.dtype, device=x.device)
         codes = torch.empty((y.numel() + 15) // 16, dtype=torch.int32, device=x.device)
         B.bt_maxpool2x2_fwd(xc, y, codes)
-        flat = y.view(-1)
         if hooks is not None and hooks.arena is not None:
-            bitmap, prefix, nnz_word, off_word, stored = _compress_arena(flat, hooks, relu_into=flat)
-            hooks.share(y, PackedActivation(bitmap, None, prefix, tuple(y.shape), y.dtype, y.device, nnz_word,
-                                            arena=hooks.arena, offset=off_word, owner=hooks, stored=stored))
+            record, stored = _compress_arena(y, hooks, relu_into=y)
+            hooks.share(y, _packed_arena(y, record, hooks, stored))
             hooks.dense_bytes += y.numel() * y.element_size()
         else:
             scratch = hooks.scratch if hooks is not None else _Scratch()
-            bitmap, values, prefix, nnz = _compress(flat, scratch, relu_into=flat,
-                                                    narrow=hooks.narrow if hooks is not None else None)
+            record, values, nnz = _compress(y, scratch, relu_into=y, narrow=hooks.narrow if hooks is not None else None)
             if hooks is not None:
-                packed = PackedActivation(bitmap, values, prefix, tuple(y.shape), y.dtype, y.device, nnz)
+                packed = _packed(y, record, values, nnz)
                 hooks.share(y, packed)
                 hooks.packed_bytes += packed.nbytes()
                 hooks.dense_bytes += y.numel() * y.element_size()
-        ctx.save_for_backward(codes, bitmap)
+        ctx.save_for_backward(codes, record.buf)
         ctx.in_shape = tuple(xc.shape)
         return y
 
