@@ -299,7 +299,8 @@ __global__ void __launch_bounds__((kWorkers + 3) * 32) compress_kernel(const Com
 
     // ---------------------------------------------------------------- workers
     OneTensor<U, Stored<CAST, U>, kTile, CtaState<kSegs, kStages>> stream{a, sh, num_tiles, cta, G};
-    if (!work<U, FUSED, WRITE_Y, CAST, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, a.tau, wait_ns) && lane == 0)
+    if (!work<U, FUSED, WRITE_Y, CAST, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, a.tau, wait_ns,
+                                                                               a.capacity != 0 || a.arena_cursor) && lane == 0)
         raise_timeout(a.ws_header, a.dev_status, &sh.abort, sh.tag);
 }
 

@@ -430,7 +430,7 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
     // ---------------------------------------------------------------- workers
     ManyTensors<U, kTile, kJobs, CtaState<kSegs, kStages>> stream{p, sh, cta, G, {}, 0};
     walk_begin(stream.w, p, cta, G);
-    if (!work<U, FUSED, WRITE_Y, 0, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, p.c.tau, wait_ns) && lane == 0)
+    if (!work<U, FUSED, WRITE_Y, 0, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, p.c.tau, wait_ns, true) && lane == 0)
         raise_timeout(p, &sh.abort, sh.tag);
 }
 

@@ -528,7 +528,8 @@ struct TileOut {
 
 // One worker warp of a CTA (worker w of kWorkers): takes the segments w, w + kWorkers, w + 2 kWorkers, ... of the CTA's
 // stream of tiles -- into registers, flags, ranks, count posted, packed into its own ring in shared memory -- and copies
-// each out once its base is known, a few tiles later.  False if a wait ran out.
+// each out once its base is known, a few tiles later.  `pack`: false where no values are wanted (a capacity of 0: the call
+// is made for bitmap, prefix and count), then neither packing nor copying takes place.  False if a wait ran out.
 //
 // Every worker does everything, so that what one waits for (a shuffle, a shared load, a base) is filled by the others;
 // a warp's chain of dependent steps per segment is about 1500 cycles, as long as a tile takes at full bandwidth, and
@@ -540,7 +541,7 @@ struct TileOut {
 // only make it wait for segments at least 2 tiles back, because the ring holds the segments nearer than that: kNear.)
 template <typename U, int FUSED, bool WRITE_Y, int CAST, int kSegs, int kWorkers, int kStages, int kRing, typename Stream>
 __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, const uint32_t ring, const uint32_t w, const uint32_t lane,
-                                     Stream &stream, const float tau, const uint64_t wait_ns)
+                                     Stream &stream, const float tau, const uint64_t wait_ns, const bool pack)
 {
     using V                  = Stored<CAST, U>;
     constexpr int      kE    = Rows<U>::kE;
@@ -621,8 +622,9 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
             rank_rows(ranks[h], flags[h]);
             run += ranks[h].count();
         }
-        // the count first: the exchange of counts waits for nothing else
-        if (it >= static_cast<uint32_t>(kQueue) && !mbar_wait(&sh.done[q], ((it / kQueue) - 1) & 1u, &sh.abort, wait_ns)) return false;
+        // the count first: the exchange of counts waits for nothing else (without values to copy out, a place in the queue
+        // is free again once the scan is done with it)
+        if (it >= static_cast<uint32_t>(kQueue) && !mbar_wait(pack ? &sh.done[q] : &sh.ready[q], ((it / kQueue) - 1) & 1u, &sh.abort, wait_ns)) return false;
         if (lane == 0) {
             sh.cnt[q][seg] = run;
             mbar_arrive(&sh.counted[q]);
@@ -635,6 +637,7 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
                 if (wd < ((t.n + 31) >> 5) && extent_of(t.bitmap, 4 * ((t.n + 31) >> 5)).holds(t.bitmap + wd, 4)) t.bitmap[wd] = word;
             }
         }
+        if (!pack) continue;
         // room in the ring: the pending segments lie one behind the other from the oldest one to `head`, each in one
         // piece, so the end of the ring may stay unused
         const uint32_t need = run ? (run * kES + 15u) & ~15u : 16u;
