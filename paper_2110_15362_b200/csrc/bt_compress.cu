@@ -67,7 +67,7 @@ struct OneTensor {
 // CAST: 0, or the 16-bit type the kept binary32 values are narrowed to (1 binary16, 2 bfloat16).
 // kSegs segments per tile, kWorkers worker warps, kStages slots of the input ring, kRing bytes of packed values per worker.
 template <typename U, int FUSED, bool WRITE_Y, int CAST, int kSegs, int kWorkers, int kStages, int kRing>
-__global__ void __launch_bounds__((kWorkers + 3) * 32) compress_kernel(const CompressArgs a, const uint32_t num_tiles)
+__global__ void __launch_bounds__((kWorkers + 3 + WRITE_Y) * 32) compress_kernel(const CompressArgs a, const uint32_t num_tiles)
 {
     constexpr int kSeg          = Rows<U>::kSeg;
     constexpr int kTile         = kSegs * kSeg;
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__((kWorkers + 3) * 32) compress_kernel(const Com
     constexpr int kSegsPerChunk = BT_CHUNK_ELEMS / kSeg;
     // warp roles
     constexpr int kScanWarp = kWorkers;                   // and kScanWarp + 1
-    constexpr int kLoadWarp = kWorkers + 2;
+    constexpr int kLoadWarp = kWorkers + 2;               // and, with the dense output, a store warp behind it
     static_assert(BT_CHUNK_ELEMS % kSeg == 0 && kTile % BT_CHUNK_ELEMS == 0, "segments tile a chunk, chunks a tile");
     static_assert(kSegs <= 32, "one lane per segment count");
 
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__((kWorkers + 3) * 32) compress_kernel(const Com
 
     // The arena's cursor is read before the barrier below: the kernel's one update of it follows the last tile's base,
     // which needs a publication from every CTA, and a CTA publishes only after this barrier.
-    if (tid == 0) sh.init();
+    if (tid == 0) sh.init(WRITE_Y);
     in_stream_order();
     if (tid == 0) sh.arena_c0 = a.arena_cursor ? *reinterpret_cast<const volatile uint64_t *>(a.arena_cursor) : 0;
     __syncthreads();
@@ -297,8 +297,15 @@ __global__ void __launch_bounds__((kWorkers + 3) * 32) compress_kernel(const Com
         return;
     }
 
-    // ---------------------------------------------------------------- workers
     OneTensor<U, Stored<CAST, U>, kTile, CtaState<kSegs, kStages>> stream{a, sh, num_tiles, cta, G};
+    if constexpr (WRITE_Y) {
+        if (warp == kLoadWarp + 1) {
+            if (!store_dense<U>(sh, tiles, lane, stream, wait_ns) && lane == 0) raise_timeout(a.ws_header, a.dev_status, &sh.abort, sh.tag);
+            return;
+        }
+    }
+
+    // ---------------------------------------------------------------- workers
     if (!work<U, FUSED, WRITE_Y, CAST, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, a.tau, wait_ns,
                                                                                a.capacity != 0 || a.arena_cursor) && lane == 0)
         raise_timeout(a.ws_header, a.dev_status, &sh.abort, sh.tag);
@@ -340,7 +347,7 @@ template <typename U, int FUSED, bool WRITE_Y, int CAST, int kSegs, int kWorkers
 cudaError_t launch_shaped(const CompressArgs &a, cudaStream_t stream)
 {
     constexpr int kTile    = kSegs * Rows<U>::kSeg;
-    constexpr int kThreads = (kWorkers + 3) * 32;
+    constexpr int kThreads = (kWorkers + 3 + WRITE_Y) * 32;
     constexpr size_t kSmem = static_cast<size_t>(kStages) * kTile * sizeof(U) + static_cast<size_t>(kWorkers) * kRing;
     static LaunchShape shape;   // one per instantiation
     auto kernel = compress_kernel<U, FUSED, WRITE_Y, CAST, kSegs, kWorkers, kStages, kRing>;

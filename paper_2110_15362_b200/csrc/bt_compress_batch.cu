@@ -128,7 +128,7 @@ struct ManyTensors {
 // kJobs: room for tensors in the kernel's parameters.
 // kSegs segments per tile, kWorkers worker warps, kStages slots of the input ring, kRing bytes of packed values per worker.
 template <typename U, int FUSED, bool WRITE_Y, int kJobs, int kSegs, int kWorkers, int kStages, int kRing>
-__global__ void __launch_bounds__((kWorkers + 3) * 32)
+__global__ void __launch_bounds__((kWorkers + 3 + WRITE_Y) * 32)
 compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
 {
     constexpr int kSeg           = Rows<U>::kSeg;
@@ -137,7 +137,7 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
     constexpr int kSegsPerChunk  = BT_CHUNK_ELEMS / kSeg;
     // warp roles
     constexpr int kScanWarp = kWorkers;                   // and kScanWarp + 1
-    constexpr int kLoadWarp = kWorkers + 2;
+    constexpr int kLoadWarp = kWorkers + 2;               // and, with the dense output, a store warp behind it
     static_assert(BT_CHUNK_ELEMS % kSeg == 0 && kTile % BT_CHUNK_ELEMS == 0, "segments tile a chunk, chunks a tile");
     static_assert(kSegs <= 32, "one lane per segment count");
 
@@ -157,7 +157,7 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
     // The arena's cursor is read before the barrier below: the launch's first update of it follows a tensor's last base,
     // which needs a publication from every CTA in front of it, and the sequence number moves only behind all of them.
     const bool in_arena = p.c.arena != nullptr;
-    if (tid == 0) sh.init();
+    if (tid == 0) sh.init(WRITE_Y);
     in_stream_order();
     if (tid == 0) sh.arena_c0 = in_arena ? *reinterpret_cast<const volatile uint64_t *>(p.c.arena_cursor) : 0;
     __syncthreads();
@@ -427,9 +427,16 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
         return;
     }
 
-    // ---------------------------------------------------------------- workers
     ManyTensors<U, kTile, kJobs, CtaState<kSegs, kStages>> stream{p, sh, cta, G, {}, 0};
     walk_begin(stream.w, p, cta, G);
+    if constexpr (WRITE_Y) {
+        if (warp == kLoadWarp + 1) {
+            if (!store_dense<U>(sh, tiles, lane, stream, wait_ns) && lane == 0) raise_timeout(p, &sh.abort, sh.tag);
+            return;
+        }
+    }
+
+    // ---------------------------------------------------------------- workers
     if (!work<U, FUSED, WRITE_Y, 0, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, p.c.tau, wait_ns, true) && lane == 0)
         raise_timeout(p, &sh.abort, sh.tag);
 }
@@ -438,7 +445,7 @@ template <typename U, int FUSED, bool WRITE_Y, int kJobs, int kSegs, int kWorker
 cudaError_t launch_shaped(const CompressCommon &c, const CompressJob *jobs, uint32_t count, void *workspace, cudaStream_t stream)
 {
     constexpr int    kTile    = kSegs * Rows<U>::kSeg;
-    constexpr int    kThreads = (kWorkers + 3) * 32;
+    constexpr int    kThreads = (kWorkers + 3 + WRITE_Y) * 32;
     constexpr size_t kSmem    = static_cast<size_t>(kStages) * kTile * sizeof(U) + static_cast<size_t>(kWorkers) * kRing;
     static LaunchShape shape;   // one per instantiation
     auto kernel = compress_kernel<U, FUSED, WRITE_Y, kJobs, kSegs, kWorkers, kStages, kRing>;

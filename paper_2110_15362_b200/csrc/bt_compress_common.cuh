@@ -186,12 +186,11 @@ __device__ __forceinline__ uint32_t relu6_saturates_pair(const uint32_t x)
     return m;
 }
 
-// The flag word of the lane's elements of a block (x: its rows, y: its dense output); the fused forms replace the elements by their forward value on the way (the
-// forms decided by one compare leave elements that are not kept as they are: their flag is clear) and, with WRITE_Y,
-// store it (kGuardY: only the first yvalid elements of the block exist).
-template <typename U, int FUSED, bool WRITE_Y, bool kGuardY>
-__device__ __forceinline__ uint32_t flag_rows(uint32_t (&rows)[8][Rows<U>::kRegs], const uint32_t lane, U *y, const uint32_t yvalid, const float tau,
-                                              const Extent yx)
+// The flag word of the lane's elements of a block (its rows); the fused forms replace the elements by their forward value
+// on the way (the forms decided by one compare leave elements that are not kept as they are: their flag is clear) and,
+// with WRITE_Y, put it in the elements' place in the input slot (`slot`: shared address of the block).
+template <typename U, int FUSED, bool WRITE_Y>
+__device__ __forceinline__ uint32_t flag_rows(uint32_t (&rows)[8][Rows<U>::kRegs], const uint32_t lane, const uint32_t slot, const float tau)
 {
     using R                = Rows<U>;
     constexpr bool kDirect = FUSED >= kFusedReluDirect;
@@ -251,22 +250,11 @@ __device__ __forceinline__ uint32_t flag_rows(uint32_t (&rows)[8][Rows<U>::kRegs
             }
         }
         if constexpr (WRITE_Y) {
-            const uint32_t e = static_cast<uint32_t>(r * 32 * R::kE) + lane * R::kE;       // the lane's first element of the row
-            if (!kGuardY || e + R::kE <= yvalid) {
-                if (yx.holds(y + e, R::kE * sizeof(U))) {
-                    if constexpr (R::kRegs == 4) *reinterpret_cast<uint4 *>(y + e) = make_uint4(yv[0], yv[1], yv[2], yv[3]);
-                    else *reinterpret_cast<uint2 *>(y + e) = make_uint2(yv[0], yv[1]);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < R::kE; ++j) {
-                    U v;
-                    if constexpr (sizeof(U) == 2) v = static_cast<U>(yv[j >> 1] >> (16 * (j & 1)));
-                    else if constexpr (sizeof(U) == 4) v = yv[j];
-                    else v = yv[2 * j] | (static_cast<uint64_t>(yv[2 * j + 1]) << 32);
-                    if (e + j < yvalid && yx.holds(y + e + j, sizeof(U))) y[e + j] = v;
-                }
-            }
+            const uint32_t at = slot + static_cast<uint32_t>(r) * (128u * R::kRegs) + lane * (4u * R::kRegs);
+            if constexpr (R::kRegs == 4)
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(yv[0]), "r"(yv[1]), "r"(yv[2]), "r"(yv[3]) : "memory");
+            else
+                asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(yv[0]), "r"(yv[1]) : "memory");
         }
     }
     return acc[0] | (acc[1] << 8) | (acc[2] << 16) | (acc[3] << 24);
@@ -476,13 +464,15 @@ __device__ __forceinline__ void copy_out_clipped(const uint32_t from, const uint
 
 // ---------------------------------------------------------------------------------------------
 // Shared memory of a CTA besides the ring of tiles and the worker warps' rings of packed values.  A tile goes round
-// through five mbarriers: its ring slot through `full` and `empty`, its place in the queue of the last kQueue tiles
-// through `counted`, `ready` and `done`.
+// through five mbarriers: its ring slot through `full` and `empty` (forms with the dense output: `written` in between),
+// its place in the queue of the last kQueue tiles through `counted`, `ready` and `done`.
 constexpr int kQueue = 8;   // tiles of a CTA between their count and the end of their copy-out
 template <int kSegs, int kStages>
 struct CtaState {
     uint64_t full[kStages];           // the bulk copy of the tile has landed               (copy engine -> workers)
-    uint64_t empty[kStages];          // every segment of the tile is in registers          (workers -> load warp)
+    uint64_t empty[kStages];          // every segment of the tile is in registers          (workers -> load warp),
+                                      // or the dense output has left the slot              (store warp -> load warp)
+    uint64_t written[kStages];        // the dense output is in the slot                    (workers -> store warp)
     uint64_t counted[kQueue];         // every segment's count is posted                    (workers -> scan warps)
     uint64_t ready[kQueue];           // base and offsets are in shared                     (scan warps -> workers)
     uint64_t done[kQueue];            // every segment has been copied out                  (workers -> workers)
@@ -497,11 +487,11 @@ struct CtaState {
     uint64_t          arena_c0;       // arena forms: the cursor as the launch found it
     volatile uint32_t abort;
     // by one thread; a CTA-wide barrier follows
-    __device__ __forceinline__ void init()
+    __device__ __forceinline__ void init(const bool dense_output)
     {
         abort = 0;
         tag   = 0;
-        for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], kSegs);
+        for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], dense_output ? 1 : kSegs), mbar_init(&written[s], kSegs);
         for (int q = 0; q < kQueue; ++q) mbar_init(&counted[q], kSegs), mbar_init(&ready[q], 1), mbar_init(&done[q], kSegs);
         fence_proxy_async();
     }
@@ -600,8 +590,10 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
         // the segment into registers; the slot is free for the next tile once every segment is
         Rows<U> rows;
         load_rows<U>(rows, smem_addr(tile + seg * kSeg), lane);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.empty[s]);
+        if constexpr (!WRITE_Y) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.empty[s]);
+        }
 
         const uint64_t e0 = t.first + seg * kSeg;                   // first element of the segment
         constexpr int  kBlocks = Rows<U>::kBlocks, kBlock = Rows<U>::kBlock;
@@ -609,18 +601,14 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
         RowRanks       ranks[kBlocks];
 #pragma unroll
         for (int h = 0; h < kBlocks; ++h) {
-            if constexpr (WRITE_Y) {
-                const uint64_t b0     = e0 + h * kBlock;            // first element of the block
-                U *const       y      = static_cast<U *>(t.y) + b0;
-                const Extent   yx     = extent_of(t.y, t.n * sizeof(U));
-                const uint32_t yvalid = b0 + kBlock <= t.n ? static_cast<uint32_t>(kBlock) : (b0 < t.n ? static_cast<uint32_t>(t.n - b0) : 0u);
-                if (yvalid == static_cast<uint32_t>(kBlock)) flags[h] = flag_rows<U, FUSED, true, false>(rows.x[h], lane, y, yvalid, tau, yx);
-                else flags[h] = flag_rows<U, FUSED, true, true>(rows.x[h], lane, y, yvalid, tau, yx);
-            } else {
-                flags[h] = flag_rows<U, FUSED, false, false>(rows.x[h], lane, nullptr, 0, tau, extent_of(nullptr, 0));
-            }
+            flags[h] = flag_rows<U, FUSED, WRITE_Y>(rows.x[h], lane, smem_addr(tile + seg * kSeg + h * kBlock), tau);
             rank_rows(ranks[h], flags[h]);
             run += ranks[h].count();
+        }
+        if constexpr (WRITE_Y) {
+            fence_proxy_async();                                    // the copy engine reads the dense output next
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.written[s]);
         }
         // the count first: the exchange of counts waits for nothing else (without values to copy out, a place in the queue
         // is free again once the scan is done with it)
@@ -678,6 +666,39 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
     }
     while (pending)
         if (!copy_oldest()) return false;
+    return true;
+}
+
+// The store warp of the forms with the dense output: sends every tile off from its slot, whole 16-byte units by ONE bulk
+// copy, and hands the slot back.  Stored by the workers themselves, 4 KB here and 4 KB there, the same bytes are slower
+// than in one piece (fp32 2^28 at half zeros 422 us against 418, fp32 2^25 without values 52.9 against 50.4, bf16
+// [61,144,57,55] 31.6 against 30.5).  False if a wait ran out.
+template <typename U, int kSegs, int kStages, typename Stream>
+__device__ __forceinline__ bool store_dense(CtaState<kSegs, kStages> &sh, const U *tiles, const uint32_t lane, Stream &stream, const uint64_t wait_ns)
+{
+    constexpr uint32_t kTile = kSegs * Rows<U>::kSeg;
+    TileIn t;
+    for (uint32_t it = 0; stream.seek(it, t); ++it) {
+        const uint32_t s    = it % kStages;
+        const U *const tile = tiles + static_cast<size_t>(s) * kTile;
+        if (!mbar_wait(&sh.written[s], (it / kStages) & 1u, &sh.abort, wait_ns)) return false;
+        const uint64_t left  = t.n - t.first;
+        const uint32_t have  = left < kTile ? static_cast<uint32_t>(left) : kTile;
+        const uint32_t whole = (have * static_cast<uint32_t>(sizeof(U))) & ~15u;
+        U *const       y     = static_cast<U *>(t.y) + t.first;
+        const Extent   yx    = extent_of(t.y, t.n * sizeof(U));
+        if (lane == 0 && whole && yx.holds(y, whole)) {
+            bulk_store(y, tile, whole);
+            bulk_commit();
+        }
+        const uint32_t e = whole / static_cast<uint32_t>(sizeof(U)) + lane;       // behind the last whole unit
+        if (e < have && yx.holds(y + e, sizeof(U))) y[e] = tile[e];
+        __syncwarp();
+        if (lane == 0) {
+            bulk_wait_read<0>();
+            mbar_arrive(&sh.empty[s]);
+        }
+    }
     return true;
 }
 
