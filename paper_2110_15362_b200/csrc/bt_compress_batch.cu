@@ -96,6 +96,12 @@ __device__ __forceinline__ void walk_next(Walk &w, const CompressParams<kJobs> &
     }
 }
 
+// values of `size` bytes that fit behind a cursor of an arena
+__device__ __forceinline__ uint64_t arena_room(const uint64_t cursor, const uint64_t bytes, const uint32_t size)
+{
+    return cursor <= bytes ? (bytes - cursor) / size : 0;
+}
+
 // The tiles of a CTA of a batched launch, as `work` takes them.
 template <typename U, int kTile, int kJobs, typename State>
 struct ManyTensors {
@@ -119,7 +125,7 @@ struct ManyTensors {
             return TileOut{j.values, j.capacity};
         }
         const uint64_t at0 = sh.dst[q];
-        return TileOut{static_cast<unsigned char *>(p.c.arena) + at0, at0 <= p.c.arena_bytes ? (p.c.arena_bytes - at0) / sizeof(U) : 0};
+        return TileOut{static_cast<unsigned char *>(p.c.arena) + at0, arena_room(at0, p.c.arena_bytes, sizeof(U))};
     }
 };
 
@@ -243,8 +249,6 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
         walk_begin(cur, p, cta, G);
         if (q == 1 && cur.valid) walk_next(cur, p, cta, G);
         uint32_t pk = 0, pj = 0, pv = 0;            // this warp's previous tile: tensor, wave, virtual CTA
-        uint64_t arena_at     = 0;                  // arena form: byte offset of the values of tensor arena_of ...
-        uint32_t arena_of     = 0xFFFFFFFFu;        // ... (none yet)
 
         for (uint32_t i = q; !failed && i <= last_i + 2; i += 2) {
             const bool has = i <= last_i;
@@ -294,47 +298,51 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
                             ld_relaxed_2xu64(desc + 2 * (from + lane + 32u * k), d0[k], d1[k]);
                 }
                 if (failed) break;
-                uint32_t part = 0;                                   // at most 160 tiles of 16384 elements
+                const uint64_t pt = pv + static_cast<uint64_t>(pj) * G;
+                if ((in_arena ? i > 2 : pj > 0) && !mbar_wait(&sh.ready[(i - 3) % kQueue], ((i - 3) / kQueue) & 1u, &sh.abort, wait_ns)) {
+                    failed = true;
+                    break;
+                }
+                // the sum of the window's counts from descriptor lo to before hi: at most 160 tiles of 16384 elements
+                auto counts = [&](const uint64_t lo, const uint64_t hi) {
+                    uint32_t part = 0;
 #pragma unroll
-                for (int k = 0; k < kMaxWindows; ++k) part += static_cast<uint32_t>(d0[k]);
-                uint64_t base = __reduce_add_sync(kFull, part);
-                if (pj > 0) {                                        // the CTA's tile before is tile pt - G of the same tensor
-                    if (!mbar_wait(&sh.ready[(i - 3) % kQueue], ((i - 3) / kQueue) & 1u, &sh.abort, wait_ns)) {
-                        failed = true;
-                        break;
+                    for (int k = 0; k < kMaxWindows; ++k) {
+                        const uint64_t at = from + lane + 32u * k;
+                        part += at >= lo && at < hi ? static_cast<uint32_t>(d0[k]) : 0u;
                     }
-                    base += sh.base[(i - 3) % kQueue];
+                    return __reduce_add_sync(kFull, part);
+                };
+                uint64_t base = 0, arena_at = 0;
+                if (!in_arena) {
+                    // the CTA's tile before is tile pt - G of the same tensor, if it is not the first here
+                    base = (pj > 0 ? sh.base[(i - 3) % kQueue] : 0ull) + counts(0, ~0ull);
+                } else {
+                    // Arena form: the tensor's values start where the tensor before it ended.  The window goes back to the
+                    // CTA's tile before, whatever tensor that is in, so every CTA adds up the tensors that end in between by
+                    // itself and nobody waits for a cursor from another CTA (MobileNetV2 layers at batch 2: 70 us with the
+                    // cursors handed on, 38 this way; at batch 64 361 and 351).
+                    uint32_t m = 0;
+                    uint64_t lo = from;
+                    arena_at    = sh.arena_c0;
+                    if (i > 2) m = sh.job[(i - 3) % kQueue], base = sh.base[(i - 3) % kQueue], arena_at = sh.dst[(i - 3) % kQueue];
+                    for (;; ++m) {
+                        const uint64_t end = static_cast<uint64_t>(p.job[m].desc0) + p.job[m].tiles, lin = jb.desc0 + pt;
+                        const uint64_t hi  = end < lin ? end : lin;
+                        base += counts(lo, hi);
+                        lo = hi;
+                        if (m == pk) break;
+                        // tensor m is complete: the cursor moves past it if it fits
+                        if (base <= arena_room(arena_at, p.c.arena_bytes, sizeof(U))) arena_at += (base * sizeof(U) + 15) & ~15ull;
+                        base = 0;
+                    }
                 }
                 const uint32_t ps = (i - 2) % kQueue;
-                const uint64_t pt = pv + static_cast<uint64_t>(pj) * G;
                 // exclusive count in front of each chunk of that tile
                 if (lane < kSegs && (lane % kSegsPerChunk) == 0) {
                     const uint64_t ch = pt * kChunksPerTile + lane / kSegsPerChunk;
                     const uint64_t chunks_total = (jb.n + BT_CHUNK_ELEMS - 1) / BT_CHUNK_ELEMS;
                     if (ch < chunks_total && extent_of(jb.prefix, 8 * chunks_total).holds(jb.prefix + ch, 8)) jb.prefix[ch] = base + sh.off[ps][lane];
-                }
-                // Arena form: the tensor's values start where the tensor before it ended.  That cursor is published,
-                // under the launch's tag, by whoever finishes that tensor's last tile; tensor 0 starts at the cursor
-                // the launch found.  Read once per tensor and warp (bounded, like every wait here).
-                if (in_arena && arena_of != pk) {
-                    uint64_t at = sh.arena_c0;
-                    if (pk > 0) {
-                        const uint64_t *const w = p.c.ws_arena + 2 * (pk - 1);
-                        uint64_t       a0 = 0, a1 = 0;
-                        const uint64_t ta = now_ns();
-                        for (;;) {
-                            ld_relaxed_2xu64(w, a0, a1);
-                            if (((a0 ^ tag_w0) >> 32) == 0 && ((a1 ^ tag_w1) >> 32) == 0) break;
-                            if (now_ns() - ta > wait_ns || ld_relaxed_u64(p.c.ws_header + kHdrAbort) == tag) {
-                                failed = true;
-                                break;
-                            }
-                            __nanosleep(100);
-                        }
-                        if (failed) break;
-                        at = (a0 & 0xFFFFFFFFull) | (a1 << 32);
-                    }
-                    arena_at = at, arena_of = pk;
                 }
                 bool bump = false;              // lane 0: this is the launch's last tile
                 if (pt == jb.tiles - 1 && lane == 0) {
@@ -344,14 +352,11 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
                     const bool aborted  = ld_relaxed_u64(p.c.ws_header + kHdrAbort) == tag;
                     uint64_t   capacity = jb.capacity;
                     if (in_arena) {
-                        // the room behind the tensor's start; the cursor moves past it only when everything fitted
-                        capacity            = arena_at <= p.c.arena_bytes ? (p.c.arena_bytes - arena_at) / sizeof(U) : 0;
-                        const bool     fits = !aborted && nnz <= capacity;
-                        const uint64_t end  = fits ? arena_at + ((nnz * sizeof(U) + 15) & ~15ull) : arena_at;
+                        // the cursor moves past the tensor only when everything fitted
+                        capacity        = arena_room(arena_at, p.c.arena_bytes, sizeof(U));
+                        const bool fits = !aborted && nnz <= capacity;
                         if (fits) *jb.offset_out = arena_at;
-                        if (pk + 1 == p.c.jobs) *p.c.arena_cursor = end;
-                        if (wsx.holds(p.c.ws_arena + 2 * pk, 16))
-                            st_relaxed_2xu64(p.c.ws_arena + 2 * pk, tag_w0 | (end & 0xFFFFFFFFull), tag_w1 | (end >> 32));
+                        if (pk + 1 == p.c.jobs) *p.c.arena_cursor = fits ? arena_at + ((nnz * sizeof(U) + 15) & ~15ull) : arena_at;
                     }
                     bump = pk + 1 == p.c.jobs;
                     if (jb.dev_status) {
@@ -411,8 +416,12 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
                     failed = true;
                     break;
                 }
-                window = cur.tile(G) < G ? cur.tile(G) : G;
-                from   = static_cast<uint64_t>(p.job[cur.k].desc0) + cur.tile(G) - window;
+                // the descriptors in front of the tile back to the CTA's tile before: in the arena form whatever tensor they
+                // belong to, else those of the tile's own tensor
+                const uint64_t lin  = static_cast<uint64_t>(p.job[cur.k].desc0) + cur.tile(G);
+                const uint64_t back = in_arena ? lin : cur.tile(G);
+                window = back < G ? static_cast<uint32_t>(back) : G;
+                from   = lin - window;
 #pragma unroll
                 for (int k = 0; k < kMaxWindows; ++k) {
                     if (lane + 32u * k < window) ld_relaxed_2xu64(desc + 2 * (from + lane + 32u * k), d0[k], d1[k]);
@@ -483,7 +492,6 @@ cudaError_t launch_shaped(const CompressCommon &c, const CompressJob *jobs, uint
     p.c.ws_header = static_cast<uint64_t *>(workspace);
     p.c.ws_desc   = reinterpret_cast<uint64_t *>(static_cast<unsigned char *>(workspace) + kWsHeaderBytes);
     p.c.ws_words  = (batch_workspace_bytes(chunks, count) - kWsHeaderBytes) / 8;
-    p.c.ws_arena  = p.c.ws_desc + 2 * dealt;                          // behind the descriptors: 16-byte aligned like them
     p.c.call_tag  = next_call_tag();
     p.c.wait_ns   = compress_wait_ns();
     // cooperative launch: the runtime guarantees that all `grid` CTAs are resident together

@@ -86,7 +86,6 @@ struct CompressCommon {
     void       *arena;
     uint64_t    arena_bytes;
     uint64_t   *arena_cursor;
-    uint64_t   *ws_arena;   // two tagged words per tensor: the cursor behind that tensor (set by launch_compress_batch)
 };
 
 // What the caller of launch_compress_batch gives for the arena form.
@@ -96,8 +95,7 @@ struct BatchArena {
     uint64_t *arena_cursor;
 };
 
-// bytes of workspace for a batched launch: the tensors' descriptors and totals, and two words per tensor for the
-// arena form's chain of cursors
+// bytes of workspace for a batched launch: the tensors' descriptors, and 16 bytes per tensor to spare
 __host__ __device__ constexpr size_t batch_workspace_bytes(uint64_t chunks, uint32_t count)
 {
     return compress_workspace_bytes(chunks) + 16 * static_cast<size_t>(count);
