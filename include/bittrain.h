@@ -90,12 +90,10 @@ size_t bt_compressed_bytes(uint64_t n, uint64_t nnz, int dtype);
 
 /*
  * Bytes of device scratch bt_compress / bt_relu_fwd_compress need for n
- * elements: the tile descriptors and per-wave totals of the single-pass scan
- * plus a small header.  The contents need no initialisation and are
- * unspecified after a call: a tile descriptor counts as written by the running
- * call only if it carries that call's 64-bit tag, which no other call shares,
- * and the per-wave totals are cleared by the running launch itself, before a
- * grid-wide meeting that precedes the first addition to them.  Two calls that
+ * elements: the tile descriptors of the single-pass scan plus a small header.
+ * The contents need no initialisation and are unspecified after a call: a tile
+ * descriptor counts as written by the running call only if it carries that
+ * call's 64-bit tag, which no other call shares.  Two calls that
  * run concurrently must not share a workspace; calls ordered on the device
  * (one stream, or events) may.  No counterpart in the paper (its scan is
  * sequential).

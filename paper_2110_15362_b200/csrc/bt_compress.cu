@@ -99,7 +99,7 @@ __global__ void __launch_bounds__((kWorkers + 3 + WRITE_Y) * 32) compress_kernel
 
     // The arena's cursor is read before the barrier below: the kernel's one update of it follows the last tile's base,
     // which needs a publication from every CTA, and a CTA publishes only after this barrier.
-    if (tid == 0) sh.init(WRITE_Y);
+    sh.init(WRITE_Y, tid);
     in_stream_order();
     if (tid == 0) sh.arena_c0 = a.arena_cursor ? *reinterpret_cast<const volatile uint64_t *>(a.arena_cursor) : 0;
     __syncthreads();
@@ -239,11 +239,17 @@ __global__ void __launch_bounds__((kWorkers + 3 + WRITE_Y) * 32) compress_kernel
                     const uint64_t ch = pt * kChunksPerTile + lane / kSegsPerChunk;
                     if (ch < chunks_total && extent_of(a.prefix, 8 * chunks_total).holds(a.prefix + ch, 8)) a.prefix[ch] = base + sh.off[ps][lane];
                 }
+                const uint32_t agg_last = sh.agg[ps];
+                __syncwarp();
+                if (lane == 0) {
+                    sh.base[ps] = base;
+                    mbar_arrive(&sh.ready[ps]);                      // the tile's values may leave; what follows takes two trips to L2 and fences
+                }
                 if (pt == num_tiles - 1 && lane == 0) {
-                    const uint64_t nnz = base + sh.agg[ps];
+                    const uint64_t nnz = base + agg_last;
                     *a.nnz_out = nnz;
-                    __threadfence();
-                    const bool aborted = ld_relaxed_u64(a.ws_header + kHdrAbort) == tag;
+                    // (the status word needs no look at the abort word here: it is looked at after the store, below)
+                    const bool aborted = a.arena_cursor && ld_relaxed_u64(a.ws_header + kHdrAbort) == tag;
                     uint64_t capacity = a.capacity;
                     if (a.arena_cursor) {
                         // arena form: the room left behind the cursor; the cursor moves only when everything fitted
@@ -265,11 +271,6 @@ __global__ void __launch_bounds__((kWorkers + 3 + WRITE_Y) * 32) compress_kernel
                     // every CTA has published all its counts by now, so every CTA has read the sequence number:
                     // the next launch on this workspace gets another tag
                     red_add_u64(a.ws_header + kHdrSeq, 1ull);
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    sh.base[ps] = base;
-                    mbar_arrive(&sh.ready[ps]);                      // the tile's values may leave
                 }
             }
             if (j <= last_it) {

@@ -163,7 +163,7 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
     // The arena's cursor is read before the barrier below: the launch's first update of it follows a tensor's last base,
     // which needs a publication from every CTA in front of it, and the sequence number moves only behind all of them.
     const bool in_arena = p.c.arena != nullptr;
-    if (tid == 0) sh.init(WRITE_Y);
+    sh.init(WRITE_Y, tid);
     in_stream_order();
     if (tid == 0) sh.arena_c0 = in_arena ? *reinterpret_cast<const volatile uint64_t *>(p.c.arena_cursor) : 0;
     __syncthreads();
@@ -344,12 +344,20 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
                     const uint64_t chunks_total = (jb.n + BT_CHUNK_ELEMS - 1) / BT_CHUNK_ELEMS;
                     if (ch < chunks_total && extent_of(jb.prefix, 8 * chunks_total).holds(jb.prefix + ch, 8)) jb.prefix[ch] = base + sh.off[ps][lane];
                 }
+                const uint32_t agg_last = sh.agg[ps];
+                __syncwarp();
+                if (lane == 0) {
+                    sh.base[ps] = base;
+                    sh.dst[ps]  = arena_at;
+                    sh.job[ps]  = pk;
+                    mbar_arrive(&sh.ready[ps]);                      // the tile's values may leave; what follows takes two trips to L2 and fences
+                }
                 bool bump = false;              // lane 0: this is the launch's last tile
                 if (pt == jb.tiles - 1 && lane == 0) {
-                    const uint64_t nnz = base + sh.agg[ps];
+                    const uint64_t nnz = base + agg_last;
                     *jb.nnz_out        = nnz;
-                    __threadfence();
-                    const bool aborted  = ld_relaxed_u64(p.c.ws_header + kHdrAbort) == tag;
+                    // (the status word needs no look at the abort word here: it is looked at after the store, below)
+                    const bool aborted = in_arena && ld_relaxed_u64(p.c.ws_header + kHdrAbort) == tag;
                     uint64_t   capacity = jb.capacity;
                     if (in_arena) {
                         // the cursor moves past the tensor only when everything fitted
@@ -397,12 +405,6 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
                         __nanosleep(200);
                     }
                     if (lane == 0) red_add_u64(p.c.ws_header + kHdrSeq, all ? 1ull : 1ull << 32);
-                }
-                if (lane == 0) {
-                    sh.base[ps] = base;
-                    sh.dst[ps]  = arena_at;
-                    sh.job[ps]  = pk;
-                    mbar_arrive(&sh.ready[ps]);                      // the tile's values may leave
                 }
             }
             if (has) {

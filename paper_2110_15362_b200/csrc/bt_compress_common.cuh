@@ -486,14 +486,17 @@ struct CtaState {
     volatile uint64_t tag;            // this launch's tag once a scan warp has it, else 0
     uint64_t          arena_c0;       // arena forms: the cursor as the launch found it
     volatile uint32_t abort;
-    // by one thread; a CTA-wide barrier follows
-    __device__ __forceinline__ void init(const bool dense_output)
+    // by the first threads of the CTA, one barrier each; a CTA-wide barrier follows
+    __device__ __forceinline__ void init(const bool dense_output, const uint32_t tid)
     {
-        abort = 0;
-        tag   = 0;
-        for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1), mbar_init(&empty[s], dense_output ? 1 : kSegs), mbar_init(&written[s], kSegs);
-        for (int q = 0; q < kQueue; ++q) mbar_init(&counted[q], kSegs), mbar_init(&ready[q], 1), mbar_init(&done[q], kSegs);
-        fence_proxy_async();
+        if (tid == 0) abort = 0, tag = 0;
+        if (tid < kStages) {
+            mbar_init(&full[tid], 1), mbar_init(&empty[tid], dense_output ? 1 : kSegs), mbar_init(&written[tid], kSegs);
+        } else if (tid - kStages < kQueue) {
+            const uint32_t q = tid - kStages;
+            mbar_init(&counted[q], kSegs), mbar_init(&ready[q], 1), mbar_init(&done[q], kSegs);
+        }
+        if (tid < kStages + kQueue) fence_proxy_async();
     }
 };
 

@@ -1,6 +1,6 @@
 // bt_compress_noalloc: Algorithm 1 for callers that may not allocate device memory.
 //
-// bt_compress needs a scratch buffer (wave totals and tile descriptors of its scan).  Normally the
+// bt_compress needs a scratch buffer (the tile descriptors of its scan).  Normally the
 // caller allocates it.  Some callers cannot: a hook that runs while its framework's allocator is
 // frozen (inside a memory plan whose every byte is already assigned, or in a region where an
 // allocation would synchronise or fail), or a plug-in that is handed its input and output buffers
