@@ -579,15 +579,20 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
         U *const       tile = tiles + static_cast<size_t>(s) * kTile;
         if (!mbar_wait(&sh.full[s], (it / kStages) & 1u, &sh.abort, wait_ns)) return false;
         if (t.n - t.first < static_cast<uint64_t>(kTile)) {
-            // Ragged last tile: each warp completes its own segment -- what the 16-byte granular bulk copy left out,
-            // zeros behind the end of the tensor -- and meets no other warp over it.  (A barrier among the workers here
-            // would never open if one of them had left the kernel because its wait ran out.)
+            // Ragged last tile: each warp completes its own segment -- the elements of the last 16 bytes that the bulk copy
+            // left out, zeros behind the end of the tensor -- and meets no other warp over it.  (A barrier among the workers
+            // here would never open if one of them had left the kernel because its wait ran out.)  One element per lane for
+            // those 16 bytes, then whole vectors: the ragged tile is the last one and everything waits for its count.
+            // (Filled element by element, 64 steps for 2-byte types: bf16 200704 elements 7.7 us, this way 6.2.)
+            constexpr uint32_t kPer = 16 / sizeof(U);
             const U *const src     = static_cast<const U *>(t.src);
             const uint32_t have    = static_cast<uint32_t>(t.n - t.first);
-            const uint32_t by_bulk = ((have * static_cast<uint32_t>(sizeof(U))) & ~15u) / sizeof(U);
+            const uint32_t by_bulk = have / kPer * kPer;
             const uint32_t seg0    = seg * kSeg;
-            for (uint32_t e = (by_bulk > seg0 ? by_bulk : seg0) + lane; e < seg0 + kSeg; e += 32)
-                tile[e] = (e < have) ? src[t.first + e] : U(0);
+            if (by_bulk >= seg0 && by_bulk < seg0 + kSeg && lane < kPer)
+                tile[by_bulk + lane] = by_bulk + lane < have ? src[t.first + by_bulk + lane] : U(0);
+            for (uint32_t e = (by_bulk >= seg0 ? by_bulk + kPer : seg0) + kPer * lane; e < seg0 + kSeg; e += 32 * kPer)
+                *reinterpret_cast<uint4 *>(tile + e) = make_uint4(0, 0, 0, 0);
             __syncwarp();
         }
         // the segment into registers; the slot is free for the next tile once every segment is

@@ -35,6 +35,24 @@ def test_sizes_around_segments_and_parts(G, oracle, kind, units, off):
 
 
 @pytest.mark.parametrize("kind", ["f32", "bf16", "f64"])
+@pytest.mark.parametrize("seg", [0, 3, 7])
+def test_ragged_tile_in_a_used_slot(G, oracle, kind, seg):
+    """The fifth tile of the only CTA ends within segment `seg`, around 16-byte units, over the dense data of the second."""
+    unit = 16 // np.dtype(W.random_patterns(1, kind, 0.0, seed=0).dtype).itemsize
+    before = B.bt_set_max_ctas(1)
+    try:
+        for off in (1, unit - 1, unit, unit + 1, UNIT[kind] // 2, UNIT[kind] - unit - 1, UNIT[kind] - 1, UNIT[kind]):
+            n = (4 * 8 + seg) * UNIT[kind] + off
+            x = W.random_patterns(n, kind, 0.01, seed=n)
+            y_ref, c = oracle.prune_fwd_compress(x, kind, 0.0)
+            g = G.gpu_compress(from_raw(x, kind), relu=True, want_y=True)
+            assert g.guards_ok and g.status == B.BT_OK and g.nnz == c.nnz and np.array_equal(g.y, y_ref)
+            assert np.array_equal(g.bitmap, c.bitmap) and np.array_equal(g.prefix, c.prefix) and np.array_equal(g.values, c.values)
+    finally:
+        B.bt_set_max_ctas(before)
+
+
+@pytest.mark.parametrize("kind", ["f32", "bf16", "f64"])
 @pytest.mark.parametrize("fused", [False, True])
 @pytest.mark.parametrize("tiles", [1, 2 * 8, 2 * 8 + 1, 2 * 19 + 1])
 def test_no_room_for_values(oracle, kind, fused, tiles):
