@@ -111,8 +111,9 @@ size_t bt_workspace_bytes(uint64_t n);
  * unspecified.  *dev_status = BT_ERR_TIMEOUT means an internal bounded wait
  * gave up (two seconds without the data it waits for; every CTA then leaves
  * the kernel) and every output is undefined; the workspace and the context
- * stay usable and the next call runs normally.  The kernel is launched
- * cooperatively (all its CTAs resident at once, one per SM at most).
+ * stay usable and the next call runs normally.  The kernel takes one CTA per
+ * SM at most; with more tiles of 32 KB than CTAs it is launched cooperatively
+ * (all its CTAs resident at once).
  */
 int bt_compress(const void *dense, uint64_t n, int dtype,
                 uint32_t *bitmap, void *values, uint64_t values_capacity,
@@ -210,8 +211,9 @@ int bt_relu_bwd_from_bitmap_batch(const bt_batch_item *items /* host */, uint32_
 /*
  * Launch configuration for callers that keep several compress calls in flight
  * (on several streams, or in the branches of a CUDA graph).  The compress
- * kernel is launched cooperatively with one CTA per SM, and a cooperative
- * launch starts only when all its CTAs can be resident: two launches of more
+ * kernel has at most one CTA per SM and, with more tiles than CTAs, is
+ * launched cooperatively; a cooperative launch starts only when all its CTAs
+ * can be resident: two such launches of more
  * than half the SMs each therefore run one after the other, whatever their
  * streams.  bt_set_max_ctas(m) limits every later compress-family launch MADE
  * BY THE CALLING THREAD to m CTAs (0: no limit, the default), so that

@@ -2,8 +2,9 @@
 // compaction pass: a persistent-CTA stream compaction whose prefix sum rides on the
 // wave structure of the grid.
 //
-// The grid is launched cooperatively with exactly as many CTAs (G) as fit on
-// the device at once, so all of them are co-resident, and CTA b takes tiles
+// The grid has exactly as many CTAs (G) as fit on the device at once and is
+// launched cooperatively, so that all of them are co-resident (a tensor of at
+// most G tiles: one CTA per tile, a plain launch), and CTA b takes tiles
 // b, b+G, b+2G, ...: iteration j of every CTA together forms "wave j", G
 // consecutive tiles.  The warps of a CTA are specialised: one load warp, two
 // scan warps, and workers for everything else (bt_compress_common.cuh: `work`).
@@ -360,11 +361,10 @@ cudaError_t launch_shaped(const CompressArgs &a, cudaStream_t stream)
     if (max_grid > 32 * kMaxWindows) max_grid = 32 * kMaxWindows;
     if (t_max_ctas != 0 && static_cast<uint32_t>(max_grid) > t_max_ctas) max_grid = static_cast<int>(t_max_ctas);
     const uint32_t grid  = num_tiles < static_cast<uint32_t>(max_grid) ? num_tiles : static_cast<uint32_t>(max_grid);
-    // cooperative launch: the runtime guarantees that all `grid` CTAs are resident together
     CompressArgs args = a;
     args.call_tag     = next_call_tag();
     args.wait_ns      = compress_wait_ns();
-    return launch_cooperative(kernel, grid, kThreads, kSmem, stream, args, num_tiles);
+    return launch_waiting(num_tiles, kernel, grid, kThreads, kSmem, stream, args, num_tiles);
 }
 
 template <typename U, int FUSED, bool WRITE_Y, int CAST = 0>

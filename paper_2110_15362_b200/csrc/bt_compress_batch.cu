@@ -496,8 +496,8 @@ cudaError_t launch_shaped(const CompressCommon &c, const CompressJob *jobs, uint
     p.c.ws_words  = (batch_workspace_bytes(chunks, count) - kWsHeaderBytes) / 8;
     p.c.call_tag  = next_call_tag();
     p.c.wait_ns   = compress_wait_ns();
-    // cooperative launch: the runtime guarantees that all `grid` CTAs are resident together
-    return launch_cooperative(kernel, grid, kThreads, kSmem, stream, p);
+    // (with no more tiles than CTAs, CTA b takes descriptor b: what launch_waiting asks for)
+    return launch_waiting(tiles, kernel, grid, kThreads, kSmem, stream, p);
 }
 
 template <typename U, int FUSED, bool WRITE_Y>

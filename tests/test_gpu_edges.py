@@ -52,6 +52,40 @@ def test_ragged_tile_in_a_used_slot(G, oracle, kind, seg):
         B.bt_set_max_ctas(before)
 
 
+@pytest.mark.parametrize("kind", ["f32", "bf16"])
+def test_one_tile_per_cta_on_two_streams(oracle, kind):
+    """Launches of one tile per CTA need not be resident as a whole: two streams, each launch with more than half the SMs,
+    alone and as batches, against the oracle; the largest such launch and the next tile."""
+    B.lib()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tile = 8 * UNIT[kind]
+    sizes = [tile * sms, tile * (sms - 1) + 1, tile * sms + 1, tile * (sms - 20) - 5]
+    raws = [W.random_patterns(n, kind, 0.5, seed=n % 1000) for n in sizes]
+    refs = [oracle.compress(r) for r in raws]
+    xs = [from_raw(r, kind) for r in raws]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    half = [from_raw(r[: r.size // 2], kind) for r in raws[:2]]      # batches: two tensors that fill the SMs together
+    for _ in range(5):
+        stashes, wss = [B.Stash(n, x.dtype) for n, x in zip(sizes, xs)], [B.new_workspace(n) for n in sizes]
+        bst = [[B.Stash(h.numel(), h.dtype) for h in half] for _ in streams]
+        bws = [torch.empty(B.bt_batch_workspace_bytes([h.numel() for h in half]), dtype=torch.uint8, device="cuda") for _ in streams]
+        torch.cuda.synchronize()
+        for k in range(len(sizes)):
+            st, s = stashes[k], streams[k % 2]
+            B.bt_compress(xs[k], st.bitmap, st.values, st.chunk_prefix, st.nnz_out, wss[k], st.dev_status, stream=s)
+            if k < 2:
+                B.bt_compress_batch(B.batch_items(half, bst[k]), half[0].dtype, bws[k], stream=s)
+        torch.cuda.synchronize()
+        for st, c in zip(stashes, refs):
+            assert st.status == B.BT_OK and st.nnz == c.nnz
+            assert np.array_equal(W.raw_numpy(st.bitmap).view(np.uint32), c.bitmap)
+            assert np.array_equal(W.raw_numpy(st.values[: c.nnz]), c.values)
+        for pair in bst:
+            for st, r in zip(pair, raws):
+                c = oracle.compress(r[: r.size // 2])
+                assert st.status == B.BT_OK and st.nnz == c.nnz and np.array_equal(W.raw_numpy(st.values[: c.nnz]), c.values)
+
+
 @pytest.mark.parametrize("kind", ["f32", "bf16", "f64"])
 @pytest.mark.parametrize("fused", [False, True])
 @pytest.mark.parametrize("tiles", [1, 2 * 8, 2 * 8 + 1, 2 * 19 + 1])
