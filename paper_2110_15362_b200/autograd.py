@@ -47,6 +47,12 @@ from typing import Dict, Optional, Tuple
 import torch
 
 from . import binding as B
+from . import build as _build
+
+try:
+    from . import _autograd as _native
+except ImportError as e:
+    raise ImportError(f"{_build.AUTOGRAD_PATH} is missing: build it with `python -m paper_2110_15362_b200.build`") from e
 
 __all__ = ["PackedActivation", "stash_saved_activations", "relu_stash", "ReLUStash", "relu6_stash", "ReLU6Stash",
            "double_mask", "DoubleMask", "maxpool2x2_stash", "MaxPool2x2Stash", "relu_maxpool2x2_stash",
@@ -59,9 +65,9 @@ class _Record:
 
     __slots__ = ("buf", "n", "_bitmap", "_prefix")
 
-    def __init__(self, n: int, device, words: int = 0):
+    def __init__(self, n: int, device=None, words: int = 0, buf: Optional[torch.Tensor] = None):
         self.n = n
-        self.buf = torch.empty(_words_at(n) + 8 * words, dtype=torch.uint8, device=device)
+        self.buf = torch.empty(_words_at(n) + 8 * words, dtype=torch.uint8, device=device) if buf is None else buf
         self._bitmap = self._prefix = None
 
     @property
@@ -130,19 +136,20 @@ class PackedActivation:
         return B.bt_compressed_bytes(self.numel, nnz, self.stored)
 
     def unpack(self) -> torch.Tensor:
-        out = torch.empty(self.shape, dtype=self.dtype, device=self.device)
-        n, at, calls, stream = self.record.n, self.record.buf.data_ptr(), B._calls(), B._stream(None)
-        prefix, code = at + _prefix_at(n), B.DTYPE_CODE[self.stored]
-        if self.arena is not None:
+        arena = self.arena is not None
+        if arena:
             self.owner.check_statuses()
-            # a stash of another type than the tensor's is a narrowed stash of a float32 tensor
-            call = calls.bt_decompress_arena if self.stored is self.dtype else calls.bt_decompress_widen_arena
-            st = call(at, self.arena, at + _words_at(n) + 8, prefix, n, code, out, stream)
-        else:
-            call = calls.bt_decompress if self.stored is self.dtype else calls.bt_decompress_widen
-            st = call(at, self.values, prefix, n, code, out, stream)
+        # a stash of another type than the tensor's is a narrowed stash of a float32 tensor
+        call = _RESTORES[arena, self.stored is not self.dtype]
+        st, out = _native.restore(B._calls().address[call], self.record.buf, self.arena if arena else self.values, arena,
+                                  B.DTYPE_CODE[self.stored], self.shape, self.dtype)
         B._check("bt_decompress (autograd stash)", st, True)
         return out
+
+
+# by (in an arena, narrowed)
+_RESTORES = {(False, False): "bt_decompress", (False, True): "bt_decompress_widen",
+             (True, False): "bt_decompress_arena", (True, True): "bt_decompress_widen_arena"}
 
 
 def _usable(t: torch.Tensor) -> bool:
@@ -253,18 +260,25 @@ def _compress(x: torch.Tensor, scratch: _Scratch, relu_into: Optional[torch.Tens
     else:
         st = calls.bt_prune_fwd_compress_narrow(x, n, code, 0.0, relu_into, *tail)
     B._check("bt_compress (autograd stash)", st, True)
-    torch.cuda.current_stream().synchronize()       # the one host read: sizes the values exactly
-    nnz, st = int(host.view[0]), int(host.view[1]) & 0xFFFFFFFF
-    if st != B.BT_OK and not (two_pass and st == B.BT_ERR_CAPACITY):
-        raise B.BitTrainError("bt_compress (autograd stash)", st)
-    if not two_pass:
-        return record, full[:nnz].clone(), nnz
-    values = torch.empty(nnz, dtype=x.dtype, device=dev)
-    if nnz:
-        st = calls.bt_mask_compress(x if relu_into is None else relu_into, n, code, at, at + _prefix_at(n), None, values, nnz,
-                                    B._stream(None))
-        B._check("bt_mask_compress (autograd stash)", st, True)
+    values, nnz = _exact_values(x if relu_into is None else relu_into, record, host, full)
     return record, values, nnz
+
+
+def _exact_values(y: torch.Tensor, record: _Record, host: _HostWords, full: Optional[torch.Tensor]):
+    """The exact-size values of the stash that is being made of `y` (the tensor as it is stashed), and their number: copied
+    from `full`, or with `full` None gathered from y under the record's bitmap."""
+    _native.synchronize()                           # the one host read: sizes the values exactly
+    nnz, st = int(host.view[0]), int(host.view[1]) & 0xFFFFFFFF
+    if st != B.BT_OK and not (full is None and st == B.BT_ERR_CAPACITY):
+        raise B.BitTrainError("bt_compress (autograd stash)", st)
+    if full is not None:
+        return full[:nnz].clone(), nnz
+    values = torch.empty(nnz, dtype=y.dtype, device=y.device)
+    if nnz:
+        at, n = record.buf.data_ptr(), record.n
+        st = B._calls().bt_mask_compress(y, n, B.DTYPE_CODE[y.dtype], at, at + _prefix_at(n), None, values, nnz, B._stream(None))
+        B._check("bt_mask_compress (autograd stash)", st, True)
+    return values, nnz
 
 
 def _compress_arena(x: torch.Tensor, owner, relu_into: Optional[torch.Tensor] = None, relu6: bool = False):
@@ -407,56 +421,65 @@ class stash_saved_activations(torch.autograd.graph.saved_tensors_hooks):
         return super().__exit__(*exc)
 
 
-class ReLUStash(torch.autograd.Function):
-    """ReLU with the stash fused into its forward pass; the backward pass reads only the bitmap."""
+class ReLUStash:
+    """ReLU with the stash fused into its forward pass; the backward pass reads only the bitmap.  Both are a node in native
+    code (csrc/bt_autograd.cpp, where the reason and the figures stand)."""
 
     @staticmethod
-    def forward(ctx, x: torch.Tensor, hooks: Optional[stash_saved_activations] = None, inplace: bool = False,
-                keep_values: bool = True):
-        if inplace and _usable(x):
-            xc = y = x                   # the kernel may write the activation over its input
-            ctx.mark_dirty(x)
-        else:
-            xc = _flat_input(x)
-            y = torch.empty_like(xc)
+    def apply(x: torch.Tensor, hooks: Optional[stash_saved_activations] = None, inplace: bool = False,
+              keep_values: bool = True) -> torch.Tensor:
+        n, dev = x.numel(), x.device
+        scratch = hooks.scratch if hooks is not None else _Scratch()
+        address = B._calls().address
+        bwd = address["bt_relu_bwd_from_bitmap"]
+        ws = scratch.workspace(n, dev)
         if not keep_values:
             # nobody will ask for the activation again (e.g. it only feeds a pooling layer that keeps winner codes):
             # the bitmap is all this ReLU's backward pass needs, so the values are not stored at all
-            n, dev = xc.numel(), xc.device
-            record = _Record(n, dev, words=2)
             statuses = hooks.loose_statuses if hooks is not None else _StatusWords()
-            scratch = hooks.scratch if hooks is not None else _Scratch()
-            at, ws = record.buf.data_ptr(), scratch.workspace(n, dev)
-            st = B._calls().bt_relu_fwd_compress(xc, n, B.DTYPE_CODE[xc.dtype], y, at, None, 0, at + _prefix_at(n),
-                                                 at + _words_at(n), ws, ws.numel(), statuses.next(dev), B._stream(None))
+            st, y, _ = _native.relu_stash(x, address["bt_relu_fwd_compress"], bwd, _PLAIN, B.DTYPE_CODE[x.dtype], inplace, None, 0,
+                                          None, None, ws, ws.numel(), statuses.next(dev))
             B._check("bt_relu_fwd_compress (bitmap only)", st, True)
             if hooks is None:                           # BT_ERR_CAPACITY is the expected answer here
                 st = statuses.drain()[0]
                 if st not in (B.BT_OK, B.BT_ERR_CAPACITY):
                     raise B.BitTrainError("bt_relu_fwd_compress (bitmap only)", st)
-            ctx.save_for_backward(record.buf)
             return y
+        narrow = hooks.narrow if hooks is not None and x.dtype is torch.float32 else None
+        stored = narrow or x.dtype
+        code = B.DTYPE_CODE[stored]
         if hooks is not None and hooks.arena is not None:
-            record, stored = _compress_arena(xc, hooks, relu_into=y)
-            ctx.save_for_backward(record.buf)
-            hooks.share(y, _packed_arena(y, record, hooks, stored))
-            hooks.dense_bytes += y.numel() * y.element_size()
+            arena = hooks.arena
+            call = "bt_prune_fwd_compress_arena" if narrow is None else "bt_prune_fwd_compress_narrow_arena"
+            st, y, buf = _native.relu_stash(x, address[call], bwd, _ARENA, code, inplace, arena, arena.numel(), hooks.cursor, None,
+                                            ws, ws.numel(), hooks.statuses.next(dev))
+            B._check("bt_*_arena (autograd stash)", st, True)
+            hooks.share(y, _packed_arena(y, _Record(n, buf=buf), hooks, stored))
+            hooks.dense_bytes += n * y.element_size()
             return y
-        scratch = hooks.scratch if hooks is not None else _Scratch()
-        record, values, nnz = _compress(xc, scratch, relu_into=y, narrow=hooks.narrow if hooks is not None else None)
-        ctx.save_for_backward(record.buf)     # released with the graph, like any saved tensor
+        full = None if n == 0 or (scratch.two_pass and narrow is None) else scratch.full_values(n, stored, dev)
+        host = _read_back()
+        nnz_word = host.words.data_ptr()
+        call = 0 if n == 0 else address["bt_relu_fwd_compress" if narrow is None else "bt_prune_fwd_compress_narrow"]
+        st, y, buf = _native.relu_stash(x, call, bwd, _PLAIN if narrow is None else _NARROW, code, inplace, full,
+                                        0 if full is None else n, None, nnz_word, ws, ws.numel(), nnz_word + 8)
+        B._check("bt_compress (autograd stash)", st, True)
+        record = _Record(n, buf=buf)
+        if n == 0:
+            values, nnz = torch.empty(0, dtype=x.dtype, device=dev), 0
+        else:
+            values, nnz = _exact_values(y, record, host, full)
         if hooks is not None:
             # the next layer will save y as its input: hand it this stash instead of compressing y again
             packed = _packed(y, record, values, nnz)
             hooks.share(y, packed)
             hooks.packed_bytes += packed.nbytes()
-            hooks.dense_bytes += y.numel() * y.element_size()
+            hooks.dense_bytes += n * y.element_size()
         return y
 
-    @staticmethod
-    def backward(ctx, grad: torch.Tensor):
-        (buf,) = ctx.saved_tensors
-        return _relu_bwd(buf, grad), None, None, None
+
+# the compressors that the native node calls
+_PLAIN, _NARROW, _ARENA = 0, 1, 2
 
 
 def relu_stash(x: torch.Tensor, hooks: Optional[stash_saved_activations] = None, inplace: bool = False,

@@ -73,11 +73,13 @@ def lib() -> ctypes.CDLL:
 
 
 class _Calls:
-    """The ABI's asynchronous calls of one build of the library (see _pycall): status codes out."""
+    """The ABI's asynchronous calls of one build of the library (see _pycall): status codes out.  `address`: their
+    addresses by name, for native code that makes the calls itself."""
 
     def __init__(self, L: ctypes.CDLL, native_call):
-        for name in CALLS:
-            setattr(self, name, native_call(ctypes.cast(getattr(L, name), ctypes.c_void_p).value))
+        self.address = {name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in CALLS}
+        for name, at in self.address.items():
+            setattr(self, name, native_call(at))
 
 
 def _calls() -> _Calls:

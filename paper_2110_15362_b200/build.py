@@ -14,6 +14,8 @@ INCLUDE = os.path.join(os.path.dirname(PKG_DIR), "include")
 LIB_PATH = os.path.join(PKG_DIR, "libbittrain.so")
 CALLER_SRC = os.path.join(CSRC, "bt_pycall.c")
 CALLER_PATH = os.path.join(PKG_DIR, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+AUTOGRAD_SRC = os.path.join(CSRC, "bt_autograd.cpp")
+AUTOGRAD_PATH = os.path.join(PKG_DIR, "_autograd" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
@@ -44,12 +46,31 @@ def build_caller(force: bool = False) -> str:
     return CALLER_PATH
 
 
+def build_autograd(force: bool = False) -> str:
+    """Compile the extension module of the autograd integration against torch's C++ headers; returns its path."""
+    newest = max(os.path.getmtime(f) for f in (AUTOGRAD_SRC, os.path.join(INCLUDE, "bittrain.h")))
+    if not force and os.path.exists(AUTOGRAD_PATH) and os.path.getmtime(AUTOGRAD_PATH) >= newest:
+        return AUTOGRAD_PATH
+    import torch
+    from torch.utils import cpp_extension
+    headers = cpp_extension.include_paths() + [os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
+    tmp = AUTOGRAD_PATH + ".tmp%d" % os.getpid()
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wall", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+                           "-I", sysconfig.get_paths()["include"], "-I", INCLUDE]
+                          + [a for h in headers for a in ("-isystem", h)] + ["-o", tmp, AUTOGRAD_SRC]
+                          + ["-L" + d for d in cpp_extension.library_paths()]
+                          + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+    os.replace(tmp, AUTOGRAD_PATH)
+    return AUTOGRAD_PATH
+
+
 def build_library(force: bool = False, verbose: bool = False, out: str = LIB_PATH, extra_flags=()) -> str:
     """Compile every .cu under csrc/ into one shared object; returns its path.  `out` and
     `extra_flags` (preprocessor defines and the like) are for the checking builds the tests use;
     the product library is the default."""
     if out == LIB_PATH:
         build_caller(force)
+        build_autograd(force)
     if not force and not is_stale(out):
         return out
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"

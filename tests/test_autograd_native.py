@@ -1,0 +1,80 @@
+"""The native node of the stashing ReLU and the native restore: what they refuse (no GPU), and on the GPU every form of the
+node against torch.relu -- inputs and gradients that are views, in place, retained and released graphs, empty tensors."""
+import pytest
+import torch
+
+from paper_2110_15362_b200 import autograd as A
+from paper_2110_15362_b200 import binding as B
+
+
+def test_arguments_are_checked():
+    x = torch.zeros(64)
+    none = (0, 0, 0, 0, False, None, 0, None, None, None, 0, None)
+    with pytest.raises(TypeError):
+        A._native.relu_stash(x)
+    with pytest.raises(TypeError):
+        A._native.relu_stash(None, *none)
+    with pytest.raises(RuntimeError, match="CUDA"):
+        A._native.relu_stash(x, *none)
+    with pytest.raises(OverflowError):
+        A._native.relu_stash(x, -1 << 70, *none[1:])
+    with pytest.raises(TypeError):
+        A._native.restore(0, x, None, False, 0, [64], torch.float32)
+    with pytest.raises(RuntimeError, match="record"):
+        A._native.restore(0, torch.zeros(8, dtype=torch.uint8), None, False, 0, (64,), torch.float32)
+
+
+def _views(kind, dtype):
+    """(a leaf, a function of it whose result the ReLU takes)"""
+    g = torch.Generator().manual_seed(7)
+    if kind == "empty":
+        return torch.zeros(0, device="cuda", dtype=dtype), lambda t: t * 1
+    t = torch.randn(96, 203, generator=g).to(dtype).cuda()
+    if kind == "transposed":
+        return t, lambda t: (t * 1).t()
+    if kind == "misaligned":
+        return t, lambda t: (t * 1).flatten()[1:]
+    return t, lambda t: t * 1
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("form", ["exact", "full", "arena", "bits", "bits_alone", "alone", "narrow", "narrow_arena"])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float64])
+@pytest.mark.parametrize("kind", ["whole", "transposed", "misaligned", "empty"])
+@pytest.mark.parametrize("inplace", [False, True])
+def test_every_form_of_the_node(form, dtype, kind, inplace):
+    opts = {"exact": {}, "full": {"two_pass": False}, "arena": {"arena_bytes": 1 << 20}, "bits": {}, "narrow": {"narrow": torch.bfloat16},
+            "narrow_arena": {"narrow": torch.bfloat16, "arena_bytes": 1 << 20}}
+    hooks = A.stash_saved_activations(min_numel=16, **opts[form]) if form in opts else None
+    t, view = _views(kind, dtype)
+    leaf, ref = t.clone().requires_grad_(), t.clone().requires_grad_()
+
+    def step():
+        h = view(leaf)
+        # an activation may be written over its input only where that is not a view of something saved
+        return A.relu_stash(h, hooks, inplace=inplace, keep_values=not form.startswith("bits"))
+
+    if hooks is not None:
+        with hooks:
+            y = step()
+    else:
+        y = step()
+    y_ref = torch.relu(view(ref))
+    assert torch.equal(y, y_ref) and y.requires_grad
+    for grad in (torch.randn_like(y_ref), torch.ones((), device="cuda", dtype=dtype).expand_as(y_ref)):
+        leaf.grad = ref.grad = None
+        y.backward(grad, retain_graph=True)
+        y_ref.backward(grad, retain_graph=True)
+        assert torch.equal(leaf.grad, ref.grad)
+    y.sum().backward()
+    with pytest.raises(RuntimeError, match="second time"):
+        y.sum().backward()
+    if hooks is not None:
+        packed = getattr(y, "_bt_packed", None)
+        assert (packed is None) == form.startswith("bits")
+        if packed is not None and t.numel():
+            back, want = packed.unpack(), y.detach()
+            assert torch.equal(back, want.bfloat16().to(dtype) if form.startswith("narrow") and dtype == torch.float32 else want)
+        hooks.check_statuses()
+    with torch.no_grad():
+        assert not A.relu_stash(view(ref), keep_values=not form.startswith("bits")).requires_grad
