@@ -73,17 +73,39 @@ def lib() -> ctypes.CDLL:
 
 
 class _Calls:
-    """The ABI's asynchronous calls of one build of the library (see _pycall): status codes out.  `address`: their
-    addresses by name, for native code that makes the calls itself."""
+    """The ABI's asynchronous calls of one build of the library (see _pycall): status codes out.  `pointer`: the kind of
+    their pointer parameters, "p" (tensors) or "a" (tensors or addresses).  `address`: their addresses by name, for native
+    code that makes the calls itself."""
 
-    def __init__(self, L: ctypes.CDLL, native_call):
+    def __init__(self, L: ctypes.CDLL, native_call, pointer: str):
         self.address = {name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in CALLS}
         for name, at in self.address.items():
-            setattr(self, name, native_call(at))
+            fn = getattr(L, name)
+            kinds = "".join({ctypes.c_void_p: pointer, ctypes.c_float: "f", ctypes.POINTER(BatchItem): "b"}.get(t, "n")
+                            for t in fn.argtypes[:-1]) + "s"
+            setattr(self, name, native_call(at, kinds, _through_ctypes(fn, kinds), BatchItem))
+
+
+def _through_ctypes(fn, kinds: str):
+    """The call of `fn` by ctypes, for arguments that are not plainly of their parameter's kind: it converts them (one-element
+    integer tensors and the like as counts) or refuses them."""
+    def pointer(kind, v):
+        if kind not in "pa" or v is None or (kind == "a" and isinstance(v, int)):
+            return v
+        return v.data_ptr()
+
+    def call(*args):
+        return fn(*[pointer(kinds[k] if k < len(kinds) else "n", v) for k, v in enumerate(args)])
+    return call
 
 
 def _calls() -> _Calls:
+    """The calls with tensors' addresses allowed in place of the tensors."""
     return (_lib or lib()).calls
+
+
+def _tensor_calls() -> _Calls:
+    return (_lib or lib()).tensor_calls
 
 
 def load_library(path: str) -> ctypes.CDLL:
@@ -96,7 +118,6 @@ def load_library(path: str) -> ctypes.CDLL:
     except ImportError as e:
         raise ImportError(f"{_build.CALLER_PATH} is missing: build it with `python -m paper_2110_15362_b200.build`") from e
     L = ctypes.CDLL(path)
-    L.calls = _Calls(L, _pycall.native_call)
     u64, vp, i32, sz = ctypes.c_uint64, ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
     L.bt_compressed_bytes.restype = sz
     L.bt_compressed_bytes.argtypes = [u64, u64, i32]
@@ -174,6 +195,8 @@ def load_library(path: str) -> ctypes.CDLL:
     L.bt_relu_fwd_compress_host.argtypes = [vp, u64, i32, vp, vp, vp, u64, vp, vp, vp, sz, vp]
     L.bt_relu_bwd_from_bitmap_host.restype = i32
     L.bt_relu_bwd_from_bitmap_host.argtypes = [vp, vp, u64, i32, vp, vp, sz, vp]
+    L.calls = _Calls(L, _pycall.native_call, "a")
+    L.tensor_calls = _Calls(L, _pycall.native_call, "p")
     return L
 
 
@@ -215,7 +238,7 @@ def bt_compress(dense: torch.Tensor, bitmap: torch.Tensor, values: torch.Tensor,
                 check: bool = True) -> int:
     n = dense.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = _calls().bt_compress(dense, n, DTYPE_CODE[dense.dtype], bitmap, values, cap,
+    st = _tensor_calls().bt_compress(dense, n, DTYPE_CODE[dense.dtype], bitmap, values, cap,
                               chunk_prefix, nnz_out, workspace,
                               workspace.numel() * workspace.element_size(), dev_status, _stream(stream))
     return _check("bt_compress", st, check)
@@ -239,14 +262,14 @@ def batch_items(dense, stashes, y_out=None) -> "ctypes.Array":
 
 def bt_compress_batch(items, dtype: torch.dtype, workspace: torch.Tensor, *, stream=None, check: bool = True) -> int:
     """bt_compress of every tensor of `items` (from batch_items) in one pass."""
-    st = _calls().bt_compress_batch(items, len(items), DTYPE_CODE[dtype], workspace, _nbytes(workspace), _stream(stream))
+    st = _tensor_calls().bt_compress_batch(items, len(items), DTYPE_CODE[dtype], workspace, _nbytes(workspace), _stream(stream))
     return _check("bt_compress_batch", st, check)
 
 
 def bt_relu_fwd_compress_batch(items, dtype: torch.dtype, workspace: torch.Tensor, *, stream=None,
                                check: bool = True) -> int:
     """bt_relu_fwd_compress of every tensor of `items` (from batch_items) in one pass."""
-    st = _calls().bt_relu_fwd_compress_batch(items, len(items), DTYPE_CODE[dtype], workspace, _nbytes(workspace),
+    st = _tensor_calls().bt_relu_fwd_compress_batch(items, len(items), DTYPE_CODE[dtype], workspace, _nbytes(workspace),
                                              _stream(stream))
     return _check("bt_relu_fwd_compress_batch", st, check)
 
@@ -256,7 +279,7 @@ def bt_compress_arena_batch(items, dtype: torch.dtype, arena: torch.Tensor, aren
                             check: bool = True) -> int:
     """The tensors of `items` pushed into the arena back to back by one pass (fused: ReLU forward first);
     values_offsets_out is a device int64 tensor with one word per item."""
-    fn = _calls().bt_relu_fwd_compress_arena_batch if fused else _calls().bt_compress_arena_batch
+    fn = _tensor_calls().bt_relu_fwd_compress_arena_batch if fused else _tensor_calls().bt_compress_arena_batch
     st = fn(items, len(items), DTYPE_CODE[dtype], arena, _nbytes(arena), arena_cursor, values_offsets_out, workspace,
             _nbytes(workspace), _stream(stream))
     return _check("bt_compress_arena_batch", st, check)
@@ -265,19 +288,19 @@ def bt_compress_arena_batch(items, dtype: torch.dtype, arena: torch.Tensor, aren
 def bt_decompress_arena_batch(items, dtype: torch.dtype, arena: torch.Tensor, values_offsets: torch.Tensor, *, stream=None,
                               check: bool = True) -> int:
     """Every item's y_out restored from (bitmap, arena + values_offsets[k], chunk_prefix) in one pass."""
-    st = _calls().bt_decompress_arena_batch(items, len(items), DTYPE_CODE[dtype], arena, values_offsets, _stream(stream))
+    st = _tensor_calls().bt_decompress_arena_batch(items, len(items), DTYPE_CODE[dtype], arena, values_offsets, _stream(stream))
     return _check("bt_decompress_arena_batch", st, check)
 
 
 def bt_decompress_batch(items, dtype: torch.dtype, *, stream=None, check: bool = True) -> int:
     """bt_decompress of every stash of `items` into its y_out, in one pass."""
-    st = _calls().bt_decompress_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
+    st = _tensor_calls().bt_decompress_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
     return _check("bt_decompress_batch", st, check)
 
 
 def bt_relu_bwd_from_bitmap_batch(items, dtype: torch.dtype, *, stream=None, check: bool = True) -> int:
     """bt_relu_bwd_from_bitmap of every item (dense: upstream gradient, y_out: input gradient), in one pass."""
-    st = _calls().bt_relu_bwd_from_bitmap_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
+    st = _tensor_calls().bt_relu_bwd_from_bitmap_batch(items, len(items), DTYPE_CODE[dtype], _stream(stream))
     return _check("bt_relu_bwd_from_bitmap_batch", st, check)
 
 
@@ -288,7 +311,7 @@ def bt_compress_noalloc(dense: torch.Tensor, bitmap: torch.Tensor, values: torch
     call allocates nothing (for callers that may not); n is limited to NOALLOC_MAX_ELEMS."""
     n = dense.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = _calls().bt_compress_noalloc(dense, n, DTYPE_CODE[dense.dtype], bitmap, values, cap,
+    st = _tensor_calls().bt_compress_noalloc(dense, n, DTYPE_CODE[dense.dtype], bitmap, values, cap,
                                       chunk_prefix, nnz_out, dev_status, _stream(stream))
     return _check("bt_compress_noalloc", st, check)
 
@@ -300,7 +323,7 @@ def bt_relu_fwd_compress(pre_act: torch.Tensor, y_out: Optional[torch.Tensor], b
                          check: bool = True) -> int:
     n = pre_act.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = _calls().bt_relu_fwd_compress(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
+    st = _tensor_calls().bt_relu_fwd_compress(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
                                        values, cap, chunk_prefix, nnz_out, workspace,
                                        workspace.numel() * workspace.element_size(), dev_status,
                                        _stream(stream))
@@ -316,7 +339,7 @@ def bt_prune_fwd_compress(x: torch.Tensor, tau: float, y_out: Optional[torch.Ten
     """Activation pruning fused with the stash: elements <= tau (a binary32 threshold) become +0."""
     n = x.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = _calls().bt_prune_fwd_compress(x, n, DTYPE_CODE[x.dtype], float(tau), y_out, bitmap,
+    st = _tensor_calls().bt_prune_fwd_compress(x, n, DTYPE_CODE[x.dtype], tau, y_out, bitmap,
                                         values, cap, chunk_prefix, nnz_out, workspace,
                                         workspace.numel() * workspace.element_size(), dev_status,
                                         _stream(stream))
@@ -339,7 +362,7 @@ def bt_compress_narrow(dense: torch.Tensor, bitmap: torch.Tensor, values: torch.
     n = dense.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
     assert dense.dtype == torch.float32
-    st = _calls().bt_compress_narrow(dense, n, DTYPE_CODE[values.dtype], bitmap, values, cap,
+    st = _tensor_calls().bt_compress_narrow(dense, n, DTYPE_CODE[values.dtype], bitmap, values, cap,
                                      chunk_prefix, nnz_out, workspace, _nbytes(workspace),
                                      dev_status, _stream(stream))
     return _check("bt_compress_narrow", st, check)
@@ -354,7 +377,7 @@ def bt_prune_fwd_compress_narrow(x: torch.Tensor, tau: float, y_out: Optional[to
     n = x.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
     assert x.dtype == torch.float32
-    st = _calls().bt_prune_fwd_compress_narrow(x, n, DTYPE_CODE[values.dtype], float(tau), y_out,
+    st = _tensor_calls().bt_prune_fwd_compress_narrow(x, n, DTYPE_CODE[values.dtype], tau, y_out,
                                                bitmap, values, cap, chunk_prefix, nnz_out,
                                                workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_prune_fwd_compress_narrow", st, check)
@@ -365,7 +388,7 @@ def bt_decompress_widen(bitmap: torch.Tensor, values: torch.Tensor, chunk_prefix
     """Restores a narrowed stash (16-bit `values`) into a float32 tensor."""
     n = dense_out.numel() if n is None else n
     assert dense_out.dtype == torch.float32
-    st = _calls().bt_decompress_widen(bitmap, values, chunk_prefix, n, DTYPE_CODE[values.dtype],
+    st = _tensor_calls().bt_decompress_widen(bitmap, values, chunk_prefix, n, DTYPE_CODE[values.dtype],
                                       dense_out, _stream(stream))
     return _check("bt_decompress_widen", st, check)
 
@@ -377,7 +400,7 @@ def bt_maxpool2x2_fwd(x: torch.Tensor, y: torch.Tensor, codes: Optional[torch.Te
     height = x.shape[-2] if height is None else height
     width = x.shape[-1] if width is None else width
     planes = x.numel() // max(1, height * width) if planes is None else planes
-    st = _calls().bt_maxpool2x2_fwd(x, planes, height, width, DTYPE_CODE[x.dtype], y, codes, _stream(stream))
+    st = _tensor_calls().bt_maxpool2x2_fwd(x, planes, height, width, DTYPE_CODE[x.dtype], y, codes, _stream(stream))
     return _check("bt_maxpool2x2_fwd", st, check)
 
 
@@ -387,7 +410,7 @@ def bt_maxpool2x2_bwd(codes: torch.Tensor, grad_out: torch.Tensor, grad_in: torc
     height = grad_in.shape[-2] if height is None else height
     width = grad_in.shape[-1] if width is None else width
     planes = grad_in.numel() // max(1, height * width) if planes is None else planes
-    st = _calls().bt_maxpool2x2_bwd(codes, grad_out, planes, height, width, DTYPE_CODE[grad_out.dtype],
+    st = _tensor_calls().bt_maxpool2x2_bwd(codes, grad_out, planes, height, width, DTYPE_CODE[grad_out.dtype],
                                     grad_in, _stream(stream))
     return _check("bt_maxpool2x2_bwd", st, check)
 
@@ -400,7 +423,7 @@ def bt_maxpool2x2_bwd_masked(codes: torch.Tensor, pooled_bitmap: torch.Tensor, g
     height = grad_in.shape[-2] if height is None else height
     width = grad_in.shape[-1] if width is None else width
     planes = grad_in.numel() // max(1, height * width) if planes is None else planes
-    st = _calls().bt_maxpool2x2_bwd_masked(codes, pooled_bitmap, grad_out, planes, height, width,
+    st = _tensor_calls().bt_maxpool2x2_bwd_masked(codes, pooled_bitmap, grad_out, planes, height, width,
                                            DTYPE_CODE[grad_out.dtype], grad_in, _stream(stream))
     return _check("bt_maxpool2x2_bwd_masked", st, check)
 
@@ -411,7 +434,7 @@ def bt_mask_compress(x: torch.Tensor, mask_bitmap: torch.Tensor, mask_chunk_pref
     """Double-mask form: the values of x at the set bits of an existing stash's bitmap (and the masked dense y)."""
     n = x.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = _calls().bt_mask_compress(x, n, DTYPE_CODE[x.dtype], mask_bitmap, mask_chunk_prefix,
+    st = _tensor_calls().bt_mask_compress(x, n, DTYPE_CODE[x.dtype], mask_bitmap, mask_chunk_prefix,
                                    y_out, values, cap, _stream(stream))
     return _check("bt_mask_compress", st, check)
 
@@ -422,7 +445,7 @@ def bt_compress_arena(dense: torch.Tensor, bitmap: torch.Tensor, arena: torch.Te
                       stream=None, check: bool = True) -> int:
     """bt_compress whose values go behind the cursor of a caller-owned arena (a uint8 device tensor)."""
     n = dense.numel() if n is None else n
-    st = _calls().bt_compress_arena(dense, n, DTYPE_CODE[dense.dtype], bitmap, arena, _nbytes(arena),
+    st = _tensor_calls().bt_compress_arena(dense, n, DTYPE_CODE[dense.dtype], bitmap, arena, _nbytes(arena),
                                     arena_cursor, values_offset_out, chunk_prefix, nnz_out,
                                     workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_compress_arena", st, check)
@@ -435,7 +458,7 @@ def bt_prune_fwd_compress_arena(x: torch.Tensor, tau: float, y_out: Optional[tor
                                 check: bool = True) -> int:
     """Fused forward (tau = 0: ReLU) whose values go behind the cursor of a caller-owned arena."""
     n = x.numel() if n is None else n
-    st = _calls().bt_prune_fwd_compress_arena(x, n, DTYPE_CODE[x.dtype], float(tau), y_out,
+    st = _tensor_calls().bt_prune_fwd_compress_arena(x, n, DTYPE_CODE[x.dtype], tau, y_out,
                                               bitmap, arena, _nbytes(arena), arena_cursor,
                                               values_offset_out, chunk_prefix, nnz_out,
                                               workspace, _nbytes(workspace), dev_status, _stream(stream))
@@ -446,7 +469,7 @@ def bt_decompress_arena(bitmap: torch.Tensor, arena: torch.Tensor, values_offset
                         chunk_prefix: torch.Tensor, dense_out: torch.Tensor, *, n: Optional[int] = None, stream=None,
                         check: bool = True) -> int:
     n = dense_out.numel() if n is None else n
-    st = _calls().bt_decompress_arena(bitmap, arena, values_offset, chunk_prefix, n,
+    st = _tensor_calls().bt_decompress_arena(bitmap, arena, values_offset, chunk_prefix, n,
                                       DTYPE_CODE[dense_out.dtype], dense_out, _stream(stream))
     return _check("bt_decompress_arena", st, check)
 
@@ -458,7 +481,7 @@ def bt_compress_narrow_arena(dense: torch.Tensor, to_dtype: torch.dtype, bitmap:
     """bt_compress_narrow whose 16-bit values (of `to_dtype`) go behind the cursor of a caller-owned arena."""
     n = dense.numel() if n is None else n
     assert dense.dtype == torch.float32
-    st = _calls().bt_compress_narrow_arena(dense, n, DTYPE_CODE[to_dtype], bitmap, arena, _nbytes(arena),
+    st = _tensor_calls().bt_compress_narrow_arena(dense, n, DTYPE_CODE[to_dtype], bitmap, arena, _nbytes(arena),
                                            arena_cursor, values_offset_out, chunk_prefix, nnz_out,
                                            workspace, _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_compress_narrow_arena", st, check)
@@ -472,7 +495,7 @@ def bt_prune_fwd_compress_narrow_arena(x: torch.Tensor, to_dtype: torch.dtype, t
     """bt_prune_fwd_compress_narrow whose 16-bit values (of `to_dtype`) go behind the cursor of a caller-owned arena."""
     n = x.numel() if n is None else n
     assert x.dtype == torch.float32
-    st = _calls().bt_prune_fwd_compress_narrow_arena(x, n, DTYPE_CODE[to_dtype], float(tau), y_out,
+    st = _tensor_calls().bt_prune_fwd_compress_narrow_arena(x, n, DTYPE_CODE[to_dtype], tau, y_out,
                                                      bitmap, arena, _nbytes(arena), arena_cursor,
                                                      values_offset_out, chunk_prefix, nnz_out,
                                                      workspace, _nbytes(workspace), dev_status, _stream(stream))
@@ -485,7 +508,7 @@ def bt_decompress_widen_arena(bitmap: torch.Tensor, arena: torch.Tensor, values_
     """Restores a narrowed stash whose 16-bit values (of `from_dtype`) sit in an arena into a float32 tensor."""
     n = dense_out.numel() if n is None else n
     assert dense_out.dtype == torch.float32
-    st = _calls().bt_decompress_widen_arena(bitmap, arena, values_offset, chunk_prefix, n,
+    st = _tensor_calls().bt_decompress_widen_arena(bitmap, arena, values_offset, chunk_prefix, n,
                                             DTYPE_CODE[from_dtype], dense_out, _stream(stream))
     return _check("bt_decompress_widen_arena", st, check)
 
@@ -497,7 +520,7 @@ def bt_relu6_fwd_compress_arena(pre_act: torch.Tensor, y_out: Optional[torch.Ten
                                 check: bool = True) -> int:
     """Fused ReLU6 forward whose values go behind the cursor of a caller-owned arena."""
     n = pre_act.numel() if n is None else n
-    st = _calls().bt_relu6_fwd_compress_arena(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
+    st = _tensor_calls().bt_relu6_fwd_compress_arena(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
                                               arena, _nbytes(arena), arena_cursor, values_offset_out,
                                               chunk_prefix, nnz_out, workspace, _nbytes(workspace),
                                               dev_status, _stream(stream))
@@ -509,7 +532,7 @@ def bt_relu6_bwd_from_stash_arena(bitmap: torch.Tensor, arena: torch.Tensor, val
                                   *, n: Optional[int] = None, stream=None, check: bool = True) -> int:
     """ReLU6 backward from a stash whose values sit in an arena."""
     n = grad_out.numel() if n is None else n
-    st = _calls().bt_relu6_bwd_from_stash_arena(bitmap, arena, values_offset, chunk_prefix,
+    st = _tensor_calls().bt_relu6_bwd_from_stash_arena(bitmap, arena, values_offset, chunk_prefix,
                                                 grad_out, n, DTYPE_CODE[grad_out.dtype], grad_in, _stream(stream))
     return _check("bt_relu6_bwd_from_stash_arena", st, check)
 
@@ -521,7 +544,7 @@ def bt_relu6_fwd_compress(pre_act: torch.Tensor, y_out: Optional[torch.Tensor], 
                           check: bool = True) -> int:
     n = pre_act.numel() if n is None else n
     cap = values.numel() if values_capacity is None else values_capacity
-    st = _calls().bt_relu6_fwd_compress(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
+    st = _tensor_calls().bt_relu6_fwd_compress(pre_act, n, DTYPE_CODE[pre_act.dtype], y_out, bitmap,
                                         values, cap, chunk_prefix, nnz_out, workspace,
                                         _nbytes(workspace), dev_status, _stream(stream))
     return _check("bt_relu6_fwd_compress", st, check)
@@ -531,7 +554,7 @@ def bt_relu6_bwd_from_stash(bitmap: torch.Tensor, values: torch.Tensor, chunk_pr
                             grad_out: torch.Tensor, grad_in: torch.Tensor, *, n: Optional[int] = None, stream=None,
                             check: bool = True) -> int:
     n = grad_out.numel() if n is None else n
-    st = _calls().bt_relu6_bwd_from_stash(bitmap, values, chunk_prefix, grad_out, n,
+    st = _tensor_calls().bt_relu6_bwd_from_stash(bitmap, values, chunk_prefix, grad_out, n,
                                           DTYPE_CODE[grad_out.dtype], grad_in, _stream(stream))
     return _check("bt_relu6_bwd_from_stash", st, check)
 
@@ -539,7 +562,7 @@ def bt_relu6_bwd_from_stash(bitmap: torch.Tensor, values: torch.Tensor, chunk_pr
 def bt_decompress(bitmap: torch.Tensor, values: torch.Tensor, chunk_prefix: torch.Tensor, dense_out: torch.Tensor,
                   *, n: Optional[int] = None, stream=None, check: bool = True) -> int:
     n = dense_out.numel() if n is None else n
-    st = _calls().bt_decompress(bitmap, values, chunk_prefix, n, DTYPE_CODE[dense_out.dtype],
+    st = _tensor_calls().bt_decompress(bitmap, values, chunk_prefix, n, DTYPE_CODE[dense_out.dtype],
                                 dense_out, _stream(stream))
     return _check("bt_decompress", st, check)
 
@@ -547,7 +570,7 @@ def bt_decompress(bitmap: torch.Tensor, values: torch.Tensor, chunk_prefix: torc
 def bt_relu_bwd_from_bitmap(bitmap: torch.Tensor, grad_out: torch.Tensor, grad_in: torch.Tensor,
                             *, n: Optional[int] = None, stream=None, check: bool = True) -> int:
     n = grad_out.numel() if n is None else n
-    st = _calls().bt_relu_bwd_from_bitmap(bitmap, grad_out, n, DTYPE_CODE[grad_out.dtype], grad_in,
+    st = _tensor_calls().bt_relu_bwd_from_bitmap(bitmap, grad_out, n, DTYPE_CODE[grad_out.dtype], grad_in,
                                           _stream(stream))
     return _check("bt_relu_bwd_from_bitmap", st, check)
 
