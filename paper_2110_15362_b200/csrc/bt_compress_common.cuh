@@ -22,7 +22,9 @@ namespace cmp {
 constexpr uint32_t kFull       = 0xFFFFFFFFu;
 constexpr int      kMaxWindows = 5;                   // the grid never exceeds 32 * kMaxWindows CTAs
 constexpr int      kHdrSeq     = 0;                   // header words (64-bit): launch sequence number,
-constexpr int      kHdrAbort   = 1;                   //   abort word (== the launch's tag once a wait ran out)
+constexpr int      kHdrAbort   = 1;                   //   abort word (== the launch's tag once a wait ran out),
+constexpr int      kHdrCursor  = 2;                   //   batched arena form: the cursor as the launch found it, and
+constexpr int      kHdrPushed  = 3;                   //   1 once its last tile is finished, 0 before
 
 __device__ __forceinline__ uint64_t now_ns()
 {

@@ -13,7 +13,8 @@ namespace bt {
 // ---------------------------------------------------------------- workspace layout
 // The workspace arrives with unspecified contents.  It holds
 //   a 256-byte header, 64-bit words: [0] seq, the launch sequence number of this workspace; [1] abort, equal to
-//     the launch's tag once a bounded wait of that launch ran out;
+//     the launch's tag once a bounded wait of that launch ran out; [2], [3] of a batched arena launch: the cursor
+//     that it found, and 1 once it is complete (read by the launch behind it);
 //   one 16-byte descriptor per tile, never cleared: word 0 = (tag >> 32) << 32 | count, word 1 = (tag & 0xFFFFFFFF)
 //     << 32 | count.  A reader takes a descriptor only if both halves carry its own launch's tag and agree on
 //     the count (the two halves may be written and read separately).

@@ -263,3 +263,48 @@ def test_fused_batch_on_every_two_byte_pattern(oracle, kind, want_y):
     B.bt_relu_fwd_compress_batch(B.batch_items(xs, sts, ys), dt, ws)
     torch.cuda.synchronize()
     check_batch(oracle, kind, raws, sts, ys, True)
+
+
+def _pushes(counts, es, room, cursor0=0):
+    """(offset or None if it does not fit) of every push, and the cursor behind the last, as single calls would leave them."""
+    at, offsets = cursor0, []
+    for z in counts:
+        fits = z * es <= room - at
+        offsets.append(at if fits else None)
+        at += (z * es + 15) // 16 * 16 if fits else 0
+    return offsets, at
+
+
+# tiles of the tensor that does not fit, and of the ones behind it; `lead`: tensors in front
+FULL = {"one_behind": (1, [40], [1]), "many_tiles": (2, [400], [30, 2]), "fits_between": (1, [200, 3, 180], [2, 90]), "at_the_launch_edge": (31, [60], [1, 1]),
+        "behind_the_launch_edge": (30, [60], [1, 50, 1])}
+
+
+@pytest.mark.parametrize("kind,fused", [("f32", False), ("bf16", True), ("f64", False), ("f16", False)])
+@pytest.mark.parametrize("shape", list(FULL))
+def test_arena_batch_values_behind_a_tensor_that_does_not_fit(oracle, kind, fused, shape):
+    """A tensor that fits behind one that does not starts at the same byte: its values are whole, as after single calls."""
+    es = np.dtype(W.random_patterns(1, kind, 0.0, seed=0).dtype).itemsize
+    tile = 32768 // es
+    lead, big, small = FULL[shape]
+    sizes = [tile // 2 + 5 * k for k in range(lead)] + [b * tile - 3 for b in big[:1]]
+    for k, t in enumerate(small):
+        sizes += [t * tile - 77 - k] + [b * tile + 9 for b in big[1 + k:2 + k]]
+    seed = 4000 + lead
+    raws = [W.random_patterns(n, kind, 0.5, seed=seed + 7 * k) for k, n in enumerate(sizes)]
+    refs = [oracle.relu_fwd_compress(r, kind)[1] if fused else oracle.compress(r) for r in raws]
+    counts = [c.nnz for c in refs]
+    # room for the tensors in front, for the small ones behind, and for nearly all of the first large one
+    need = sum((z * es + 15) // 16 * 16 for z in counts[:lead]) + 48
+    room = max(need + sum((counts[k] * es + 15) // 16 * 16 for k in range(lead + 1, len(sizes)) if sizes[k] < sizes[lead] // 2),
+               need + counts[lead] * es - 64 - 48) // 16 * 16
+    offsets, end = _pushes(counts, es, room, 48)
+    assert offsets[lead] is None and all(o is not None for o in offsets[:lead]) and any(o is not None for o in offsets[lead + 1:])
+    for _ in range(6):
+        _, sts, _, arena, cursor, offs = _arena_batch(kind, sizes, seed, fused, room, cursor0=48)
+        assert [st.status for st in sts] == [B.BT_ERR_CAPACITY if o is None else B.BT_OK for o in offsets]
+        assert offs.tolist() == [-7 if o is None else o for o in offsets] and int(cursor.item()) == end
+        for o, c, raw in zip(offsets, refs, raws):
+            if o is not None:
+                assert np.array_equal(arena[o:o + c.nnz * es].cpu().numpy().view(raw.dtype), c.values)
+        assert bool((arena[:48] == 0x5A).all().item()) and bool((arena[room:] == 0x5A).all().item())
