@@ -42,7 +42,7 @@ from __future__ import annotations
 
 import threading
 import weakref
-from typing import Dict, Optional, Tuple
+from typing import Dict, NamedTuple, Optional, Tuple
 
 import torch
 
@@ -185,30 +185,48 @@ class _Scratch:
         return v
 
 
+class _StatusWord(NamedTuple):
+    address: int
+    block: torch.Tensor
+    index: int
+
+
 class _StatusWords:
-    """Device status words of the calls of a pass, handed out from blocks; fresh blocks after every check."""
+    """Device status words of the calls of a pass, handed out from blocks; fresh blocks after every check.  A word counts
+    once its call is made (nothing ever writes the word of a call that failed), and holds its block until then."""
 
     BLOCK = 64
 
     def __init__(self):
-        self.blocks: list = []           # (block, words handed out)
+        self._lock = threading.Lock()
+        self._block: Optional[torch.Tensor] = None
+        self._used = 0
+        self._made: list = []
 
     def __bool__(self) -> bool:
-        return bool(self.blocks)
+        return bool(self._made)
 
-    def next(self, device) -> int:
-        """The address of a new word on `device`."""
-        if not self.blocks or self.blocks[-1][1] == self.BLOCK or self.blocks[-1][0].device != device:
-            self.blocks.append([torch.empty(self.BLOCK, dtype=torch.int32, device=device), 0])
-        last = self.blocks[-1]
-        last[1] += 1
-        return last[0].data_ptr() + 4 * (last[1] - 1)
+    def next(self, device) -> _StatusWord:
+        """A new word on `device`."""
+        with self._lock:
+            if self._block is None or self._used == self.BLOCK or self._block.device != device:
+                self._block, self._used = torch.empty(self.BLOCK, dtype=torch.int32, device=device), 0
+            k, block = self._used, self._block
+            self._used += 1
+        return _StatusWord(block.data_ptr() + 4 * k, block, k)
+
+    def made(self, word: _StatusWord) -> None:
+        """The call that reports in `word` is on its stream."""
+        with self._lock:
+            self._made.append(word)
 
     def drain(self) -> list:
-        """The words handed out since the last time (one host read per block)."""
-        words = [w for block, used in self.blocks for w in block[:used].tolist()]
-        self.blocks = []
-        return words
+        """The words of the calls made since the last time (one host read per block)."""
+        with self._lock:
+            made, self._made, self._block = self._made, [], None
+        blocks = {id(w.block): w.block for w in made}
+        read = {at: block.tolist() for at, block in blocks.items()}
+        return [read[id(w.block)][w.index] for w in made]
 
 
 class _HostWords(threading.local):
@@ -290,8 +308,9 @@ def _compress_arena(x: torch.Tensor, owner, relu_into: Optional[torch.Tensor] = 
     ws, calls, arena = owner.scratch.workspace(n, dev), B._calls(), owner.arena
     at = record.buf.data_ptr()
     words = at + _words_at(n)
-    tail = (at, arena, arena.numel(), owner.cursor, words + 8, at + _prefix_at(n), words, ws, ws.numel(),
-            owner.statuses.next(dev), B._stream(None))
+    status = owner.statuses.next(dev)
+    tail = (at, arena, arena.numel(), owner.cursor, words + 8, at + _prefix_at(n), words, ws, ws.numel(), status.address,
+            B._stream(None))
     code = B.DTYPE_CODE[narrow or x.dtype]
     if relu6:
         st = calls.bt_relu6_fwd_compress_arena(x, n, code, relu_into, *tail)
@@ -301,6 +320,7 @@ def _compress_arena(x: torch.Tensor, owner, relu_into: Optional[torch.Tensor] = 
         st = (calls.bt_prune_fwd_compress_arena if narrow is None else calls.bt_prune_fwd_compress_narrow_arena)(
             x, n, code, 0.0, relu_into, *tail)
     B._check("bt_*_arena (autograd stash)", st, True)
+    owner.statuses.made(status)
     return record, narrow or x.dtype
 
 
@@ -437,9 +457,11 @@ class ReLUStash:
             # nobody will ask for the activation again (e.g. it only feeds a pooling layer that keeps winner codes):
             # the bitmap is all this ReLU's backward pass needs, so the values are not stored at all
             statuses = hooks.loose_statuses if hooks is not None else _StatusWords()
+            status = statuses.next(dev)
             st, y, _ = _native.relu_stash(x, address["bt_relu_fwd_compress"], bwd, _PLAIN, B.DTYPE_CODE[x.dtype], inplace, None, 0,
-                                          None, None, ws, ws.numel(), statuses.next(dev))
+                                          None, None, ws, ws.numel(), status.address)
             B._check("bt_relu_fwd_compress (bitmap only)", st, True)
+            statuses.made(status)
             if hooks is None:                           # BT_ERR_CAPACITY is the expected answer here
                 st = statuses.drain()[0]
                 if st not in (B.BT_OK, B.BT_ERR_CAPACITY):
@@ -451,9 +473,11 @@ class ReLUStash:
         if hooks is not None and hooks.arena is not None:
             arena = hooks.arena
             call = "bt_prune_fwd_compress_arena" if narrow is None else "bt_prune_fwd_compress_narrow_arena"
+            status = hooks.statuses.next(dev)
             st, y, buf = _native.relu_stash(x, address[call], bwd, _ARENA, code, inplace, arena, arena.numel(), hooks.cursor, None,
-                                            ws, ws.numel(), hooks.statuses.next(dev))
+                                            ws, ws.numel(), status.address)
             B._check("bt_*_arena (autograd stash)", st, True)
+            hooks.statuses.made(status)
             hooks.share(y, _packed_arena(y, _Record(n, buf=buf), hooks, stored))
             hooks.dense_bytes += n * y.element_size()
             return y
