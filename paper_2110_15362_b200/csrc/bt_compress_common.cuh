@@ -721,17 +721,17 @@ struct LaunchShape {
     cudaError_t max_grid(Kernel kernel, int threads, size_t smem, int &grid)
     {
         int         dev = 0;
-        cudaError_t e   = cudaGetDevice(&dev);
+        cudaError_t e   = reported(cudaGetDevice(&dev));
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
         std::lock_guard<std::mutex> g(lock);
         if (grid_of_device[dev] == 0) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+            e = reported(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
             if (e != cudaSuccess) return e;
             int sms = 0, per_sm = 0;
-            e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            e = reported(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
             if (e != cudaSuccess) return e;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+            e = reported(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
             if (e != cudaSuccess) return e;
             if (per_sm < 1 || sms < 1) return cudaErrorLaunchOutOfResources;
             grid_of_device[dev] = sms * per_sm;

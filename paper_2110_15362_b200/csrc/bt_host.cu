@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(kCopyThreads)
 copy_values_sized(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst, const uint64_t *__restrict__ nnz,
                   const uint64_t capacity, const uint64_t n, const uint32_t es)
 {
+    bt::in_stream_order();
     uint64_t count = *nnz < capacity ? *nnz : capacity;
     count          = count < n ? count : n;     // src holds n elements whatever a failed launch left in *nnz
     const uint64_t   bytes = count * es;
@@ -71,7 +72,7 @@ struct Staging {
     }
 };
 
-inline bool ok(cudaError_t e) { return e == cudaSuccess; }
+inline bool ok(cudaError_t e) { return bt::reported(e) == cudaSuccess; }
 
 int compress_host_common(bool relu, const void *host_in, uint64_t n, int dtype, void *host_y, uint32_t *host_bitmap,
                          void *host_values, uint64_t host_values_capacity, uint64_t *host_prefix, uint64_t *host_nnz,
@@ -123,9 +124,9 @@ int compress_host_common(bool relu, const void *host_in, uint64_t n, int dtype, 
         // page-locked value buffer: the device copies exactly min(nnz, capacity) values; one synchronisation
         int dev = 0, sms = 0;
         if (!ok(cudaGetDevice(&dev)) || !ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return fail();
-        copy_values_sized<<<sms * 4, kCopyThreads, 0, s>>>(g.values, mapped, reinterpret_cast<const uint64_t *>(g.nnz),
-                                                            host_values_capacity, n, static_cast<uint32_t>(es));
-        if (!ok(cudaGetLastError())) return fail();
+        if (!ok(bt::launch(copy_values_sized, static_cast<unsigned>(sms) * 4, kCopyThreads, 0, s, g.values, mapped,
+                           reinterpret_cast<const uint64_t *>(g.nnz), host_values_capacity, n, static_cast<uint32_t>(es))))
+            return fail();
     }
     if (!ok(cudaStreamSynchronize(s))) return BT_ERR_CUDA;
     if (status != BT_OK) return status;

@@ -152,6 +152,14 @@ cudaError_t launch_relu_bwd(const uint32_t *bitmap, const void *gout, uint64_t n
 // (cudaTriggerProgrammaticLaunchCompletion): the launch begins when the last CTAs exit.  With leave given at the start
 // the next kernel's CTAs take SM slots from the streaming kernels' own: four calls on fp32 2^28 elements 1093 -> 1164 us,
 // against 1090 this way; three calls on fp16 [64,512,28,28] 66.0 -> 61.5 us this way.
+//
+// A failed runtime call is reported by the call of the library it belongs to, through its own result, and taken out of the
+// runtime's last-error word; no launch is judged by that word, which may hold the error of an earlier call.
+inline cudaError_t reported(const cudaError_t e)
+{
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
 template <typename... P, typename... A>
 inline cudaError_t launch_as(bool cooperative, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)
 {
@@ -163,7 +171,7 @@ inline cudaError_t launch_as(bool cooperative, void (*kernel)(P...), unsigned gr
     cudaLaunchConfig_t c{};
     c.gridDim = dim3(grid), c.blockDim = dim3(threads), c.dynamicSmemBytes = smem, c.stream = stream;
     c.attrs = attr, c.numAttrs = cooperative ? 2 : 1;
-    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+    return reported(cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...));
 }
 template <typename... P, typename... A>
 inline cudaError_t launch(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)

@@ -235,12 +235,10 @@ cudaError_t launch_typed(const void *x, const uint32_t *bitmap, const uint64_t *
     const uint64_t grid     = (quarters + kWarps - 1) / kWarps;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     if (y)
-        launch(mask_gather_kernel<U, kE, kWarps, true>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
-            static_cast<const U *>(x), bitmap, prefix, n, static_cast<U *>(y), static_cast<U *>(values), capacity);
-    else
-        launch(mask_gather_kernel<U, kE, kWarps, false>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, 
-            static_cast<const U *>(x), bitmap, prefix, n, nullptr, static_cast<U *>(values), capacity);
-    return cudaGetLastError();
+        return launch(mask_gather_kernel<U, kE, kWarps, true>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, static_cast<const U *>(x), bitmap,
+                      prefix, n, static_cast<U *>(y), static_cast<U *>(values), capacity);
+    return launch(mask_gather_kernel<U, kE, kWarps, false>, static_cast<unsigned>(grid), kWarps * 32, 0, stream, static_cast<const U *>(x), bitmap,
+                  prefix, n, nullptr, static_cast<U *>(values), capacity);
 }
 
 }  // namespace

@@ -126,9 +126,8 @@ cudaError_t launch_typed(const uint32_t *bitmap, const void *gout, uint64_t n, v
     uint64_t       grid = (vecs + kThreads * kUnroll - 1) / (kThreads * kUnroll);
     if (grid == 0) grid = 1;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    launch(relu_bwd_kernel<U>, static_cast<unsigned>(grid), kThreads, 0, stream, bitmap, static_cast<const U *>(gout), n,
-                                                                             static_cast<U *>(gin));
-    return cudaGetLastError();
+    return launch(relu_bwd_kernel<U>, static_cast<unsigned>(grid), kThreads, 0, stream, bitmap, static_cast<const U *>(gout), n,
+                  static_cast<U *>(gin));
 }
 
 }  // namespace
@@ -156,10 +155,9 @@ cudaError_t launch_relu_bwd_batch(const DecompressJob *jobs, uint32_t count, int
     }
     p.jobs = count;
     const unsigned grid = static_cast<unsigned>(blocks);
-    if (elem_size == 8) launch(relu_bwd_batch_kernel<uint64_t, kMaxBatch>, grid, kThreads, 0, stream, p);
-    else if (elem_size == 4) launch(relu_bwd_batch_kernel<uint32_t, kMaxBatch>, grid, kThreads, 0, stream, p);
-    else launch(relu_bwd_batch_kernel<uint16_t, kMaxBatch>, grid, kThreads, 0, stream, p);
-    return cudaGetLastError();
+    if (elem_size == 8) return launch(relu_bwd_batch_kernel<uint64_t, kMaxBatch>, grid, kThreads, 0, stream, p);
+    if (elem_size == 4) return launch(relu_bwd_batch_kernel<uint32_t, kMaxBatch>, grid, kThreads, 0, stream, p);
+    return launch(relu_bwd_batch_kernel<uint16_t, kMaxBatch>, grid, kThreads, 0, stream, p);
 }
 
 }  // namespace bt
