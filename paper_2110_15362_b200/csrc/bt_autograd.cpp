@@ -59,6 +59,7 @@ struct Request {
     void     *status;
     Tensor    record;        // out
     int       result = 0;    // out: the ABI's status code
+    bool      called = false;   // out: the compressor is on its stream (or has refused)
 };
 
 struct ReLUStash : torch::autograd::Function<ReLUStash> {
@@ -80,7 +81,8 @@ struct ReLUStash : torch::autograd::Function<ReLUStash> {
         auto *const words  = reinterpret_cast<uint64_t *>(rec + words_at(n));
         auto *const nnz    = r->nnz ? static_cast<uint64_t *>(r->nnz) : words;
         auto *const status = static_cast<int32_t *>(r->status);
-        if (r->call == 0) r->result = BT_OK;
+        r->called              = r->call != 0;
+        if (!r->called) r->result = BT_OK;
         else if (r->form == kArena)
             r->result = reinterpret_cast<decltype(&bt_prune_fwd_compress_arena)>(r->call)(
                 in.data_ptr(), n, r->code, 0.0f, y.data_ptr(), bitmap, r->store, r->room, static_cast<uint64_t *>(r->cursor), words + 1, prefix, nnz,
@@ -146,7 +148,15 @@ PyObject *relu_stash(PyObject *, PyObject *const *a, const Py_ssize_t count)
     Tensor y;
     {
         pybind11::gil_scoped_release no_gil;
-        y = ReLUStash::apply(x, &r);
+        try {
+            y = ReLUStash::apply(x, &r);
+        } catch (...) {
+            // A saved-tensor hook raised behind the launch (a recomputation under a checkpoint ends that way).  With a count
+            // word of the caller's the kernel still has to store into memory that the caller's next call waits on: not later
+            // than here.
+            if (r.called && r.nnz) c10::cuda::getCurrentCUDAStream().synchronize();
+            throw;
+        }
     }
     return Py_BuildValue("(iNN)", r.result, THPVariable_Wrap(y), THPVariable_Wrap(r.record));
     END_HANDLE_TH_ERRORS

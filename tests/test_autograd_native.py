@@ -78,3 +78,33 @@ def test_every_form_of_the_node(form, dtype, kind, inplace):
         hooks.check_statuses()
     with torch.no_grad():
         assert not A.relu_stash(view(ref), keep_values=not form.startswith("bits")).requires_grad
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("two_pass", [True, False])
+def test_a_hook_that_raises_leaves_no_kernel_writing_the_threads_words(two_pass):
+    """The count of an exact-size stash goes to page-locked words of the thread; a hook that raises behind the launch must not
+    leave that store to a later moment, when the thread may be waiting for another stash's count on another stream."""
+    class Raised(Exception):
+        pass
+
+    def pack(t):
+        raise Raised
+
+    x = torch.randn(1 << 16, device="cuda").requires_grad_()
+    hooks = A.stash_saved_activations(min_numel=16, two_pass=two_pass)
+    with hooks:
+        A.relu_stash(x * 1, hooks).sum().backward()
+    torch.cuda.synchronize()
+    h, host = x.detach().clone().requires_grad_() * 1, A._read_back()
+    host.view[:] = -1
+    torch.cuda._sleep(100_000_000)
+    with torch.autograd.graph.saved_tensors_hooks(pack, lambda t: t):
+        with pytest.raises(Raised):
+            A.relu_stash(h, hooks)
+    seen = int(host.view[0])
+    torch.cuda.synchronize()
+    assert seen == int((h > 0).sum())
+    with hooks:
+        y = A.relu_stash(x * 1, hooks)
+    assert torch.equal(y, torch.relu(x)) and y._bt_packed.nnz == seen
