@@ -163,17 +163,27 @@ def _flat_input(t: torch.Tensor) -> torch.Tensor:
 
 
 class _Scratch:
-    """Per-device reusable buffers of the packing calls: workspace and a full-capacity values buffer."""
+    """Per-device reusable buffers of the packing calls: workspace and a full-capacity values buffer.  `kept`: the context's
+    own buffers.  All of them may be used on other streams than the one they were allocated on, and are given back as soon
+    as the context goes: the allocator is told of every stream."""
 
-    def __init__(self, two_pass: bool = True):
+    def __init__(self, two_pass: bool = True, kept: Tuple[torch.Tensor, ...] = ()):
         self.ws: Dict[torch.device, torch.Tensor] = {}
         self.ws_for: Dict[torch.device, int] = {}        # the largest element count a device's workspace serves
         self.values: Dict[Tuple[torch.device, torch.dtype], torch.Tensor] = {}
+        self.kept = kept
+        self.streams: Dict[Tuple[int, int], torch.cuda.Stream] = {}      # those of the calls so far, by device and handle
         self.two_pass = two_pass         # exact-size values without a full-capacity buffer (see _compress)
 
     def workspace(self, n: int, device) -> torch.Tensor:
+        if device.type == "cuda" and (device.index, torch._C._cuda_getCurrentRawStream(device.index)) not in self.streams:
+            stream = torch.cuda.current_stream(device)
+            self.streams[device.index, stream.cuda_stream] = stream
+            for t in (*self.kept, *self.ws.values(), *self.values.values()):
+                if t.device == device:
+                    t.record_stream(stream)
         if self.ws_for.get(device, -1) < n:
-            self.ws[device] = torch.empty(B.bt_workspace_bytes(n), dtype=torch.uint8, device=device)
+            self.ws[device] = self._new(B.bt_workspace_bytes(n), torch.uint8, device)
             self.ws_for[device] = n
         return self.ws[device]
 
@@ -181,8 +191,15 @@ class _Scratch:
         key = (device, dtype)
         v = self.values.get(key)
         if v is None or v.numel() < n:
-            v = self.values[key] = torch.empty(n, dtype=dtype, device=device)
+            v = self.values[key] = self._new(n, dtype, device)
         return v
+
+    def _new(self, n: int, dtype, device) -> torch.Tensor:
+        t = torch.empty(n, dtype=dtype, device=device)
+        for stream in self.streams.values():
+            if stream.device == device:
+                t.record_stream(stream)
+        return t
 
 
 class _StatusWord(NamedTuple):
@@ -349,6 +366,10 @@ class stash_saved_activations(torch.autograd.graph.saved_tensors_hooks):
     `two_pass` (exact-size mode): size the values by a first pass without values and fill them with a masked
     gather, instead of compacting into a buffer of full capacity that stays allocated (default)."""
 
+    # The base class would keep the bound method in the object, a reference cycle: a context that is dropped would hold its
+    # arena until the cyclic collector runs.  What an entered context needs is held by torch's stack of hooks.
+    pack_hook = property(lambda self: self._pack, lambda self, hook: None)
+
     def __init__(self, min_numel: int = 1 << 14, min_saving: float = 0.1, arena_bytes: Optional[int] = None,
                  device="cuda", narrow: Optional[torch.dtype] = None, two_pass: bool = True):
         if narrow not in (None, torch.float16, torch.bfloat16):
@@ -360,7 +381,7 @@ class stash_saved_activations(torch.autograd.graph.saved_tensors_hooks):
         if arena_bytes is not None:
             self.arena = torch.empty((arena_bytes + 15) // 16 * 16, dtype=torch.uint8, device=device)
             self.cursor = torch.zeros(1, dtype=torch.int64, device=device)
-        self.scratch = _Scratch(two_pass)
+        self.scratch = _Scratch(two_pass, () if self.arena is None else (self.arena, self.cursor))
         self.packed_bytes = 0            # bytes kept in compressed form so far
         self.dense_bytes = 0             # bytes the same tensors would have taken
         self._shared: Dict[int, Tuple[weakref.ref, weakref.ref]] = {}

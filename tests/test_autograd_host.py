@@ -1,5 +1,7 @@
 """Host side of the autograd integration, without a GPU: the words that calls report in, and what a context keeps alive."""
+import gc
 import threading
+import weakref
 
 import pytest
 import torch
@@ -73,3 +75,45 @@ def test_status_words_of_several_threads():
         t.join()
     got = sorted(seen + words.drain())
     assert got == sorted(1000 * t + k for t in range(4) for k in range(500))
+
+
+@pytest.mark.parametrize("entered", [False, True])
+def test_a_dropped_context_frees_its_arena_at_once(entered):
+    gc.collect()
+    gc.disable()
+    try:
+        hooks = _hooks(arena_bytes=1 << 16)
+        arena = weakref.ref(hooks.arena)
+        if entered:
+            x = torch.randn(64, requires_grad=True)
+            with hooks:
+                y = (x * x).sum()
+            y.backward()
+            assert torch.equal(x.grad, 2 * x)
+        del hooks
+        assert arena() is None
+    finally:
+        gc.enable()
+
+
+def test_an_entered_context_needs_no_other_reference():
+    """Entered by hand and dropped: its hooks stay in force until it is left."""
+    class Counted(A.stash_saved_activations):
+        packed = 0
+
+        def _pack(self, t):
+            Counted.packed += 1
+            return super()._pack(t)
+
+    gone = weakref.ref(Counted(device="cpu"))
+    assert gone() is None
+    h = Counted(device="cpu")
+    h.__enter__()
+    leave = torch._C._autograd._pop_saved_tensors_default_hooks
+    del h
+    try:
+        x = torch.randn(8, requires_grad=True)
+        (x * x).sum().backward()
+        assert Counted.packed == 2
+    finally:
+        leave()

@@ -108,3 +108,34 @@ def test_a_hook_that_raises_leaves_no_kernel_writing_the_threads_words(two_pass)
     with hooks:
         y = A.relu_stash(x * 1, hooks)
     assert torch.equal(y, torch.relu(x)) and y._bt_packed.nnz == seen
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", ["arena", "full"])
+def test_a_dropped_context_on_a_side_stream(mode):
+    """A context's buffers go back to the allocator as soon as it is dropped, but to no other stream before the one that the
+    pass ran on is done with them."""
+    n, opts = 3 << 20, {"arena": {"arena_bytes": 37 << 20}, "full": {"two_pass": False}}[mode]
+    x = torch.randn(n, device="cuda").requires_grad_()
+    hooks = A.stash_saved_activations(min_numel=16, **opts)
+    with hooks:
+        A.relu_stash(x.detach(), hooks)                                  # the scratch buffers: the default stream's
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    used = {t.data_ptr(): t.numel() * t.element_size() for t in (*hooks.scratch.kept, *hooks.scratch.ws.values(), *hooks.scratch.values.values())}
+    assert len(used) == (3 if mode == "arena" else 2)
+    with torch.cuda.stream(side):
+        with hooks:
+            y = A.relu_stash(x * 1, hooks) * 2
+            z = (y * y).sum()
+        hooks.check_statuses()                                           # its host read here, not behind the pause
+        torch.cuda._sleep(400_000_000)
+        z.backward()
+    del hooks, y, z
+    taken = [torch.empty(size, dtype=torch.uint8, device="cuda") for size in used.values() for _ in range(4)]
+    assert not side.query()                                              # the backward pass is still to run
+    assert not set(used) & {t.data_ptr() for t in taken}
+    torch.cuda.synchronize()
+    r = x.detach().clone().requires_grad_()
+    ((torch.relu(r * 1) * 2) ** 2).sum().backward()
+    assert torch.equal(x.grad, r.grad)
