@@ -108,15 +108,23 @@ def _tensor_calls() -> _Calls:
     return (_lib or lib()).tensor_calls
 
 
+def _native_call():
+    """What wraps a call of the library: the extension's native_call, or on a host without the extension ctypes alone."""
+    if not _build.native_calls():
+        return lambda address, kinds, through_ctypes, item: through_ctypes
+    try:
+        from . import _pycall
+    except ImportError as e:
+        raise ImportError(f"{_build.CALLER_PATH} is missing: build it with `python -m paper_2110_15362_b200.build`") from e
+    return _pycall.native_call
+
+
 def load_library(path: str) -> ctypes.CDLL:
     """Open a build of the library and declare the C ABI's signatures on it."""
     if not os.path.exists(path):
         raise ImportError(f"{path} is missing: build it with "
                           "`python -m paper_2110_15362_b200.build` (needs nvcc); there is no CPU fallback")
-    try:
-        from . import _pycall
-    except ImportError as e:
-        raise ImportError(f"{_build.CALLER_PATH} is missing: build it with `python -m paper_2110_15362_b200.build`") from e
+    native_call = _native_call()
     L = ctypes.CDLL(path)
     u64, vp, i32, sz = ctypes.c_uint64, ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
     L.bt_compressed_bytes.restype = sz
@@ -195,8 +203,8 @@ def load_library(path: str) -> ctypes.CDLL:
     L.bt_relu_fwd_compress_host.argtypes = [vp, u64, i32, vp, vp, vp, u64, vp, vp, vp, sz, vp]
     L.bt_relu_bwd_from_bitmap_host.restype = i32
     L.bt_relu_bwd_from_bitmap_host.argtypes = [vp, vp, u64, i32, vp, vp, sz, vp]
-    L.calls = _Calls(L, _pycall.native_call, "a")
-    L.tensor_calls = _Calls(L, _pycall.native_call, "p")
+    L.calls = _Calls(L, native_call, "a")
+    L.tensor_calls = _Calls(L, native_call, "p")
     return L
 
 

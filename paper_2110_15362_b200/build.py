@@ -4,6 +4,7 @@ from __future__ import annotations
 
 import glob
 import os
+import platform
 import shutil
 import subprocess
 import sysconfig
@@ -36,8 +37,15 @@ def is_stale(path: str = LIB_PATH) -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def native_calls() -> bool:
+    """Is there an extension module for calls on this host?  (It rests on the argument passing of x86-64.)"""
+    return platform.machine() == "x86_64"
+
+
 def build_caller(force: bool = False) -> str:
     """Compile the extension module the binding calls the library through; returns its path."""
+    if not native_calls():
+        return CALLER_PATH
     if not force and os.path.exists(CALLER_PATH) and os.path.getmtime(CALLER_PATH) >= os.path.getmtime(CALLER_SRC):
         return CALLER_PATH
     tmp = CALLER_PATH + ".tmp%d" % os.getpid()

@@ -18,10 +18,12 @@
  *
  * On x86-64 integer and pointer arguments travel in one sequence (six registers, then the stack) and float arguments in
  * another, so one prototype -- a float and kMax integer words -- fits every such function: the callee does not look at
- * words behind its own, and the caller clears the stack.
+ * words behind its own, and the caller clears the stack.  On other hosts the module is not built, and the binding calls
+ * through ctypes alone.
  */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <structmember.h>   /* T_PYSSIZET and READONLY: the names that Python versions before 3.12 have, too */
 #include <stddef.h>
 #include <stdint.h>
 #include <string.h>
@@ -181,7 +183,7 @@ fail:
 }
 
 static PyMemberDef native_call_members[] = {
-    {"__vectorcalloffset__", Py_T_PYSSIZET, offsetof(NativeCall, vectorcall), Py_READONLY, NULL},
+    {"__vectorcalloffset__", T_PYSSIZET, offsetof(NativeCall, vectorcall), READONLY, NULL},
     {NULL, 0, 0, 0, NULL},
 };
 

@@ -1,7 +1,9 @@
 """Arguments of the binding's calls: what ctypes refuses is refused, what it converts is converted the same way, and nothing
 reaches the library in another argument's place (no GPU needed: the called library is a stub that records its arguments)."""
 import ctypes
+import platform
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -14,10 +16,10 @@ WORDS = 18
 N = 5000
 
 
-@pytest.fixture(scope="module")
-def stub(tmp_path_factory):
-    """A library with the exported names, opened as a build of the product library; every function records what it gets."""
-    build.build_caller()
+@pytest.fixture(scope="module", params=["x86_64", "aarch64"])
+def stub(tmp_path_factory, request):
+    """A library with the exported names, opened as a build of the product library; every function records what it gets.
+    On a host that the native call path is not for, the binding calls through ctypes alone."""
     d = tmp_path_factory.mktemp("stub")
     args = ", ".join("W a%d" % k for k in range(WORDS))
     lines = ["typedef unsigned long long W;", "W seen[%d], called; float f_seen;" % WORDS]
@@ -29,7 +31,13 @@ def stub(tmp_path_factory):
             lines.append("int %s(void) { return 0; }" % name)
     (d / "s.c").write_text("\n".join(lines))
     subprocess.check_call(["gcc", "-O1", "-shared", "-fPIC", "-o", str(d / "s.so"), str(d / "s.c")])
-    return B.load_library(str(d / "s.so"))
+    with pytest.MonkeyPatch.context() as m:
+        m.setattr(platform, "machine", lambda: request.param)
+        if request.param != "x86_64":                # nothing is compiled or loaded there
+            m.setattr(subprocess, "check_call", None)
+            m.setitem(sys.modules, "paper_2110_15362_b200._pycall", None)
+        build.build_caller(force=request.param != "x86_64")
+        return B.load_library(str(d / "s.so"))
 
 
 @pytest.fixture
