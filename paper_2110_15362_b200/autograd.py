@@ -52,7 +52,8 @@ from . import build as _build
 try:
     from . import _autograd as _native
 except ImportError as e:
-    raise ImportError(f"{_build.AUTOGRAD_PATH} is missing: build it with `python -m paper_2110_15362_b200.build`") from e
+    raise ImportError(f"{_build.AUTOGRAD_PATH} is missing or does not load (built for torch {_build.autograd_built_for() or 'unknown'}, this is "
+                      f"{torch.__version__}): build it with `python -m paper_2110_15362_b200.build`") from e
 
 __all__ = ["PackedActivation", "stash_saved_activations", "relu_stash", "ReLUStash", "relu6_stash", "ReLU6Stash",
            "double_mask", "DoubleMask", "maxpool2x2_stash", "MaxPool2x2Stash", "relu_maxpool2x2_stash",

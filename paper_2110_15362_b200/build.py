@@ -17,6 +17,7 @@ CALLER_SRC = os.path.join(CSRC, "bt_pycall.c")
 CALLER_PATH = os.path.join(PKG_DIR, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 AUTOGRAD_SRC = os.path.join(CSRC, "bt_autograd.cpp")
 AUTOGRAD_PATH = os.path.join(PKG_DIR, "_autograd" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+AUTOGRAD_BUILT_FOR = os.path.join(PKG_DIR, "_autograd.built_for")      # the torch version that AUTOGRAD_PATH fits
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
@@ -54,12 +55,22 @@ def build_caller(force: bool = False) -> str:
     return CALLER_PATH
 
 
+def autograd_built_for() -> str:
+    """The torch version that the extension module of the autograd integration was built for ("" if unknown)."""
+    try:
+        with open(AUTOGRAD_BUILT_FOR) as f:
+            return f.read()
+    except FileNotFoundError:
+        return ""
+
+
 def build_autograd(force: bool = False) -> str:
-    """Compile the extension module of the autograd integration against torch's C++ headers; returns its path."""
-    newest = max(os.path.getmtime(f) for f in (AUTOGRAD_SRC, os.path.join(INCLUDE, "bittrain.h")))
-    if not force and os.path.exists(AUTOGRAD_PATH) and os.path.getmtime(AUTOGRAD_PATH) >= newest:
-        return AUTOGRAD_PATH
+    """Compile the extension module of the autograd integration against torch's C++ headers; returns its path.  It fits the
+    torch that it was built for only, whatever the age of the files."""
     import torch
+    newest = max(os.path.getmtime(f) for f in (AUTOGRAD_SRC, os.path.join(INCLUDE, "bittrain.h")))
+    if not force and os.path.exists(AUTOGRAD_PATH) and os.path.getmtime(AUTOGRAD_PATH) >= newest and autograd_built_for() == torch.__version__:
+        return AUTOGRAD_PATH
     from torch.utils import cpp_extension
     headers = cpp_extension.include_paths() + [os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
     tmp = AUTOGRAD_PATH + ".tmp%d" % os.getpid()
@@ -69,6 +80,8 @@ def build_autograd(force: bool = False) -> str:
                           + ["-L" + d for d in cpp_extension.library_paths()]
                           + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
     os.replace(tmp, AUTOGRAD_PATH)
+    with open(AUTOGRAD_BUILT_FOR, "w") as f:
+        f.write(torch.__version__)
     return AUTOGRAD_PATH
 
 
