@@ -40,6 +40,7 @@ those calls); a ReLU6 stash is never narrowed.
 """
 from __future__ import annotations
 
+import math
 import threading
 import weakref
 from typing import Dict, NamedTuple, Optional, Tuple
@@ -104,9 +105,26 @@ class PackedActivation:
 
     __slots__ = ("record", "values", "shape", "dtype", "device", "_nnz", "arena", "owner", "stored", "__weakref__")
 
-    def __init__(self, record: _Record, values, shape, dtype, device, nnz, arena=None, owner=None, stored=None):
+    def __init__(self, bitmap, values, chunk_prefix, shape, dtype, device, nnz, arena=None, offset=None, owner=None,
+                 stored=None):
+        """A stash made elsewhere: its bitmap and prefix array (arena mode: and the words nnz and offset) are copied."""
+        words = () if arena is None else (nnz, offset)
+        record = _Record(math.prod(shape), device, words=len(words))
+        record.bitmap.copy_(bitmap.view(torch.int32)[:record.bitmap.numel()])
+        record.chunk_prefix.copy_(chunk_prefix.view(torch.int64)[:record.chunk_prefix.numel()])
+        for k, word in enumerate(words):
+            record.word(k).copy_(word)
+        self._set(record, values, shape, dtype, device, nnz if arena is None else None, arena, owner, stored)
+
+    @classmethod
+    def of_record(cls, record: _Record, values, shape, dtype, device, nnz, arena=None, owner=None, stored=None):
+        packed = cls.__new__(cls)
+        packed._set(record, values, shape, dtype, device, nnz, arena, owner, stored)
+        return packed
+
+    def _set(self, record, values, shape, dtype, device, nnz, arena, owner, stored) -> None:
         self.record, self.values = record, values
-        self.shape, self.dtype, self.device, self._nnz = shape, dtype, device, nnz
+        self.shape, self.dtype, self.device, self._nnz = tuple(shape), dtype, device, nnz
         self.arena, self.owner = arena, owner
         self.stored = stored if stored is not None else (dtype if values is None else values.dtype)
 
@@ -343,11 +361,11 @@ def _compress_arena(x: torch.Tensor, owner, relu_into: Optional[torch.Tensor] = 
 
 
 def _packed(y: torch.Tensor, record: _Record, values, nnz) -> PackedActivation:
-    return PackedActivation(record, values, tuple(y.shape), y.dtype, y.device, nnz)
+    return PackedActivation.of_record(record, values, y.shape, y.dtype, y.device, nnz)
 
 
 def _packed_arena(y: torch.Tensor, record: _Record, owner, stored) -> PackedActivation:
-    return PackedActivation(record, None, tuple(y.shape), y.dtype, y.device, None, owner.arena, owner, stored)
+    return PackedActivation.of_record(record, None, y.shape, y.dtype, y.device, None, owner.arena, owner, stored)
 
 
 def _relu_bwd(bitmap: torch.Tensor, grad: torch.Tensor) -> torch.Tensor:

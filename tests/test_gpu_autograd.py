@@ -375,3 +375,32 @@ def test_relu_and_pooling_commuted_is_bit_identical(A, dtype):
         assert torch.equal(xs.grad.view(iv), xr.grad.view(iv))
     with pytest.raises(ValueError):
         A.relu_maxpool2x2_stash(torch.zeros(2, 3, 5, 4, device="cuda"))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("form", ["exact", "narrow", "arena"])
+def test_a_stash_made_elsewhere_is_shared_and_restored(A, form, dtype):
+    """PackedActivation of a stash that the caller made with the codec's own calls, with a bitmap that is a view at an odd word."""
+    x = torch.relu(torch.randn(7, 1003, device="cuda")).to(dtype)
+    n, stored = x.numel(), torch.float16 if form == "narrow" and dtype == torch.float32 else dtype
+    st, ws = B.Stash(n, stored), B.new_workspace(n)
+    bitmap = torch.empty((n + 31) // 32 + 1, dtype=torch.int32, device="cuda")[1:]
+    hooks = A.stash_saved_activations(min_numel=16, arena_bytes=1 << 20 if form == "arena" else None)
+    if form == "arena":
+        offset = torch.empty(1, dtype=torch.int64, device="cuda")
+        hooks.cursor.fill_(64)
+        B.bt_compress_arena(x, bitmap, hooks.arena, hooks.cursor, offset, st.chunk_prefix, st.nnz_out, ws, st.dev_status)
+        packed = A.PackedActivation(bitmap, None, st.chunk_prefix, tuple(x.shape), dtype, x.device, st.nnz_out, arena=hooks.arena, offset=offset,
+                                    owner=hooks, stored=stored)
+        assert int(packed.nnz) == st.nnz and int(packed.offset) == 64
+    else:
+        call = B.bt_compress if stored is dtype else B.bt_compress_narrow
+        call(x, bitmap, st.values, st.chunk_prefix, st.nnz_out, ws, st.dev_status)
+        packed = A.PackedActivation(bitmap, st.values, st.chunk_prefix, tuple(x.shape), dtype, x.device, st.nnz)
+        assert packed.nnz == st.nnz
+    assert packed.numel == n and packed.shape == (7, 1003) and packed.stored == stored and packed.nbytes() == B.bt_compressed_bytes(n, st.nnz, stored)
+    assert torch.equal(packed.bitmap, bitmap) and torch.equal(packed.chunk_prefix, st.chunk_prefix)
+    want = x if stored is dtype else x.to(stored).to(dtype)
+    assert torch.equal(packed.unpack(), want)
+    hooks.share(x, packed)
+    assert hooks._lookup(x) is packed
