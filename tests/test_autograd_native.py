@@ -121,18 +121,25 @@ def test_a_dropped_context_on_a_side_stream(mode):
     with hooks:
         A.relu_stash(x.detach(), hooks)                                  # the scratch buffers: the default stream's
     side = torch.cuda.Stream()
-    torch.cuda.synchronize()
     used = {t.data_ptr(): t.numel() * t.element_size() for t in (*hooks.scratch.kept, *hooks.scratch.ws.values(), *hooks.scratch.values.values())}
     assert len(used) == (3 if mode == "arena" else 2)
-    with torch.cuda.stream(side):
-        with hooks:
-            y = A.relu_stash(x * 1, hooks) * 2
-            z = (y * y).sum()
-        hooks.check_statuses()                                           # its host read here, not behind the pause
-        torch.cuda._sleep(400_000_000)
-        z.backward()
-    del hooks, y, z
-    taken = [torch.empty(size, dtype=torch.uint8, device="cuda") for size in used.values() for _ in range(4)]
+
+    def spare():
+        return [torch.empty(size, dtype=torch.uint8, device="cuda") for size in used.values() for _ in range(4)]
+    spare()                                                              # (device allocations would wait for the pause below)
+    for pause in (0, 400_000_000):
+        torch.cuda.synchronize()
+        x.grad = None
+        with torch.cuda.stream(side):
+            with hooks:
+                y = A.relu_stash(x * 1, hooks) * 2
+                z = (y * y).sum()
+            hooks.check_statuses()                                       # its host read here, not behind the pause
+            torch.cuda._sleep(pause)
+            z.backward()
+        del y, z
+    del hooks
+    taken = spare()
     assert not side.query()                                              # the backward pass is still to run
     assert not set(used) & {t.data_ptr() for t in taken}
     torch.cuda.synchronize()
