@@ -40,10 +40,11 @@ those calls); a ReLU6 stash is never narrowed.
 """
 from __future__ import annotations
 
+import collections
 import math
 import threading
 import weakref
-from typing import Dict, NamedTuple, Optional, Tuple
+from typing import Dict, Optional, Tuple
 
 import torch
 
@@ -221,48 +222,60 @@ class _Scratch:
         return t
 
 
-class _StatusWord(NamedTuple):
-    address: int
-    block: torch.Tensor
-    index: int
+class _StatusBlock:
+    SIZE = 64
+
+    __slots__ = ("words", "device", "address", "left")
+
+    def __init__(self, device):
+        self.words, self.device = torch.empty(self.SIZE, dtype=torch.int32, device=device), device
+        self.address, self.left = self.words.data_ptr(), iter(range(self.SIZE))
 
 
 class _StatusWords:
     """Device status words of the calls of a pass, handed out from blocks; fresh blocks after every check.  A word counts
-    once its call is made (nothing ever writes the word of a call that failed), and holds its block until then."""
-
-    BLOCK = 64
+    once its call is made (nothing ever writes the word of a call that failed), and holds its block until then.  Several
+    threads may take, list and read words: each step on the shared state is one indivisible operation."""
 
     def __init__(self):
-        self._lock = threading.Lock()
-        self._block: Optional[torch.Tensor] = None
-        self._used = 0
-        self._made: list = []
+        self._lock = threading.Lock()                    # for a new block
+        self._block: Optional[_StatusBlock] = None
+        self._made: collections.deque = collections.deque()
 
     def __bool__(self) -> bool:
         return bool(self._made)
 
-    def next(self, device) -> _StatusWord:
-        """A new word on `device`."""
-        with self._lock:
-            if self._block is None or self._used == self.BLOCK or self._block.device != device:
-                self._block, self._used = torch.empty(self.BLOCK, dtype=torch.int32, device=device), 0
-            k, block = self._used, self._block
-            self._used += 1
-        return _StatusWord(block.data_ptr() + 4 * k, block, k)
+    def next(self, device) -> Tuple[int, _StatusBlock, int]:
+        """A new word on `device`: its address, and where it lies."""
+        while True:
+            block = self._block
+            if block is not None and block.device == device:
+                k = next(block.left, None)
+                if k is not None:
+                    return block.address + 4 * k, block, k
+            with self._lock:
+                if self._block is block:
+                    self._block = _StatusBlock(device)
 
-    def made(self, word: _StatusWord) -> None:
+    def made(self, word: Tuple[int, _StatusBlock, int]) -> None:
         """The call that reports in `word` is on its stream."""
-        with self._lock:
-            self._made.append(word)
+        self._made.append(word)
 
     def drain(self) -> list:
         """The words of the calls made since the last time (one host read per block)."""
-        with self._lock:
-            made, self._made, self._block = self._made, [], None
-        blocks = {id(w.block): w.block for w in made}
-        read = {at: block.tolist() for at, block in blocks.items()}
-        return [read[id(w.block)][w.index] for w in made]
+        self._block = None
+        read: Dict[_StatusBlock, list] = {}
+        words = []
+        for _ in range(len(self._made)):
+            try:
+                _, block, k = self._made.popleft()
+            except IndexError:                           # another thread reads them too
+                break
+            words.append((block, k))
+        for block, _ in words:
+            if block not in read:
+                read[block] = block.words.tolist()
+        return [read[block][k] for block, k in words]
 
 
 class _HostWords(threading.local):
@@ -345,7 +358,7 @@ def _compress_arena(x: torch.Tensor, owner, relu_into: Optional[torch.Tensor] = 
     at = record.buf.data_ptr()
     words = at + _words_at(n)
     status = owner.statuses.next(dev)
-    tail = (at, arena, arena.numel(), owner.cursor, words + 8, at + _prefix_at(n), words, ws, ws.numel(), status.address,
+    tail = (at, arena, arena.numel(), owner.cursor, words + 8, at + _prefix_at(n), words, ws, ws.numel(), status[0],
             B._stream(None))
     code = B.DTYPE_CODE[narrow or x.dtype]
     if relu6:
@@ -499,7 +512,7 @@ class ReLUStash:
             statuses = hooks.loose_statuses if hooks is not None else _StatusWords()
             status = statuses.next(dev)
             st, y, _ = _native.relu_stash(x, address["bt_relu_fwd_compress"], bwd, _PLAIN, B.DTYPE_CODE[x.dtype], inplace, None, 0,
-                                          None, None, ws, ws.numel(), status.address)
+                                          None, None, ws, ws.numel(), status[0])
             B._check("bt_relu_fwd_compress (bitmap only)", st, True)
             statuses.made(status)
             if hooks is None:                           # BT_ERR_CAPACITY is the expected answer here
@@ -515,7 +528,7 @@ class ReLUStash:
             call = "bt_prune_fwd_compress_arena" if narrow is None else "bt_prune_fwd_compress_narrow_arena"
             status = hooks.statuses.next(dev)
             st, y, buf = _native.relu_stash(x, address[call], bwd, _ARENA, code, inplace, arena, arena.numel(), hooks.cursor, None,
-                                            ws, ws.numel(), status.address)
+                                            ws, ws.numel(), status[0])
             B._check("bt_*_arena (autograd stash)", st, True)
             hooks.statuses.made(status)
             hooks.share(y, _packed_arena(y, _Record(n, buf=buf), hooks, stored))

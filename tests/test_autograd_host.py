@@ -43,17 +43,17 @@ def test_a_call_that_fails_leaves_no_status_word(call, monkeypatch):
 
 def test_status_words_are_distinct_and_read_once_made():
     words = A._StatusWords()
-    taken = [words.next(torch.device("cpu")) for _ in range(3 * A._StatusWords.BLOCK + 5)]
-    assert len({w.address for w in taken}) == len(taken) and not words
+    taken = [words.next(torch.device("cpu")) for _ in range(3 * A._StatusBlock.SIZE + 5)]
+    assert len({w[0] for w in taken}) == len(taken) and not words
     for k, w in enumerate(taken):
-        w.block[w.index] = k
+        w[1].words[w[2]] = k
         if k % 3 == 0:
             words.made(w)
     assert words and sorted(words.drain()) == list(range(0, len(taken), 3)) and not words
     # a word handed out before a check and made after it still has its memory
     w = words.next(torch.device("cpu"))
     assert words.drain() == []
-    w.block[w.index] = 7
+    w[1].words[w[2]] = 7
     words.made(w)
     assert words.drain() == [7] and words.drain() == []
 
@@ -64,7 +64,7 @@ def test_status_words_of_several_threads():
     def take(base):
         for k in range(500):
             w = words.next(torch.device("cpu"))
-            w.block[w.index] = base + k
+            w[1].words[w[2]] = base + k
             words.made(w)
             if k % 50 == 49:
                 seen.extend(words.drain())
