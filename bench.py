@@ -9,12 +9,12 @@ gradient -- four launches per tensor on one stream, about 27 ms per step, so tha
 last half a second and the clock samples fall inside the timed region.  The metric
 is dense-equivalent GB/s: N * sizeof(dtype) per call, summed over the step, divided by the step time.
 
-The same JSON line carries, under roofline.kernels, every kernel of the five workload configurations
-timed on its own: CUDA events around ONE launch, the L2 flushed before it, median over repetitions --
-the single fp32 layer, the ResNet-18 step (batched launches), the sparsity sweep (i.i.d. and clustered),
-the VGG-16 tensors in bf16 and fp16 (fused forward with and without the dense output, backward), and the
-MobileNetV2 forward-then-reverse trace.  `roofline` itself is the row with the lowest fraction among
-the five graded calls on tensors of at least 256 MB.
+Before that JSON line, the only one on standard output, every kernel of the five workload configurations
+timed on its own goes to standard error, a JSON object per line: CUDA events around ONE launch, the L2
+flushed before it, median over repetitions -- the single fp32 layer, the ResNet-18 step (batched launches),
+the sparsity sweep (i.i.d. and clustered), the VGG-16 tensors in bf16 and fp16 (fused forward with and
+without the dense output, backward), and the MobileNetV2 forward-then-reverse trace.  `roofline` of the
+line is the row with the lowest fraction among the five graded calls on tensors of at least 256 MB.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
     python bench.py --case <f32|f16|bf16|f64> <op> [--log2n 26] [--zeros 0.5] [--reps 3]     # one kernel, for a profiler
@@ -710,6 +710,16 @@ def run_e2e(batch: Batch, steps: int = 3, warmup: int = 1, workers: int = 4):
             "workers": workers}
 
 
+def report(line: dict, rows: list) -> None:
+    """The line on standard output, the per-kernel rows on standard error: with its 163 rows the line took 47 KB, more than is
+    kept by a reader of the end of a program's output."""
+    for r in rows:
+        print(json.dumps(r), file=sys.stderr)
+    sys.stderr.flush()
+    line["roofline"]["rows_on_stderr"] = len(rows)
+    print(json.dumps(line), flush=True)
+
+
 def run_ours(args):
     import torch
     import torch.distributed as dist
@@ -778,16 +788,15 @@ def run_ours(args):
                                 "traffic": None if per_el is None else round(per_el * low["elements"]),
                                 "traffic_source": src,
                                 "how": "the lowest fraction among the five graded calls on tensors of at least 256 MB; "
-                                       "each row: CUDA events around one launch, L2 flushed before it, median of 9",
-                                "kernels": rows}
+                                       "each row: CUDA events around one launch, L2 flushed before it, median of 9"}
         else:
             # without the table: the headline tensor's own four kernels, timed one by one
             T = KernelTimer(dev, peak)
             codec_rows(T, B, "cfg3_iid", batch.x[0], batch.pre[0], batch.g, ZEROS, ops=("compress", "decompress", "fwd", "bwd"))
             low = min(T.rows, key=lambda r: r["frac_of_measured"])
             line["roofline"] = {"bound": "hbm", "kernel": low["kernel"], "dtype": "f32", "achieved": low["gbs"], "peak": peak,
-                                "unit": "GB/s", "frac": low["frac_of_measured"], "peak_kind": peak_kind, "traffic": None,
-                                "kernels": T.rows}
+                                "unit": "GB/s", "frac": low["frac_of_measured"], "peak_kind": peak_kind, "traffic": None}
+            rows = T.rows
         line.update(extras)
         if not args.no_e2e:
             e = run_e2e(batch)
@@ -807,7 +816,7 @@ def run_ours(args):
                                     "kind": "oracle", "seconds": round(sec, 2),
                                     "sample": "the first %d elements of one tensor of the batch (of %d), all four operations, "
                                               "single thread; host has %d cores" % (m, 1 << LOG2N, os.cpu_count())}
-        print(json.dumps(line))
+        report(line, rows)
     barrier()
     if world > 1:
         dist.destroy_process_group()

@@ -73,3 +73,14 @@ def test_default_arguments():
     assert (a.gpus, a.steps, a.warmup, a.impl) == (1, 20, 5, "ours") and a.case is None
     c = bench.parse_args(["--case", "bf16", "relu", "--log2n", "27"])
     assert c.case == ["bf16", "relu"] and c.log2n == 27
+
+
+def test_the_line_is_short_and_the_rows_are_on_stderr(capsys):
+    import json
+    rows = [{"kernel": "bt_relu_fwd_compress", "median_ms": 0.1 * k, "note": "x" * 80} for k in range(163)]
+    line = {"metric": bench.METRIC, "value": 1.0, "roofline": {"kernel": "bt_compress"}, "config": bench.workload_config()}
+    bench.report(line, rows)
+    out, err = capsys.readouterr()
+    assert out.count("\n") == 1 and len(out) < 4096
+    assert json.loads(out)["value"] == 1.0 and json.loads(out)["roofline"] == {"kernel": "bt_compress", "rows_on_stderr": 163}
+    assert [json.loads(x) for x in err.splitlines()] == rows
