@@ -25,7 +25,6 @@ namespace bt {
 // per word for the tag, and the repeated count on top.
 // Sized for the smallest tile, with 8 bytes per 4096 elements to spare: 24 bytes per 4096 elements.
 constexpr size_t   kWsHeaderBytes = 256;
-constexpr uint32_t kMinTileElems  = BT_CHUNK_ELEMS;
 constexpr uint32_t kMaxBatch      = 32;                        // tensors of one batched launch
 constexpr uint64_t kDefaultWaitNs = 2000000000ull;             // bound of every in-kernel wait: 2 s
 // bytes of workspace for tensors holding `chunks` 4096-element chunks in all
@@ -298,11 +297,6 @@ __device__ __forceinline__ void bulk_wait_read()
 {
     asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
-template <int N>
-__device__ __forceinline__ void bulk_wait_all()
-{
-    asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
-}
 
 __device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t *p)
 {
@@ -323,18 +317,7 @@ __device__ __forceinline__ void st_relaxed_2xu64(uint64_t *p, uint64_t w0, uint6
 {
     asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(w0), "l"(w1) : "memory");
 }
-__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p)
-{
-    uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_relaxed_u32(uint32_t *p, uint32_t v)
-{
-    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 
-__device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 __device__ __forceinline__ uint32_t lanemask_lt()
 {
     uint32_t m;

@@ -39,16 +39,6 @@ struct Pair<uint64_t> {
     __device__ static T make(uint64_t a, uint64_t b) { return make_ulonglong2(a, b); }
 };
 
-template <typename U>
-__device__ __forceinline__ void unpack16(const uint4 v, U (&e)[16 / sizeof(U)])
-{
-    if constexpr (sizeof(U) == 4) {
-        e[0] = v.x, e[1] = v.y, e[2] = v.z, e[3] = v.w;
-    } else {
-        e[0] = static_cast<U>(v.x), e[1] = static_cast<U>(v.x >> 16), e[2] = static_cast<U>(v.y), e[3] = static_cast<U>(v.y >> 16);
-        e[4] = static_cast<U>(v.z), e[5] = static_cast<U>(v.z >> 16), e[6] = static_cast<U>(v.w), e[7] = static_cast<U>(v.w >> 16);
-    }
-}
 // Two windows of 2-byte elements at once: A, B, C, D hold the two windows' elements (0,0), (0,1), (1,0), (1,1), one
 // window per half.  The comparison rule on packed pairs in the element's own type (an exact widening changes no
 // comparison); `code` receives the winner's position per half.
@@ -299,9 +289,8 @@ maxpool2x2_fwd_vec_kernel(const U *__restrict__ x, const uint64_t groups, const 
                                        __byte_perm(q.z, q.w, 0x7632), c1);
                 bits = __dp4a(c0, 0x00040001u, __dp4a(c1, 0x00400010u, 0u));
             } else {
-                U t[2 * kOut], b[2 * kOut], win[kOut];
-                unpack16<U>(top[u], t);
-                unpack16<U>(bot[u], b);
+                const U t[4] = {top[u].x, top[u].y, top[u].z, top[u].w}, b[4] = {bot[u].x, bot[u].y, bot[u].z, bot[u].w};
+                U       win[kOut];
 #pragma unroll
                 for (int j = 0; j < kOut; ++j) {
                     const U  e[4]  = {t[2 * j], t[2 * j + 1], b[2 * j], b[2 * j + 1]};
