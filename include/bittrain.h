@@ -113,7 +113,9 @@ size_t bt_workspace_bytes(uint64_t n);
  * the kernel) and every output is undefined; the workspace and the context
  * stay usable and the next call runs normally.  The kernel takes one CTA per
  * SM at most; with more tiles of 32 KB than CTAs it is launched cooperatively
- * (all its CTAs resident at once).
+ * (all its CTAs resident at once).  With no more tiles than CTAs it is a plain
+ * launch whose CTAs wait for CTAs of a lower index alone, which rests on CTAs
+ * being dispatched in the order of their index; the wait is bounded as well.
  */
 int bt_compress(const void *dense, uint64_t n, int dtype,
                 uint32_t *bitmap, void *values, uint64_t values_capacity,

@@ -1,6 +1,7 @@
 // What the single-tensor and the batched compress kernels share: constants of the workspace protocol, small PTX
-// wrappers, the bounded mbarrier wait, the in-place compaction of one segment by one warp, the copy-out of a
-// packed segment, and the host-side launch shape.
+// wrappers, the bounded mbarrier wait, the steps of a worker warp on a segment (into registers, flags, ranks, bitmap
+// words, survivors packed into the worker's own ring in shared memory, copy-out from there), the worker and the store
+// warp built of them, and the host-side launch shape.
 #pragma once
 
 #include <mutex>

@@ -91,7 +91,9 @@ decompress_body(const uint32_t *__restrict__ bitmap, const U *values, const uint
     }
 }
 
-constexpr int kWarps = 4;   // warps per CTA; twelve CTAs per SM: 42 registers at most
+// Warps per CTA.  The bound of twelve CTAs per SM keeps the registers at 42 at most.  Twelve fit with 4- and 8-byte elements
+// (17.6 and 17.1 KB of shared memory each); with 2-byte elements the table of words takes 18.6 KB, and eleven do.
+constexpr int kWarps = 4;
 
 template <typename U, int WIDEN = 0>
 __global__ void __launch_bounds__(kWarps * 32, 12)

@@ -118,7 +118,7 @@ cudaError_t launch_relu6_bwd(const uint32_t *bitmap, const void *values, const u
                              cudaStream_t stream)
 {
     // 64 bytes of gradient ahead per lane: 8 steps of 2-byte elements on 10 CTAs per SM ([61,144,57,55] bf16: 23.5 us; 4
-    // steps on 12 CTAs 27.1, 12 on 8 23.2, 16 on 8 23.8), 4 steps of wider ones on 8 (fp32 2^27: 197.8 us; 8 steps on 10
+    // steps on 11 CTAs 27.1, 12 on 8 23.2, 16 on 8 23.8), 4 steps of wider ones on 8 (fp32 2^27: 197.8 us; 8 steps on 10
     // CTAs 205.6, 2 on 12 204.4).  Gathered from global memory the two took 28.8 and 217.7 us.
     switch (dtype) {
     case BT_F64: return launch_typed<uint64_t, BT_F64, 4, 8>(bitmap, values, values_offset, prefix, gout, n, gin, stream);

@@ -11,7 +11,8 @@
 // elements came before the first element (restore of [64,128,112,112] bf16: 59 us with a quarter chunk per warp, 51 this
 // way).  4-byte elements: the gathered values of a quarter occupy 32 registers a lane until they arrive, which keeps 35
 // warps on an SM with two dependent round trips each (fp32 2^28 at half zeros: 266 us gathered from global memory, 243
-// this way; 2^27 at 90 % zeros 108 and 94; 200704 elements 4.2 and 2.3).  4096 bytes a warp keep 48 warps on an SM.
+// this way; 2^27 at 90 % zeros 108 and 94; 200704 elements 4.2 and 2.3).  4096 bytes a warp keep 48 warps on an SM (44 with
+// 2-byte elements, whose table is larger).
 #pragma once
 
 #include "bt_internal.cuh"
