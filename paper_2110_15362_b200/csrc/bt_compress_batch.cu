@@ -466,10 +466,18 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
 // tensor starts where the one that did not fit started, and that one's first values went there as well (its tiles leave
 // before its count is known), in no order.  Once the launch is complete they are gathered again, from the dense input under
 // the bitmap: a kept element is the input's own pattern, in the fused ReLU too, whose dense output may lie over the input.
-// Where everything fitted, as the counts and the cursor tell, there is nothing to do: a launch and two trips to L2
-// (52 layers of MobileNetV2 at batch 128, two launches and their restore: 1268.5 us without, 1271.7 with).  (Ordering the launch's own stores instead would take a published end of every CTA's copy-out, fences
-// included, in every launch.)
-constexpr int kAgainThreads = 256;
+//
+// Where everything fitted, as the counts and the cursor tell, there is nothing to do, and what it costs is a launch: 2 us
+// with few CTAs, 2.9 with one per SM (35 layers of MobileNetV2 at batch 1, two such launches: 39.0 us without, 43.1, 44.8).
+// So the CTAs go by the tiles of the launch, one per 64 and at least 8 (8 take 10 ms for 400 MB, one per SM 0.6).  Leave
+// to start early, given by the launch in front, costs 0.2 us more.  Ordering the launch's own stores instead would take a
+// published end of every CTA's copy-out, fences included, in every launch.
+constexpr uint32_t kAgainThreads = 256;
+inline uint32_t again_ctas(const uint64_t tiles, const uint32_t grid)
+{
+    const uint64_t n = tiles / 64 < 8 ? 8 : tiles / 64;
+    return n < grid ? static_cast<uint32_t>(n) : grid;
+}
 template <typename U, int kJobs>
 __global__ void __launch_bounds__(kAgainThreads) values_again_kernel(const __grid_constant__ CompressParams<kJobs> p)
 {
@@ -494,13 +502,26 @@ __global__ void __launch_bounds__(kAgainThreads) values_again_kernel(const __gri
             U *const           to   = reinterpret_cast<U *>(static_cast<unsigned char *>(p.c.arena) + at);
             const Extent       vx   = extent_of(to, count * sizeof(U));
             const uint64_t     step = static_cast<uint64_t>(gridDim.x) * (kAgainThreads / 32);
+            // a chunk per warp and turn, its bitmap words four per lane
             for (uint64_t ch = static_cast<uint64_t>(blockIdx.x) * (kAgainThreads / 32) + (threadIdx.x >> 5); ch * BT_CHUNK_ELEMS < j.n; ch += step) {
-                uint64_t rank = j.prefix[ch];
-                for (uint64_t e = ch * BT_CHUNK_ELEMS; e < j.n && e < (ch + 1) * BT_CHUNK_ELEMS; e += 32) {
-                    const uint32_t word = j.bitmap[e / 32];
-                    const uint64_t r    = rank + __popc(word & lanemask_lt());
-                    if (((word >> lane) & 1u) && e + lane < j.n && r < count && vx.holds(to + r, sizeof(U))) to[r] = src[e + lane];
-                    rank += __popc(word);
+                const uint64_t e0   = ch * BT_CHUNK_ELEMS + lane;
+                const uint4    w4   = load_words4(j.bitmap, ch * (BT_CHUNK_ELEMS / 32) + 4 * lane, (j.n + 31) >> 5);
+                uint64_t       rank = j.prefix[ch];
+#pragma unroll 2
+                for (uint32_t q = 0; q < 32; ++q) {
+                    const uint32_t w[4] = {__shfl_sync(kFull, w4.x, q), __shfl_sync(kFull, w4.y, q), __shfl_sync(kFull, w4.z, q), __shfl_sync(kFull, w4.w, q)};
+                    U              v[4];
+#pragma unroll
+                    for (uint32_t i = 0; i < 4; ++i) {
+                        const uint64_t e = e0 + 32 * (4 * q + i);
+                        v[i]             = ((w[i] >> lane) & 1u) && e < j.n ? src[e] : U(0);
+                    }
+#pragma unroll
+                    for (uint32_t i = 0; i < 4; ++i) {
+                        const uint64_t e = e0 + 32 * (4 * q + i), at_rank = rank + __popc(w[i] & lanemask_lt());
+                        if (((w[i] >> lane) & 1u) && e < j.n && at_rank < count && vx.holds(to + at_rank, sizeof(U))) to[at_rank] = v[i];
+                        rank += __popc(w[i]);
+                    }
                 }
             }
         }
@@ -555,7 +576,7 @@ cudaError_t launch_shaped(const CompressCommon &c, const CompressJob *jobs, uint
     // (with no more tiles than CTAs, CTA b takes descriptor b: what launch_waiting asks for)
     e = launch_waiting(tiles, kernel, grid, kThreads, kSmem, stream, p);
     if (e != cudaSuccess || p.c.arena == nullptr || count < 2) return e;
-    return launch(values_again_kernel<U, kJobs>, grid, kAgainThreads, 0, stream, p);
+    return launch(values_again_kernel<U, kJobs>, again_ctas(tiles, grid), kAgainThreads, 0, stream, p);
 }
 
 template <typename U, int FUSED, bool WRITE_Y>

@@ -276,7 +276,7 @@ def _pushes(counts, es, room, cursor0=0):
 
 
 # tiles of the tensor that does not fit, and of the ones behind it; `lead`: tensors in front
-FULL = {"one_behind": (1, [40], [1]), "many_tiles": (2, [400], [30, 2]), "fits_between": (1, [200, 3, 180], [2, 90]), "at_the_launch_edge": (31, [60], [1, 1]),
+FULL = {"one_behind": (1, [40], [1]), "many_tiles": (2, [400], [30, 2]), "more_ctas_behind": (1, [900], [300]), "fits_between": (1, [200, 3, 180], [2, 90]), "at_the_launch_edge": (31, [60], [1, 1]),
         "behind_the_launch_edge": (30, [60], [1, 50, 1])}
 
 
