@@ -65,7 +65,7 @@ NCU_DRAM_BYTES_PER_ELEMENT = {
     ("f32", "bt_compress"): (5.529, "profiles/bt_compress_ncu.md"),
     ("f32", "bt_relu_fwd_compress"): (5.529, "profiles/bt_compress_ncu.md (plain compressor; same kernel body)"),
     ("f32", "bt_decompress"): (5.277, "profiles/bt_staged_walk_ncu.md"),
-    ("f32", "bt_relu_bwd_from_bitmap"): (7.382, "an earlier capture of the same kernel (2^26 elements, ncu dram bytes)"),
+    ("f32", "bt_relu_bwd_from_bitmap"): (7.372, "profiles/bt_relu_bwd_ncu.md"),
 }
 
 

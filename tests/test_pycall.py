@@ -1,5 +1,6 @@
-"""The extension the binding calls the library through (csrc/bt_pycall.c): every kind of argument, in registers and on
-the stack, arrives where the called function expects it (no GPU needed: the called functions are compiled here)."""
+"""The extension the binding calls the library through (csrc/bt_pycall.c), functions wrapped without their parameters'
+kinds: every kind of argument, in registers and on the stack, arrives where the called function expects it (no GPU needed:
+the called functions are compiled here).  What a wrapped call of the library refuses: test_call_arguments.py."""
 import ctypes
 import subprocess
 
