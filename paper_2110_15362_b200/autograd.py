@@ -115,19 +115,18 @@ class PackedActivation:
         record.chunk_prefix.copy_(chunk_prefix.view(torch.int64)[:record.chunk_prefix.numel()])
         for k, word in enumerate(words):
             record.word(k).copy_(word)
-        self._set(record, values, shape, dtype, device, nnz if arena is None else None, arena, owner, stored)
+        made = PackedActivation.of_record(record, values, shape, dtype, device, nnz if arena is None else None, arena, owner, stored)
+        for name in PackedActivation.__slots__[:-1]:
+            setattr(self, name, getattr(made, name))
 
     @classmethod
     def of_record(cls, record: _Record, values, shape, dtype, device, nnz, arena=None, owner=None, stored=None):
-        packed = cls.__new__(cls)
-        packed._set(record, values, shape, dtype, device, nnz, arena, owner, stored)
-        return packed
-
-    def _set(self, record, values, shape, dtype, device, nnz, arena, owner, stored) -> None:
+        self = cls.__new__(cls)
         self.record, self.values = record, values
         self.shape, self.dtype, self.device, self._nnz = tuple(shape), dtype, device, nnz
         self.arena, self.owner = arena, owner
         self.stored = stored if stored is not None else (dtype if values is None else values.dtype)
+        return self
 
     @property
     def bitmap(self) -> torch.Tensor:
@@ -182,6 +181,9 @@ def _flat_input(t: torch.Tensor) -> torch.Tensor:
     return t if _usable(t) else t.clone(memory_format=torch.contiguous_format)
 
 
+_raw_stream = torch._C._cuda_getCurrentRawStream     # the handle of a device's current stream
+
+
 class _Scratch:
     """Per-device reusable buffers of the packing calls: workspace and a full-capacity values buffer.  `kept`: the context's
     own buffers.  All of them may be used on other streams than the one they were allocated on, and are given back as soon
@@ -194,9 +196,15 @@ class _Scratch:
         self.kept = kept
         self.streams: Dict[Tuple[int, int], torch.cuda.Stream] = {}      # those of the calls so far, by device and handle
         self.two_pass = two_pass         # exact-size values without a full-capacity buffer (see _compress)
+        # the workspace of the last call, the elements it serves, its device and the stream of that call (by handle)
+        self.last: tuple = (None, -1, None, 0, 0)
 
     def workspace(self, n: int, device) -> torch.Tensor:
-        if device.type == "cuda" and (device.index, torch._C._cuda_getCurrentRawStream(device.index)) not in self.streams:
+        ws, served, of, index, stream = self.last
+        if n <= served and device == of and _raw_stream(index) == stream:
+            return ws
+        cuda = device.type == "cuda"
+        if cuda and (device.index, _raw_stream(device.index)) not in self.streams:
             stream = torch.cuda.current_stream(device)
             self.streams[device.index, stream.cuda_stream] = stream
             for t in (*self.kept, *self.ws.values(), *self.values.values()):
@@ -205,7 +213,10 @@ class _Scratch:
         if self.ws_for.get(device, -1) < n:
             self.ws[device] = self._new(B.bt_workspace_bytes(n), torch.uint8, device)
             self.ws_for[device] = n
-        return self.ws[device]
+        ws = self.ws[device]
+        if cuda:
+            self.last = ws, self.ws_for[device], device, device.index, _raw_stream(device.index)
+        return ws
 
     def full_values(self, n: int, dtype, device) -> torch.Tensor:
         key = (device, dtype)
