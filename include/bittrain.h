@@ -112,10 +112,12 @@ size_t bt_workspace_bytes(uint64_t n);
  * gave up (two seconds without the data it waits for; every CTA then leaves
  * the kernel) and every output is undefined; the workspace and the context
  * stay usable and the next call runs normally.  The kernel takes one CTA per
- * SM at most; with more tiles of 32 KB than CTAs it is launched cooperatively
- * (all its CTAs resident at once).  With no more tiles than CTAs it is a plain
- * launch whose CTAs wait for CTAs of a lower index alone, which rests on CTAs
- * being dispatched in the order of their index; the wait is bounded as well.
+ * SM at most.  It is a plain launch of one CTA per tile of 32 KB, whose CTAs
+ * wait for tiles of a lower index alone, which rests on CTAs being handed out
+ * in the order of their index, to an SM or to a CTA that runs and takes the
+ * tile over; the wait is bounded as well.  Above 20 tiles per SM without a
+ * dense output, and under bt_set_max_ctas, it is launched cooperatively (all
+ * its CTAs resident at once).
  */
 int bt_compress(const void *dense, uint64_t n, int dtype,
                 uint32_t *bitmap, void *values, uint64_t values_capacity,
@@ -213,7 +215,7 @@ int bt_relu_bwd_from_bitmap_batch(const bt_batch_item *items /* host */, uint32_
 /*
  * Launch configuration for callers that keep several compress calls in flight
  * (on several streams, or in the branches of a CUDA graph).  The compress
- * kernel has at most one CTA per SM and, with more tiles than CTAs, is
+ * kernel fills the SMs with one CTA each, and from a size on (bt_compress) is
  * launched cooperatively; a cooperative launch starts only when all its CTAs
  * can be resident: two such launches of more
  * than half the SMs each therefore run one after the other, whatever their

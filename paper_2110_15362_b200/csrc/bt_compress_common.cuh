@@ -21,7 +21,8 @@ uint64_t compress_wait_ns();
 namespace cmp {
 
 constexpr uint32_t kFull       = 0xFFFFFFFFu;
-constexpr int      kMaxWindows = 5;                   // the grid never exceeds 32 * kMaxWindows CTAs
+constexpr int      kMaxWindows = 5;                   // 32 * kMaxWindows descriptors are read at a time (six: bf16 2^27 82.4 us, five: 80.1)
+constexpr uint32_t kMaxGrid    = 32 * kMaxWindows;    // CTAs that tiles are dealt to
 constexpr int      kHdrSeq     = 0;                   // header words (64-bit): launch sequence number,
 constexpr int      kHdrAbort   = 1;                   //   abort word (== the launch's tag once a wait ran out),
 constexpr int      kHdrCursor  = 2;                   //   batched arena form: the cursor as the launch found it, and
@@ -79,6 +80,7 @@ static __device__ __noinline__ void raise_timeout(uint64_t *ws_header, int32_t *
 // (-DBT_TEST_HOOKS) can set such a limit, and only that build carries the code for it: the product's waits
 // are the same instructions with or without it.
 constexpr uint64_t kStrictLimitNs = 1000;
+constexpr uint64_t kLastNs        = 20000000;         // the last wait for a copy that is in flight
 #ifdef BT_TEST_HOOKS
 constexpr bool kTestHooks = true;
 #else
@@ -470,6 +472,11 @@ __device__ __forceinline__ void copy_out_clipped(const uint32_t from, const uint
 // through five mbarriers: its ring slot through `full` and `empty` (forms with the dense output: `written` in between),
 // its place in the queue of the last kQueue tiles through `counted`, `ready` and `done`.
 constexpr int kQueue = 8;   // tiles of a CTA between their count and the end of their copy-out
+// The numbers of a CTA's last kTiles tiles.  The load warp writes the number of tile `it` once tile it - kStages is in
+// registers.  Every worker has then posted the counts up to tile it - 2 kStages, and so all is done with the tiles kQueue
+// before that one.
+constexpr int      kTiles  = 16;
+constexpr uint32_t kNoTile = 0xFFFFFFFFu;             // behind a CTA's last tile, kStages times
 template <int kSegs, int kStages>
 struct CtaState {
     uint64_t full[kStages];           // the bulk copy of the tile has landed               (copy engine -> workers)
@@ -477,28 +484,31 @@ struct CtaState {
                                       // or the dense output has left the slot              (store warp -> load warp)
     uint64_t written[kStages];        // the dense output is in the slot                    (workers -> store warp)
     uint64_t counted[kQueue];         // every segment's count is posted                    (workers -> scan warps)
-    uint64_t ready[kQueue];           // base and offsets are in shared                     (scan warps -> workers)
+    uint64_t ready[kQueue];           // base and offsets are in shared, the count is out   (scan, publishing warps -> workers)
     uint64_t done[kQueue];            // every segment has been copied out                  (workers -> workers)
     uint64_t base[kQueue];            // exclusive base of the tile
     uint64_t dst[kQueue];             // batched arena form: byte offset of the tile's tensor in the arena
     uint32_t job[kQueue];             // batched form: the tile's tensor
-    uint32_t agg[kQueue];             // packed count of the tile
     uint32_t cnt[kQueue][kSegs];      // packed count of each segment
     uint32_t off[kQueue][kSegs];      // exclusive offset of each segment in the tile
     uint32_t at[kQueue][kSegs];       // where in its worker's ring a segment's values start
-    volatile uint64_t tag;            // this launch's tag once a scan warp has it, else 0
+    uint32_t tile[kTiles];            // the tiles' numbers (kNoTile: the stream has ended)
+    __align__(16) uint64_t offer[2];  // the answer to the load warp's request for the tile of a CTA that has not started,
+    uint64_t offered;                 // and the barrier that it arrives on
+    volatile uint64_t tag;            // this launch's tag once the first scan warp has it, else 0
     uint64_t          arena_c0;       // arena forms: the cursor as the launch found it
     volatile uint32_t abort;
     // by the first threads of the CTA, one barrier each; a CTA-wide barrier follows
-    __device__ __forceinline__ void init(const bool dense_output, const uint32_t tid)
+    __device__ __forceinline__ void init(const bool dense_output, const bool publisher, const uint32_t tid)
     {
         if (tid == 0) abort = 0, tag = 0;
         if (tid < kStages) {
             mbar_init(&full[tid], 1), mbar_init(&empty[tid], dense_output ? 1 : kSegs), mbar_init(&written[tid], kSegs);
         } else if (tid - kStages < kQueue) {
             const uint32_t q = tid - kStages;
-            mbar_init(&counted[q], kSegs), mbar_init(&ready[q], 1), mbar_init(&done[q], kSegs);
+            mbar_init(&counted[q], kSegs), mbar_init(&ready[q], publisher ? 2 : 1), mbar_init(&done[q], kSegs);
         }
+        static_assert(2 * kStages + kQueue <= kTiles, "a tile's number outlives the tile");
         if (tid < kStages + kQueue) fence_proxy_async();
     }
 };
@@ -509,6 +519,186 @@ struct CtaState {
 struct Shape {
     static constexpr int kSegs = 8, kWorkers = 24, kStages = 3, kRing = 5376;
 };
+// Do the CTAs have a warp for publishing the counts (see scan_tiles)?
+template <typename U>
+constexpr bool kPublisher = sizeof(U) >= 4;
+// load warp, two scan warps, and as the form has them a publishing and a store warp
+template <typename U>
+constexpr int warps_of(const bool dense_output)
+{
+    return Shape::kWorkers + 3 + (kPublisher<U> ? 1 : 0) + (dense_output ? 1 : 0);
+}
+
+// A tile's descriptor: its count under the launch's tag, twice.
+__device__ __forceinline__ void post(uint64_t *desc, const uint32_t count, const uint64_t tag)
+{
+    st_relaxed_2xu64(desc, (tag & 0xFFFFFFFF00000000ull) | count, (tag << 32) | count);
+}
+
+// The launch's tag as the first scan warp left it in shared memory (bounded wait; 0 if the CTA is aborting).
+__device__ __forceinline__ uint64_t wait_tag(volatile uint64_t *s_tag, volatile uint32_t *s_abort, const uint64_t limit_ns)
+{
+    uint64_t t = *s_tag;
+    if (t) return t;
+    const uint64_t t0 = now_ns();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 32; ++i) {
+            t = *s_tag;
+            if (t) return t;
+        }
+        if (*s_abort || now_ns() - t0 > limit_ns) return 0;
+    }
+}
+
+// The counts in front of a tile, as a scan warp reads them: d0[k], d1[k], lane l <-> descriptor from + l + 32k.
+struct Window {
+    uint64_t d0[kMaxWindows], d1[kMaxWindows];
+    uint32_t from, size;
+    __device__ static __forceinline__ bool valid(const uint64_t w0, const uint64_t w1, const uint64_t tag)
+    {
+        return ((w0 ^ tag) >> 32) == 0 && ((w1 >> 32) ^ (tag & 0xFFFFFFFFull)) == 0 && static_cast<uint32_t>(w0) == static_cast<uint32_t>(w1);
+    }
+    // One batch of independent loads, from `from` on towards tile `to`.
+    __device__ __forceinline__ void read(const uint64_t *desc, const uint32_t to, const uint64_t tag, const uint32_t lane)
+    {
+        size = to - from < 32u * kMaxWindows ? to - from : 32u * kMaxWindows;
+#pragma unroll
+        for (int k = 0; k < kMaxWindows; ++k) {
+            if (lane + 32u * k < size) ld_relaxed_2xu64(desc + 2 * (static_cast<uint64_t>(from) + lane + 32u * k), d0[k], d1[k]);
+            else d0[k] = tag & 0xFFFFFFFF00000000ull, d1[k] = tag << 32;             // no such tile: a valid count of 0
+        }
+    }
+    // Polls until all are published.  False if the wait ran out or the launch is giving up.
+    __device__ __forceinline__ bool settle(const uint64_t *desc, const uint64_t *header, const uint64_t tag, const uint32_t lane, const uint32_t pause_ns,
+                                           const uint64_t wait_ns)
+    {
+        uint32_t polls = 0;
+        uint64_t t0    = 0;
+        for (;;) {
+            bool missing = false;
+#pragma unroll
+            for (int k = 0; k < kMaxWindows; ++k) missing |= !valid(d0[k], d1[k], tag);
+            if (!__any_sync(kFull, missing)) return true;
+            __nanosleep(pause_ns);
+            if ((++polls & 255u) == 0 || (kTestHooks && wait_ns < kStrictLimitNs)) {
+                if (t0 == 0) t0 = now_ns();
+                if (__any_sync(kFull, (now_ns() - t0 > wait_ns) || ld_relaxed_u64(header + kHdrAbort) == tag)) return false;
+            }
+#pragma unroll
+            for (int k = 0; k < kMaxWindows; ++k)
+                if (!valid(d0[k], d1[k], tag)) ld_relaxed_2xu64(desc + 2 * (static_cast<uint64_t>(from) + lane + 32u * k), d0[k], d1[k]);
+        }
+    }
+    // The sum of the counts (of those from tile lo to before hi): at most 160 tiles of 16384 elements.
+    __device__ __forceinline__ uint32_t sum() const
+    {
+        uint32_t part = 0;
+#pragma unroll
+        for (int k = 0; k < kMaxWindows; ++k) part += static_cast<uint32_t>(d0[k]);
+        return __reduce_add_sync(kFull, part);
+    }
+    __device__ __forceinline__ uint32_t sum(const uint32_t lo, const uint32_t hi, const uint32_t lane) const
+    {
+        uint32_t part = 0;
+#pragma unroll
+        for (int k = 0; k < kMaxWindows; ++k) {
+            const uint64_t at = static_cast<uint64_t>(from) + lane + 32u * k;
+            part += at >= lo && at < hi ? static_cast<uint32_t>(d0[k]) : 0u;
+        }
+        return __reduce_add_sync(kFull, part);
+    }
+};
+
+// A scan warp's tag: the first one makes it from the sequence number, which changes only once all counts of the launch are
+// published, or two seconds into a failure; a CTA publishes none before it has the tag.  0 if the CTA is aborting.
+template <int kSegs, int kStages>
+__device__ __forceinline__ uint64_t scan_tag(CtaState<kSegs, kStages> &sh, const uint32_t p, const uint32_t lane, const uint64_t call_tag,
+                                             const uint64_t *header, const uint64_t wait_ns)
+{
+    uint64_t tag = 0;
+    if (lane == 0) {
+        if (p == 0) sh.tag = tag = mix64(call_tag + ld_relaxed_u64(header + kHdrSeq) * 0x9E3779B97F4A7C15ull) | 1ull;
+        else tag = wait_tag(&sh.tag, &sh.abort, wait_ns);
+    }
+    return __shfl_sync(kFull, tag, 0);
+}
+
+// What the two scan warps of a CTA do.  Warp p takes the CTA's tiles p, p + 2, p + 4, ... (in the order the CTA takes them).
+// Its turn for the CTA's tile j:
+//   wait until tile j + 1 is counted -- about one tile later, when the tiles in front of tile j, taken at about the same
+//     time by other CTAs, are counted and published too -- and read, in ONE batch of independent loads, the descriptors
+//     from the CTA's tile j - 1 up to tile j.  2-byte types and dense tiles (11/16 and more survive), whose CTAs are further
+//     apart, read 0.1 us later, so that the first read usually finds everything: fp32 2^26 without zeros 94.1 -> 88.7 us,
+//     2^27 at 30 % zeros with the restore 290.9 -> 281.9, bf16 2^27 78.4 -> 76.8 (fp32 at 90 % zeros 51.6 and 51.8);
+//   wait until tile j + 2 is counted: the loads have arrived by then (the round trip to L2 takes 1.3 us under load).
+//     Handed to the workers as soon as the loads are there, bases come before the workers are through with the counting,
+//     and dense tensors, whose values then leave in smaller pieces, lose what sparse ones gain: fp32 2^26 without zeros
+//     103 us against 94, with 90 % zeros 53 against 54;
+//   finish tile j: its base is that of tile j - 1, which is the other scan warp's, plus the counts.
+// Each warp has two tiles' time for a turn.  What the workers wait for most is this exchange, not data (fp32 2^26 at half
+// zeros: a third of their time for bases, a tenth for tiles), so nothing else is done between the last wait and the base.
+//
+// Who publishes the counts.  All CTAs wait for every count, so nothing may hold it up.  4- and 8-byte types: a warp of its own
+// (publish_tiles).  2-byte types: the scan warps, in the wait for tile j + 2; their SMs are short of issue slots, and another
+// warp costs more than it gives (bf16 2^27 82.7 us against 81; fp32 2^26 with 90 % zeros 54 against 58 the other way).
+//
+// Stream: tile numbers and tensors.  Scan: what a kernel does with a tile,
+//   begin(tile, j)   what does not depend on the counts in front of it,
+//   resume(j)        the base of the CTA's tile before,
+//   add(window)      the counts from there on,
+//   finish(tile, j)  base and offsets for the workers, prefix entries; at a tensor's end nnz and status.
+// False if a wait ran out.
+template <typename U, bool LISTED, int kSegs, int kStages, typename Stream, typename Scan>
+__device__ __forceinline__ bool scan_tiles(CtaState<kSegs, kStages> &sh, const uint32_t p, const uint32_t lane, Stream &stream, Scan &scan,
+                                           const uint64_t *desc, const uint64_t *header, const uint64_t tag, const bool one_wave, const uint64_t wait_ns)
+{
+    auto counted = [&](const uint32_t j) { return mbar_wait(&sh.counted[j % kQueue], (j / kQueue) & 1u, &sh.abort, wait_ns); };
+    // waits until tile j is counted and publishes it; its number, or kNoTile behind the last one
+    auto next = [&](const uint32_t j, uint32_t &tile) {
+        tile = LISTED ? 0u : stream.dealt(j);
+        if (tile == kNoTile) return true;
+        if (!counted(j)) return false;
+        if constexpr (LISTED) tile = sh.tile[j % kTiles];
+        if constexpr (!kPublisher<U>) {
+            const uint32_t count = __reduce_add_sync(kFull, lane < kSegs ? sh.cnt[j % kQueue][lane] : 0u);
+            if (lane == 0 && tile != kNoTile) stream.publish(tile, count, tag);
+        }
+        return true;
+    };
+    uint32_t tile, after;
+    if (!next(p, tile)) return false;
+    for (uint32_t j = p; tile != kNoTile; j += 2, tile = after) {
+        uint32_t behind = LISTED ? 0u : stream.dealt(j + 1);
+        if (behind != kNoTile && !counted(j + 1)) return false;
+        if constexpr (LISTED) behind = sh.tile[(j + 1) % kTiles];
+        // The CTA's last tile: there is no next tile to wait for.  A short pause gives the counts in front of it
+        // time to land, so that the reads below usually succeed at once instead of costing a second
+        // round trip; a launch of one wave, whose counts come all at once, does not pause (fp32 200704
+        // elements 7.2 -> 6.7 us; 2.4 M elements, two waves: 9.9 -> 10.4 without the pause).
+        if (behind == kNoTile) __nanosleep(one_wave ? 20 : 300);
+        Window w;
+        w.from = j == 0 ? 0u : LISTED ? sh.tile[(j - 1) % kTiles] : tile - gridDim.x;
+        scan.begin(tile, j);
+        if (behind != kNoTile && (sizeof(U) == 2 || scan.count * 16u >= 11u * kSegs * Rows<U>::kSeg)) __nanosleep(100);
+        w.read(desc, tile, tag, lane);
+        after = kNoTile;
+        if (behind != kNoTile && !next(j + 2, after)) return false;
+        if (!w.settle(desc, header, tag, lane, one_wave ? 20 : 100, wait_ns)) return false;
+        if (j > 0 && !mbar_wait(&sh.ready[(j - 1) % kQueue], ((j - 1) / kQueue) & 1u, &sh.abort, wait_ns)) return false;
+        scan.resume(j);
+        // (a window is cut only where a CTA was slow or started late, behind a kernel that took its SM for a while)
+        for (;;) {
+            scan.add(w);
+            if (w.from + w.size == tile) break;
+            w.from += w.size;
+            w.read(desc, tile, tag, lane);
+            if (!w.settle(desc, header, tag, lane, 100, wait_ns)) return false;
+        }
+        scan.finish(tile, j);
+    }
+    return true;
+}
 
 // The tile a worker looks at, and where a tile's values go.
 struct TileIn {
@@ -521,6 +711,109 @@ struct TileOut {
     void    *values;
     uint64_t capacity;          // in values
 };
+
+// ---------------------------------------------------------------------------------------------
+// Which tiles a CTA takes (deal_of says when).  Stealing: the launch has one CTA per tile; a CTA that runs takes its own tile
+// first and then, while it works, those of CTAs that have not started (clusterlaunchcontrol.try_cancel), until none is
+// left.  Tiles are handed out in ascending order, so whoever waits for the counts of lower tiles waits for tiles that are
+// done or in the hands of CTAs that run: no CTA needs another one to be resident.  Else CTA b takes the tiles b, b + G, ...
+__device__ __forceinline__ void ask_for_tile(uint64_t (&offer)[2], uint64_t *bar)
+{
+    fence_proxy_async();                               // the answer before was read by an ordinary load
+    mbar_arrive_expect_tx(bar, 16);
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(smem_addr(offer)),
+                 "r"(smem_addr(bar))
+                 : "memory");
+}
+// kNoTile: refused.  No request may follow a refusal.
+__device__ __forceinline__ uint32_t offered_tile(const uint64_t (&offer)[2])
+{
+    uint32_t tile;
+    asm volatile(
+        "{\n\t.reg .b128 r;\n\t.reg .pred p;\n\t"
+        "ld.shared.b128 r, [%1];\n\t"
+        "mov.u32 %0, 0xFFFFFFFF;\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}"
+        : "=r"(tile)
+        : "r"(smem_addr(offer))
+        : "memory");
+    return tile;
+}
+
+// The first request goes out before the CTA waits for the kernel in front (by the load warp's lane).
+template <int kSegs, int kStages>
+__device__ __forceinline__ void ask_first(CtaState<kSegs, kStages> &sh)
+{
+    mbar_init(&sh.offered, 1);
+    ask_for_tile(sh.offer, &sh.offered);
+}
+
+// The load warp's lane: one bulk copy per tile into the ring, kStages tiles ahead of the workers at most.  One request for a
+// tile is under way at a time, so that a CTA's tiles ascend; its answer has a tile's time to arrive (two or four under way
+// are no faster: bf16 64 MiB with dense output 31.2 us, 31.5, 31.9).
+template <typename U, bool LISTED, int kSegs, int kStages, typename Stream>
+__device__ __forceinline__ void load_tiles(CtaState<kSegs, kStages> &sh, U *tiles, Stream &stream, const uint32_t num_tiles, const bool stealing,
+                                           const uint64_t wait_ns)
+{
+    constexpr uint32_t kTile = kSegs * Rows<U>::kSeg;
+    uint64_t tile = blockIdx.x;                        // 64-bit: running past the end cannot wrap
+    uint32_t it = 0, ends = 0, answers = 0;
+    bool     asked = stealing;
+    for (; ends < kStages; ++it) {
+        const uint32_t s = it % kStages;
+        if (it >= static_cast<uint32_t>(kStages) && !mbar_wait(&sh.empty[s], ((it / kStages) - 1) & 1u, &sh.abort, wait_ns)) break;
+        if (tile >= num_tiles) {
+            if (!LISTED) break;
+            sh.tile[it % kTiles] = kNoTile;
+            mbar_arrive(&sh.full[s]);
+            ++ends;
+            continue;
+        }
+        if (LISTED) sh.tile[it % kTiles] = static_cast<uint32_t>(tile);
+        TileIn t;
+        stream.locate(static_cast<uint32_t>(tile), t);
+        const uint64_t left  = t.n - t.first;
+        const uint32_t valid = left < static_cast<uint64_t>(kTile) ? static_cast<uint32_t>(left) : kTile;
+        const uint32_t bytes = (valid * static_cast<uint32_t>(sizeof(U))) & ~15u;   // whole 16-byte units
+        fence_proxy_async();                       // the workers' accesses to the slot come first
+        mbar_arrive_expect_tx(&sh.full[s], bytes);  // bytes == 0 simply completes the phase
+        if (bytes) bulk_load(tiles + static_cast<size_t>(s) * kTile, static_cast<const U *>(t.src) + t.first, bytes, &sh.full[s]);
+        if (!LISTED || !stealing) {
+            tile += gridDim.x;
+            continue;
+        }
+        const uint64_t before = tile;
+        tile                  = kNoTile;
+        if (asked) {
+            if (!mbar_wait(&sh.offered, answers & 1u, &sh.abort, wait_ns)) {
+                ++it;
+                break;
+            }
+            ++answers;
+            tile  = offered_tile(sh.offer);
+            asked = tile != kNoTile;
+            if (asked) ask_for_tile(sh.offer, &sh.offered);
+            if (tile <= before) {                  // not in ascending order: the launch gives up
+                sh.abort = 1u;
+                ++it;
+                break;
+            }
+        }
+    }
+    // This lane stays until everything it asked for has landed, whatever the other warps do (they may leave early once a
+    // bounded wait has run out somewhere): the CTA never retires with a copy into its shared memory in flight.  Behind the
+    // markers of the end all is in; before them, the last kStages copies can be pending.  A launch that gives up takes the
+    // CTAs that have not started with it, else each of them would wait anew.  Every wait is bounded.
+    if (ends == 0)
+        for (uint32_t i = it > static_cast<uint32_t>(kStages) ? it - kStages : 0; i < it; ++i)
+            mbar_wait<false>(&sh.full[i % kStages], (i / kStages) & 1u, &sh.abort, kLastNs);
+    while (asked && mbar_wait<false>(&sh.offered, answers & 1u, &sh.abort, kLastNs)) {
+        ++answers;
+        asked = offered_tile(sh.offer) != kNoTile;
+        if (asked) ask_for_tile(sh.offer, &sh.offered);
+    }
+}
 
 // One worker warp of a CTA (worker w of kWorkers): takes the segments w, w + kWorkers, w + 2 kWorkers, ... of the CTA's
 // stream of tiles -- into registers, flags, ranks, count posted, packed into its own ring in shared memory -- and copies
@@ -535,7 +828,7 @@ struct TileOut {
 // tiles up to t + 2 are counted, and a worker that waits for tile t has posted its segments of the tiles up to t + 2.
 // (After placing a segment of tile `it` it copies out what is left of tiles up to it - 3; a lack of room in its ring can
 // only make it wait for segments at least 2 tiles back, because the ring holds the segments nearer than that: kNear.)
-template <typename U, int FUSED, bool WRITE_Y, int CAST, int kSegs, int kWorkers, int kStages, int kRing, typename Stream>
+template <typename U, int FUSED, bool WRITE_Y, int CAST, bool LISTED, int kSegs, int kWorkers, int kStages, int kRing, typename Stream>
 __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, const uint32_t ring, const uint32_t w, const uint32_t lane,
                                      Stream &stream, const float tau, const uint64_t wait_ns, const bool pack)
 {
@@ -576,11 +869,16 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
         return true;
     };
 
-    TileIn t;
-    for (; stream.seek(it, t); next(it, seg)) {
+    for (TileIn t;; next(it, seg)) {
         const uint32_t s    = it % kStages, q = it % kQueue;
         U *const       tile = tiles + static_cast<size_t>(s) * kTile;
+        if (!LISTED && !stream.seek(it, t)) break;
         if (!mbar_wait(&sh.full[s], (it / kStages) & 1u, &sh.abort, wait_ns)) return false;
+        if constexpr (LISTED) {
+            const uint32_t number = sh.tile[it % kTiles];
+            if (number == kNoTile) break;
+            stream.locate(number, t);
+        }
         if (t.n - t.first < static_cast<uint64_t>(kTile)) {
             // Ragged last tile: each warp completes its own segment -- the elements of the last 16 bytes that the bulk copy
             // left out, zeros behind the end of the tensor -- and meets no other warp over it.  (A barrier among the workers
@@ -675,9 +973,42 @@ __device__ __forceinline__ bool work(CtaState<kSegs, kStages> &sh, U *tiles, con
         while (pending && o_it + 3 <= it)
             if (!copy_oldest()) return false;
     }
+    if constexpr (LISTED) {
+        // the end goes on to the scan and store warps like a tile (each worker has a segment in one of its markers)
+        const uint32_t s = it % kStages, q = it % kQueue;
+        if (it >= static_cast<uint32_t>(kQueue) && !mbar_wait(pack ? &sh.done[q] : &sh.ready[q], ((it / kQueue) - 1) & 1u, &sh.abort, wait_ns)) return false;
+        if (lane == 0) {
+            if constexpr (WRITE_Y) mbar_arrive(&sh.written[s]);
+            mbar_arrive(&sh.counted[q]);
+        }
+    }
     while (pending)
         if (!copy_oldest()) return false;
     return true;
+}
+
+// The publishing warp of the 4- and 8-byte types: sends a tile's count out to the other CTAs as soon as every segment is
+// counted.  Published by the worker that counts last, whose chain of steps that lengthens, bf16 2^27 takes 88 us instead of 78;
+// by the store warp, behind its wait for the copy engine, fp32 8 MiB with the dense output 7.2 instead of 5.7.  False if a
+// wait ran out.
+template <typename U, bool LISTED, int kSegs, int kStages, typename Stream>
+__device__ __forceinline__ bool publish_tiles(CtaState<kSegs, kStages> &sh, const uint32_t lane, Stream &stream, const uint64_t wait_ns)
+{
+    const uint64_t tag = wait_tag(&sh.tag, &sh.abort, wait_ns);
+    if (tag == 0) return false;
+    for (uint32_t it = 0;; ++it) {
+        const uint32_t q      = it % kQueue;
+        uint32_t       number = LISTED ? 0u : stream.dealt(it);
+        if (number == kNoTile) return true;
+        if (!mbar_wait(&sh.counted[q], (it / kQueue) & 1u, &sh.abort, wait_ns)) return false;
+        if constexpr (LISTED) number = sh.tile[it % kTiles];
+        if (number == kNoTile) return true;
+        const uint32_t count = __reduce_add_sync(kFull, lane < kSegs ? sh.cnt[q][lane] : 0u);
+        if (lane == 0) {
+            stream.publish(number, count, tag);
+            mbar_arrive(&sh.ready[q]);             // (until then the counts of the tile's segments stay)
+        }
+    }
 }
 
 // The store warp of the forms with the dense output: sends every tile off from its slot, whole 16-byte units by ONE bulk
@@ -689,10 +1020,13 @@ __device__ __forceinline__ bool store_dense(CtaState<kSegs, kStages> &sh, const 
 {
     constexpr uint32_t kTile = kSegs * Rows<U>::kSeg;
     TileIn t;
-    for (uint32_t it = 0; stream.seek(it, t); ++it) {
+    for (uint32_t it = 0;; ++it) {
         const uint32_t s    = it % kStages;
         const U *const tile = tiles + static_cast<size_t>(s) * kTile;
         if (!mbar_wait(&sh.written[s], (it / kStages) & 1u, &sh.abort, wait_ns)) return false;
+        const uint32_t number = sh.tile[it % kTiles];
+        if (number == kNoTile) return true;
+        stream.locate(number, t);
         const uint64_t left  = t.n - t.first;
         const uint32_t have  = left < kTile ? static_cast<uint32_t>(left) : kTile;
         const uint32_t whole = (have * static_cast<uint32_t>(sizeof(U))) & ~15u;
@@ -710,7 +1044,6 @@ __device__ __forceinline__ bool store_dense(CtaState<kSegs, kStages> &sh, const 
             mbar_arrive(&sh.empty[s]);
         }
     }
-    return true;
 }
 
 // Launch shape of one kernel instantiation on one device: the opt-in shared
@@ -742,6 +1075,37 @@ struct LaunchShape {
     }
 };
 
+// How a compressor of `tiles` tiles is launched.
+//   No more tiles than CTAs that fit: a CTA per tile.  A CTA waits for the counts of lower CTAs alone; those are dispatched
+//     first and retire without waiting for it (single-pass scans with look-back rest on that order as well; and the waits
+//     are bounded), so a plain launch will do.
+//   Stealing: a CTA per tile too, of which those that run take over the others' (load_tiles).  A plain launch, which takes the
+//     device 2.2 us less than a cooperative one, and a slow SM takes fewer tiles.  With the dense output at every size
+//     (f32 64 MiB 33.5 -> 30.2 us, 1 GiB 421 -> 416); without it up to kStealWaves tiles per CTA: beyond, the CTAs no longer read and
+//     write in step, which costs the DRAM more than the launch is worth (f32 8 MiB 8.2 us dealt out, 5.4 stolen; 64 MiB, 14 waves,
+//     23.7 and 22.6; 128 MiB, 28 waves, 40.2 and 40.9; 1 GiB 270 and 299; bf16 64 MiB 24.8 and 23.9, 128 MiB 44.5 and 44.8).
+//   Else, or under a limit on the CTAs that is in force: the tiles are dealt to CTAs that wait for one another and must be
+//     resident together: a cooperative launch, or an error.
+struct Deal {
+    uint32_t grid, resident, stealing;
+    bool     cooperative;
+};
+constexpr uint32_t kStealWaves = 20;
+template <typename Kernel>
+inline cudaError_t deal_of(const uint32_t tiles, const bool dense_output, Kernel dealt, Kernel listed, LaunchShape (&shapes)[2], const int threads,
+                           const size_t smem, Deal &d)
+{
+    int         resident = 0;
+    cudaError_t e        = shapes[0].max_grid(dealt, threads, smem, resident);
+    if (e != cudaSuccess) return e;
+    const uint32_t limit = compress_max_ctas(), all = static_cast<uint32_t>(resident) < kMaxGrid ? static_cast<uint32_t>(resident) : kMaxGrid;
+    const bool     limited = limit != 0 && limit < all;
+    d.resident = limited ? limit : all;
+    d.stealing = !limited && tiles > all && tiles <= 0x7FFFFFFFu && (dense_output || tiles <= kStealWaves * all);   // (a grid has fewer than 2^31 CTAs)
+    d.grid     = d.stealing || tiles < d.resident ? tiles : d.resident;
+    d.cooperative = tiles > d.grid;
+    return d.stealing ? shapes[1].max_grid(listed, threads, smem, resident) : cudaSuccess;
+}
 
 }  // namespace cmp
 }  // namespace bt

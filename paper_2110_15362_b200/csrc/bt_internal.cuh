@@ -53,6 +53,7 @@ struct CompressArgs {
     uint64_t   *values_offset_out;
     uint64_t    arena_bytes;
     uint64_t    n;
+    uint32_t    stealing;   // one CTA per tile, of which those that run take over the others' (set by launch_compress)
 };
 
 // One tensor of a batched launch.
@@ -69,8 +70,7 @@ struct CompressJob {
     uint64_t   *offset_out; // arena form: where the byte offset of the tensor's values in the arena goes
     // set by launch_compress_batch:
     uint32_t    tiles;      // number of tiles of the tensor
-    uint32_t    rot;        // the CTA that takes the tensor's tile 0 (tile t goes to CTA (rot + t) mod grid)
-    uint32_t    desc0;      // index of the tensor's first tile descriptor
+    uint32_t    desc0;      // number of the tensor's first tile (and of its descriptor): tiles are counted through the batch
 };
 
 // What the tensors of a batched launch share (all set by launch_compress_batch but tau).
@@ -81,6 +81,8 @@ struct CompressCommon {
     uint32_t    jobs;       // number of tensors
     uint64_t    call_tag;   // unique to the call
     uint64_t    wait_ns;    // bound of every in-kernel wait
+    uint32_t    tiles;      // of all tensors
+    uint32_t    stealing;   // one CTA per tile, of which those that run take over the others'
     float       tau;        // fused form: elements <= tau become +0 (0 for plain ReLU)
     // arena form (arena != nullptr): the tensors' values go back to back behind *arena_cursor
     void       *arena;
@@ -176,17 +178,6 @@ template <typename... P, typename... A>
 inline cudaError_t launch(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)
 {
     return launch_as(false, kernel, grid, threads, smem, stream, static_cast<A &&>(args)...);
-}
-// The compressors: CTAs that wait for counts of others.  With more tiles than CTAs a CTA waits for CTAs of a higher index
-// too, so all must be resident together: a cooperative launch, or an error.  With one tile per CTA it waits for CTAs of a
-// lower index alone.  Those are dispatched first and retire without waiting for it, so it needs no more than that order
-// (which single-pass scans with look-back rest on as well; and the waits are bounded).  Such a launch goes out as a plain
-// one: a cooperative launch takes the device 2.2 us longer and starts no earlier than the whole grid fits
-// (fp32 200704 elements 6.20 us cooperative, 4.09 plain; bf16 7.9 and 4.0).
-template <typename... P, typename... A>
-inline cudaError_t launch_waiting(uint64_t tiles, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, A &&...args)
-{
-    return launch_as(tiles > grid, kernel, grid, threads, smem, stream, static_cast<A &&>(args)...);
 }
 __device__ __forceinline__ void in_stream_order() { cudaGridDependencySynchronize(); }
 
