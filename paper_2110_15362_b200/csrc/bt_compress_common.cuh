@@ -802,12 +802,11 @@ __device__ __forceinline__ void load_tiles(CtaState<kSegs, kStages> &sh, U *tile
         }
     }
     // This lane stays until everything it asked for has landed, whatever the other warps do (they may leave early once a
-    // bounded wait has run out somewhere): the CTA never retires with a copy into its shared memory in flight.  Behind the
-    // markers of the end all is in; before them, the last kStages copies can be pending.  A launch that gives up takes the
-    // CTAs that have not started with it, else each of them would wait anew.  Every wait is bounded.
-    if (ends == 0)
-        for (uint32_t i = it > static_cast<uint32_t>(kStages) ? it - kStages : 0; i < it; ++i)
-            mbar_wait<false>(&sh.full[i % kStages], (i / kStages) & 1u, &sh.abort, kLastNs);
+    // bounded wait has run out somewhere): the CTA never retires with a copy into its shared memory in flight.  The last
+    // kStages copies can be pending, behind the first markers of the end too; a marker's phase is complete.  A launch that
+    // gives up takes the CTAs that have not started with it, else each of them would wait anew.  Every wait is bounded.
+    for (uint32_t i = it > static_cast<uint32_t>(kStages) ? it - kStages : 0; i < it; ++i)
+        mbar_wait<false>(&sh.full[i % kStages], (i / kStages) & 1u, &sh.abort, kLastNs);
     while (asked && mbar_wait<false>(&sh.offered, answers & 1u, &sh.abort, kLastNs)) {
         ++answers;
         asked = offered_tile(sh.offer) != kNoTile;

@@ -68,6 +68,34 @@ def test_wait_runs_out_then_workspace_is_reusable(hooks, oracle, kind, limit_ns)
     assert all(g.guards_intact() for g in (bitmap, values, prefix, nnz, status))
 
 
+@pytest.mark.parametrize("kind,limit_ns", [("f32", 0), ("f32", 50), ("f16", 20), ("f64", 100)])
+@pytest.mark.parametrize("tiles", [1, 3, 25, 148])
+def test_one_tile_per_cta_with_the_dense_output(hooks, oracle, kind, limit_ns, tiles):
+    """A CTA with one tile comes to the end of its stream with its only copy still under way; the first wait that runs out
+    there finds the end markers already in place.  It stays until the copy has landed all the same."""
+    n = tiles * 32768 // {"f32": 4, "f16": 2, "f64": 8}[kind] - 3
+    raws = [W.random_patterns(n, kind, 0.5, seed=60 + i) for i in range(2)]
+    x_a, x_b = (from_raw(r, kind) for r in raws)
+    ws, y = B.new_workspace(n), Guarded(n, x_a.dtype)
+    bitmap, values, prefix, nnz, status = _buffers(n, x_a.dtype)
+    status.inner.fill_(-1)
+    hooks.bt_test_set_wait_ns(limit_ns)
+    t0 = time.perf_counter()
+    for _ in range(20):                          # the CTAs of one launch take the place of those of the one before
+        rc = B.bt_relu_fwd_compress(x_a, y.inner, bitmap.inner, values.inner, prefix.inner, nnz.inner, ws, status.inner, check=False)
+        assert rc == B.BT_OK
+    torch.cuda.synchronize()
+    assert time.perf_counter() - t0 < 1.0 and int(status.inner.item()) == B.BT_ERR_TIMEOUT
+    hooks.bt_test_set_wait_ns(2_000_000_000)
+    B.bt_relu_fwd_compress(x_b, y.inner, bitmap.inner, values.inner, prefix.inner, nnz.inner, ws, status.inner)
+    torch.cuda.synchronize()
+    y_ref, c = oracle.relu_fwd_compress(raws[1], kind)
+    assert int(status.inner.item()) == B.BT_OK and int(nnz.inner.item()) == c.nnz
+    assert np.array_equal(bitmap.raw().view(np.uint32), c.bitmap) and np.array_equal(prefix.raw().view(np.uint64), c.prefix)
+    assert np.array_equal(values.raw()[:c.nnz], c.values) and np.array_equal(y.raw(), y_ref)
+    assert all(g.guards_intact() for g in (bitmap, values, prefix, nnz, status, y))
+
+
 def test_fused_and_batched_forms_time_out_cleanly(hooks, oracle):
     sizes = [8192 * 300 + 77, 5, 8192 * 40, 4096 * 3 + 1]
     raws = [W.random_patterns(n, "f16", 0.5, seed=50 + i) for i, n in enumerate(sizes)]
