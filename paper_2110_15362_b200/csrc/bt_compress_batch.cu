@@ -76,11 +76,6 @@ struct ManyTensors {
     }
     __device__ __forceinline__ void publish(const uint32_t tile, const uint32_t count, const uint64_t tag) const
     {
-        if (tile == 0 && p.c.arena != nullptr) {
-            // (before the launch's first count: whoever finishes its last tile has seen it)
-            st_relaxed_u64(p.c.ws_header + kHdrPushed, 0);
-            __threadfence();
-        }
         uint64_t *const d = p.c.ws_desc + 2 * static_cast<uint64_t>(tile);
         if (extent_of(p.c.ws_desc, 8 * p.c.ws_words).holds(d, 16)) post(d, count, tag);
     }
@@ -176,7 +171,7 @@ struct ManyScan {
                 *p.c.arena_cursor = fits ? at + ((nnz * sizeof(U) + 15) & ~15ull) : at;
                 __threadfence();
                 st_relaxed_u64(p.c.ws_header + kHdrCursor, sh.arena_c0);
-                if (!aborted) st_relaxed_u64(p.c.ws_header + kHdrPushed, 1);
+                if (!aborted) st_relaxed_u64(p.c.ws_header + kHdrPushed, tag);
             }
         }
         if (jb.dev_status) {
@@ -289,7 +284,9 @@ __global__ void __launch_bounds__(kAgainThreads) values_again_kernel(const __gri
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t nnz  = lane < p.c.jobs ? *p.job[lane].nnz_out : 0;
     const uint64_t at0  = p.c.ws_header[kHdrCursor];
-    if (p.c.ws_header[kHdrPushed] != 1) return;                     // a wait ran out: every output is undefined
+    // A launch that finished moved the sequence number by one, one that gave up by more (and may not have come to this word,
+    // which then holds an earlier launch's tag, beside that launch's cursor): every output of it is undefined.
+    if (p.c.ws_header[kHdrPushed] != tag_of(p.c.call_tag, p.c.ws_header[kHdrSeq] - 1)) return;
     const uint64_t all = warp_sum_u64((nnz * sizeof(U) + 15) & ~15ull);
     if (at0 <= p.c.arena_bytes && all <= p.c.arena_bytes - at0) return;
     uint64_t at      = at0;

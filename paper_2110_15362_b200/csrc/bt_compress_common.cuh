@@ -26,7 +26,7 @@ constexpr uint32_t kMaxGrid    = 32 * kMaxWindows;    // CTAs that tiles are dea
 constexpr int      kHdrSeq     = 0;                   // header words (64-bit): launch sequence number,
 constexpr int      kHdrAbort   = 1;                   //   abort word (== the launch's tag once a wait ran out),
 constexpr int      kHdrCursor  = 2;                   //   batched arena form: the cursor as the launch found it, and
-constexpr int      kHdrPushed  = 3;                   //   1 once its last tile is finished, 0 before
+constexpr int      kHdrPushed  = 3;                   //   its tag once its last tile is finished
 
 __device__ __forceinline__ uint64_t now_ns()
 {
@@ -61,6 +61,12 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t x)
     x *= 0x94D049BB133111EBull;
     x ^= x >> 31;
     return x;
+}
+
+// The tag of a launch that found the sequence number `seq` in its workspace (never 0).
+__device__ __forceinline__ uint64_t tag_of(const uint64_t call_tag, const uint64_t seq)
+{
+    return mix64(call_tag + seq * 0x9E3779B97F4A7C15ull) | 1ull;
 }
 
 // Raise the abort flag (shared, and global under this launch's tag if a scan warp got as far as reading it),
@@ -618,7 +624,7 @@ __device__ __forceinline__ uint64_t scan_tag(CtaState<kSegs, kStages> &sh, const
 {
     uint64_t tag = 0;
     if (lane == 0) {
-        if (p == 0) sh.tag = tag = mix64(call_tag + ld_relaxed_u64(header + kHdrSeq) * 0x9E3779B97F4A7C15ull) | 1ull;
+        if (p == 0) sh.tag = tag = tag_of(call_tag, ld_relaxed_u64(header + kHdrSeq));
         else tag = wait_tag(&sh.tag, &sh.abort, wait_ns);
     }
     return __shfl_sync(kFull, tag, 0);

@@ -158,3 +158,45 @@ def test_batched_arena_form_times_out_cleanly(hooks, oracle):
         assert np.array_equal(raw_arena[at:at + 4 * c.nnz].cpu().numpy().view(np.uint32), c.values)
         at += (4 * c.nnz + 15) // 16 * 16
     assert int(cursor.item()) == at and arena.guards_intact()
+
+
+def test_batch_that_times_out_leaves_earlier_stashes_alone(hooks, oracle):
+    """An arena batch that gives up may leave anything behind the cursor, but nothing in front of it: there lie the values
+    of calls that reported BT_OK.  Its counts are whatever the caller's memory held; here they are such that the second tensor
+    would fit behind a first one that does not, which is what the launch behind a batch looks for."""
+    sizes = [8192 * 160 + 5, 8192 * 140 + 1]
+    raws = [W.random_patterns(n, "f32", 0.5, seed=70 + i) for i, n in enumerate(sizes)]
+    xs = [from_raw(r, "f32") for r in raws]
+    new_stashes = lambda: [B.Stash(n, torch.float32, "cuda", values_capacity=1) for n in sizes]
+    first, second = new_stashes(), new_stashes()
+    refs = [oracle.compress(r) for r in raws]
+    step = [(4 * c.nnz + 15) // 16 * 16 for c in refs]
+    # room for the first batch and, behind it, for the second tensor of another one but not for the first
+    arena = Guarded((sum(step) + step[1] + 64) // 4, torch.float32)
+    assert step[0] > step[1] + 64
+    raw_arena = arena.inner.view(torch.uint8)
+    cursor = torch.zeros(1, dtype=torch.int64, device="cuda")
+    offsets = torch.zeros(len(sizes), dtype=torch.int64, device="cuda")
+    ws = torch.empty(B.bt_batch_workspace_bytes(sizes), dtype=torch.uint8, device="cuda")
+    B.bt_compress_arena_batch(B.batch_items(xs, first), torch.float32, raw_arena, cursor, offsets, ws)
+    torch.cuda.synchronize()
+    assert [st.status for st in first] == [B.BT_OK] * 2 and int(cursor.item()) == sum(step)
+    before = raw_arena[:sum(step)].clone()
+
+    for st, left in zip(second, (sum(sizes), 5000)):
+        st.nnz_out.fill_(left)
+        st.bitmap.fill_(-1)
+        st.chunk_prefix.zero_()
+    hooks.bt_test_set_wait_ns(30)
+    assert B.bt_compress_arena_batch(B.batch_items(xs, second), torch.float32, raw_arena, cursor, offsets, ws, check=False) == B.BT_OK
+    torch.cuda.synchronize()
+    assert second[0].status == B.BT_ERR_TIMEOUT and int(cursor.item()) == sum(step)
+    assert torch.equal(raw_arena[:sum(step)], before) and arena.guards_intact()
+
+    # and the launch behind a batch is back at work in the next one: the second tensor whole behind a first that does not fit
+    hooks.bt_test_set_wait_ns(2_000_000_000)
+    B.bt_compress_arena_batch(B.batch_items(xs, second), torch.float32, raw_arena, cursor, offsets, ws)
+    torch.cuda.synchronize()
+    assert [st.status for st in second] == [B.BT_ERR_CAPACITY, B.BT_OK] and int(offsets[1].item()) == sum(step)
+    assert np.array_equal(raw_arena[sum(step):sum(step) + 4 * refs[1].nnz].cpu().numpy().view(np.uint32), refs[1].values)
+    assert int(cursor.item()) == sum(step) + step[1] and torch.equal(raw_arena[:sum(step)], before) and arena.guards_intact()
