@@ -131,7 +131,7 @@ int compress_batch_common(const bt_batch_item *items, uint32_t count, int dtype,
             j.offset_out       = arena ? offsets_out + k : nullptr;
         }
         if (m == bt::kMaxBatch || (k + 1 == count && m > 0)) {
-            if (bt::launch_compress_batch(jobs, m, 0.0f, workspace, dtype, fused, arena, s) != cudaSuccess) return BT_ERR_CUDA;
+            if (bt::launch_compress_batch(jobs, m, workspace, dtype, fused, arena, s) != cudaSuccess) return BT_ERR_CUDA;
             m = 0;
         }
     }

@@ -257,7 +257,7 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
     }
 
     // ---------------------------------------------------------------- workers
-    if (!work<U, FUSED, WRITE_Y, 0, LISTED, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, p.c.tau, wait_ns, true) && lane == 0)
+    if (!work<U, FUSED, WRITE_Y, 0, LISTED, kSegs, kWorkers, kStages, kRing>(sh, tiles, packed + warp * kRing, warp, lane, stream, 0.0f, wait_ns, true) && lane == 0)
         raise_timeout(p, &sh.abort, sh.tag);
 }
 
@@ -390,17 +390,16 @@ cudaError_t launch_typed(const CompressCommon &c, const CompressJob *jobs, uint3
 
 }  // namespace
 
-cudaError_t launch_compress_batch(const CompressJob *jobs, uint32_t count, float tau, void *workspace, int dtype, int fused,
+cudaError_t launch_compress_batch(const CompressJob *jobs, uint32_t count, void *workspace, int dtype, int fused,
                                   const BatchArena *arena, cudaStream_t stream)
 {
-    // fused: 0 plain compressor, 1 threshold form (ReLU at tau = 0)
+    // fused: 0 plain compressor, 1 ReLU
     // the dense output is written for all tensors of a launch or for none
     if (count == 0 || count > kMaxBatch || fused > 1) return cudaErrorInvalidValue;
     const bool y = jobs[0].y != nullptr;
     for (uint32_t k = 1; k < count; ++k)
         if ((jobs[k].y != nullptr) != y) return cudaErrorInvalidValue;
     CompressCommon c{};
-    c.tau = tau;
     if (arena) {
         c.arena        = arena->arena;
         c.arena_bytes  = arena->arena_bytes;
@@ -411,31 +410,21 @@ cudaError_t launch_compress_batch(const CompressJob *jobs, uint32_t count, float
                : dtype == BT_F32 ? launch_typed<uint32_t, -1, false>(c, jobs, count, workspace, stream)
                                  : launch_typed<uint16_t, -1, false>(c, jobs, count, workspace, stream);
     }
-    if (tau == 0.0f && dtype != BT_F64) {
-        // the ReLU itself: decided by one compare in the element's own type (as in the single-tensor kernel)
-        constexpr int kd = kFusedReluDirect;
-        if (dtype == BT_F32)
-            return y ? launch_typed<uint32_t, kd + BT_F32, true>(c, jobs, count, workspace, stream)
-                     : launch_typed<uint32_t, kd + BT_F32, false>(c, jobs, count, workspace, stream);
-        if (dtype == BT_F16)
-            return y ? launch_typed<uint16_t, kd + BT_F16, true>(c, jobs, count, workspace, stream)
-                     : launch_typed<uint16_t, kd + BT_F16, false>(c, jobs, count, workspace, stream);
-        return y ? launch_typed<uint16_t, kd + BT_BF16, true>(c, jobs, count, workspace, stream)
-                 : launch_typed<uint16_t, kd + BT_BF16, false>(c, jobs, count, workspace, stream);
-    }
+    // the ReLU: for 2- and 4-byte types decided by one compare in the element's own type (as in the single-tensor kernel)
+    constexpr int kd = kFusedReluDirect;
     switch (dtype) {
     case BT_F64:
         return y ? launch_typed<uint64_t, BT_F64, true>(c, jobs, count, workspace, stream)
                  : launch_typed<uint64_t, BT_F64, false>(c, jobs, count, workspace, stream);
     case BT_F32:
-        return y ? launch_typed<uint32_t, BT_F32, true>(c, jobs, count, workspace, stream)
-                 : launch_typed<uint32_t, BT_F32, false>(c, jobs, count, workspace, stream);
+        return y ? launch_typed<uint32_t, kd + BT_F32, true>(c, jobs, count, workspace, stream)
+                 : launch_typed<uint32_t, kd + BT_F32, false>(c, jobs, count, workspace, stream);
     case BT_F16:
-        return y ? launch_typed<uint16_t, BT_F16, true>(c, jobs, count, workspace, stream)
-                 : launch_typed<uint16_t, BT_F16, false>(c, jobs, count, workspace, stream);
+        return y ? launch_typed<uint16_t, kd + BT_F16, true>(c, jobs, count, workspace, stream)
+                 : launch_typed<uint16_t, kd + BT_F16, false>(c, jobs, count, workspace, stream);
     default:
-        return y ? launch_typed<uint16_t, BT_BF16, true>(c, jobs, count, workspace, stream)
-                 : launch_typed<uint16_t, BT_BF16, false>(c, jobs, count, workspace, stream);
+        return y ? launch_typed<uint16_t, kd + BT_BF16, true>(c, jobs, count, workspace, stream)
+                 : launch_typed<uint16_t, kd + BT_BF16, false>(c, jobs, count, workspace, stream);
     }
 }
 

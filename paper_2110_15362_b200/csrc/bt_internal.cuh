@@ -73,7 +73,7 @@ struct CompressJob {
     uint32_t    desc0;      // number of the tensor's first tile (and of its descriptor): tiles are counted through the batch
 };
 
-// What the tensors of a batched launch share (all set by launch_compress_batch but tau).
+// What the tensors of a batched launch share (set by launch_compress_batch).
 struct CompressCommon {
     uint64_t   *ws_header;
     uint64_t   *ws_desc;    // tile descriptors
@@ -83,7 +83,6 @@ struct CompressCommon {
     uint64_t    wait_ns;    // bound of every in-kernel wait
     uint32_t    tiles;      // of all tensors
     uint32_t    stealing;   // one CTA per tile, of which those that run take over the others'
-    float       tau;        // fused form: elements <= tau become +0 (0 for plain ReLU)
     // arena form (arena != nullptr): the tensors' values go back to back behind *arena_cursor
     void       *arena;
     uint64_t    arena_bytes;
@@ -106,9 +105,9 @@ __host__ __device__ constexpr size_t batch_workspace_bytes(uint64_t chunks, uint
 // fused: 0 plain compressor, 1 threshold form (ReLU at tau = 0), 2 ReLU6
 cudaError_t launch_compress(const CompressArgs &a, int dtype, int fused, cudaStream_t s);
 // `jobs` (count of them: 1 .. kMaxBatch, every n > 0) are the tensors of one launch; `workspace` holds at least
-// batch_workspace_bytes() of their chunks; fused: 0 plain compressor, 1 threshold form; arena: nullptr, or the arena
+// batch_workspace_bytes() of their chunks; fused: 0 plain compressor, 1 ReLU; arena: nullptr, or the arena
 // the values go to (the jobs' values / capacity are then ignored and their offset_out must be set)
-cudaError_t launch_compress_batch(const CompressJob *jobs, uint32_t count, float tau, void *workspace, int dtype, int fused,
+cudaError_t launch_compress_batch(const CompressJob *jobs, uint32_t count, void *workspace, int dtype, int fused,
                                   const BatchArena *arena, cudaStream_t s);
 // the calling thread's limit on the CTAs of one compress launch (0: none); returns the limit it replaces
 uint32_t set_compress_max_ctas(uint32_t max_ctas);
