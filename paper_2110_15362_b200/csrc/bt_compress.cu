@@ -79,26 +79,17 @@ struct OneTensor {
 
 // What a scan warp of a single-tensor launch does with a tile (see scan_tiles).
 template <typename V, int kSegs, int kChunksPerTile, typename State>
-struct OneScan {
+struct OneScan : TileCounts<kSegs> {
     const CompressArgs &a;
     State              &sh;
     const uint32_t      num_tiles, lane;
     const uint64_t      tag;
-    uint32_t            own, upto;     // lane s: the count of the tile's segment s, and of its segments up to s
-    uint32_t            count;         // of the tile
     uint64_t            base;
-    __device__ __forceinline__ void begin(const uint32_t, const uint32_t j)
+    __device__ __forceinline__ OneScan(const CompressArgs &args, State &state, uint32_t tiles, uint32_t l, uint64_t t)
+        : a(args), sh(state), num_tiles(tiles), lane(l), tag(t)
     {
-        own  = lane < kSegs ? sh.cnt[j % kQueue][lane] : 0u;
-        upto = own;
-#pragma unroll
-        for (int o = 1; o < kSegs; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(kFull, upto, o);
-            if (lane >= static_cast<uint32_t>(o)) upto += u;
-        }
-        if (lane < kSegs) sh.off[j % kQueue][lane] = upto - own;
-        count = __shfl_sync(kFull, upto, kSegs - 1);
     }
+    __device__ __forceinline__ void begin(const uint32_t, const uint32_t j) { this->take(sh, j, lane); }
     __device__ __forceinline__ void resume(const uint32_t j) { base = j ? sh.base[(j - 1) % kQueue] : 0ull; }
     __device__ __forceinline__ void add(const Window &w) { base += w.sum(); }
     __device__ __forceinline__ void finish(const uint32_t tile, const uint32_t j)
@@ -109,14 +100,14 @@ struct OneScan {
         // exclusive count in front of each chunk of the tile
         if (lane < kSegs && (lane % kSegsPerChunk) == 0) {
             const uint64_t ch = static_cast<uint64_t>(tile) * kChunksPerTile + lane / kSegsPerChunk;
-            if (ch < chunks_total && extent_of(a.prefix, 8 * chunks_total).holds(a.prefix + ch, 8)) a.prefix[ch] = base + (upto - own);
+            if (ch < chunks_total && extent_of(a.prefix, 8 * chunks_total).holds(a.prefix + ch, 8)) a.prefix[ch] = base + (this->upto - this->own);
         }
         __syncwarp();
         if (lane != 0) return;
         sh.base[ps] = base;
         mbar_arrive(&sh.ready[ps]);                      // the tile's values may leave; what follows takes two trips to L2 and fences
         if (tile != num_tiles - 1) return;
-        const uint64_t nnz = base + count;
+        const uint64_t nnz = base + this->count;
         *a.nnz_out = nnz;
         // (the status word needs no look at the abort word here: it is looked at after the store, below)
         const bool aborted = a.arena_cursor && ld_relaxed_u64(a.ws_header + kHdrAbort) == tag;
@@ -154,7 +145,6 @@ __global__ void __launch_bounds__(warps_of<U>(WRITE_Y) * 32) compress_kernel(con
     constexpr int kSeg          = Rows<U>::kSeg;
     constexpr int kTile         = kSegs * kSeg;
     constexpr int kChunksPerTile = kTile / BT_CHUNK_ELEMS;
-    constexpr int kSegsPerChunk = BT_CHUNK_ELEMS / kSeg;
     // warp roles
     constexpr int kScanWarp = kWorkers;                   // and kScanWarp + 1
     constexpr int kLoadWarp = kWorkers + 2;               // and behind it a publishing and a store warp, as the form has them
@@ -170,7 +160,6 @@ __global__ void __launch_bounds__(warps_of<U>(WRITE_Y) * 32) compress_kernel(con
     const uint32_t lane = tid & 31u;
     // broadcast from lane 0 so that the compiler knows the role branches below are warp-uniform
     const uint32_t warp = __shfl_sync(kFull, tid >> 5, 0);
-    const uint64_t n    = a.n;
     const uint64_t wait_ns = a.wait_ns;          // bound of every wait below
 
     // The arena's cursor is read before the barrier below: the kernel's one update of it follows the last tile's base,
@@ -192,7 +181,7 @@ __global__ void __launch_bounds__(warps_of<U>(WRITE_Y) * 32) compress_kernel(con
         // ------------------------------------------------------------ scan warps
         const uint32_t p   = warp - kScanWarp;
         const uint64_t tag = scan_tag(sh, p, lane, a.call_tag, a.ws_header, wait_ns);
-        OneScan<Stored<CAST, U>, kSegs, kChunksPerTile, CtaState<kSegs, kStages>> scan{a, sh, num_tiles, lane, tag};
+        OneScan<Stored<CAST, U>, kSegs, kChunksPerTile, CtaState<kSegs, kStages>> scan(a, sh, num_tiles, lane, tag);
         if ((tag == 0 || !scan_tiles<U, LISTED>(sh, p, lane, stream, scan, a.ws_desc, a.ws_header, tag, num_tiles <= gridDim.x && !a.stealing, wait_ns)) && lane == 0)
             raise_timeout(a.ws_header, a.dev_status, &sh.abort, sh.tag);
         return;

@@ -93,29 +93,20 @@ struct ManyTensors {
 // What a scan warp of a batched launch does with a tile (see scan_tiles).  A window covers the tiles from the CTA's tile
 // before on, whatever tensors they belong to.
 template <typename U, int kSegs, int kChunksPerTile, int kJobs, typename State>
-struct ManyScan {
+struct ManyScan : TileCounts<kSegs> {
     const CompressParams<kJobs> &p;
     State                       &sh;
     const uint32_t               lane;
     const uint64_t               tag;
     uint32_t                     k = 0;         // the tile's tensor
-    uint32_t                     own, upto;     // lane s: the count of the tile's segment s, and of its segments up to s
-    uint32_t            count;         // of the tile
     uint32_t                     m;             // as far as add() has come: tensor m, `base` values of it, which start at
     uint64_t                     base, at;      // byte `at` of the arena
+    __device__ __forceinline__ ManyScan(const CompressParams<kJobs> &params, State &state, uint32_t l, uint64_t t) : p(params), sh(state), lane(l), tag(t) {}
     __device__ __forceinline__ bool in_arena() const { return p.c.arena != nullptr; }
     __device__ __forceinline__ void begin(const uint32_t tile, const uint32_t j)
     {
-        k    = tensor_of(p, k, tile);
-        own  = lane < kSegs ? sh.cnt[j % kQueue][lane] : 0u;
-        upto = own;
-#pragma unroll
-        for (int o = 1; o < kSegs; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(kFull, upto, o);
-            if (lane >= static_cast<uint32_t>(o)) upto += u;
-        }
-        if (lane < kSegs) sh.off[j % kQueue][lane] = upto - own;
-        count = __shfl_sync(kFull, upto, kSegs - 1);
+        k = tensor_of(p, k, tile);
+        this->take(sh, j, lane);
     }
     __device__ __forceinline__ void resume(const uint32_t j)
     {
@@ -148,7 +139,7 @@ struct ManyScan {
         // exclusive count in front of each chunk of the tile
         if (lane < kSegs && (lane % kSegsPerChunk) == 0) {
             const uint64_t ch = static_cast<uint64_t>(pt) * kChunksPerTile + lane / kSegsPerChunk;
-            if (ch < chunks_total && extent_of(jb.prefix, 8 * chunks_total).holds(jb.prefix + ch, 8)) jb.prefix[ch] = base + (upto - own);
+            if (ch < chunks_total && extent_of(jb.prefix, 8 * chunks_total).holds(jb.prefix + ch, 8)) jb.prefix[ch] = base + (this->upto - this->own);
         }
         __syncwarp();
         if (lane != 0) return;
@@ -157,7 +148,7 @@ struct ManyScan {
         sh.job[ps]  = k;
         mbar_arrive(&sh.ready[ps]);                      // the tile's values may leave; what follows takes two trips to L2 and fences
         if (pt != jb.tiles - 1) return;
-        const uint64_t nnz = base + count;
+        const uint64_t nnz = base + this->count;
         *jb.nnz_out        = nnz;
         // (the status word needs no look at the abort word here: it is looked at after the store, below)
         const bool aborted  = in_arena() && ld_relaxed_u64(p.c.ws_header + kHdrAbort) == tag;
@@ -199,7 +190,6 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
     constexpr int kSeg           = Rows<U>::kSeg;
     constexpr int kTile          = kSegs * kSeg;
     constexpr int kChunksPerTile = kTile / BT_CHUNK_ELEMS;
-    constexpr int kSegsPerChunk  = BT_CHUNK_ELEMS / kSeg;
     // warp roles
     constexpr int kScanWarp = kWorkers;                   // and kScanWarp + 1
     constexpr int kLoadWarp = kWorkers + 2;               // and behind it a publishing and a store warp, as the form has them
@@ -237,7 +227,7 @@ compress_kernel(const __grid_constant__ CompressParams<kJobs> p)
         // ------------------------------------------------------------ scan warps
         const uint32_t q   = warp - kScanWarp;
         const uint64_t tag = scan_tag(sh, q, lane, p.c.call_tag, p.c.ws_header, wait_ns);
-        ManyScan<U, kSegs, kChunksPerTile, kJobs, CtaState<kSegs, kStages>> scan{p, sh, lane, tag};
+        ManyScan<U, kSegs, kChunksPerTile, kJobs, CtaState<kSegs, kStages>> scan(p, sh, lane, tag);
         if ((tag == 0 || !scan_tiles<U, LISTED>(sh, q, lane, stream, scan, p.c.ws_desc, p.c.ws_header, tag, false, wait_ns)) && lane == 0)
             raise_timeout(p, &sh.abort, tag);
         return;

@@ -616,6 +616,27 @@ struct Window {
     }
 };
 
+// A tile's counts as a scan warp has them.
+template <int kSegs>
+struct TileCounts {
+    uint32_t own, upto;       // lane s: the count of the tile's segment s, and of its segments up to s
+    uint32_t count;           // of the tile
+    // from the counts of the CTA's tile j; leaves the segments' offsets in the tile for the workers
+    template <typename State>
+    __device__ __forceinline__ void take(State &sh, const uint32_t j, const uint32_t lane)
+    {
+        own  = lane < kSegs ? sh.cnt[j % kQueue][lane] : 0u;
+        upto = own;
+#pragma unroll
+        for (int o = 1; o < kSegs; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(kFull, upto, o);
+            if (lane >= static_cast<uint32_t>(o)) upto += u;
+        }
+        if (lane < kSegs) sh.off[j % kQueue][lane] = upto - own;
+        count = __shfl_sync(kFull, upto, kSegs - 1);
+    }
+};
+
 // A scan warp's tag: the first one makes it from the sequence number, which changes only once all counts of the launch are
 // published, or two seconds into a failure; a CTA publishes none before it has the tag.  0 if the CTA is aborting.
 template <int kSegs, int kStages>
