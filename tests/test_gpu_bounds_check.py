@@ -15,7 +15,7 @@ from paper_2110_15362_b200 import binding as B
 from tests import checking_libs as C
 from tests import gpu_util
 from tests import test_gpu_arena, test_gpu_batch, test_gpu_host_forms, test_gpu_mask, test_gpu_maxpool
-from tests import test_gpu_narrow, test_gpu_parity, test_gpu_prune, test_gpu_relu6
+from tests import test_gpu_narrow, test_gpu_parity, test_gpu_prune, test_gpu_relu6, test_gpu_tile_deal
 
 pytestmark = pytest.mark.gpu
 
@@ -39,6 +39,14 @@ def test_compress_and_decompress(checked, oracle, kind):
     test_gpu_parity.test_compress_decompress_edge_sizes(gpu_util, oracle, kind, RAGGED)
     test_gpu_parity.test_compress_decompress_edge_sizes(gpu_util, oracle, kind, 33)
     test_gpu_parity.test_compress_decompress_sparsity_levels(gpu_util, oracle, kind, 0.99)
+
+
+@pytest.mark.parametrize("kind", ["f32", "bf16", "f64"])
+def test_compress_beyond_twenty_waves(checked, oracle, kind):
+    n = 148 * 21 * (32768 // {"f32": 4, "bf16": 2, "f64": 8}[kind]) + 4097 + 13       # the kernel whose tiles are dealt out
+    test_gpu_parity.test_compress_decompress_edge_sizes(gpu_util, oracle, kind, n)
+    test_gpu_tile_deal.test_batch_beyond_twenty_waves(oracle, kind, False, False)
+    test_gpu_tile_deal.test_arena_batch_beyond_twenty_waves(oracle, kind)
 
 
 @pytest.mark.parametrize("kind", ["bf16", "f16"])

@@ -40,6 +40,39 @@ def test_two_streams_compress_concurrently(oracle, n):
             assert np.array_equal(W.raw_numpy(st.values[:c.nnz]), c.values)
 
 
+def test_two_streams_of_launches_that_need_every_sm(oracle):
+    """Launches of more than twenty waves of tiles are cooperative, one CTA per SM: from two streams they run one after the
+    other, interleaved with launches of a few waves that need no SM of their own."""
+    B.lib()
+    dev = torch.device("cuda")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    sizes = [8192 * sms * 21 + 77, 8192 * sms * 3 + 5]
+    raws = [[W.random_patterns(n, "f32", 0.5 + 0.1 * k, seed=93 + k) for n in sizes] for k in range(2)]
+    refs = [[oracle.compress(r) for r in rs] for rs in raws]
+    xs = [[torch.from_numpy(r.view(np.int32)).to(dev).view(torch.float32) for r in rs] for rs in raws]
+    reps = 6
+    stashes = [[[B.Stash(n, torch.float32, dev) for n in sizes] for _ in range(reps)] for _ in range(2)]
+    wss = [B.new_workspace(max(sizes), dev) for _ in range(2)]
+    torch.cuda.synchronize()
+    for rep in range(reps):
+        for i in range(2):
+            for k, s in enumerate(streams):
+                st = stashes[k][rep][i]
+                with torch.cuda.stream(s):
+                    B.bt_compress(xs[k][i], st.bitmap, st.values, st.chunk_prefix, st.nnz_out, wss[k], st.dev_status, stream=s)
+    torch.cuda.synchronize()
+    for k in range(2):
+        for i in range(2):
+            c = refs[k][i]
+            bitmap, prefix, values = (torch.from_numpy(a.view(np.int64 if a.dtype.itemsize == 8 else np.int32)).to(dev) for a in (c.bitmap, c.prefix, c.values))
+            for rep in range(reps):
+                st = stashes[k][rep][i]
+                assert st.status == B.BT_OK and st.nnz == c.nnz
+                assert torch.equal(st.bitmap, bitmap) and torch.equal(st.chunk_prefix, prefix)
+                assert torch.equal(st.values[:c.nnz].view(torch.int32), values)
+
+
 def test_graph_replays_share_one_workspace_across_sizes():
     """A captured graph of launches of different sizes and element types that share ONE workspace, replayed many
     times with the inputs changed in between: every replay's words in the workspace must be told from the
@@ -47,7 +80,8 @@ def test_graph_replays_share_one_workspace_across_sizes():
     B.lib()
     dev = torch.device("cuda")
     sizes = [(8192 * 300 + 11, torch.float32), (8192 * 3 + 5, torch.float32), (16384 * 200 + 3, torch.bfloat16),
-             (8192 * 149, torch.float32), (77, torch.float32), (4096 * 148 * 3 + 1, torch.float64)]
+             (8192 * 149, torch.float32), (77, torch.float32), (4096 * 148 * 3 + 1, torch.float64),
+             (16384 * 148 * 21 + 5, torch.bfloat16), (8192 * 148 * 21 + 9, torch.float32)]      # beyond 20 waves: dealt out
     xs = [torch.zeros(n, dtype=dt, device=dev) for n, dt in sizes]
     stashes = [B.Stash(n, dt, dev) for n, dt in sizes]
     ws = B.new_workspace(max(n for n, _ in sizes), dev)

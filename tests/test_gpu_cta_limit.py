@@ -92,3 +92,26 @@ def test_two_limited_launches_side_by_side_and_in_a_graph(oracle):
         assert np.array_equal(W.raw_numpy(st.bitmap).view(np.uint32), c.bitmap)
         assert np.array_equal(W.raw_numpy(st.chunk_prefix).view(np.uint64), c.prefix)
         assert np.array_equal(W.raw_numpy(st.values[:c.nnz]).view(np.uint32), c.values)
+
+
+@pytest.mark.parametrize("kind", ["f32", "bf16", "f64"])
+@pytest.mark.parametrize("want_y", [False, True])
+@pytest.mark.parametrize("kept", [(2688, 2688), (2688, 2704), (2704, 2688), (4096, 1280), (1280, 4096), (1296, 4096), (4096, 4096), (0, 4096), (16, 5360 // 2)])
+def test_packed_segments_that_just_fit_together(G, oracle, kind, want_y, kept):
+    """A worker packs 4096-byte segments into a ring of 5376 bytes, from either end in turn, and its segments are three tiles apart:
+    bytes kept of a segment alternate every three tiles of the one CTA, so that two fit exactly, or miss by a vector."""
+    es = {"f32": 4, "bf16": 2, "f64": 8}[kind]
+    per_seg, rng = 4096 // es, np.random.default_rng(sum(kept) + es)
+    x = np.zeros((17 * 8, per_seg), dtype={2: np.uint16, 4: np.uint32, 8: np.uint64}[es])
+    for s in range(x.shape[0]):
+        k = kept[s // 24 % 2] // es
+        x[s, rng.permutation(per_seg)[:k]] = rng.integers(1, 0x7C00, size=k)       # greater than zero in every type
+    x = x.reshape(-1)
+    y_ref, c = oracle.relu_fwd_compress(x, kind)
+    B.bt_set_max_ctas(1)
+    g = G.gpu_compress(G.from_raw(x, kind), relu=True, want_y=want_y)
+    assert g.guards_ok and g.status == B.BT_OK and g.nnz == c.nnz
+    assert np.array_equal(g.bitmap, c.bitmap) and np.array_equal(g.prefix, c.prefix)
+    assert np.array_equal(g.values.view(c.values.dtype), c.values)
+    if want_y:
+        assert np.array_equal(g.y, y_ref)

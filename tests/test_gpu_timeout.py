@@ -27,16 +27,22 @@ def hooks(monkeypatch):
     monkeypatch.setattr(B, "_lib", L)
     yield L
     L.bt_test_set_wait_ns(2_000_000_000)
+    B.bt_set_max_ctas(0)
 
 
+# How a launch's tiles are shared out: `ctas` 0: as its size has it; 74: dealt out to that many CTAs, a cooperative launch
 def _buffers(n, dtype, cap=None):
     return (Guarded((n + 31) // 32, torch.int32), Guarded(n if cap is None else cap, dtype),
             Guarded((n + 4095) // 4096, torch.int64), Guarded(1, torch.int64), Guarded(1, torch.int32))
 
 
 @pytest.mark.parametrize("kind,limit_ns", [("f32", 0), ("f32", 50), ("bf16", 100), ("f64", 50)])
-def test_wait_runs_out_then_workspace_is_reusable(hooks, oracle, kind, limit_ns):
+@pytest.mark.parametrize("waves,ctas", [(5, 0), (5, 74), (21, 0)])
+def test_wait_runs_out_then_workspace_is_reusable(hooks, oracle, kind, limit_ns, waves, ctas):
     n = 148 * 8192 * 5 + 4097 * 3 + 5          # several waves of tiles on every SM and a ragged tail
+    if waves > 20:                             # without the dense output: dealt out to a CTA per SM, a cooperative launch
+        n = 148 * (32768 // {"f32": 4, "bf16": 2, "f64": 8}[kind]) * waves + 4097 * 3 + 5
+    B.bt_set_max_ctas(ctas)
     raw_a = W.random_patterns(n, kind, 0.5, seed=41)
     raw_b = W.random_patterns(n, kind, 0.7, seed=42)
     x_a, x_b = from_raw(raw_a, kind), from_raw(raw_b, kind)
@@ -96,7 +102,9 @@ def test_one_tile_per_cta_with_the_dense_output(hooks, oracle, kind, limit_ns, t
     assert all(g.guards_intact() for g in (bitmap, values, prefix, nnz, status, y))
 
 
-def test_fused_and_batched_forms_time_out_cleanly(hooks, oracle):
+@pytest.mark.parametrize("ctas", [0, 74])
+def test_fused_and_batched_forms_time_out_cleanly(hooks, oracle, ctas):
+    B.bt_set_max_ctas(ctas)
     sizes = [8192 * 300 + 77, 5, 8192 * 40, 4096 * 3 + 1]
     raws = [W.random_patterns(n, "f16", 0.5, seed=50 + i) for i, n in enumerate(sizes)]
     xs = [from_raw(r, "f16") for r in raws]
@@ -125,38 +133,41 @@ def test_fused_and_batched_forms_time_out_cleanly(hooks, oracle):
         assert np.array_equal(y.raw(), y_ref) and y.guards_intact()
 
 
-def test_batched_arena_form_times_out_cleanly(hooks, oracle):
-    """The batched arena form has one more wait (a tensor's place in the arena comes from the tensor before it):
-    under a limit of a few nanoseconds the launch gives up by itself, and the next ordinary launch on the same
-    workspace and arena is the oracle's."""
+@pytest.mark.parametrize("ctas", [0, 74])
+@pytest.mark.parametrize("kind", ["f32", "bf16"])
+def test_batched_arena_form_times_out_cleanly(hooks, oracle, kind, ctas):
+    """The batched arena form under a limit of a few nanoseconds: the launch gives up by itself, and the next ordinary launch
+    on the same workspace and arena is the oracle's."""
+    B.bt_set_max_ctas(ctas)
+    es, dt = {"f32": (4, torch.float32), "bf16": (2, torch.bfloat16)}[kind]
     sizes = [8192 * 200 + 5, 8192 * 150, 4097, 8192 * 170 + 1]
-    raws = [W.random_patterns(n, "f32", 0.5, seed=90 + i) for i, n in enumerate(sizes)]
-    xs = [from_raw(r, "f32") for r in raws]
-    stashes = [B.Stash(n, torch.float32, "cuda", values_capacity=1) for n in sizes]
+    raws = [W.random_patterns(n, kind, 0.5, seed=90 + i) for i, n in enumerate(sizes)]
+    xs = [from_raw(r, kind) for r in raws]
+    stashes = [B.Stash(n, dt, "cuda", values_capacity=1) for n in sizes]
     items = B.batch_items(xs, stashes)
-    arena = Guarded(sum(sizes), torch.float32)
+    arena = Guarded(sum(sizes) + 3, dt)
     cursor = torch.zeros(1, dtype=torch.int64, device="cuda")
     offsets = torch.zeros(len(sizes), dtype=torch.int64, device="cuda")
     ws = torch.empty(B.bt_batch_workspace_bytes(sizes), dtype=torch.uint8, device="cuda")
 
     hooks.bt_test_set_wait_ns(30)
     t0 = time.perf_counter()
-    rc = B.bt_compress_arena_batch(items, torch.float32, arena.inner.view(torch.uint8), cursor, offsets, ws, check=False)
+    rc = B.bt_compress_arena_batch(items, dt, arena.inner.view(torch.uint8), cursor, offsets, ws, check=False)
     torch.cuda.synchronize()
     assert rc == B.BT_OK and time.perf_counter() - t0 < 1.0
     assert stashes[0].status == B.BT_ERR_TIMEOUT and arena.guards_intact()
 
     hooks.bt_test_set_wait_ns(2_000_000_000)
     cursor.zero_()
-    B.bt_compress_arena_batch(items, torch.float32, arena.inner.view(torch.uint8), cursor, offsets, ws)
+    B.bt_compress_arena_batch(items, dt, arena.inner.view(torch.uint8), cursor, offsets, ws)
     torch.cuda.synchronize()
     at = 0
     raw_arena = arena.inner.view(torch.uint8)
     for k, raw in enumerate(raws):
         c = oracle.compress(raw)
         assert stashes[k].status == B.BT_OK and stashes[k].nnz == c.nnz and int(offsets[k].item()) == at
-        assert np.array_equal(raw_arena[at:at + 4 * c.nnz].cpu().numpy().view(np.uint32), c.values)
-        at += (4 * c.nnz + 15) // 16 * 16
+        assert np.array_equal(raw_arena[at:at + es * c.nnz].cpu().numpy().view(raw.dtype), c.values)
+        at += (es * c.nnz + 15) // 16 * 16
     assert int(cursor.item()) == at and arena.guards_intact()
 
 
