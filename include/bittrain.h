@@ -115,9 +115,9 @@ size_t bt_workspace_bytes(uint64_t n);
  * SM at most.  It is a plain launch of one CTA per tile of 32 KB, whose CTAs
  * wait for tiles of a lower index alone, which rests on CTAs being handed out
  * in the order of their index, to an SM or to a CTA that runs and takes the
- * tile over; the wait is bounded as well.  Above 20 tiles per SM without a
- * dense output, and under bt_set_max_ctas, it is launched cooperatively (all
- * its CTAs resident at once).
+ * tile over; the wait is bounded as well.  Without a dense output above 28
+ * tiles per SM (2-byte types: 80; a batch: 20), and under bt_set_max_ctas, it
+ * is launched cooperatively (all its CTAs resident at once).
  */
 int bt_compress(const void *dense, uint64_t n, int dtype,
                 uint32_t *bitmap, void *values, uint64_t values_capacity,

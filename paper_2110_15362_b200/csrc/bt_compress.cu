@@ -218,10 +218,9 @@ uint64_t next_call_tag()
     return counter.fetch_add(1, std::memory_order_relaxed);
 }
 
-// The calling thread's limit on the CTAs of one compress launch (0: none).  A cooperative launch needs all its
-// CTAs resident at once and a CTA of this kernel fills an SM, so two launches of more than half the SMs each run
-// one after the other even on different streams; a caller that keeps several launches in flight gives each a
-// share of the SMs.
+// The calling thread's limit on the CTAs of one compress launch (0: none).  A launch of this kernel fills the SMs with one CTA
+// each, and a cooperative one (deal_of) starts only when all its CTAs can be resident, so two launches of more than half the
+// SMs each run one after the other even on different streams; a caller that keeps several in flight gives each a share of the SMs.
 thread_local uint32_t t_max_ctas = 0;
 uint32_t compress_max_ctas() { return t_max_ctas; }
 uint32_t set_compress_max_ctas(uint32_t max_ctas)
@@ -250,7 +249,7 @@ cudaError_t launch_shaped(const CompressArgs &a, cudaStream_t stream)
 
     const uint32_t num_tiles = static_cast<uint32_t>((a.n + kTile - 1) / kTile);
     Deal           deal;
-    cudaError_t    e = deal_of(num_tiles, WRITE_Y, dealt, listed, shapes, kThreads, kSmem, deal);
+    cudaError_t    e = deal_of(num_tiles, WRITE_Y, kStealWaves<U>, dealt, listed, shapes, kThreads, kSmem, deal);
     if (e != cudaSuccess) return e;
     CompressArgs args = a;
     args.call_tag     = next_call_tag();

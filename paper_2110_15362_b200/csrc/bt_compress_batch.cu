@@ -350,7 +350,7 @@ cudaError_t launch_shaped(const CompressCommon &c, const CompressJob *jobs, uint
     for (uint32_t k = count; k < static_cast<uint32_t>(kJobs); ++k) p.job[k] = CompressJob{};
 
     Deal        deal;
-    cudaError_t e = deal_of(static_cast<uint32_t>(tiles), WRITE_Y, dealt, listed, shapes, kThreads, kSmem, deal);
+    cudaError_t e = deal_of(static_cast<uint32_t>(tiles), WRITE_Y, kBatchStealWaves, dealt, listed, shapes, kThreads, kSmem, deal);
     if (e != cudaSuccess) return e;
     p.c.stealing = deal.stealing;
 

@@ -1097,18 +1097,25 @@ struct LaunchShape {
 //     are bounded), so a plain launch will do.
 //   Stealing: a CTA per tile too, of which those that run take over the others' (load_tiles).  A plain launch, which takes the
 //     device 2.2 us less than a cooperative one, and a slow SM takes fewer tiles.  With the dense output at every size
-//     (f32 64 MiB 33.5 -> 30.2 us, 1 GiB 421 -> 416); without it up to kStealWaves tiles per CTA: beyond, the CTAs no longer read and
-//     write in step, which costs the DRAM more than the launch is worth (f32 8 MiB 8.2 us dealt out, 5.4 stolen; 64 MiB, 14 waves,
-//     23.7 and 22.6; 128 MiB, 28 waves, 40.2 and 40.9; 1 GiB 270 and 299; bf16 64 MiB 24.8 and 23.9, 128 MiB 44.5 and 44.8).
+//     (f32 64 MiB 33.5 -> 30.2 us, 1 GiB 421 -> 416); without it up to `steal_waves` tiles per CTA: beyond, the CTAs no longer read
+//     and write in step, which costs the DRAM more than the launch is worth.  Dealt out and stolen, half zeros, us:
+//       f32 8 MiB 6.5 5.2, 64 21.3 20.2, 128 (28 waves) 37.1 36.1, 196 52.5 52.6 (2 % zeros 69.2 72.8), 256 65.8 66.3, 1 GiB 246 256;
+//       f64 128 MiB 35.9 34.8, 256 64.5 64.6, 1 GiB 235 244;
+//       bf16, whose kernel is bound by the SM before the DRAM, 128 MiB 42.1 38.5, 256 78.2 74.6, 384 (83 waves) 118.2 113.8 (2 % zeros
+//       149.1 148.9), 768 226.7 223.1 (30 % zeros 263.9 268.7), 1 GiB 294 292;
+//       batches, where a CTA looks for each tile's tensor: ResNet-18 f32 batch 16 (30 waves) 42.0 41.8, 32 73.9 77.5, bf16 batch 32
+//       (30 waves) 44.8 45.5, 64 81.5 85.2.
 //   Else, or under a limit on the CTAs that is in force: the tiles are dealt to CTAs that wait for one another and must be
 //     resident together: a cooperative launch, or an error.
 struct Deal {
     uint32_t grid, resident, stealing;
     bool     cooperative;
 };
-constexpr uint32_t kStealWaves = 20;
+template <typename U>
+constexpr uint32_t kStealWaves      = sizeof(U) == 2 ? 80 : 28;       // one tensor
+constexpr uint32_t kBatchStealWaves = 20;
 template <typename Kernel>
-inline cudaError_t deal_of(const uint32_t tiles, const bool dense_output, Kernel dealt, Kernel listed, LaunchShape (&shapes)[2], const int threads,
+inline cudaError_t deal_of(const uint32_t tiles, const bool dense_output, const uint32_t steal_waves, Kernel dealt, Kernel listed, LaunchShape (&shapes)[2], const int threads,
                            const size_t smem, Deal &d)
 {
     int         resident = 0;
@@ -1117,7 +1124,7 @@ inline cudaError_t deal_of(const uint32_t tiles, const bool dense_output, Kernel
     const uint32_t limit = compress_max_ctas(), all = static_cast<uint32_t>(resident) < kMaxGrid ? static_cast<uint32_t>(resident) : kMaxGrid;
     const bool     limited = limit != 0 && limit < all;
     d.resident = limited ? limit : all;
-    d.stealing = !limited && tiles > all && tiles <= 0x7FFFFFFFu && (dense_output || tiles <= kStealWaves * all);   // (a grid has fewer than 2^31 CTAs)
+    d.stealing = !limited && tiles > all && tiles <= 0x7FFFFFFFu && (dense_output || tiles <= steal_waves * all);   // (a grid has fewer than 2^31 CTAs)
     d.grid     = d.stealing || tiles < d.resident ? tiles : d.resident;
     d.cooperative = tiles > d.grid;
     return d.stealing ? shapes[1].max_grid(listed, threads, smem, resident) : cudaSuccess;

@@ -42,8 +42,8 @@ def test_compress_and_decompress(checked, oracle, kind):
 
 
 @pytest.mark.parametrize("kind", ["f32", "bf16", "f64"])
-def test_compress_beyond_twenty_waves(checked, oracle, kind):
-    n = 148 * 21 * (32768 // {"f32": 4, "bf16": 2, "f64": 8}[kind]) + 4097 + 13       # the kernel whose tiles are dealt out
+def test_compress_whose_tiles_are_dealt_out(checked, oracle, kind):
+    n = 148 * (test_gpu_tile_deal.LINE[kind] + 1) * (32768 // test_gpu_tile_deal.SIZE[kind]) + 4097 + 13
     test_gpu_parity.test_compress_decompress_edge_sizes(gpu_util, oracle, kind, n)
     test_gpu_tile_deal.test_batch_beyond_twenty_waves(oracle, kind, False, False)
     test_gpu_tile_deal.test_arena_batch_beyond_twenty_waves(oracle, kind)

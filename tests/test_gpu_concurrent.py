@@ -41,13 +41,13 @@ def test_two_streams_compress_concurrently(oracle, n):
 
 
 def test_two_streams_of_launches_that_need_every_sm(oracle):
-    """Launches of more than twenty waves of tiles are cooperative, one CTA per SM: from two streams they run one after the
+    """Launches of more than 28 waves of tiles are cooperative, one CTA per SM: from two streams they run one after the
     other, interleaved with launches of a few waves that need no SM of their own."""
     B.lib()
     dev = torch.device("cuda")
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
-    sizes = [8192 * sms * 21 + 77, 8192 * sms * 3 + 5]
+    sizes = [8192 * sms * 29 + 77, 8192 * sms * 3 + 5]
     raws = [[W.random_patterns(n, "f32", 0.5 + 0.1 * k, seed=93 + k) for n in sizes] for k in range(2)]
     refs = [[oracle.compress(r) for r in rs] for rs in raws]
     xs = [[torch.from_numpy(r.view(np.int32)).to(dev).view(torch.float32) for r in rs] for rs in raws]
@@ -81,7 +81,7 @@ def test_graph_replays_share_one_workspace_across_sizes():
     dev = torch.device("cuda")
     sizes = [(8192 * 300 + 11, torch.float32), (8192 * 3 + 5, torch.float32), (16384 * 200 + 3, torch.bfloat16),
              (8192 * 149, torch.float32), (77, torch.float32), (4096 * 148 * 3 + 1, torch.float64),
-             (16384 * 148 * 21 + 5, torch.bfloat16), (8192 * 148 * 21 + 9, torch.float32)]      # beyond 20 waves: dealt out
+             (16384 * 148 * 81 + 5, torch.bfloat16), (8192 * 148 * 29 + 9, torch.float32)]      # beyond 80 and 28 waves: dealt out
     xs = [torch.zeros(n, dtype=dt, device=dev) for n, dt in sizes]
     stashes = [B.Stash(n, dt, dev) for n, dt in sizes]
     ws = B.new_workspace(max(n for n, _ in sizes), dev)

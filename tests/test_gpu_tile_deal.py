@@ -1,6 +1,6 @@
 """How the compress launches share out their tiles: a CTA per tile up to one wave, tiles of CTAs that have not started taken
-over by those that run above it (always with the dense output, up to twenty waves without), dealt out beforehand to resident
-CTAs beyond that.  Sizes on both sides of every line, ragged last tiles, against the oracle; and launches that get
+over by those that run above it (always with the dense output; without it up to 28 waves, 80 of 2-byte types, 20 of a batch), dealt
+out beforehand to resident CTAs beyond that.  Sizes on both sides of every line, ragged last tiles, against the oracle; and launches that get
 the SMs late, because others on streams of their own hold them."""
 import numpy as np
 import pytest
@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
 
 TILE_BYTES = 32768
 SIZE = {"f32": 4, "bf16": 2, "f64": 8}
+LINE = {"f32": 28, "bf16": 80, "f64": 28}                        # waves of tiles of one tensor without the dense output
 
 
 @pytest.fixture(scope="module")
@@ -31,8 +32,9 @@ def _sms():
 
 @pytest.mark.parametrize("kind", ["f32", "bf16", "f64"])
 @pytest.mark.parametrize("want_y", [False, True])
-@pytest.mark.parametrize("waves,more", [(1, -1), (1, 0), (1, 1), (2, 1), (20, 0), (20, 1)])
+@pytest.mark.parametrize("waves,more", [(1, -1), (1, 0), (1, 1), (2, 1), (None, 0), (None, 1)])
 def test_lines_of_the_rule(G, oracle, kind, want_y, waves, more):
+    waves = waves or (20 if want_y else LINE[kind])
     tiles = waves * _sms() + more
     n = tiles * TILE_BYTES // SIZE[kind] - 1027                  # the last tile is ragged
     assert -(-n * SIZE[kind] // TILE_BYTES) == tiles
