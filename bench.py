@@ -54,16 +54,16 @@ CASE_OPS = ("compress", "relu", "relu_y", "prune", "narrow", "relu6", "relu6_bwd
 # little below the algorithmic bytes because the tail of what a launch writes is still in the L2 when it ends.
 # The capture and its command are summarised in the file named beside each figure.
 NCU_DRAM_BYTES_PER_ELEMENT = {
-    ("bf16", "bt_relu_fwd_compress"): (2.823, "profiles/bt_compress_ncu.md"),
-    ("f16", "bt_relu_fwd_compress"): (2.823, "profiles/bt_compress_ncu.md (bf16 capture; same kernel)"),
-    ("bf16", "bt_relu_fwd_compress+y"): (4.694, "profiles/bt_compress_ncu.md"),
-    ("f16", "bt_relu_fwd_compress+y"): (4.694, "profiles/bt_compress_ncu.md (bf16 capture; same kernel)"),
-    ("bf16", "bt_compress"): (2.823, "profiles/bt_compress_ncu.md (fused capture; same bytes)"),
-    ("f16", "bt_compress"): (2.823, "profiles/bt_compress_ncu.md (bf16 fused capture; same bytes)"),
+    ("bf16", "bt_relu_fwd_compress"): (2.830, "profiles/bt_compress_ncu.md"),
+    ("f16", "bt_relu_fwd_compress"): (2.830, "profiles/bt_compress_ncu.md (bf16 capture; same kernel)"),
+    ("bf16", "bt_relu_fwd_compress+y"): (4.709, "profiles/bt_compress_ncu.md"),
+    ("f16", "bt_relu_fwd_compress+y"): (4.709, "profiles/bt_compress_ncu.md (bf16 capture; same kernel)"),
+    ("bf16", "bt_compress"): (2.830, "profiles/bt_compress_ncu.md (fused capture; same bytes)"),
+    ("f16", "bt_compress"): (2.830, "profiles/bt_compress_ncu.md (bf16 fused capture; same bytes)"),
     ("bf16", "bt_decompress"): (2.708, "profiles/bt_staged_walk_ncu.md"),
     ("f16", "bt_decompress"): (2.708, "profiles/bt_staged_walk_ncu.md (bf16 capture; same kernel)"),
-    ("f32", "bt_compress"): (5.529, "profiles/bt_compress_ncu.md"),
-    ("f32", "bt_relu_fwd_compress"): (5.529, "profiles/bt_compress_ncu.md (plain compressor; same kernel body)"),
+    ("f32", "bt_compress"): (5.443, "profiles/bt_compress_ncu.md"),
+    ("f32", "bt_relu_fwd_compress"): (5.443, "profiles/bt_compress_ncu.md (plain compressor; same kernel body)"),
     ("f32", "bt_decompress"): (5.277, "profiles/bt_staged_walk_ncu.md"),
     ("f32", "bt_relu_bwd_from_bitmap"): (7.372, "profiles/bt_relu_bwd_ncu.md"),
 }
