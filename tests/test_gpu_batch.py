@@ -308,3 +308,43 @@ def test_arena_batch_values_behind_a_tensor_that_does_not_fit(oracle, kind, fuse
             if o is not None:
                 assert np.array_equal(arena[o:o + c.nnz * es].cpu().numpy().view(raw.dtype), c.values)
         assert bool((arena[:48] == 0x5A).all().item()) and bool((arena[room:] == 0x5A).all().item())
+
+
+@pytest.mark.parametrize("kind", ["f32", "bf16"])
+def test_arena_batch_replayed_from_a_graph(oracle, kind):
+    """A captured arena batch whose first tensor does not fit, replayed with other inputs: every replay has the same call's words in the
+    workspace and its own place in the sequence, and the tensors behind are whole in each."""
+    dt, es = TDT[kind], W.random_patterns(1, kind, 0.0, seed=0).dtype.itemsize
+    sizes = [8192 * 170 + 3, 8192 * 9 + 1, 5, 8192 * 2]
+    xs = [torch.zeros(n, dtype=dt, device="cuda") for n in sizes]
+    sts = [B.Stash(n, dt, values_capacity=1) for n in sizes]
+    items = B.batch_items(xs, sts)
+    arena = torch.zeros(8192 * 11 * es // 16 * 16, dtype=torch.uint8, device="cuda")
+    cursor = torch.zeros(1, dtype=torch.int64, device="cuda")
+    offsets = torch.zeros(len(sizes), dtype=torch.int64, device="cuda")
+    ws = torch.empty(B.bt_batch_workspace_bytes(sizes), dtype=torch.uint8, device="cuda")
+    ws.random_(0, 255)
+
+    def push():
+        cursor.zero_()
+        B.bt_compress_arena_batch(items, dt, arena, cursor, offsets, ws)
+
+    push()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        push()
+    for rep in range(6):
+        raws = [W.random_patterns(n, kind, 0.4, seed=800 + 10 * rep + k) for k, n in enumerate(sizes)]
+        for x, r in zip(xs, raws):
+            x.copy_(from_raw(r, kind))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert [st.status for st in sts] == [B.BT_ERR_CAPACITY] + [B.BT_OK] * 3
+        at = 0
+        for k, raw in list(enumerate(raws))[1:]:
+            c = oracle.compress(raw)
+            assert sts[k].nnz == c.nnz and int(offsets[k].item()) == at, (rep, k)
+            assert np.array_equal(arena[at:at + c.nnz * es].cpu().numpy().view(raw.dtype), c.values), (rep, k)
+            at += (c.nnz * es + 15) // 16 * 16
+        assert int(cursor.item()) == at
